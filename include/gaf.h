@@ -107,14 +107,13 @@ enum {
                                    wait on other CTAs is bounded: GAF_STATUS_TIMEOUT if it ever runs out
                                    (only when something else, another process say, keeps part of the
                                    device busy for seconds).
-                                   With K = 2 (the setting of the paper's experiments, Section 4) the
-                                   result is either the mean of both gradients or the seed alone, and
-                                   the first pass writes one of the two while it reads: the one the
-                                   latest two such calls on the same workspace both ended with (a word
-                                   in the workspace; a fresh workspace guesses "both"; no guess while
-                                   the latest two differ).  A call whose decision matches the guess
-                                   moves (2 b + 4) D bytes and has no second pass; one that does not
-                                   rewrites the output.  The values never depend on the guess.
+                                   Which gradients will be accepted is predicted inside the call from the
+                                   Gram sums of a sample of the elements, and the mean under that pattern is
+                                   written while the inputs are read for the full sums.  A call whose
+                                   decisions come out as predicted moves (K b + 4) D bytes and has no second
+                                   pass over the gradients; one that does not rewrites the output.  The
+                                   values never depend on the prediction.  (GAF_SCHED_GRAM with K <= 8
+                                   does the same; its second launch then has nothing to do.)
                                    GAF_SCHED_AUTO takes this form for K = 2 at every length. */
 };
 

@@ -171,6 +171,7 @@ size_t gram_partials_bytes(int K) {
     return pairs * kGramMaxSlices * 64 * sizeof(double);
 }
 size_t gram_matrix_bytes(int K) { return round_up(size_t(K) * K * sizeof(double), 256); }
+static_assert(size_t(36) * kFilterMaxCtas <= size_t(kGramMaxSlices) * 64, "the one-pass kernel's [pair][CTA] partial sums");
 // Bucketed variant: partial slots [ctas + buckets][64] doubles and one bit mask per bucket.
 size_t bucketed_extra_bytes() {
     return size_t(kBkMaxCtas + kBkMaxBuckets) * 64 * sizeof(double) + size_t(kBkMaxBuckets) * 8;
@@ -393,60 +394,11 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
     return cudaGetLastError() == cudaSuccess ? GAF_OK : GAF_ERR_CUDA;
 }
 
-template <typename T, int KT>
-int launch_gram_small_kt(GramSmallArgs a, const DeviceInfo &di, cudaStream_t st) {
-    // 7 or 8 bfloat16 gradients go through the warp-level tensor-core kernel (with fewer, the lanes of the
-    // absent rows fetch nothing and too few bytes are in flight: measured slower than the register tile)
-    constexpr bool kMma = std::is_same<T, __nv_bfloat16>::value && KT >= 7;
-    void (*kernel)(GramSmallArgs) = nullptr;
-    if constexpr (kMma) kernel = gram_mma_kernel<KT>;
-    else kernel = gram_small_kernel<T, KT>;
-    static PerDevice<OccPlan> table;
-    plan_once(table.plan[di.dev], table.ready[di.dev], [kernel](OccPlan &pl) {
-        int occ = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kGsThreads, 0) != cudaSuccess || occ < 1)
-            occ = 1;
-        pl.occ = occ > 2 ? 2 : occ;
-        return GAF_OK;
-    });
-    const int occ = table.plan[di.dev].occ;
-    int64_t grid = int64_t(di.sms) * occ;
-    if (grid > kGsMaxCtas) grid = kGsMaxCtas;
-    // elements one CTA consumes per trip of its loop
-    const int64_t per_cta = kMma ? int64_t(kGsThreads / 32) * kMmaTileElems * 2 : int64_t(kGsThreads) * GsVec<T>::N;
-    const int64_t work = (a.D + per_cta - 1) / per_cta;
-    if (grid > work) grid = work;
-    if (grid < 1) grid = 1;
-    // long vectors: runs of several trips per CTA (address-translation locality), once every CTA gets
-    // at least eight such runs; otherwise one trip at a time
-    a.mma_run = (kMma && a.D >= int64_t(8) * kMmaLongRun / 2 * per_cta * grid) ? kMmaLongRun : 2;
-    kernel<<<int(grid), kGsThreads, 0, st>>>(a);
-    ++g_launches;
-    return cudaGetLastError() == cudaSuccess ? GAF_OK : GAF_ERR_CUDA;
-}
-
-template <typename T>
-int launch_gram_small(const GramSmallArgs &a, int K, const DeviceInfo &di, cudaStream_t st) {
-    switch (K) {
-        case 2: return launch_gram_small_kt<T, 2>(a, di, st);
-        case 3: return launch_gram_small_kt<T, 3>(a, di, st);
-        case 4: return launch_gram_small_kt<T, 4>(a, di, st);
-        case 5: return launch_gram_small_kt<T, 5>(a, di, st);
-        case 6: return launch_gram_small_kt<T, 6>(a, di, st);
-        case 7: return launch_gram_small_kt<T, 7>(a, di, st);
-        case 8: return launch_gram_small_kt<T, 8>(a, di, st);
-        default: return GAF_ERR_ARG;
-    }
-}
-
 // One-launch form of the Gram-first schedule (gaf_fused.cuh).  Returns GAF_OK when it was
 // launched, GAF_ERR_UNSUPPORTED when this device or K does not allow it, or an error code.
 constexpr int kKeepL2Pct = 10;          // share of L2 the Gram pass asks to keep for the second pass
                                         // ("evict last" lines live in the persisting part of L2, 24.9 MB by
                                         // default on this GPU; larger shares slow both passes down)
-// Shared memory of one SM given to parked rounds.  The rest of the L1/shared array stays L1, which the
-// loads in flight need: beyond about 60 % shared memory both passes lose more than parking gains.
-constexpr int kParkBytesPerSm = 128 << 10;
 // AUTO takes the one-launch form for binary32 inputs up to this many bytes in all: beyond, what stays
 // on chip between the passes is a negligible share and the two-launch form is as fast or slightly
 // faster.  For bfloat16 with up to 6 gradients the one-launch form stays ahead at every length measured;
@@ -466,55 +418,56 @@ struct FusedGuard {
 };
 FusedGuard g_fused_guard[kMaxDevices];
 
+// Tiles, rounds and sample of gram_filter_kernel (one- and two-launch form alike: same sums, same order).
+#ifndef GAF_SAMPLE_SHORT
+#define GAF_SAMPLE_SHORT 2
+#endif
+#ifndef GAF_FILTER_RUN
+#define GAF_FILTER_RUN 1
+#endif
+template <typename T, int KT>
+int filter_shape(GramFusedArgs &a, const DeviceInfo &di, bool predict) {
+    using Tile = FilterTile<T, KT>;
+    // at least 256 elements per CTA; tiles cut so that all CTAs get the same number of equally long ones
+    int64_t grid = (a.D + 255) / 256;
+    if (grid > di.sms) grid = di.sms;
+    if (grid > kFilterMaxCtas) grid = kFilterMaxCtas;
+    if (grid < 1) grid = 1;
+    int64_t rounds = (a.D + grid * Tile::kElems - 1) / (grid * Tile::kElems);
+    if (rounds < 1) rounds = 1;
+    const int64_t te = (a.D + grid * rounds - 1) / (grid * rounds);
+    a.tile_elems = int((te + 63) / 64 * 64);
+    if (a.tile_elems < 64) a.tile_elems = 64;
+    a.run = rounds >= 256 ? GAF_FILTER_RUN : 1;
+    a.rounds = int((rounds + a.run - 1) / a.run * a.run);
+    a.sample = 0;
+    if (predict && a.rounds > Tile::kStages) a.sample = a.rounds < 64 ? GAF_SAMPLE_SHORT : Tile::kStages / 2;
+    return int(grid);
+}
+
+// Shared-memory attributes of one instantiation, once per device; GAF_ERR_UNSUPPORTED when no CTA of it fits an SM.
+template <typename T, int KT, bool ONE>
+int filter_plan(const DeviceInfo &di) {
+    static PerDevice<DynSmemPlan> table;
+    return plan_once(table.plan[di.dev], table.ready[di.dev], [&](DynSmemPlan &pl) {
+        auto kernel = gram_filter_kernel<T, KT, ONE>;
+        pl.dyn = FilterTile<T, KT>::kStages * FilterTile<T, KT>::kBytes;
+        if (pl.dyn > di.smem_per_cta_max) return GAF_ERR_UNSUPPORTED;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.dyn) != cudaSuccess) return GAF_ERR_CUDA;
+        int occ = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kFilterThreads, pl.dyn) != cudaSuccess || occ < 1)
+            return GAF_ERR_UNSUPPORTED;
+        return GAF_OK;
+    });
+}
+
 template <typename T, int KT>
 int launch_gram_fused_kt(GramFusedArgs &a, const DeviceInfo &di, cudaStream_t st) {
-    auto kernel = gram_fused_kernel<T, KT>;
-    // The plan of this instantiation on this device: CTAs per SM by registers alone, then as many parked
-    // rounds as shared memory allows; the kernel's shared-memory attributes are set on the way.
-    static PerDevice<FusedPlan> table;
-    if (int rc = plan_once(table.plan[di.dev], table.ready[di.dev], [&](FusedPlan &pl) {
-            int occ = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kGsThreads, 0) != cudaSuccess || occ < 1)
-                return GAF_ERR_UNSUPPORTED;
-            if (occ > 2) occ = 2;
-            cudaFuncAttributes fa{};
-            if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return GAF_ERR_CUDA;
-            const int round_bytes = KT * kGsThreads * 16;
-            int64_t budget = di.smem_per_sm / occ - 1024 - int64_t(fa.sharedSizeBytes);
-            if (budget > di.smem_per_cta_max - int64_t(fa.sharedSizeBytes))
-                budget = di.smem_per_cta_max - int64_t(fa.sharedSizeBytes);
-            if (budget > kParkBytesPerSm / occ) budget = kParkBytesPerSm / occ;
-            const int park = budget > 0 ? int(budget / round_bytes) : 0;
-            const int dyn = park * round_bytes;
-            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) != cudaSuccess)
-                return GAF_ERR_CUDA;
-            // shared memory share of the L1/shared array: what the CTAs of one SM need, no more (the rest is L1)
-            int pct = int((int64_t(dyn + fa.sharedSizeBytes + 1024) * occ * 100 + di.smem_per_sm - 1) / di.smem_per_sm);
-            if (pct > 100) pct = 100;
-            if (cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, pct) != cudaSuccess)
-                return GAF_ERR_CUDA;
-            int occ2 = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, kernel, kGsThreads, dyn) != cudaSuccess || occ2 < 1)
-                return GAF_ERR_UNSUPPORTED;
-            pl.occ = occ2 < occ ? occ2 : occ;
-            pl.park = park;
-            pl.dyn = dyn;
-            return GAF_OK;
-        }))
-        return rc;
-    const FusedPlan &pl = table.plan[di.dev];
-    int64_t grid = int64_t(di.sms) * pl.occ;
-    if (grid > kGsMaxCtas) grid = kGsMaxCtas;
-    const int64_t work = (a.D / FusedVec<T>::N + kGsThreads - 1) / kGsThreads;
-    if (grid > work) grid = work;
-    if (grid < 1) grid = 1;
-    a.park_rounds = pl.park;
+    if (int rc = filter_plan<T, KT, true>(di)) return rc;
+    auto kernel = gram_filter_kernel<T, KT, true>;
+    const int grid = filter_shape<T, KT>(a, di, true);
     a.spin_limit = g_test_wait_limit ? g_test_wait_limit : kFusedSpinLimit;
     a.test_withhold = g_test_withhold;
-    // the last stretch is asked to stay in L2 for the second pass
-    const int64_t per_elem = int64_t(KT) * int64_t(sizeof(T));
-    const int64_t keep_elems = int64_t(di.l2_bytes) * kKeepL2Pct / 100 / per_elem;
-    a.keep_from = a.D > keep_elems ? a.D - keep_elems : 0;
     // The grid is no larger than what the device holds at once (occupancy above), so all its CTAs become
     // resident and the one wait on other CTAs ends; it is bounded in any case.  Programmatic stream
     // serialisation: the kernel waits for its predecessor on the stream itself (griddepcontrol.wait, first
@@ -534,8 +487,8 @@ int launch_gram_fused_kt(GramFusedArgs &a, const DeviceInfo &di, cudaStream_t st
         if (q != cudaSuccess) cudaGetLastError();       // that stream no longer exists: nothing of it is in flight
     }
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(unsigned(grid)); cfg.blockDim = dim3(kGsThreads);
-    cfg.dynamicSmemBytes = size_t(pl.dyn); cfg.stream = st;
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kFilterThreads);
+    cfg.dynamicSmemBytes = size_t(FilterTile<T, KT>::kStages * FilterTile<T, KT>::kBytes); cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -562,6 +515,33 @@ int launch_gram_fused(GramFusedArgs &a, int K, const DeviceInfo &di, cudaStream_
     }
 }
 
+// Two-launch form: the same kernel without the wait at its end; masked_mean_kernel behind it.  Also the pairwise
+// distances of up to 8 gradients (no mean, nothing behind it).
+template <typename T, int KT>
+int launch_gram_filter_kt(GramFusedArgs &a, const DeviceInfo &di, cudaStream_t st) {
+    if (int rc = filter_plan<T, KT, false>(di)) return rc;
+    const int grid = filter_shape<T, KT>(a, di, a.pair_dist_out == nullptr);
+    a.test_withhold = 0;
+    const cudaError_t err = launch_dependent_smem(gram_filter_kernel<T, KT, false>, grid, kFilterThreads,
+                                                  size_t(FilterTile<T, KT>::kStages * FilterTile<T, KT>::kBytes), st, a);
+    ++g_launches;
+    if (err != cudaSuccess) { cudaGetLastError(); return GAF_ERR_CUDA; }
+    return GAF_OK;
+}
+template <typename T>
+int launch_gram_filter(GramFusedArgs &a, int K, const DeviceInfo &di, cudaStream_t st) {
+    switch (K) {
+        case 2: return launch_gram_filter_kt<T, 2>(a, di, st);
+        case 3: return launch_gram_filter_kt<T, 3>(a, di, st);
+        case 4: return launch_gram_filter_kt<T, 4>(a, di, st);
+        case 5: return launch_gram_filter_kt<T, 5>(a, di, st);
+        case 6: return launch_gram_filter_kt<T, 6>(a, di, st);
+        case 7: return launch_gram_filter_kt<T, 7>(a, di, st);
+        case 8: return launch_gram_filter_kt<T, 8>(a, di, st);
+        default: return GAF_ERR_ARG;
+    }
+}
+
 // Gram-first schedule: Gram matrix, scalar walk of Algorithm 1, masked mean.
 // `seed_out` non-null selects the any-seed variant (ord must then be the identity).
 template <typename T>
@@ -582,8 +562,9 @@ int launch_gram_first(const void *const *g, int K, int64_t D, int dtype, double 
     double *gram_by_index = reinterpret_cast<double *>(base + kExtraOffset + gram_partials_bytes(K));
     double *gram_by_step = reinterpret_cast<double *>(base + kExtraOffset + gram_partials_bytes(K) +
                                                       gram_matrix_bytes(K));
-    if (one_launch) {
-        if (K < 2 || K > kGsMaxK) return GAF_ERR_UNSUPPORTED;
+    if (one_launch && (K < 2 || K > kGsMaxK)) return GAF_ERR_UNSUPPORTED;
+    const bool filter_pass = K >= 2 && K <= kGsMaxK;
+    if (filter_pass) {
         GramFusedArgs f{};
         for (int t = 0; t < K; ++t) f.g[t] = g[ord[t]];
         f.D = D; f.out = macro_out;
@@ -591,21 +572,8 @@ int launch_gram_first(const void *const *g, int K, int64_t D, int dtype, double 
         f.gram = gram_by_step;
         f.replay = r;
         f.ring = ring;
-        return launch_gram_fused<T>(f, K, di, st);
-    }
-    if (use_small_gram(K, D, dtype)) {
-        GramSmallArgs a{};
-        for (int t = 0; t < K; ++t) a.g[t] = g[ord[t]];
-        a.D = D;
-        // how much of the tail of the Gram pass should stay in L2 for the masked-mean pass
-        const int64_t per_elem = int64_t(K) * int64_t(sizeof(T));
-        const int64_t keep_elems = int64_t(di.l2_bytes) * kKeepL2Pct / 100 / per_elem;
-        a.keep_from = D > keep_elems ? D - keep_elems : 0;
-        a.partials = reinterpret_cast<double *>(base + kExtraOffset);
-        a.gram = gram_by_step;
-        a.replay = r;
-        a.ring = ring;
-        if (int rc = launch_gram_small<T>(a, K, di, st)) return rc;
+        if (one_launch) return launch_gram_fused<T>(f, K, di, st);
+        if (int rc = launch_gram_filter<T>(f, K, di, st)) return rc;
     } else {
         if (int rc = launch_gram_tiles(g, K, D, dtype, nullptr, nullptr, base, di, st)) return rc;
         if (seed_out) gram_ring_replay_kernel<<<1, GAF_MAX_K, 0, st>>>(ring, gram_by_index);
@@ -614,7 +582,7 @@ int launch_gram_first(const void *const *g, int K, int64_t D, int dtype, double 
     }
     MaskedMeanArgs m{};
     for (int t = 0; t < K; ++t) m.g[t] = g[ord[t]];
-    m.K = K; m.D = D; m.out = macro_out; m.ctl = ctl;
+    m.K = K; m.D = D; m.out = macro_out; m.ctl = ctl; m.may_be_done = filter_pass ? 1 : 0;
     const int grid = stream_grid(D, kMsThreads, sms);
     {
         // runs of 8 chunks per CTA once every CTA gets at least eight such runs, else one trip at a time
@@ -1109,18 +1077,17 @@ int gaf_pairwise_cosdist(const void *const *grads, int K, int64_t D, int dtype, 
     auto *base = static_cast<unsigned char *>(workspace);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if (use_small_gram(K, D, dtype)) {
-        // few gradients: the one-pass register-tiled Gram kernel, distances in its last CTA
-        GramSmallArgs a{};
+        // few gradients: the one-pass kernel, distances in its last CTA
+        GramFusedArgs a{};
         for (int i = 0; i < K; ++i) a.g[i] = grads[i];
         a.D = D;
-        a.keep_from = D;                                    // nothing is read again: stream everything
         a.partials = reinterpret_cast<double *>(base + kExtraOffset);
         a.gram = reinterpret_cast<double *>(base + kExtraOffset + gram_partials_bytes(K));
         a.replay.ctl = reinterpret_cast<Control *>(base);
         a.pair_dist_out = dist_out;
         a.pair_gram_out = gram_out;
-        return dtype == GAF_F32 ? launch_gram_small<float>(a, K, di, st)
-                                : launch_gram_small<__nv_bfloat16>(a, K, di, st);
+        return dtype == GAF_F32 ? launch_gram_filter<float>(a, K, di, st)
+                                : launch_gram_filter<__nv_bfloat16>(a, K, di, st);
     }
     return launch_gram_tiles(grads, K, D, dtype, dist_out, gram_out, base, di, st);
 }

@@ -17,8 +17,8 @@ constexpr int kOct = 8;                 // elements handled per inner step
 // Control block at the start of the caller's workspace.
 struct Control {
     unsigned int ticket;                // last-block election, wraps to 0 by itself
-    unsigned int pair_hint;             // one-launch schedule with two gradients: what the latest two calls kept (0 both, 1 the seed alone, 2 | latest: they differed)
-    unsigned int reserved1;
+    unsigned int written_ctas;          // two-launch form: CTAs that wrote the predicted mean of all their elements
+    int mean_done;                      // two-launch form: 1 = the first launch has written the result
     int status;                         // GAF_STATUS_* bits of the latest call
     int count;                          // running c of Algorithm 1
     int ring_seed;                      // any-seed variant: the winning seed, else -1
@@ -33,6 +33,11 @@ struct Control {
     // 12..31 count calls and bits 0..11 the CTAs of the running call that have arrived.
     alignas(128) unsigned int fused_arrivals;
     unsigned int fused_pad[31];
+    // Prediction of the accept pattern from a sample (gaf_fused.cuh): an arrival counter like the one above for
+    // the CTAs whose sample sums are in, and the sums, two sets that calls use in turn.
+    alignas(128) unsigned int sample_arrivals;
+    unsigned int sample_pad[31];
+    double sample_sums[2][36];
 };
 constexpr size_t kControlBytes = 4096;  // sizeof(Control) rounded up
 static_assert(sizeof(Control) <= kControlBytes, "control block");

@@ -1,53 +1,99 @@
-// Gram-first schedule of Algorithm 1 as ONE launch (K <= 8).
+// Gram-first schedule of Algorithm 1 for 2 to 8 gradients in (mostly) ONE pass over the inputs.
 //
-// The two-launch form (gaf_gramfilter.cuh) reads every gradient once for the Gram
-// matrix and the accepted ones a second time for g/c (Eq. 5).  When the whole call
-// lasts tens of microseconds, what the second pass has to fetch again is a large part
-// of the cost.  Here one grid whose CTAs are all resident at once does both passes, so
-// that part of what the first pass read is still ON CHIP when the second pass starts:
-//   pass 1   every thread walks its vectors (grid-stride), accumulating the Gram
-//            partial sums exactly as gram_small_kernel does, and parks the raw loads
-//            of its FIRST R rounds in shared memory (the last rounds are the ones L2
-//            still holds afterwards: shared memory and L2 then keep different data);
-//   decide   every CTA stores its partial sums and adds itself to an arrival counter;
-//            when the counter is full every CTA totals the partials in the same fixed
-//            order and walks Algorithm 1 (Eq. 4 in binary64) on the Gram matrix ITSELF --
-//            all CTAs get the same bits, nobody waits for a published result (one trip
-//            through L2 less than electing a CTA to decide); CTA 0 writes the outputs;
-//   pass 2   the same thread visits the same vectors: the rounds that were not parked
-//            from the last one down (the end of the vectors was loaded "keep in L2"),
-//            then the parked rounds straight from shared memory, adding the accepted
-//            gradients in processing order in binary32 and dividing by c.
-// Same sums, same order of additions as the two-launch form: identical outputs.
+// Every gradient is needed for the Gram matrix before the first decision of Algorithm 1 is known, and the
+// accepted ones again for g/c (Eq. 5).  What that second pass fetches is most of what a call costs beyond reading
+// the inputs once.  But WHICH gradients will be accepted can be told from a part of them: cosines estimated on m
+// elements are off by about 1/sqrt(m), a thousandth on a million.  So:
+//   stream   one CTA per SM; a producer thread keeps a ring of tiles (all K gradients x a chunk of D) in shared
+//            memory filled with bulk copies (cp.async.bulk), about 200 KB in flight per SM;
+//   sample   the first few tiles of every CTA are spread evenly over the vectors (every CTA at another phase, so
+//            that all parts of a network are represented); the consumer warps take their Gram sums and KEEP them;
+//   predict  the CTAs exchange the sample's sums, each walks Algorithm 1 on them, while the ring fills: the
+//            exchange takes about as long as HBM needs for the rest of the ring;
+//   write    the mean under the predicted pattern is written for the kept tiles, and from then on for every
+//            tile together with its Gram sums;
+//   decide   at the end Algorithm 1 is walked on the full Gram matrix.  If it decides as predicted the
+//            result is complete; otherwise the mean is formed again from the accepted gradients.
+// The prediction decides which stores are made early, never a value: mask, distances and count come from the
+// full sums, and the mean is the same additions in the same order (binary32, processing order, one division by
+// c) whichever pass writes it.  Nothing is carried over from call to call.  Vectors that fit into the rings of
+// all SMs (about 29 MB of gradients) need no prediction: the mean is written from shared memory after the decision.
 //
-// The grid is sized by the host to what the device holds at once.  The kernel is launched with
-// programmatic stream serialisation: it waits for whatever precedes it on the stream before it
-// touches memory, and lets the launch behind it be placed as soon as its own decisions are taken
-// (that launch waits in turn), which hides most of the launch latency of back-to-back calls.
-// The one wait on other CTAs is bounded and ends in GAF_STATUS_TIMEOUT.
+// Two forms of one kernel, with the same sums in the same order, hence the same outputs:
+//   ONE      every CTA is resident at once.  At the end every CTA stores its partial sums, adds itself to an
+//            arrival counter, waits (bounded, GAF_STATUS_TIMEOUT) until it is full, totals the partials and walks
+//            Algorithm 1 ITSELF -- all CTAs get the same bits, nobody waits for a published result; CTA 0 writes
+//            the outputs.  After a wrong prediction the ring is run once more over the accepted gradients, the
+//            last tiles first (what L2 still holds).
+//   two      the last CTA to take a ticket decides, and masked_mean_kernel, launched behind, returns at once when
+//            the result is already written.  The only wait for other CTAs is the prediction's, and it is short:
+//            a CTA that does not get one goes on without.  The same form gives the pairwise distances.
+// The kernel is launched with programmatic stream serialisation: it waits for whatever precedes it on the stream
+// before it touches global memory, and lets the launch behind it be placed once its own streaming (two) or
+// deciding (ONE) is over.
+//
+// Gram sums of a tile: up to 4 binary32 gradients in binary64 registers (products exact); otherwise binary32
+// chains (64 products; 128 of bfloat16 values, whose products are exact), two to a register pair, widened to
+// binary64 in shared memory; 7 and 8 bfloat16 gradients by warp-level MMAs (gaf_gram_mma.cuh's mapping, operands
+// from shared memory, chains of 128).
 #pragma once
 
 #include <type_traits>
 
 #include "gaf_device.cuh"
+#include "gaf_gram_mma.cuh"
+#include "gaf_gram_tc.cuh"
 #include "gaf_gramfilter.cuh"
 
 namespace gaf {
 
 constexpr unsigned int kFusedSpinLimit = 1u << 23;   // polls of an L2 round trip plus a 20 ns sleep each: seconds
-constexpr unsigned int kFusedCallUnit = 4096;        // what one call adds to the arrival counter in all
+constexpr unsigned int kFusedSampleLimit = 64;       // two-launch form: polls for the prediction, some tens of microseconds
+constexpr unsigned int kFusedCopyLimit = 1u << 19;   // attempts of up to 2 us at a ring barrier
+constexpr unsigned int kFusedCallUnit = 4096;        // what one call adds to an arrival counter in all
 constexpr int kFusedCallShift = 12;
 
+// Consumer warps work in groups; a tile belongs to one group, the groups take the tiles in turn.  One more warp
+// produces.  15 warps of at most 128 registers.
+constexpr int kFilterGroups = 2;
+constexpr int kFilterGroupWarps = 7;
+constexpr int kFilterGroupThreads = kFilterGroupWarps * 32;
+constexpr int kFilterWarps = kFilterGroups * kFilterGroupWarps;
+constexpr int kFilterConsumers = kFilterWarps * 32;
+constexpr int kFilterThreads = kFilterConsumers + 32;
+constexpr int kFilterMaxStages = 24;
+constexpr int kFilterMaxCtas = 160;
+constexpr int kFilterRingBytes = 206 << 10;
+
+// Tile of K gradients: kVecs groups of 4 elements per thread of a group and gradient, about 28 KB in all.
+template <typename T, int KT> struct FilterTile {
+    static constexpr bool kMma = std::is_same<T, __nv_bfloat16>::value && KT >= 7;
+    static constexpr int kVecs = KT == 2 ? 16 / int(sizeof(T)) : (KT <= 4 ? 8 / int(sizeof(T)) : 4 / int(sizeof(T)));
+    static constexpr int kElems = kVecs * 4 * kFilterGroupThreads;
+    // (the MMA fragments of eight rows are read together: 64 bytes between rows keep them apart in the banks)
+    static constexpr int kPitch = kElems * int(sizeof(T)) + (kMma ? 64 : 0);
+    static constexpr int kBytes = KT * kPitch;
+    // A multiple of the groups: a stage then always belongs to the same group, which has seen its previous tile land
+    // before it waits for the next one (copies complete in any order; a barrier's parity tells only two phases apart).
+    static constexpr int kFit = kFilterRingBytes / kBytes < kFilterMaxStages ? kFilterRingBytes / kBytes : kFilterMaxStages;
+    static constexpr int kStages = kFit / kFilterGroups * kFilterGroups;
+    static constexpr int kBatch = KT == 2 ? 4 : (KT <= 4 ? 2 : 1);  // groups of 4 elements a thread loads together
+};
+
 struct GramFusedArgs {
-    const void *g[kGsMaxK];                 // processing order (original order in any-seed mode)
+    const void *g[kGsMaxK];                 // processing order (original order in any-seed and pairwise mode)
     int64_t D;
-    int64_t keep_from;                      // elements from here on are loaded "keep in L2"
-    int park_rounds;                        // R: rounds per thread parked in shared memory
-    double *partials;                       // [pair][kGsPartialStride]
+    int tile_elems;                         // elements of a tile per gradient (a multiple of 64, at most FilterTile::kElems)
+    int rounds;                             // tiles per CTA
+    int run;                                // consecutive tiles a CTA takes before it jumps ahead by the grid's share
+    int sample;                             // tiles per CTA in the sample; 0 = no prediction
+    double *partials;                       // [pair][kFilterMaxCtas]
     double *gram;                           // [K][K]
     float *out;                             // D floats
     ReplayArgs replay;                      // used when ring.K == 0
     RingArgs ring;                          // any-seed mode when ring.K > 0
+    float *pair_dist_out;                   // pairwise mode: K x K distances instead of the walk and the mean
+    double *pair_gram_out;                  // pairwise mode: optional copy of the Gram matrix
     unsigned int spin_limit;                // polls a waiting CTA makes before it gives up
     int test_withhold;                      // test hook, normally 0: the waiting CTAs are never shown the full
                                             // counter, so that every wait runs out
@@ -68,306 +114,630 @@ __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int *p) {
 __device__ __forceinline__ void red_release_add_u32(unsigned int *p, unsigned int v) {
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
+// Bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) into shared memory, counted on `bar`.
+__device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void *src, uint32_t bytes, uint64_t *bar, uint64_t policy) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
+                 ::"r"(dst_smem), "l"(src), "r"(bytes), "r"(tc_smem_u32(bar)), "l"(policy)
+                 : "memory");
+}
 
-template <typename T> struct FusedVec;      // one 16-byte vector of a gradient, widened
-template <> struct FusedVec<float> {
-    static constexpr int N = 4;
-    static __device__ __forceinline__ void widen(const uint4 &r, float (&v)[4]) {
-        v[0] = __uint_as_float(r.x); v[1] = __uint_as_float(r.y);
-        v[2] = __uint_as_float(r.z); v[3] = __uint_as_float(r.w);
+// The consumer warps among themselves (barrier 0 is the whole CTA's).
+struct FilterConsumers {
+    static __device__ __forceinline__ void sync() {
+        asm volatile("barrier.cta.sync 1, %0;" ::"n"(kFilterConsumers) : "memory");
+    }
+    static __device__ __forceinline__ int threads() { return kFilterConsumers; }
+};
+
+// Two binary32 values in one register pair, and the two-wide instructions on them (each half rounds as the scalar
+// instruction does).
+typedef unsigned long long Pair;
+__device__ __forceinline__ Pair pair_of(float lo, float hi) {
+    Pair r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void pair_split(Pair p, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p)); }
+__device__ __forceinline__ Pair pair_fma(Pair a, Pair b, Pair c) {
+    Pair r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
+    Pair r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
+    Pair r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+template <typename T> struct Quad;          // four consecutive elements as they lie in a tile, widened to two pairs
+template <> struct Quad<float> {
+    static __device__ __forceinline__ void load(const unsigned char *p, Pair (&x)[2]) {
+        const ulonglong2 r = *reinterpret_cast<const ulonglong2 *>(p);
+        x[0] = r.x; x[1] = r.y;
     }
 };
-template <> struct FusedVec<__nv_bfloat16> {
-    static constexpr int N = 8;
-    static __device__ __forceinline__ void widen(const uint4 &r, float (&v)[8]) {
-        const unsigned int w[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            v[2 * k] = bf16_bits_to_float(w[k] & 0xFFFFu);
-            v[2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u);
+template <> struct Quad<__nv_bfloat16> {
+    static __device__ __forceinline__ void load(const unsigned char *p, Pair (&x)[2]) {
+        const uint2 r = *reinterpret_cast<const uint2 *>(p);
+        x[0] = pair_of(bf16_bits_to_float(r.x & 0xFFFFu), __uint_as_float(r.x & 0xFFFF0000u));
+        x[1] = pair_of(bf16_bits_to_float(r.y & 0xFFFFu), __uint_as_float(r.y & 0xFFFF0000u));
+    }
+};
+
+// Division of binary32 values by a count c of 1 to 8, correctly rounded.  A power of two: multiplication by its
+// inverse.  Else x / c = RN(x zh + RN(x zl)) with zh = RN(1 / c), zl = RN(1 / c - zh) (Brisebarre, Muller and
+// Raina, "Accelerating correctly rounded floating-point division when the divisor is known in advance", IEEE
+// Trans. Computers 2004), which holds for c = 3, 5, 6 and 7 for every significand (all 2^23 checked) as long as x zl
+// is a normal number; values outside [2^-90, 2^100] (zeros, infinities among them) take the division.
+struct CountDivider {
+    float c;
+    Pair zh2, zl2;
+    bool pow2;
+    __device__ __forceinline__ explicit CountDivider(int count) {
+        c = (float)count;
+        const float zh = 1.0f / c, zl = fmaf(-zh, c, 1.0f) / c;
+        zh2 = pair_of(zh, zh);
+        zl2 = pair_of(zl, zl);
+        pow2 = (count & (count - 1)) == 0;
+    }
+    __device__ __forceinline__ void divide(Pair (&x)[2]) const {
+        if (pow2) {
+            x[0] = pair_mul(x[0], zh2); x[1] = pair_mul(x[1], zh2);
+            return;
+        }
+        float v[4];
+        pair_split(x[0], v[0], v[1]);
+        pair_split(x[1], v[2], v[3]);
+        const float least = fminf(fminf(fabsf(v[0]), fabsf(v[1])), fminf(fabsf(v[2]), fabsf(v[3])));
+        const float most = fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3])));
+        if (least >= 8.077935669463161e-28f && most <= 1.2676506002282294e+30f) {      // 2^-90, 2^100
+            x[0] = pair_fma(x[0], zh2, pair_mul(x[0], zl2));
+            x[1] = pair_fma(x[1], zh2, pair_mul(x[1], zl2));
+        } else {
+            x[0] = pair_of(v[0] / c, v[1] / c);
+            x[1] = pair_of(v[2] / c, v[3] / c);
         }
     }
 };
 
-template <int N>
-__device__ __forceinline__ void store_vec_streaming(float *dst, const float (&v)[N]) {
-#pragma unroll
-    for (int h = 0; h < N / 4; ++h)
-        __stcs(reinterpret_cast<float4 *>(dst) + h, make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]));
+// An accept pattern in one word: the rows, and the row the order starts at.  0 = not known.
+__device__ __forceinline__ unsigned int pack_pattern(unsigned int bits, int start) {
+    return 0x80000000u | ((unsigned int)start << 8) | bits;
 }
 
-// Rounds of the second pass a thread keeps in flight, by the number of gradients it has to fetch per
-// round (8 loads of 16 bytes per thread at most, 2 rounds at least up to 4 gradients).
-template <int NN> struct FusedInFlight { static constexpr int U = NN <= 1 ? 8 : (NN == 2 ? 4 : (NN <= 4 ? 2 : 1)); };
+// Order of a CTA's tiles: the S sample rounds (one in each of S segments of `seg` rounds, at the CTA's phase), then
+// the others in ascending order.
+__device__ __forceinline__ int round_of_visit(int v, int S, int seg, int phase) {
+    if (v < S) return v * seg + phase;
+    const int u = v - S, m = seg - 1;
+    if (u >= S * m) return u + S;
+    const int b = u / m, i = u - b * m;
+    return b * seg + i + (i >= phase ? 1 : 0);
+}
 
-template <typename T, int KT>
-__global__ void __launch_bounds__(kGsThreads, (KT <= 4 ? 2 : 1))
-gram_fused_kernel(const __grid_constant__ GramFusedArgs a) {
+// Algorithm 1 on a small Gram matrix in shared memory by one warp, for the prediction: decisions only, binary32.
+// Lane j carries <g_j, running sum>.  Returns the packed pattern in every lane.
+template <int KT>
+__device__ __forceinline__ unsigned int warp_guess(const double *gram, double tau) {
+    const int lane = threadIdx.x & 31, j = lane < KT ? lane : 0;
+    float pj = (float)gram[j], na = (float)gram[0];
+    const float ng_j = (float)gram[j * KT + j], bound = 1.0f - (float)tau;
+    unsigned int bits = 1u;
+    for (int t = 1; t < KT; ++t) {
+        const float p = __shfl_sync(0xFFFFFFFFu, pj, t), ng = __shfl_sync(0xFFFFFFFFu, ng_j, t);
+        float cosv = (na > 0.0f && ng > 0.0f) ? p * rsqrtf(na) * rsqrtf(ng) : 0.0f;
+        cosv = fminf(fmaxf(cosv, -1.0f), 1.0f);
+        if (cosv >= bound) {
+            bits |= 1u << t;
+            na += 2.0f * p + ng;
+            pj += (float)gram[t * KT + j];
+        }
+    }
+    return pack_pattern(bits, 0);
+}
+// ... and of its order-indifferent variant: lane s walks seed s, the largest count wins, ties to the smallest seed.
+template <int KT>
+__device__ __forceinline__ unsigned int warp_ring_guess(const RingArgs &r, const double *gram) {
+    const int lane = threadIdx.x & 31;
+    int count = 0, status = 0;
+    unsigned long long bits = 0;
+    if (lane < KT) ring_walk_one_seed(r, gram, lane, count, bits, status, nullptr);
+    const unsigned int key = lane < KT ? ((unsigned int)count << 8) | (unsigned int)(KT - 1 - lane) : 0u;
+    const unsigned int best = __reduce_max_sync(0xFFFFFFFFu, key);
+    const int seed = KT - 1 - (int)(best & 0xFFu);
+    return pack_pattern(__shfl_sync(0xFFFFFFFFu, (unsigned int)bits, seed), seed);
+}
+
+// Warp-wide sums of NP per-lane values by recursive halving, added to dst: in each round a lane keeps the half of its
+// values chosen by one bit of its number, adding its partner's copy of that half, so about NP shuffles (not 5 NP)
+// leave every sum in one lane.  A fixed tree.
+template <int NP, int D, typename Acc>
+struct HalvingSums {
+    static constexpr int H = (NP + 1) / 2;
+    static __device__ __forceinline__ void run(Acc *v, int lane, int base, int limit, double *dst) {
+        const bool upper = (lane & D) != 0;
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            const Acc hi = i + H < NP ? v[i + H] : Acc(0);
+            const Acc send = upper ? v[i] : hi, keep = upper ? hi : v[i];
+            v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, D);
+        }
+        // this lane now holds entries base .. of the half it chose; the upper half may be one shorter
+        HalvingSums<H, D / 2, Acc>::run(v, lane, base + (upper ? H : 0), upper ? min(limit, base + NP) : min(limit, base + H), dst);
+    }
+};
+template <int NP, typename Acc>
+struct HalvingSums<NP, 0, Acc> {
+    static __device__ __forceinline__ void run(Acc *v, int, int base, int limit, double *dst) {
+#pragma unroll
+        for (int i = 0; i < NP; ++i)
+            if (base + i < limit) dst[base + i] += (double)v[i];
+    }
+};
+
+template <typename T, int KT, bool ONE>
+__global__ void __launch_bounds__(kFilterThreads, 1)
+gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
+    using Tile = FilterTile<T, KT>;
+    using Sync = FilterConsumers;
     constexpr int NP = KT * (KT + 1) / 2;
-    constexpr int N = FusedVec<T>::N;
-    // With two gradients (the paper's own experiments: Section 4) the output can only be the mean of both or the
-    // seed alone, so the first pass writes one of the two while it forms the sums -- the one the latest two calls on
-    // this workspace both ended with (decisions of consecutive training steps go together; no guess while they
-    // differ) -- and the second pass runs only when this call decides otherwise: 12 bytes per fp32 element instead
-    // of 20 (16 for the seed alone) when the guess holds, 24 when it does not, the usual 20 / 16 without a guess.
-    // The guess changes which stores happen, never their values.
-    constexpr bool kSpeculative = KT == 2;
-    extern __shared__ uint4 parked[];       // [round][gradient][thread]
-    __shared__ double sacc[kGsThreads / 32][NP];
+    constexpr int CW = kFilterWarps, NG = kFilterGroups, kStages = Tile::kStages, kPitch = Tile::kPitch;
+    extern __shared__ __align__(128) unsigned char ring[];      // [stage][gradient][pitch]
+    __shared__ uint64_t full[kStages], empty[kStages];
+    __shared__ int64_t stage_e0[kStages];   // first element and length of the tile in a stage (written by the producer)
+    __shared__ int stage_n[kStages];
+    __shared__ double ssum[CW][NP];         // per-warp sums
     __shared__ double sgram[KT * KT];
     __shared__ const T *list[kGsMaxK];      // accepted gradients in the order they are added
-    __shared__ int list_row[kGsMaxK];       // ... and their row in `parked`
-    __shared__ int n_list;                  // c, or -1 when the wait ran out
+    __shared__ int n_list;                  // c
+    __shared__ int sh_ok, sh_again;         // outcome of a wait; whether the accepted gradients are run once more
+    __shared__ unsigned int sh_pred, sh_final;      // predicted and decided pattern
+    __shared__ volatile int abort_flag;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     Control *ctl = a.replay.ctl;
 
+    if (tid == 0) {
+        for (int s = 0; s < kStages; ++s) { tc_mbar_init(&full[s], 1); tc_mbar_init(&empty[s], kFilterGroupWarps); }
+        sh_pred = 0u; sh_again = 0; abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    for (int i = tid; i < CW * NP; i += kFilterThreads) (&ssum[0][0])[i] = 0.0;
+    __syncthreads();
     // Launched with programmatic stream serialisation, this grid may be placed while the launch before
     // it on the stream is still winding down: nothing that launch (or the producer of the gradients)
     // wrote may be touched before it has completed.  A no-op after an ordinary predecessor.
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
-    // call generation before this CTA has arrived: it cannot change until every CTA has, this one included
-    unsigned int gen0 = 0;
-    if (tid == 0) {
-        gen0 = ld_relaxed_u32(&ctl->fused_arrivals) >> kFusedCallShift;
-        if (blockIdx.x == 0) ctl->status = 0;
+    const int rounds = a.rounds, S = a.sample;
+    constexpr int kAlign = 16 / (int)sizeof(T);
+    const int64_t Dv = a.D / kAlign * kAlign;                   // what the copies cover
+    const bool resident = rounds <= kStages;                    // every tile stays in the ring
+
+    if (warp == CW) {
+        // ------------------------------------------------------------------ producer ----
+        const int te = a.tile_elems, seg = S > 0 ? rounds / S : 1, phase = S > 0 ? (int)blockIdx.x % seg : 0;
+        int it = 0;                         // tiles since the start, of both passes
+        const uint64_t policy = l2_policy_evict_first();
+        auto fill = [&](int v, const void *const *rows, int n_rows) {
+            const int s = it % kStages;
+            if (it >= kStages && !tc_mbar_wait(&empty[s], (uint32_t)((it / kStages - 1) & 1), &abort_flag, kFusedCopyLimit))
+                return false;
+            const int r = round_of_visit(v, S, seg, phase);
+            int64_t tile = (int64_t)r * gridDim.x + blockIdx.x;
+            if (a.run > 1) tile = ((int64_t)(r / a.run) * gridDim.x + blockIdx.x) * a.run + r % a.run;
+            const int64_t e0 = tile * te, left = Dv - e0;
+            const int n = left >= te ? te : (left > 0 ? (int)left : 0);
+            stage_e0[s] = e0;
+            stage_n[s] = n;
+            if (n > 0) {
+                const uint32_t bytes = (uint32_t)n * (uint32_t)sizeof(T), dst = tc_smem_u32(ring + (size_t)s * Tile::kBytes);
+                tc_mbar_arrive_expect_tx(&full[s], bytes * (uint32_t)n_rows);
+                for (int g = 0; g < n_rows; ++g)
+                    bulk_load(dst + (uint32_t)(g * kPitch), static_cast<const T *>(rows[g]) + e0, bytes, &full[s], policy);
+            } else {
+                tc_mbar_arrive(&full[s]);
+            }
+            ++it;
+            return true;
+        };
+        if (lane == 0)
+            for (int v = 0; v < rounds; ++v)
+                if (!fill(v, a.g, KT)) break;
+        __syncwarp();
+        __syncthreads();                    // the consumers have decided whether there is a second pass
+        if (ONE && sh_again && lane == 0)
+            for (int v = rounds - 1; v >= 0; --v)
+                if (!fill(v, reinterpret_cast<const void *const *>(list), n_list)) break;
+        // after a wait that gave up: the copies in flight must land before the CTA leaves its shared memory
+        if (lane == 0 && abort_flag)
+            for (int i = it > kStages ? it - kStages : 0; i < it; ++i)
+                for (unsigned int spin = 0; spin < kFusedCopyLimit; ++spin)
+                    if (tc_mbar_try(&full[i % kStages], (uint32_t)((i / kStages) & 1), 2000u)) break;
+        return;
     }
-    for (int p = lane; p < NP; p += 32) sacc[warp][p] = 0.0;
-    __syncwarp();
-    // (read before this CTA arrives, hence before any CTA can have decided and written the next guess)
-    // 0 / 1: the latest two such calls both kept both gradients / the seed alone: write that now;
-    // 2 / 3: they differed (the latest kept both / the seed alone): no guess, two passes as with more gradients
-    const unsigned int hint = kSpeculative ? ld_relaxed_u32(&ctl->pair_hint) : 2u;
-    const bool guessing = hint < 2u, guess_seed_alone = (hint & 1u) != 0;
 
-    const T *row[KT];
-#pragma unroll
-    for (int r = 0; r < KT; ++r) row[r] = static_cast<const T *>(a.g[r]);
+    // ---------------------------------------------------------------------- consumers ----
+    const int group = warp / kFilterGroupWarps, gwarp = warp - group * kFilterGroupWarps, gtid = gwarp * 32 + lane;
+    unsigned int gen0 = 0, gen_s = 0;       // call generations: they cannot change before this CTA has arrived
+    if (ONE && tid == 0) gen0 = ld_relaxed_u32(&ctl->fused_arrivals) >> kFusedCallShift;
+    if (S > 0) gen_s = ld_relaxed_u32(&ctl->sample_arrivals) >> kFusedCallShift;
+    if (blockIdx.x == 0 && tid == 0) ctl->status = 0;
+    // (two sets of sample sums, used by calls in turn: this one clears the next call's)
+    if (S > 0 && blockIdx.x == 0 && tid < NP) ctl->sample_sums[(gen_s + 1u) & 1u][tid] = 0.0;
 
-    const uint64_t pol_first = l2_policy_evict_first(), pol_last = l2_policy_evict_last();
-    const int64_t n_vec = a.D / N;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // rounds of this warp (the same for all its lanes: the flush shuffles across the warp)
-    const int64_t warp_first = (int64_t)blockIdx.x * blockDim.x + (tid & ~31);
-    const int64_t rounds = warp_first < n_vec ? (n_vec - warp_first + stride - 1) / stride : 0;
-    const int64_t parked_rounds = rounds < a.park_rounds ? rounds : a.park_rounds;   // the FIRST ones
-    using Acc = typename GsAcc<T, KT>::type;
-    Acc acc[NP];
+    // Accumulators: binary64, pairs of binary32 chains, or (MMA) this lane's fragment of the 8 x 8 matrix.
+    constexpr bool kF64 = !GsAcc<T, KT>::kPeriodicFlush;
+    using Acc = typename std::conditional<kF64, double, Pair>::type;
+    constexpr int NA = Tile::kMma ? 1 : NP;
+    // tiles between flushes: each half of a pair sums 64 products (128 of bfloat16 values)
+    constexpr int kChainTiles = 128 / int(sizeof(T)) / Tile::kVecs > 0 ? 128 / int(sizeof(T)) / Tile::kVecs : 1;
+    Acc acc[NA];
 #pragma unroll
-    for (int p = 0; p < NP; ++p) acc[p] = Acc(0);
+    for (int p = 0; p < NA; ++p) acc[p] = Acc(0);
+    float frag[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    double frag_sum[2] = {0.0, 0.0};
+    int chain = 0;
     auto flush = [&]() {
+        if constexpr (Tile::kMma) {
+            const int g = lane >> 2, t = lane & 3;
 #pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            Acc v = acc[p];
+            for (int h = 0; h < 2; ++h) {
+                const int j = 2 * t + h;
+                if (g <= j && j < KT) ssum[warp][g * KT - g * (g - 1) / 2 + (j - g)] += frag_sum[h];
+                frag_sum[h] = 0.0;
+            }
+        } else if constexpr (kF64) {
+            HalvingSums<NP, 16, double>::run(acc, lane, 0, NP, ssum[warp]);
 #pragma unroll
-            for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, d);
-            if (lane == 0) sacc[warp][p] += (double)v;
-            acc[p] = Acc(0);
+            for (int p = 0; p < NP; ++p) acc[p] = 0.0;
+        } else {
+            float v[NP];
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                float lo, hi;
+                pair_split(acc[p], lo, hi);
+                v[p] = lo + hi;
+                acc[p] = Pair(0);
+            }
+            HalvingSums<NP, 16, float>::run(v, lane, 0, NP, ssum[warp]);
+        }
+        chain = 0;
+    };
+    // One tile: its Gram sums (GRAM) and the mean of its rows under a pattern (MEAN).
+    auto process = [&](auto gram_tag, auto mean_tag, int s, unsigned int from, unsigned int before, const CountDivider &div) {
+        constexpr bool GRAM = decltype(gram_tag)::value, MEAN = decltype(mean_tag)::value;
+        constexpr int B = Tile::kBatch;
+        const unsigned char *tile = ring + (size_t)s * Tile::kBytes;
+        const int n = stage_n[s];
+        float *out = a.out + stage_e0[s];
+        if constexpr (GRAM && Tile::kMma) {
+            const int g = lane >> 2, t = lane & 3;
+            const unsigned char *row = tile + (g < KT ? g : 0) * kPitch;
+#pragma unroll
+            for (int u = 0; u < Tile::kElems / 32 / kFilterGroupWarps; ++u) {
+                const int e = (u * kFilterGroupWarps + gwarp) * 32 + t * 8;
+                uint4 r = make_uint4(0u, 0u, 0u, 0u);
+                if (g < KT && e < n) r = *reinterpret_cast<const uint4 *>(row + e * 2);
+                mma_bf16_16816(frag, r.x, r.y);
+                mma_bf16_16816(frag, r.z, r.w);
+                if (u % 4 == 3) {
+                    frag_sum[0] += (double)frag[0]; frag_sum[1] += (double)frag[1];
+                    frag[0] = frag[1] = frag[2] = frag[3] = 0.0f;
+                }
+            }
+            static_assert(!Tile::kMma || Tile::kElems / 32 / kFilterGroupWarps % 4 == 0, "chains end inside a tile");
+        }
+        if constexpr (MEAN || !Tile::kMma) {
+            constexpr bool SUMS = GRAM && !Tile::kMma;
+#pragma unroll
+            for (int u0 = 0; u0 < Tile::kVecs; u0 += B) {
+                Pair x[B][KT][2];
+                int e[B];
+#pragma unroll
+                for (int b = 0; b < B; ++b) {
+                    e[b] = ((u0 + b) * kFilterGroupThreads + gtid) * 4;
+                    if (e[b] < n) {
+#pragma unroll
+                        for (int g = 0; g < KT; ++g)
+                            if (SUMS || (((from | before) >> g) & 1u)) Quad<T>::load(tile + g * kPitch + e[b] * (int)sizeof(T), x[b][g]);
+                    }
+                }
+#pragma unroll
+                for (int b = 0; b < B; ++b)
+                    if (SUMS && e[b] < n) {
+                        if constexpr (kF64) {
+                            float f[KT][4];
+#pragma unroll
+                            for (int g = 0; g < KT; ++g) { pair_split(x[b][g][0], f[g][0], f[g][1]); pair_split(x[b][g][1], f[g][2], f[g][3]); }
+                            int p = 0;
+#pragma unroll
+                            for (int g = 0; g < KT; ++g)
+#pragma unroll
+                                for (int h = g; h < KT; ++h, ++p)
+#pragma unroll
+                                    for (int k = 0; k < 4; ++k) acc[p] = gs_fma(f[g][k], f[h][k], acc[p]);
+                        } else if constexpr (!Tile::kMma) {
+                            int p = 0;
+#pragma unroll
+                            for (int g = 0; g < KT; ++g)
+#pragma unroll
+                                for (int h = g; h < KT; ++h, ++p)
+                                    acc[p] = pair_fma(x[b][g][1], x[b][h][1], pair_fma(x[b][g][0], x[b][h][0], acc[p]));
+                        }
+                    }
+                if constexpr (MEAN) {
+                    // in processing order (-0 + x = x for every x, so the first addition is a copy)
+                    Pair v[B][2];
+#pragma unroll
+                    for (int b = 0; b < B; ++b) v[b][0] = v[b][1] = 0x8000000080000000ull;
+#pragma unroll
+                    for (int g = 0; g < KT; ++g)
+                        if ((from >> g) & 1u) {
+#pragma unroll
+                            for (int b = 0; b < B; ++b) { v[b][0] = pair_add(v[b][0], x[b][g][0]); v[b][1] = pair_add(v[b][1], x[b][g][1]); }
+                        }
+                    if (before) {
+#pragma unroll
+                        for (int g = 0; g < KT; ++g)
+                            if ((before >> g) & 1u) {
+#pragma unroll
+                                for (int b = 0; b < B; ++b) { v[b][0] = pair_add(v[b][0], x[b][g][0]); v[b][1] = pair_add(v[b][1], x[b][g][1]); }
+                            }
+                    }
+#pragma unroll
+                    for (int b = 0; b < B; ++b)
+                        if (e[b] < n) {
+                            div.divide(v[b]);
+                            float4 r;
+                            pair_split(v[b][0], r.x, r.y);
+                            pair_split(v[b][1], r.z, r.w);
+                            __stcs(reinterpret_cast<float4 *>(out + e[b]), r);
+                        }
+                }
+            }
+        }
+        if constexpr (GRAM && !Tile::kMma && !kF64) {
+            if (++chain == kChainTiles) flush();
         }
     };
-
-    const int64_t tail0 = n_vec * N;
-    // ---- pass 1: Gram partial sums; the first rounds stay in shared memory ----
-    // (with two gradients a thread would have only two 16-byte loads in flight: it fetches two rounds at a time;
-    // the rounds are still consumed in order, so the sums are the same)
-    constexpr int U1 = KT <= 2 ? 2 : 1;
-    int since_flush = 0;
-    for (int64_t j0 = 0; j0 < rounds; j0 += U1) {
-        int64_t q[U1];
-        bool ok[U1];
-        uint4 raw[U1][KT];
+    using std::false_type;
+    using std::true_type;
+    auto wait_full = [&](int it) {
+        const uint32_t parity = (uint32_t)((it / kStages) & 1);
+        if (!tc_mbar_try(&full[it % kStages], parity, 2000u) &&
+            !tc_mbar_wait(&full[it % kStages], parity, &abort_flag, kFusedCopyLimit) && lane == 0)
+            atomicOr(&ctl->status, GAF_STATUS_TIMEOUT);
+        __syncwarp();
+    };
+    auto release = [&](int it) {
+        __syncwarp();
+        if (lane == 0) tc_mbar_arrive(&empty[it % kStages]);
+    };
+    // This CTA's sum of pair `tid` so far, over its warps in a fixed order (threads below NP).
+    auto cta_sum = [&]() {
+        double s = 0.0;
 #pragma unroll
-        for (int u = 0; u < U1; ++u) {
-            q[u] = warp_first + (j0 + u) * stride + lane;
-            ok[u] = j0 + u < rounds && q[u] < n_vec;
-            if (ok[u]) {
-                const uint64_t pol = (q[u] * N >= a.keep_from) ? pol_last : pol_first;
-#pragma unroll
-                for (int r = 0; r < KT; ++r) raw[u][r] = ld16_policy(row[r] + q[u] * N, pol);
-            }
+        for (int w = 0; w < CW; ++w) s += ssum[w][tid];
+        return s;
+    };
+    auto arrive = [&](unsigned int *counter) {
+        red_release_add_u32(counter, blockIdx.x == 0 ? kFusedCallUnit - (gridDim.x - 1) : 1u);
+    };
+    // (the acquire orders the loads behind it, through a barrier for other threads, after every CTA's stores)
+    auto wait_all = [&](const unsigned int *counter, unsigned int gen, unsigned int limit) {
+        unsigned int polls = 0;
+        while ((ld_acquire_u32(counter) >> kFusedCallShift) == gen || a.test_withhold) {
+            __nanosleep(20);
+            if (++polls > limit) return false;
         }
-#pragma unroll
-        for (int u = 0; u < U1; ++u) {
-            const int64_t j = j0 + u;
-            if (j >= rounds) break;
-            if (ok[u]) {
-                if (j < parked_rounds) {
-                    uint4 *slot = parked + (size_t)j * KT * kGsThreads + tid;
-#pragma unroll
-                    for (int r = 0; r < KT; ++r) slot[r * kGsThreads] = raw[u][r];
-                }
-                float x[KT][N];
-#pragma unroll
-                for (int r = 0; r < KT; ++r) FusedVec<T>::widen(raw[u][r], x[r]);
-                if (kSpeculative && guessing) {
-                    // two gradients: the guessed result is written now
-                    float v[N];
-#pragma unroll
-                    for (int k = 0; k < N; ++k) v[k] = guess_seed_alone ? x[0][k] : (x[0][k] + x[1][k]) / 2.0f;
-                    store_vec_streaming<N>(a.out + q[u] * N, v);
-                }
-                int p = 0;
-#pragma unroll
-                for (int r = 0; r < KT; ++r)
-#pragma unroll
-                    for (int c = r; c < KT; ++c, ++p) {
-                        Acc s = acc[p];
-#pragma unroll
-                        for (int k = 0; k < N; ++k) s = gs_fma(x[r][k], x[c][k], s);
-                        acc[p] = s;
-                    }
-            }
-            if (GsAcc<T, KT>::kPeriodicFlush && ++since_flush == kGsFlushEvery) { flush(); since_flush = 0; }
+        return true;
+    };
+
+    unsigned int pred = 0;
+    int v = group;
+    {
+        const CountDivider none(1);
+        for (; v < S; v += NG) {
+            wait_full(v);
+            process(true_type(), false_type(), v % kStages, 0u, 0u, none);
         }
     }
-    // ragged tail (D mod N elements), first CTA
-    if (blockIdx.x == 0 && tail0 + tid < a.D) {
-        const int64_t e = tail0 + tid;
-        float x[KT];
-#pragma unroll
-        for (int r = 0; r < KT; ++r) x[r] = load1<T>(row[r], e);
-        if (kSpeculative && guessing) a.out[e] = guess_seed_alone ? x[0] : (x[0] + x[1]) / 2.0f;
-        int p = 0;
-#pragma unroll
-        for (int r = 0; r < KT; ++r)
-#pragma unroll
-            for (int c = r; c < KT; ++c, ++p) acc[p] = gs_fma(x[r], x[c], acc[p]);
+    if (S > 0) {
+        // The sample's sums are totalled by atomic additions: their last bits depend on the order, but they only
+        // serve a guess.
+        flush();
+        Sync::sync();
+        if (tid < NP) atomicAdd(&ctl->sample_sums[gen_s & 1u][tid], cta_sum());
+        Sync::sync();
+        if (warp == 0) {
+            int ok = 0;
+            if (lane == 0) {
+                arrive(&ctl->sample_arrivals);
+                ok = wait_all(&ctl->sample_arrivals, gen_s, ONE ? a.spin_limit : kFusedSampleLimit) ? 1 : 0;
+            }
+            if (__shfl_sync(0xFFFFFFFFu, ok, 0)) {
+                for (int p = lane; p < NP; p += 32) {
+                    int i = 0, rem = p;
+                    while (rem >= KT - i) { rem -= KT - i; ++i; }
+                    const double s = __ldcg(&ctl->sample_sums[gen_s & 1u][p]);
+                    sgram[i * KT + i + rem] = s;
+                    sgram[(i + rem) * KT + i] = s;
+                }
+                __syncwarp();
+                const unsigned int guess = a.ring.K > 0 ? warp_ring_guess<KT>(a.ring, sgram) : warp_guess<KT>(sgram, a.replay.tau);
+                if (lane == 0) sh_pred = guess;
+            }
+        }
+        Sync::sync();
+        pred = sh_pred;
+    }
+    if (pred) {
+        const unsigned int bits = pred & 0xFFu, before = bits & ((1u << ((pred >> 8) & 0xFu)) - 1u), from = bits ^ before;
+        const CountDivider div(__popc(bits));
+        for (int w = group; w < S; w += NG) {
+            process(false_type(), true_type(), w % kStages, from, before, div);
+            release(w);
+        }
+        for (; v < rounds; v += NG) {
+            wait_full(v);
+            process(true_type(), true_type(), v % kStages, from, before, div);
+            release(v);
+        }
+    } else {
+        const CountDivider none(1);
+        for (int w = group; w < S; w += NG) release(w);
+        for (; v < rounds; v += NG) {
+            wait_full(v);
+            process(true_type(), false_type(), v % kStages, 0u, 0u, none);
+            release(v);
+        }
     }
     flush();
-    __syncthreads();
+    if constexpr (!ONE) {
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        __syncthreads();                    // (lets the producer go)
+    } else {
+        Sync::sync();
+    }
     if (tid < NP) {
-        // the 16 warps' sums in four short chains (a fixed order, so still reproducible)
-        double s4[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            s4[c] = sacc[4 * c][tid];
-#pragma unroll
-            for (int w = 1; w < 4; ++w) s4[c] += sacc[4 * c + w][tid];
+        double s = cta_sum();
+        if (blockIdx.x == 0 && Dv < a.D) {
+            // the last elements, which no copy covers
+            int i = 0, rem = tid;
+            while (rem >= KT - i) { rem -= KT - i; ++i; }
+            const T *x = static_cast<const T *>(a.g[i]), *y = static_cast<const T *>(a.g[i + rem]);
+            for (int64_t e = Dv; e < a.D; ++e) s += (double)load1<T>(x, e) * (double)load1<T>(y, e);
         }
-        a.partials[(size_t)tid * kGsPartialStride + blockIdx.x] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+        a.partials[(size_t)tid * kFilterMaxCtas + blockIdx.x] = s;
     }
-    __syncthreads();
+    Sync::sync();
 
-    // ---- decide: arrive, wait until every CTA has, then total the partials and walk Algorithm 1 here ----
+    // ---- decide ----
     if (tid == 0) {
-        red_release_add_u32(&ctl->fused_arrivals, blockIdx.x == 0 ? kFusedCallUnit - (gridDim.x - 1) : 1u);
-        unsigned int polls = 0;
-        bool ok = true;
-        // (the acquire orders the loads of the partials below, through the barrier, after every CTA's stores)
-        while ((ld_acquire_u32(&ctl->fused_arrivals) >> kFusedCallShift) == gen0 || a.test_withhold) {
-            __nanosleep(20);
-            if (++polls > a.spin_limit) { ok = false; break; }
+        if constexpr (ONE) {
+            arrive(&ctl->fused_arrivals);
+            sh_ok = wait_all(&ctl->fused_arrivals, gen0, a.spin_limit) ? 1 : 0;
+        } else {
+            if (pred) atomicAdd(&ctl->written_ctas, 1u);
+            sh_ok = take_last_ticket(&ctl->ticket, gridDim.x) ? 1 : 0;
         }
-        n_list = ok ? 0 : -1;
-        if (!ok) atomicOr(&ctl->status, GAF_STATUS_TIMEOUT);
     }
-    __syncthreads();
-    if (n_list < 0) return;                 // every CTA has arrived all the same: the counter is whole again
-    const bool publisher = blockIdx.x == 0;
-    total_gram_partials<KT>(a.partials, gridDim.x, sgram, publisher ? a.gram : nullptr);
-    __syncthreads();
+    Sync::sync();
+    if (!sh_ok) {
+        if constexpr (ONE) {
+            // every CTA has arrived all the same: the counter is whole again
+            if (tid == 0) atomicOr(&ctl->status, GAF_STATUS_TIMEOUT);
+            __syncthreads();
+        }
+        return;
+    }
+    const bool publisher = !ONE || blockIdx.x == 0;
     {
-        // every CTA takes the same sums in the same order, hence the same decisions; one of them writes them out
-        auto take = [&](int seed, unsigned long long bits) {
+        // totals of all CTAs' sums in a fixed order: one warp per pair, all its loads issued before the first addition
+        constexpr int PW = (NP + CW - 1) / CW, R = kFilterMaxCtas / 32;
+        double part[PW][R];
+#pragma unroll
+        for (int w = 0; w < PW; ++w)
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                const int p = warp + w * CW, i = lane + 32 * k;
+                part[w][k] = (p < NP && i < (int)gridDim.x) ? __ldcg(a.partials + (size_t)p * kFilterMaxCtas + i) : 0.0;
+            }
+#pragma unroll
+        for (int w = 0; w < PW; ++w) {
+            const int p = warp + w * CW;
+            double s = 0.0;
+#pragma unroll
+            for (int k = 0; k < R; ++k) s += part[w][k];
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) s += shfl_down_f64(s, d);
+            if (lane == 0 && p < NP) {
+                int i = 0, rem = p;
+                while (rem >= KT - i) { rem -= KT - i; ++i; }
+                const int j = i + rem;
+                sgram[i * KT + j] = s;
+                sgram[j * KT + i] = s;
+                if (publisher) { a.gram[i * KT + j] = s; a.gram[j * KT + i] = s; }
+            }
+        }
+        Sync::sync();
+    }
+    if constexpr (!ONE) {
+        if (a.pair_dist_out != nullptr) {
+            // pairwise mode: Eq. 4 for every pair
+            if (tid < KT * KT) {
+                const int i = tid / KT, j = tid % KT;
+                const double gii = sgram[i * KT + i], gjj = sgram[j * KT + j], gij = sgram[tid];
+                int status = 0;
+                const double d = (i == j && gii > 0.0) ? 0.0 : cosine_distance(gij, gii, gjj, &status);
+                a.pair_dist_out[tid] = (float)d;
+                if (a.pair_gram_out) a.pair_gram_out[tid] = gij;
+                if (status) atomicOr(&ctl->status, status);
+            }
+            return;
+        }
+    }
+    // (one-launch form: every CTA takes the same sums in the same order, hence the same decisions)
+    {
+        auto known = [&](int seed, unsigned long long bits) {
             const int start = seed < 0 ? 0 : seed;
             int n = 0;
             for (int t = 0; t < KT; ++t) {
                 const int i = (start + t) % KT;
-                if ((bits >> i) & 1ull) { list[n] = static_cast<const T *>(a.g[i]); list_row[n] = i; ++n; }
+                if ((bits >> i) & 1ull) list[n++] = static_cast<const T *>(a.g[i]);
             }
             n_list = n;
+            sh_final = pack_pattern((unsigned int)bits, start);
+            if (ONE) sh_again = (!resident && sh_final != pred) ? 1 : 0;
         };
         if (a.ring.K > 0) {
-            __shared__ RingTable<KT> ring_table;
-            ring_replay_parallel<KT>(a.ring, sgram, ring_table, take, publisher);
+            __shared__ RingTable<KT> table;
+            ring_replay_parallel<KT, Sync>(a.ring, sgram, table, known, publisher);
         } else {
             __shared__ ReplayTable table;
-            replay_on_gram_parallel<KT>(a.replay, sgram, table, [&](unsigned long long bits) { take(-1, bits); }, publisher);
+            replay_on_gram_parallel<KT, Sync>(a.replay, sgram, table, [&](unsigned long long bits) { known(-1, bits); }, publisher);
         }
+        Sync::sync();
     }
-    __syncthreads();
-    const int n = n_list;
-    const float cdiv = (float)n;
-    // the launch behind this one on the stream may be placed from here on (it waits for this grid itself)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // two gradients: when the first pass guessed right, it has written the result already (the same additions and
-    // the same division as below).  Otherwise every thread overwrites, below, exactly what it wrote then.
-    if constexpr (kSpeculative) {
-        const bool seed_alone = n == 1 && list_row[0] == 0;     // (the order-indifferent variant may keep row 1 alone)
-        const unsigned int outcome = n == 1 ? 1u : 0u;
-        if (publisher && tid == 0) ctl->pair_hint = outcome == (hint & 1u) ? outcome : (2u | outcome);
-        if (guessing && (guess_seed_alone ? seed_alone : n == 2)) return;
+    const int c = n_list;
+    if constexpr (!ONE) {
+        if (tid == 0) {
+            // (the ticket ordered every CTA's count before this read)
+            const unsigned int written = __ldcg(&ctl->written_ctas);
+            ctl->written_ctas = 0u;
+            ctl->mean_done = (written == gridDim.x && pred == sh_final) ? 1 : 0;
+        }
+    } else {
+        // the launch behind this one on the stream may be placed from here on (it waits for this grid itself)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        __syncthreads();                    // the producer learns whether it is wanted again
     }
-
-    // ---- pass 2a: the rounds that were not parked, last first (what pass 1 read last is what L2 still
-    //      holds), several rounds in flight per thread; specialised on the number of accepted gradients ----
-    auto pass2a = [&](auto nn_tag) {
-        constexpr int NN = decltype(nn_tag)::value;
-        constexpr int U = FusedInFlight<NN>::U;
-        for (int64_t j0 = rounds - 1; j0 >= parked_rounds; j0 -= U) {
-            int64_t q[U];
-            bool ok[U];
-            uint4 w[U][NN];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int64_t ju = j0 - u;
-                q[u] = warp_first + ju * stride + lane;
-                ok[u] = ju >= parked_rounds && q[u] < n_vec;
-#pragma unroll
-                for (int i = 0; i < NN; ++i)
-                    if (ok[u]) w[u][i] = ld16_policy(list[i] + q[u] * N, pol_first);
+    // the last elements, which no copy covers (two launches: the second may have nothing to do)
+    if ((!ONE || blockIdx.x == 0) && Dv + tid < a.D) {
+        const int64_t e = Dv + tid;
+        float x = load1<T>(list[0], e);
+        for (int i = 1; i < c; ++i) x += load1<T>(list[i], e);
+        a.out[e] = x / (float)c;
+    }
+    if constexpr (ONE) {
+        const CountDivider div(c);
+        if (resident) {
+            const unsigned int bits = sh_final & 0xFFu, before = bits & ((1u << ((sh_final >> 8) & 0xFu)) - 1u);
+            for (int w = group; w < rounds; w += NG) process(false_type(), true_type(), w, bits ^ before, before, div);
+        } else if (sh_again) {
+            // the accepted gradients again, compacted to the first rows of a tile in the order they are added (the
+            // tiles go on alternating between the groups)
+            for (int it = rounds + (group + NG - rounds % NG) % NG; it < 2 * rounds; it += NG) {
+                wait_full(it);
+                process(false_type(), true_type(), it % kStages, (1u << c) - 1u, 0u, div);
+                release(it);
             }
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (ok[u]) {
-                    float v[N];
-                    FusedVec<T>::widen(w[u][0], v);
-#pragma unroll
-                    for (int i = 1; i < NN; ++i) {
-                        float x[N];
-                        FusedVec<T>::widen(w[u][i], x);
-#pragma unroll
-                        for (int k = 0; k < N; ++k) v[k] += x[k];
-                    }
-#pragma unroll
-                    for (int k = 0; k < N; ++k) v[k] = v[k] / cdiv;
-                    store_vec_streaming<N>(a.out + q[u] * N, v);
-                }
         }
-    };
-    switch (n) {
-        case 1: pass2a(std::integral_constant<int, 1>()); break;
-        case 2: if constexpr (KT >= 2) pass2a(std::integral_constant<int, 2>()); break;
-        case 3: if constexpr (KT >= 3) pass2a(std::integral_constant<int, 3>()); break;
-        case 4: if constexpr (KT >= 4) pass2a(std::integral_constant<int, 4>()); break;
-        case 5: if constexpr (KT >= 5) pass2a(std::integral_constant<int, 5>()); break;
-        case 6: if constexpr (KT >= 6) pass2a(std::integral_constant<int, 6>()); break;
-        case 7: if constexpr (KT >= 7) pass2a(std::integral_constant<int, 7>()); break;
-        default: if constexpr (KT >= 8) pass2a(std::integral_constant<int, 8>()); break;
-    }
-    // ---- pass 2b: the parked rounds, from shared memory ----
-    for (int64_t j = 0; j < parked_rounds; ++j) {
-        const int64_t q = warp_first + j * stride + lane;
-        if (q < n_vec) {
-            const uint4 *slot = parked + (size_t)j * KT * kGsThreads + tid;
-            float v[N];
-            FusedVec<T>::widen(slot[list_row[0] * kGsThreads], v);
-            for (int i = 1; i < n; ++i) {
-                float x[N];
-                FusedVec<T>::widen(slot[list_row[i] * kGsThreads], x);
-#pragma unroll
-                for (int k = 0; k < N; ++k) v[k] += x[k];
-            }
-#pragma unroll
-            for (int k = 0; k < N; ++k) v[k] = v[k] / cdiv;
-            store_vec_streaming<N>(a.out + q * N, v);
-        }
-    }
-    if (blockIdx.x == 0 && tail0 + tid < a.D) {
-        const int64_t e = tail0 + tid;
-        float v = load1<T>(list[0], e);
-        for (int i = 1; i < n; ++i) v += load1<T>(list[i], e);
-        a.out[e] = v / cdiv;
     }
 }
 

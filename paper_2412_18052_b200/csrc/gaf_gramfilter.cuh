@@ -90,7 +90,7 @@ __device__ __forceinline__ unsigned long long replay_on_gram(const ReplayArgs &r
 // accept pattern of steps 1..t-1) evaluates Eq. 4 for that case -- 2^(K-1) - 1 threads, all at once --
 // and thread 0 then only follows the decisions through the table.  Every case repeats the sums of
 // the sequential walk in the same order, so the results are the same to the last bit.
-// All threads of the block call (blockDim.x >= 128).  `early(bits)` is called by thread 0 as soon as
+// `Sync` stands for the threads that call (at least 128, thread 0 among them).  `early(bits)` is called by thread 0 as soon as
 // the accept bits are known, before the outputs are written.  With `publish` false nothing is written
 // to global memory (the one-launch schedule runs the walk in every CTA and lets one of them publish).
 struct ReplayTable {
@@ -100,7 +100,7 @@ struct ReplayTable {
 struct NoEarlyBits {
     __device__ __forceinline__ void operator()(unsigned long long) const {}
 };
-template <int KT, typename Early = NoEarlyBits>
+template <int KT, typename Sync, typename Early = NoEarlyBits>
 __device__ __forceinline__ void replay_on_gram_parallel(const ReplayArgs &r, const double *gram, ReplayTable &tb,
                                                         Early early = Early(), bool publish = true) {
     constexpr int K = KT;
@@ -139,7 +139,7 @@ __device__ __forceinline__ void replay_on_gram_parallel(const ReplayArgs &r, con
         tb.accept[tid] = (unsigned char)accept;
         tb.status[tid] = (unsigned char)status;
     }
-    __syncthreads();
+    Sync::sync();
     if (tid == 0) {
         unsigned int m = 0;
         int node[kReplayMaxK];
@@ -261,7 +261,7 @@ __device__ __forceinline__ void ring_replay_on_gram(const RingArgs &r, const vol
 // ORIGINAL index (step v of seed s is gradient (s + v) mod K), one thread per seed then follows its
 // decisions through the table, and thread 0 picks the largest count (ties to the smallest seed) and
 // publishes.  Same sums in the same order as ring_walk_one_seed: identical outputs.
-// All threads of the block call; `early(seed, bits)` as in ring_replay_on_gram; `publish` as in
+// All threads of `Sync` call; `early(seed, bits)` as in ring_replay_on_gram; `publish` as in
 // replay_on_gram_parallel.
 template <int KT>
 struct RingTable {
@@ -271,11 +271,11 @@ struct RingTable {
     int count[KT];
     unsigned int steps[KT];                                     // bit t-1 = step t of this seed accepted
 };
-template <int KT, typename Early = NoEarlyNotice>
+template <int KT, typename Sync, typename Early = NoEarlyNotice>
 __device__ __forceinline__ void ring_replay_parallel(const RingArgs &r, const double *gram, RingTable<KT> &tb,
                                                      Early early = Early(), bool publish = true) {
     constexpr int K = KT, C = RingTable<KT>::kCases;
-    for (int idx = threadIdx.x; idx < K * C; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < K * C; idx += Sync::threads()) {
         const int s = idx / C, cs = idx - s * C;
         const int t = 32 - __clz(cs + 1);
         const unsigned int m = (unsigned int)(cs + 1) - (1u << (t - 1));
@@ -306,7 +306,7 @@ __device__ __forceinline__ void ring_replay_parallel(const RingArgs &r, const do
         tb.accept[idx] = (unsigned char)accept;
         tb.status[idx] = (unsigned char)status;
     }
-    __syncthreads();
+    Sync::sync();
     if ((int)threadIdx.x < K) {
         const int s = threadIdx.x;
         unsigned int m = 0;
@@ -318,7 +318,7 @@ __device__ __forceinline__ void ring_replay_parallel(const RingArgs &r, const do
         tb.count[s] = count;
         tb.steps[s] = m;
     }
-    __syncthreads();
+    Sync::sync();
     if (threadIdx.x == 0) {
         int best = 0;
         for (int s = 1; s < K; ++s)
@@ -349,21 +349,6 @@ __device__ __forceinline__ void ring_replay_parallel(const RingArgs &r, const do
         __threadfence();
     }
 }
-
-// ------------------------------------------------ one-pass Gram for K <= 8 ----
-
-struct GramSmallArgs {
-    const void *g[kGsMaxK];                 // processing order
-    int64_t D;
-    int64_t keep_from;                      // elements from here on are loaded "keep in L2"
-    double *partials;                       // [pair][kGsPartialStride]
-    double *gram;                           // [K][K]
-    ReplayArgs replay;                      // used when pair_dist_out is null and ring.K == 0
-    float *pair_dist_out;                   // pairwise mode: K x K distances instead of the walk
-    double *pair_gram_out;                  // pairwise mode: optional copy of the Gram matrix
-    RingArgs ring;                          // any-seed mode when ring.K > 0 (rows are in original order)
-    int mma_run;                            // gram_mma_kernel: trips per run of a CTA (even, >= 2)
-};
 
 // 16-byte read-only load with an explicit L2 eviction policy.
 __device__ __forceinline__ uint4 ld16_policy(const void *p, uint64_t policy) {
@@ -407,49 +392,6 @@ template <> struct GsVec<__nv_bfloat16> {
     }
 };
 
-// Fixed-order totals of the per-CTA partial sums ([pair][CTA] layout), by the whole calling block:
-// one warp per pair (several pairs per warp when there are more pairs than warps, all loads issued
-// before the first add: this is the serial tail of the call), lane-strided sums, then a shuffle tree.
-// Fills the symmetric K x K matrix in shared memory and, when `gram_out` is given, in global memory.
-template <int KT>
-__device__ __forceinline__ void total_gram_partials(const double *part, int n_ctas, double *sgram, double *gram_out) {
-    constexpr int NP = KT * (KT + 1) / 2;
-    constexpr int kWarps = kGsThreads / 32;
-    constexpr int PW = (NP + kWarps - 1) / kWarps;             // pairs per warp
-    constexpr int kRounds = (kGsMaxCtas + 31) / 32;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double v[PW][kRounds];
-#pragma unroll
-    for (int w = 0; w < PW; ++w) {
-        const int p = warp + w * kWarps;
-#pragma unroll
-        for (int k = 0; k < kRounds; ++k) {
-            const int i = lane + 32 * k;
-            v[w][k] = (p < NP && i < n_ctas) ? __ldcg(part + (size_t)p * kGsPartialStride + i) : 0.0;
-        }
-    }
-#pragma unroll
-    for (int w = 0; w < PW; ++w) {
-        const int p = warp + w * kWarps;
-        double s = 0.0;
-#pragma unroll
-        for (int k = 0; k < kRounds; ++k) s += v[w][k];
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) s += shfl_down_f64(s, d);
-        if (lane == 0 && p < NP) {
-            int r = 0, rem = p;                                 // decode p -> (r, c), r <= c
-            while (rem >= KT - r) { rem -= KT - r; ++r; }
-            const int c = r + rem;
-            sgram[r * KT + c] = s;
-            sgram[c * KT + r] = s;
-            if (gram_out) {
-                gram_out[r * KT + c] = s;
-                gram_out[c * KT + r] = s;
-            }
-        }
-    }
-}
-
 // Accumulator of the register-tiled Gram kernels (K <= 8).
 // binary32 inputs, up to 4 gradients: binary64.  A product of two binary32 values is exact in binary64, so
 // the Gram sums are exact up to binary64 rounding and need no periodic flush; binary64 FMAs (half the
@@ -468,139 +410,6 @@ template <> struct GsAcc<float, 3> { using type = double; static constexpr bool 
 template <> struct GsAcc<float, 4> { using type = double; static constexpr bool kPeriodicFlush = false; };
 __device__ __forceinline__ float gs_fma(float a, float b, float s) { return fmaf(a, b, s); }
 __device__ __forceinline__ double gs_fma(float a, float b, double s) { return fma((double)a, (double)b, s); }
-
-// What every one-pass Gram kernel for K <= 8 does once its warps have left their sums in
-// sacc[warp][pair] (upper triangle, row-major pair index): per-CTA partial sums in a fixed order,
-// last-CTA election, fixed-order totals, then the walk of Algorithm 1 (or the any-seed walks, or the
-// pairwise distances).  All threads of the block call.
-template <int KT>
-__device__ __forceinline__ void gram_small_tail(const GramSmallArgs &a, double (*sacc)[KT * (KT + 1) / 2]) {
-    constexpr int NP = KT * (KT + 1) / 2;
-    __shared__ bool is_last;
-    // the streaming part of this CTA is over: a kernel launched as a programmatic dependent
-    // (the masked-mean pass) may start occupying SMs; it still waits for this whole grid
-    // before it reads anything
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    __syncthreads();
-    if (threadIdx.x < NP) {
-        // the 16 warps' sums in four short chains (a fixed order, so still reproducible)
-        double s4[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            s4[c] = sacc[4 * c][threadIdx.x];
-#pragma unroll
-            for (int w = 1; w < 4; ++w) s4[c] += sacc[4 * c + w][threadIdx.x];
-        }
-        a.partials[(size_t)threadIdx.x * kGsPartialStride + blockIdx.x] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = take_last_ticket(&a.replay.ctl->ticket, gridDim.x);
-    __syncthreads();
-    if (!is_last) return;
-
-    // last CTA: fixed-order totals (one warp per pair; all of a lane's loads are issued together,
-    // this is the serial tail of the call), then the scalar walk out of shared memory
-    __shared__ double sgram[KT * KT];
-    total_gram_partials<KT>(a.partials, gridDim.x, sgram, a.gram);
-    __syncthreads();
-    if (a.ring.K > 0) {
-        __shared__ RingTable<KT> ring_table;
-        ring_replay_parallel<KT>(a.ring, sgram, ring_table);
-        return;
-    }
-    if (a.pair_dist_out == nullptr) {
-        __shared__ ReplayTable table;
-        replay_on_gram_parallel<KT>(a.replay, sgram, table);
-        return;
-    }
-    // pairwise mode: Eq. 4 for every pair
-    if (threadIdx.x < KT * KT) {
-        const int i = threadIdx.x / KT, j = threadIdx.x % KT;
-        const double gii = sgram[i * KT + i], gjj = sgram[j * KT + j], gij = sgram[threadIdx.x];
-        int status = 0;
-        const double d = (i == j && gii > 0.0) ? 0.0 : cosine_distance(gij, gii, gjj, &status);
-        a.pair_dist_out[threadIdx.x] = (float)d;
-        if (a.pair_gram_out) a.pair_gram_out[threadIdx.x] = gij;
-        if (status) atomicOr(&a.replay.ctl->status, status);
-    }
-}
-
-template <typename T, int KT>
-__global__ void __launch_bounds__(kGsThreads, (KT <= 4 ? 2 : 1)) gram_small_kernel(const __grid_constant__ GramSmallArgs a) {
-    constexpr int NP = KT * (KT + 1) / 2;   // upper triangle
-    constexpr int N = GsVec<T>::N;
-    __shared__ double sacc[kGsThreads / 32][NP];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.replay.ctl->status = 0;      // first kernel of the operation
-    for (int p = lane; p < NP; p += 32) sacc[warp][p] = 0.0;
-    __syncwarp();
-
-    const T *row[KT];
-#pragma unroll
-    for (int r = 0; r < KT; ++r) row[r] = static_cast<const T *>(a.g[r]);
-
-    using Acc = typename GsAcc<T, KT>::type;
-    Acc acc[NP];
-#pragma unroll
-    for (int p = 0; p < NP; ++p) acc[p] = Acc(0);
-
-    auto flush = [&]() {
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            Acc v = acc[p];
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, d);
-            if (lane == 0) sacc[warp][p] += (double)v;
-            acc[p] = Acc(0);
-        }
-    };
-
-    // The masked-mean pass that follows walks the vectors from their end: the tail of
-    // this pass is loaded "evict last" so that it is still in L2 then; the head, which
-    // cannot survive anyway, is loaded "evict first".
-    const uint64_t pol_first = l2_policy_evict_first(), pol_last = l2_policy_evict_last();
-    const int64_t n_vec = a.D / N;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    int since_flush = 0;
-    // The trip count is the same for all lanes of a warp (the bound is tested on the warp's first
-    // vector): the flush below shuffles across the whole warp, so the lanes must reach it together.
-    const int64_t warp_first = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31);
-    for (int64_t qw = warp_first; qw < n_vec; qw += stride) {
-        const int64_t q = qw + lane;
-        if (q < n_vec) {
-            float x[KT][N];
-            const uint64_t pol = (q * N >= a.keep_from) ? pol_last : pol_first;
-#pragma unroll
-            for (int r = 0; r < KT; ++r) GsVec<T>::load(row[r], q * N, pol, x[r]);
-            int p = 0;
-#pragma unroll
-            for (int r = 0; r < KT; ++r)
-#pragma unroll
-                for (int c = r; c < KT; ++c, ++p) {
-                    Acc s = acc[p];
-#pragma unroll
-                    for (int k = 0; k < N; ++k) s = gs_fma(x[r][k], x[c][k], s);
-                    acc[p] = s;
-                }
-        }
-        if (GsAcc<T, KT>::kPeriodicFlush && ++since_flush == kGsFlushEvery) { flush(); since_flush = 0; }
-    }
-    // ragged tail (D mod N elements), first CTA
-    const int64_t tail0 = n_vec * N;
-    if (blockIdx.x == 0 && tail0 + threadIdx.x < a.D) {
-        const int64_t e = tail0 + threadIdx.x;
-        float x[KT];
-#pragma unroll
-        for (int r = 0; r < KT; ++r) x[r] = load1<T>(row[r], e);
-        int p = 0;
-#pragma unroll
-        for (int r = 0; r < KT; ++r)
-#pragma unroll
-            for (int c = r; c < KT; ++c, ++p) acc[p] = gs_fma(x[r], x[c], acc[p]);
-    }
-    flush();
-    gram_small_tail<KT>(a, sacc);
-}
 
 // Scalar walk as its own launch (Gram matrix produced by the tiled pairwise kernels).
 // `perm` maps processing step -> row of `gram_by_index` (K x K by original index).
@@ -660,6 +469,7 @@ struct MaskedMeanArgs {
     float *out;
     const Control *ctl;
     int run;                                // chunks (of one CTA's 512 groups of 8 elements) a CTA takes in a row
+    int may_be_done;                        // the Gram pass may have written the mean already (ctl->mean_done)
 };
 
 // out = (((g_0 + g_a) + g_b) + ...) / c over the accepted steps a < b < ..., binary32,
@@ -680,15 +490,16 @@ __global__ void __launch_bounds__(kMsThreads, 2) masked_mean_kernel(const __grid
     // completed and its writes (the accept bits) are visible; otherwise a no-op
     asm volatile("griddepcontrol.wait;" ::: "memory");
     unsigned long long bits = 0;
-    int seed = -1;
+    int seed = -1, done = 0;
     if (threadIdx.x == 0) {
-        bits = __ldcg(&a.ctl->accept_bits);                      // (two independent L2 loads)
+        bits = __ldcg(&a.ctl->accept_bits);                      // (independent L2 loads)
         seed = __ldcg(&a.ctl->ring_seed);
+        if (a.may_be_done) done = __ldcg(&a.ctl->mean_done);
     }
     if (threadIdx.x == 0) {
         const int start = seed < 0 ? 0 : seed;
         int n = 0;
-        for (int t = 0; t < a.K; ++t) {
+        for (int t = 0; t < a.K && !done; ++t) {
             const int i = (start + t) % a.K;
             if ((bits >> i) & 1ull) list[n++] = static_cast<const T *>(a.g[i]);
         }
@@ -697,6 +508,7 @@ __global__ void __launch_bounds__(kMsThreads, 2) masked_mean_kernel(const __grid
     }
     __syncthreads();
     const int n = n_list;
+    if (n == 0) return;                             // written by the Gram pass
     const float cdiv = cdiv_s;
     const int64_t n_oct = a.D / kOct;
     // U groups of 8 elements per thread and round (two for 2-byte inputs, so that as many bytes

@@ -683,6 +683,54 @@ def test_two_gradients_mean_written_in_the_first_pass(ws, dtype):
     check_filter(big.grads, 0.0, ws)
 
 
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("K", [2, 3, 4, 5, 6, 7, 8])
+def test_predicted_accept_pattern_right_and_wrong(ws, K, dtype):
+    """The Gram-first forms for up to 8 gradients write the mean under a pattern predicted from a sample.  Lengths on
+    both sides of what stays in shared memory as a whole, ragged and whole last tiles, and two kinds of inputs: mixtures, which a
+    sample predicts, and gradients whose last few elements outweigh all others, which it cannot.  Mask, distances and
+    mean against the oracle, and the mean bit for bit against the stepwise schedule."""
+    b = 4 if dtype == "f32" else 2
+    ring = 190_000 // (K * b) * 148                                  # elements the SMs' shared memory holds, roughly
+    for n, D in enumerate((ring * 3 // 4 + 5, ring + ring // 8 + 64, 3 * ring + 3)):
+        w = _mix(K, D, dtype, seed=50 * K + n, rho=[0.8] + [0.7, -0.6, 0.5, 0.0, 0.6, -0.2, 0.4][:K - 1])
+        misled = [g.clone() for g in w.grads]
+        for i, g in enumerate(misled):                               # every decision turns round at the end of the vectors
+            g[-40:] = (1.0 if i % 3 == 2 else -1.0) * (1.0 if i else -1.0) * 4.0 * (D ** 0.5) * 1e-3 / 6.0
+        for grads in (w.grads, misled):
+            for tau in (0.9, 2.0):
+                plain = gaf.gaf_filter_accumulate(grads, tau, ws, schedule=gaf.GAF_SCHED_STEPWISE)
+                plain = [t.clone() for t in plain]
+                for schedule in (gaf.GAF_SCHED_GRAM_FUSED, gaf.GAF_SCHED_GRAM):
+                    got = gaf.gaf_filter_accumulate(grads, tau, ws, schedule=schedule)
+                    assert torch.equal(got[1], plain[1]) and torch.equal(got[3], plain[3])
+                    assert torch.equal(got[0], plain[0]), (K, D, tau, schedule)
+                    assert float((got[2] - plain[2]).abs().max()) < 2e-5
+            if n == 1:
+                check_filter(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM_FUSED)
+                check_any_seed(grads, 0.9, ws)
+
+
+def test_division_by_the_count_is_correctly_rounded(ws):
+    """The mean's division by c (3, 5, 6, 7: two multiply-adds; powers of two: a multiplication) against the division
+    itself: significands across the range, zeros, subnormal and huge values, infinities."""
+    torch.manual_seed(3)
+    for c in range(2, 9):
+        x = torch.randint(-(1 << 31), (1 << 31) - 1, (400_003,), dtype=torch.int64, device="cuda").to(torch.int32).view(torch.float32)
+        x = torch.where(torch.isnan(x), torch.zeros_like(x), x)
+        x[100_000:300_000] = torch.randn(200_000, device="cuda") * 1e-3
+        x[:8] = torch.tensor([0.0, -0.0, 1e-45, -1e-45, 3.4e38, float("inf"), float("-inf"), 1e-38], device="cuda")
+        zeros = torch.zeros_like(x)                                  # tau = 2 accepts them: the sum stays x
+        macro, mask, dist, count = gaf.gaf_filter_accumulate([x] + [zeros] * (c - 1), 2.0, ws, schedule=gaf.GAF_SCHED_GRAM_FUSED)
+        if int(count.item()) != c:                                   # (infinite sums: everything but the seed is rejected)
+            x[5:7] = 1.0
+            x = x.clamp(-1e15, 1e15)
+            macro, mask, dist, count = gaf.gaf_filter_accumulate([x] + [zeros] * (c - 1), 2.0, ws, schedule=gaf.GAF_SCHED_GRAM_FUSED)
+        assert int(count.item()) == c
+        want = x / torch.full_like(x, float(c))
+        assert torch.equal(macro, want), c
+
+
 def test_wide_mma_gram_kernel_shapes_and_long_runs(ws):
     """9..16 bfloat16 gradients (and the first counts of the tcgen05 tile behind them): absent rows feed zeros;
     lengths below one tile, ragged ends, and a length from which the CTAs walk in runs of several trips."""
