@@ -112,8 +112,11 @@ enum {
                                    written while the inputs are read for the full sums.  A call whose
                                    decisions come out as predicted moves (K b + 4) D bytes and has no second
                                    pass over the gradients; one that does not rewrites the output.  The
-                                   values never depend on the prediction.  (GAF_SCHED_GRAM with K <= 8
-                                   does the same; its second launch then has nothing to do.)
+                                   values never depend on the prediction.  With K = 2, where the result
+                                   can only be the mean of both or the seed alone, a call takes the
+                                   pattern that the latest two such calls on the workspace both ended
+                                   with, if they did, instead of a sample's.  (GAF_SCHED_GRAM with K <= 8
+                                   predicts too; its second launch then has nothing to do.)
                                    GAF_SCHED_AUTO takes this form for K = 2 at every length. */
 };
 

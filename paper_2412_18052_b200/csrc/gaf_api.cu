@@ -171,7 +171,12 @@ size_t gram_partials_bytes(int K) {
     return pairs * kGramMaxSlices * 64 * sizeof(double);
 }
 size_t gram_matrix_bytes(int K) { return round_up(size_t(K) * K * sizeof(double), 256); }
-static_assert(size_t(36) * kFilterMaxCtas <= size_t(kGramMaxSlices) * 64, "the one-pass kernel's [pair][CTA] partial sums");
+// One-pass kernel for 2 to 8 gradients: [pair][CTA] sums of the whole vectors, then those of the sample (both inside
+// what gram_partials_bytes reserves).
+// (the CTAs' lines lie where the stepwise schedule has its partial sums)
+constexpr size_t kFilterSumsBytes = size_t(36) * kFilterMaxCtas * sizeof(TaggedSum);
+static_assert(kFilterSumsBytes + size_t(36) * kFilterMaxCtas * 8 <= size_t(kGramMaxSlices) * 64 * sizeof(double), "workspace layout");
+static_assert(size_t(2) * kFilterMaxCtas * 128 <= kPartialsBytes, "workspace layout");
 // Bucketed variant: partial slots [ctas + buckets][64] doubles and one bit mask per bucket.
 size_t bucketed_extra_bytes() {
     return size_t(kBkMaxCtas + kBkMaxBuckets) * 64 * sizeof(double) + size_t(kBkMaxBuckets) * 8;
@@ -417,14 +422,17 @@ struct FusedGuard {
     bool any = false;
 };
 FusedGuard g_fused_guard[kMaxDevices];
+std::atomic<unsigned int> g_fused_tag{1};               // tags the sums that the CTAs of one launch exchange
 
 // Tiles, rounds and sample of gram_filter_kernel (one- and two-launch form alike: same sums, same order).
-#ifndef GAF_SAMPLE_SHORT
-#define GAF_SAMPLE_SHORT 2
-#endif
-#ifndef GAF_FILTER_RUN
-#define GAF_FILTER_RUN 1
-#endif
+// The accept pattern is predicted from kPredictRings ring fillings on (50 MB of gradients).  The wait for the prediction costs
+// about 6 us; a second pass over what has left the rings costs little as long as L2 holds it.  Measured without / with:
+// 4 fp32 gradients of 2 / 3 / 5 / 8 / 11.2 M elements 14.6 / 19.1 / 29.3 / 45.5 / 62.5 against 16.9 / 19.7 / 25.9 / 36.6 / 46.6 us.
+// The sample is two tiles per CTA (half a million elements with 4 gradients; one tile is no faster), half a ring on
+// vectors so long that the wait does not count.
+constexpr int kPredictRings = 2;
+constexpr int kSampleTiles = 2;
+constexpr int kLongRounds = 64;
 template <typename T, int KT>
 int filter_shape(GramFusedArgs &a, const DeviceInfo &di, bool predict) {
     using Tile = FilterTile<T, KT>;
@@ -438,10 +446,11 @@ int filter_shape(GramFusedArgs &a, const DeviceInfo &di, bool predict) {
     const int64_t te = (a.D + grid * rounds - 1) / (grid * rounds);
     a.tile_elems = int((te + 63) / 64 * 64);
     if (a.tile_elems < 64) a.tile_elems = 64;
-    a.run = rounds >= 256 ? GAF_FILTER_RUN : 1;
-    a.rounds = int((rounds + a.run - 1) / a.run * a.run);
+    a.rounds = int(rounds);
     a.sample = 0;
-    if (predict && a.rounds > Tile::kStages) a.sample = a.rounds < 64 ? GAF_SAMPLE_SHORT : Tile::kStages / 2;
+    // (two gradients: the kernel has a guess without a sample most of the time)
+    if (predict && rounds > (KT == 2 ? 1 : kPredictRings) * Tile::kStages)
+        a.sample = rounds < kLongRounds ? kSampleTiles : Tile::kStages / 2;
     return int(grid);
 }
 
@@ -468,6 +477,7 @@ int launch_gram_fused_kt(GramFusedArgs &a, const DeviceInfo &di, cudaStream_t st
     const int grid = filter_shape<T, KT>(a, di, true);
     a.spin_limit = g_test_wait_limit ? g_test_wait_limit : kFusedSpinLimit;
     a.test_withhold = g_test_withhold;
+    a.tag = g_fused_tag.fetch_add(1, std::memory_order_relaxed);
     // The grid is no larger than what the device holds at once (occupancy above), so all its CTAs become
     // resident and the one wait on other CTAs ends; it is bounded in any case.  Programmatic stream
     // serialisation: the kernel waits for its predecessor on the stream itself (griddepcontrol.wait, first
@@ -521,6 +531,7 @@ template <typename T, int KT>
 int launch_gram_filter_kt(GramFusedArgs &a, const DeviceInfo &di, cudaStream_t st) {
     if (int rc = filter_plan<T, KT, false>(di)) return rc;
     const int grid = filter_shape<T, KT>(a, di, a.pair_dist_out == nullptr);
+    a.spin_limit = kFusedSpinLimit;
     a.test_withhold = 0;
     const cudaError_t err = launch_dependent_smem(gram_filter_kernel<T, KT, false>, grid, kFilterThreads,
                                                   size_t(FilterTile<T, KT>::kStages * FilterTile<T, KT>::kBytes), st, a);
@@ -568,7 +579,9 @@ int launch_gram_first(const void *const *g, int K, int64_t D, int dtype, double 
         GramFusedArgs f{};
         for (int t = 0; t < K; ++t) f.g[t] = g[ord[t]];
         f.D = D; f.out = macro_out;
-        f.partials = reinterpret_cast<double *>(base + kExtraOffset);
+        f.partials = base + kExtraOffset;
+        f.sample_partials = reinterpret_cast<unsigned long long *>(base + kExtraOffset + kFilterSumsBytes);
+        f.verdicts = reinterpret_cast<unsigned long long *>(base + kPartialsOffset);
         f.gram = gram_by_step;
         f.replay = r;
         f.ring = ring;
@@ -1081,7 +1094,7 @@ int gaf_pairwise_cosdist(const void *const *grads, int K, int64_t D, int dtype, 
         GramFusedArgs a{};
         for (int i = 0; i < K; ++i) a.g[i] = grads[i];
         a.D = D;
-        a.partials = reinterpret_cast<double *>(base + kExtraOffset);
+        a.partials = base + kExtraOffset;
         a.gram = reinterpret_cast<double *>(base + kExtraOffset + gram_partials_bytes(K));
         a.replay.ctl = reinterpret_cast<Control *>(base);
         a.pair_dist_out = dist_out;

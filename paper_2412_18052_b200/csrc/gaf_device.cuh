@@ -17,6 +17,7 @@ constexpr int kOct = 8;                 // elements handled per inner step
 // Control block at the start of the caller's workspace.
 struct Control {
     unsigned int ticket;                // last-block election, wraps to 0 by itself
+    unsigned int pair_hint;             // one-launch schedule with two gradients: what the latest two calls kept (0 both, 1 the seed alone, 2 | latest: they differed)
     unsigned int written_ctas;          // two-launch form: CTAs that wrote the predicted mean of all their elements
     int mean_done;                      // two-launch form: 1 = the first launch has written the result
     int status;                         // GAF_STATUS_* bits of the latest call
@@ -28,16 +29,7 @@ struct Control {
     float stream_dist[GAF_MAX_K];       // streaming form: distance of arrival t
     uint8_t stream_mask[GAF_MAX_K];     // streaming form: decision of arrival t
     double norm_sq_sum;                 // stepwise and streaming forms: sum of |g_i|^2 over the accepted gradients
-    // One-launch Gram-first schedule: the arrival counter its CTAs add to and poll, alone in its cache
-    // line.  Every call adds 4096 in all (one per CTA, the first CTA makes up the difference), so bits
-    // 12..31 count calls and bits 0..11 the CTAs of the running call that have arrived.
-    alignas(128) unsigned int fused_arrivals;
-    unsigned int fused_pad[31];
-    // Prediction of the accept pattern from a sample (gaf_fused.cuh): an arrival counter like the one above for
-    // the CTAs whose sample sums are in, and the sums, two sets that calls use in turn.
-    alignas(128) unsigned int sample_arrivals;
-    unsigned int sample_pad[31];
-    double sample_sums[2][36];
+    unsigned int two_launch_calls;      // calls of the two-launch form of gaf_fused.cuh so far: the tag of their sample sums
 };
 constexpr size_t kControlBytes = 4096;  // sizeof(Control) rounded up
 static_assert(sizeof(Control) <= kControlBytes, "control block");
@@ -194,20 +186,24 @@ __device__ __forceinline__ Sums3 warp_sum_partials(const double *partials, int n
 // --------------------------------------------------------------- decision ---
 
 // Eq. 4 on the three sums, in binary64:  D_c = 1 - p / (sqrt(na) sqrt(ng)),
-// with the zero-norm and clamping conventions of the header.  Returns the
+// with the zero-norm and clamping conventions of the header (`root_*` = sqrt of the norms).  Returns the
 // distance and ORs status bits into *status.
-__device__ __forceinline__ double cosine_distance(double p, double na, double ng, int *status) {
+__device__ __forceinline__ double cosine_distance(double p, double na, double ng, double root_na, double root_ng, int *status) {
     double cosv;
     if (na == 0.0 || ng == 0.0) {
         cosv = 0.0;
         *status |= GAF_STATUS_ZERO_NORM;
     } else {
-        cosv = p / (sqrt(na) * sqrt(ng));
+        cosv = p / (root_na * root_ng);
         cosv = cosv > 1.0 ? 1.0 : cosv;
         cosv = cosv < -1.0 ? -1.0 : cosv;
     }
     if (!(isfinite(p) && isfinite(na) && isfinite(ng))) *status |= GAF_STATUS_NONFINITE;
     return 1.0 - cosv;
+}
+
+__device__ __forceinline__ double cosine_distance(double p, double na, double ng, int *status) {
+    return cosine_distance(p, na, ng, sqrt(na), sqrt(ng), status);
 }
 
 // Conditioning of a running sum g of c accepted gradients.  Every schedule forms |g|^2 (and g itself)

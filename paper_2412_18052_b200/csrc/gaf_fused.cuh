@@ -8,22 +8,20 @@
 //            memory filled with bulk copies (cp.async.bulk), about 200 KB in flight per SM;
 //   sample   the first few tiles of every CTA are spread evenly over the vectors (every CTA at another phase, so
 //            that all parts of a network are represented); the consumer warps take their Gram sums and KEEP them;
-//   predict  the CTAs exchange the sample's sums, each walks Algorithm 1 on them, while the ring fills: the
-//            exchange takes about as long as HBM needs for the rest of the ring;
+//   predict  CTA 0 totals the sample's sums, walks Algorithm 1 on them and tells every CTA, while the ring fills;
 //   write    the mean under the predicted pattern is written for the kept tiles, and from then on for every
 //            tile together with its Gram sums;
 //   decide   at the end Algorithm 1 is walked on the full Gram matrix.  If it decides as predicted the
 //            result is complete; otherwise the mean is formed again from the accepted gradients.
 // The prediction decides which stores are made early, never a value: mask, distances and count come from the
 // full sums, and the mean is the same additions in the same order (binary32, processing order, one division by
-// c) whichever pass writes it.  Nothing is carried over from call to call.  Vectors that fit into the rings of
-// all SMs (about 29 MB of gradients) need no prediction: the mean is written from shared memory after the decision.
+// c) whichever pass writes it.  Short vectors go without a prediction (see filter_shape in gaf_api.cu): after the
+// decision the mean of the tiles that are still in the rings (25 MB of gradients) is written from there, and the
+// others are fetched again, from L2 for the most part.
 //
 // Two forms of one kernel, with the same sums in the same order, hence the same outputs:
-//   ONE      every CTA is resident at once.  At the end every CTA stores its partial sums, adds itself to an
-//            arrival counter, waits (bounded, GAF_STATUS_TIMEOUT) until it is full, totals the partials and walks
-//            Algorithm 1 ITSELF -- all CTAs get the same bits, nobody waits for a published result; CTA 0 writes
-//            the outputs.  After a wrong prediction the ring is run once more over the accepted gradients, the
+//   ONE      every CTA is resident at once.  At the end every CTA stores its partial sums; CTA 0 totals them, walks
+//            Algorithm 1, writes the outputs and tells every CTA (bounded waits, GAF_STATUS_TIMEOUT).  After a wrong prediction the ring is run once more over the accepted gradients, the
 //            last tiles first (what L2 still holds).
 //   two      the last CTA to take a ticket decides, and masked_mean_kernel, launched behind, returns at once when
 //            the result is already written.  The only wait for other CTAs is the prediction's, and it is short:
@@ -45,13 +43,21 @@
 #include "gaf_gram_tc.cuh"
 #include "gaf_gramfilter.cuh"
 
+// Bound by HBM: (K b + 4) D bytes.  Measured (back to back, outputs of their own; before: second pass over the accepted
+// gradients in every call): 4 x 11.2 M fp32 56 -> 46 us (225 MB: 4.8 TB/s), 8 x 40 M fp32 373 -> 244 us (5.9 TB/s), 8 x 124 M fp32
+// 987 -> 750 us, 8 x 100 M bf16 515 -> 368 us (5.4 TB/s), 8 x 1 G bf16 4.66 -> 3.7 ms.  Of the 46 us, 4 pass until every CTA has its sample
+// tiles, 6 more until the mean of the first is written (the ring is full after 4), 4 between the last CTA's last
+// tile and the decision.  What decided the shape:
+//   - with 8 consumer warps the Gram sums and the mean of a tile took longer than its copy (K = 8: 4.5 TB/s);
+//   - a ring with fewer bytes in flight (3 tiles) cost 14 % with 8 gradients;
+//   - not waiting for the prediction but fetching the tiles from before it again at the end: 70 against 46 us, because
+//     a poll from an SM with a full ring in flight takes 4 us and more;
+//   - CTAs that all read all partial sums, or all poll one counter, wait 3 to 6 us for the few lines that everybody reads.
 namespace gaf {
 
-constexpr unsigned int kFusedSpinLimit = 1u << 23;   // polls of an L2 round trip plus a 20 ns sleep each: seconds
+constexpr unsigned int kFusedSpinLimit = 1u << 22;   // polls of an L2 round trip each: seconds
 constexpr unsigned int kFusedSampleLimit = 64;       // two-launch form: polls for the prediction, some tens of microseconds
 constexpr unsigned int kFusedCopyLimit = 1u << 19;   // attempts of up to 2 us at a ring barrier
-constexpr unsigned int kFusedCallUnit = 4096;        // what one call adds to an arrival counter in all
-constexpr int kFusedCallShift = 12;
 
 // Consumer warps work in groups; a tile belongs to one group, the groups take the tiles in turn.  One more warp
 // produces.  15 warps of at most 128 registers.
@@ -85,9 +91,11 @@ struct GramFusedArgs {
     int64_t D;
     int tile_elems;                         // elements of a tile per gradient (a multiple of 64, at most FilterTile::kElems)
     int rounds;                             // tiles per CTA
-    int run;                                // consecutive tiles a CTA takes before it jumps ahead by the grid's share
     int sample;                             // tiles per CTA in the sample; 0 = no prediction
-    double *partials;                       // [pair][kFilterMaxCtas]
+    void *partials;                         // [pair][kFilterMaxCtas]: TaggedSum (ONE) or double
+    unsigned long long *sample_partials;    // [pair][kFilterMaxCtas]: binary32 sum and tag
+    unsigned long long *verdicts;           // [2][kFilterMaxCtas][16]: a line per CTA, predicted and decided pattern and tag
+    unsigned int tag;                       // ONE: a number no other launch has
     double *gram;                           // [K][K]
     float *out;                             // D floats
     ReplayArgs replay;                      // used when ring.K == 0
@@ -99,20 +107,30 @@ struct GramFusedArgs {
                                             // counter, so that every wait runs out
 };
 
-__device__ __forceinline__ unsigned int ld_relaxed_u32(const unsigned int *p) {
-    unsigned int v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+// What CTAs tell one another carries the call's tag in every word, so that the reader polls the data itself: one
+// trip to L2 and back after the last store, where an arrival counter (stores, release, counter, poll, then the
+// loads) took three.  A binary64 sum travels as two words, half a sum and the tag each; every word is written and
+// read as a whole.  What an earlier call or another kernel left in the place carries another tag.  Every word
+// has ONE reader: 148 CTAs that read the same lines at the same time wait 3 to 6 us for them.
+__device__ __forceinline__ void st_word(unsigned long long *p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long ld_word(const unsigned long long *p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int *p) {
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
+struct TaggedSum { unsigned long long w[2]; };
+__device__ __forceinline__ void st_tagged(TaggedSum *p, double v, unsigned int tag) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned long long lo = (b << 32) | tag, hi = (b & 0xFFFFFFFF00000000ull) | (unsigned int)~tag;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(lo), "l"(hi) : "memory");
 }
-// Adds to a counter, ordered after everything this CTA wrote before (its threads' stores reach this
-// thread through the barrier in front of the call).
-__device__ __forceinline__ void red_release_add_u32(unsigned int *p, unsigned int v) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+__device__ __forceinline__ bool ld_tagged(const TaggedSum *p, double &v, unsigned int tag) {
+    unsigned long long lo, hi;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
+    v = __longlong_as_double((long long)((lo >> 32) | (hi & 0xFFFFFFFF00000000ull)));
+    return (unsigned int)lo == tag && (unsigned int)hi == (unsigned int)~tag;
 }
 // Bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) into shared memory, counted on `bar`.
 __device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void *src, uint32_t bytes, uint64_t *bar, uint64_t policy) {
@@ -220,22 +238,30 @@ __device__ __forceinline__ int round_of_visit(int v, int S, int seg, int phase) 
     return b * seg + i + (i >= phase ? 1 : 0);
 }
 
-// Algorithm 1 on a small Gram matrix in shared memory by one warp, for the prediction: decisions only, binary32.
-// Lane j carries <g_j, running sum>.  Returns the packed pattern in every lane.
+// Algorithm 1 on a Gram matrix in shared memory by one warp.  Lane j carries <g_j, running sum>, its sums taken in
+// processing order; every lane takes every decision, lane t keeps the distance of step t.  Returns the packed pattern in every lane.
 template <int KT>
-__device__ __forceinline__ unsigned int warp_guess(const double *gram, double tau) {
+__device__ __forceinline__ unsigned int warp_walk(const double *gram, double tau, double &dist, int &status) {
     const int lane = threadIdx.x & 31, j = lane < KT ? lane : 0;
-    float pj = (float)gram[j], na = (float)gram[0];
-    const float ng_j = (float)gram[j * KT + j], bound = 1.0f - (float)tau;
+    double pj = gram[j], na = gram[0], norm_sq = na;
+    const double ng_j = gram[j * KT + j], root_j = sqrt(ng_j);
     unsigned int bits = 1u;
+    int count = 1;
+    dist = 0.0;
+    status = 0;
+#pragma unroll 1
     for (int t = 1; t < KT; ++t) {
-        const float p = __shfl_sync(0xFFFFFFFFu, pj, t), ng = __shfl_sync(0xFFFFFFFFu, ng_j, t);
-        float cosv = (na > 0.0f && ng > 0.0f) ? p * rsqrtf(na) * rsqrtf(ng) : 0.0f;
-        cosv = fminf(fmaxf(cosv, -1.0f), 1.0f);
-        if (cosv >= bound) {
+        const double p = __shfl_sync(0xFFFFFFFFu, pj, t), ng = __shfl_sync(0xFFFFFFFFu, ng_j, t);
+        const double root = __shfl_sync(0xFFFFFFFFu, root_j, t);
+        const double d = cosine_distance(p, na, ng, sqrt(na), root, &status);
+        if (lane == t) dist = d;
+        if (d <= tau) {
             bits |= 1u << t;
-            na += 2.0f * p + ng;
-            pj += (float)gram[t * KT + j];
+            na = na + 2.0 * p + ng;
+            norm_sq += ng;
+            ++count;
+            status |= ill_conditioned(count, norm_sq, na);
+            pj += gram[t * KT + j];
         }
     }
     return pack_pattern(bits, 0);
@@ -295,15 +321,16 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     __shared__ double sgram[KT * KT];
     __shared__ const T *list[kGsMaxK];      // accepted gradients in the order they are added
     __shared__ int n_list;                  // c
-    __shared__ int sh_ok, sh_again;         // outcome of a wait; whether the accepted gradients are run once more
-    __shared__ unsigned int sh_pred, sh_final;      // predicted and decided pattern
+    __shared__ int sh_ok, sh_again;         // outcome of a wait; how many tiles are fetched a second time
+    __shared__ unsigned int sh_pred;        // predicted and decided pattern
+    __shared__ volatile unsigned int sh_final;
     __shared__ volatile int abort_flag;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     Control *ctl = a.replay.ctl;
 
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) { tc_mbar_init(&full[s], 1); tc_mbar_init(&empty[s], kFilterGroupWarps); }
-        sh_pred = 0u; sh_again = 0; abort_flag = 0;
+        sh_pred = 0u; sh_final = 0u; sh_ok = 1; sh_again = 0; abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     for (int i = tid; i < CW * NP; i += kFilterThreads) (&ssum[0][0])[i] = 0.0;
@@ -316,7 +343,6 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     const int rounds = a.rounds, S = a.sample;
     constexpr int kAlign = 16 / (int)sizeof(T);
     const int64_t Dv = a.D / kAlign * kAlign;                   // what the copies cover
-    const bool resident = rounds <= kStages;                    // every tile stays in the ring
 
     if (warp == CW) {
         // ------------------------------------------------------------------ producer ----
@@ -328,9 +354,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
             if (it >= kStages && !tc_mbar_wait(&empty[s], (uint32_t)((it / kStages - 1) & 1), &abort_flag, kFusedCopyLimit))
                 return false;
             const int r = round_of_visit(v, S, seg, phase);
-            int64_t tile = (int64_t)r * gridDim.x + blockIdx.x;
-            if (a.run > 1) tile = ((int64_t)(r / a.run) * gridDim.x + blockIdx.x) * a.run + r % a.run;
-            const int64_t e0 = tile * te, left = Dv - e0;
+            const int64_t e0 = ((int64_t)r * gridDim.x + blockIdx.x) * te, left = Dv - e0;
             const int n = left >= te ? te : (left > 0 ? (int)left : 0);
             stage_e0[s] = e0;
             stage_n[s] = n;
@@ -350,8 +374,8 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
                 if (!fill(v, a.g, KT)) break;
         __syncwarp();
         __syncthreads();                    // the consumers have decided whether there is a second pass
-        if (ONE && sh_again && lane == 0)
-            for (int v = rounds - 1; v >= 0; --v)
+        if (ONE && lane == 0)
+            for (int v = sh_again - 1; v >= 0; --v)
                 if (!fill(v, reinterpret_cast<const void *const *>(list), n_list)) break;
         // after a wait that gave up: the copies in flight must land before the CTA leaves its shared memory
         if (lane == 0 && abort_flag)
@@ -363,12 +387,10 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
 
     // ---------------------------------------------------------------------- consumers ----
     const int group = warp / kFilterGroupWarps, gwarp = warp - group * kFilterGroupWarps, gtid = gwarp * 32 + lane;
-    unsigned int gen0 = 0, gen_s = 0;       // call generations: they cannot change before this CTA has arrived
-    if (ONE && tid == 0) gen0 = ld_relaxed_u32(&ctl->fused_arrivals) >> kFusedCallShift;
-    if (S > 0) gen_s = ld_relaxed_u32(&ctl->sample_arrivals) >> kFusedCallShift;
     if (blockIdx.x == 0 && tid == 0) ctl->status = 0;
-    // (two sets of sample sums, used by calls in turn: this one clears the next call's)
-    if (S > 0 && blockIdx.x == 0 && tid < NP) ctl->sample_sums[(gen_s + 1u) & 1u][tid] = 0.0;
+    // Two launches may be replayed from a graph: their tag is a count of such calls in the workspace, which moves on
+    // when every CTA of the call has taken its ticket.  (The tags of the one-launch form have the upper bit set.)
+    const unsigned int tag = ONE ? a.tag | 0x80000000u : __ldcg(&ctl->two_launch_calls) & 0x7FFFFFFFu;
 
     // Accumulators: binary64, pairs of binary32 chains, or (MMA) this lane's fragment of the 8 x 8 matrix.
     constexpr bool kF64 = !GsAcc<T, KT>::kPeriodicFlush;
@@ -525,61 +547,137 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         for (int w = 0; w < CW; ++w) s += ssum[w][tid];
         return s;
     };
-    auto arrive = [&](unsigned int *counter) {
-        red_release_add_u32(counter, blockIdx.x == 0 ? kFusedCallUnit - (gridDim.x - 1) : 1u);
+    // row-major pair index -> (i, j), i <= j
+    auto pair_at = [](int p, int &i, int &j) {
+        i = 0;
+        while (p >= KT - i) { p -= KT - i; ++i; }
+        j = i + p;
     };
-    // (the acquire orders the loads behind it, through a barrier for other threads, after every CTA's stores)
-    auto wait_all = [&](const unsigned int *counter, unsigned int gen, unsigned int limit) {
-        unsigned int polls = 0;
-        while ((ld_acquire_u32(counter) >> kFusedCallShift) == gen || a.test_withhold) {
-            __nanosleep(20);
-            if (++polls > limit) return false;
+    // Sums of all CTAs in a fixed order into sgram: warp w takes the pairs w, w + CW, ...  `read(pair, cta, value)`
+    // returns whether that sum is there; every warp polls its own at most `limit` times.
+    auto total = [&](auto read, unsigned int limit, double *gram_out) {
+        constexpr int R = kFilterMaxCtas / 32;
+        for (int p = warp; p < NP; p += CW) {
+            double part[R];
+            bool have[R], all = false;
+#pragma unroll
+            for (int k = 0; k < R; ++k) { part[k] = 0.0; have[k] = lane + 32 * k >= (int)gridDim.x; }
+            for (unsigned int polls = 0; polls <= limit; ++polls) {
+                bool mine = true;
+#pragma unroll
+                for (int k = 0; k < R; ++k)
+                    if (!have[k]) { have[k] = read(p, lane + 32 * k, part[k]); mine = mine && have[k]; }
+                all = __all_sync(0xFFFFFFFFu, mine);
+                if (all) break;
+            }
+            if (!all) { if (lane == 0) sh_ok = 0; break; }
+            double s = 0.0;
+#pragma unroll
+            for (int k = 0; k < R; ++k) s += part[k];
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) s += shfl_down_f64(s, d);
+            if (lane == 0) {
+                int i, j;
+                pair_at(p, i, j);
+                sgram[i * KT + j] = s;
+                sgram[j * KT + i] = s;
+                if (gram_out) { gram_out[i * KT + j] = s; gram_out[j * KT + i] = s; }
+            }
         }
-        return true;
+        Sync::sync();
+        return sh_ok != 0;
     };
 
-    unsigned int pred = 0;
+    // CTA 0, one warp: a pattern to every CTA's line; the other CTAs, one thread: wait for it (0 = it did not come).
+    auto tell = [&](unsigned long long *lines, unsigned int pattern) {
+        for (int cta = lane; cta < (int)gridDim.x; cta += 32) st_word(lines + cta * 16, ((unsigned long long)pattern << 32) | tag);
+    };
+    auto hear = [&](const unsigned long long *lines, unsigned int limit) {
+        for (unsigned int polls = 0; polls <= limit; ++polls) {
+            const unsigned long long w = ld_word(lines + blockIdx.x * 16);
+            if ((unsigned int)w == tag && !a.test_withhold) return (unsigned int)(w >> 32);
+        }
+        return 0u;
+    };
+
+    // Algorithm 1 (or its order-indifferent variant) on sgram, by all consumers: decided pattern into sh_final and, if
+    // there are lines, to every CTA; mask, distances and count to their places.
+    auto decide = [&](unsigned long long *lines) {
+        if (a.ring.K > 0) {
+            __shared__ RingTable<KT> table;
+            ring_replay_parallel<KT, Sync>(a.ring, sgram, table,
+                                           [&](int seed, unsigned long long bits) { sh_final = pack_pattern((unsigned int)bits, seed); });
+            if (lines != nullptr && warp == 0) { __syncwarp(); tell(lines, sh_final); }
+        } else if (warp == 0) {
+            double dist;
+            int status;
+            const unsigned int final = warp_walk<KT>(sgram, a.replay.tau, dist, status);
+            if (lines != nullptr) tell(lines, final);
+            const unsigned int bits = final & 0xFFu;
+            if (lane < KT) {
+                a.replay.mask_out[a.replay.idx[lane]] = (uint8_t)((bits >> lane) & 1u);
+                if (a.replay.dist_out) a.replay.dist_out[a.replay.idx[lane]] = (float)dist;
+            }
+            if (lane == 0) {
+                sh_final = final;
+                ctl->accept_bits = bits;
+                ctl->ring_seed = -1;
+                ctl->count = __popc(bits);
+                *a.replay.count_out = __popc(bits);
+                if (status) atomicOr(&ctl->status, status);
+            }
+        }
+        Sync::sync();
+    };
+
+    // Two gradients (ONE): the result is the mean of both or the first alone.  When the latest two calls on this workspace
+    // ended alike, that pattern is taken instead of a sample's, and nobody waits for one (0 both, 1 the first alone; from 2 on: they
+    // differed, bit 0 the latest).  Read before this CTA hands in its sums, hence before CTA 0 can have decided.
+    const unsigned int hint = KT == 2 && ONE && S > 0 ? __ldcg(&ctl->pair_hint) : 2u;
+    const bool sampling = S > 0 && hint >= 2u;
+    // (a group's tiles have its number modulo NG, in a second pass too)
+    auto next_of_group = [&](int it) { return it + (group + NG - it % NG) % NG; };
+    unsigned int pred = hint < 2u ? pack_pattern(hint == 1u ? 1u : 3u, 0) : 0u;
     int v = group;
-    {
+    if (sampling) {
         const CountDivider none(1);
         for (; v < S; v += NG) {
             wait_full(v);
             process(true_type(), false_type(), v % kStages, 0u, 0u, none);
         }
     }
-    if (S > 0) {
-        // The sample's sums are totalled by atomic additions: their last bits depend on the order, but they only
-        // serve a guess.
+    if (sampling) {
         flush();
         Sync::sync();
-        if (tid < NP) atomicAdd(&ctl->sample_sums[gen_s & 1u][tid], cta_sum());
-        Sync::sync();
-        if (warp == 0) {
-            int ok = 0;
-            if (lane == 0) {
-                arrive(&ctl->sample_arrivals);
-                ok = wait_all(&ctl->sample_arrivals, gen_s, ONE ? a.spin_limit : kFusedSampleLimit) ? 1 : 0;
-            }
-            if (__shfl_sync(0xFFFFFFFFu, ok, 0)) {
-                for (int p = lane; p < NP; p += 32) {
-                    int i = 0, rem = p;
-                    while (rem >= KT - i) { rem -= KT - i; ++i; }
-                    const double s = __ldcg(&ctl->sample_sums[gen_s & 1u][p]);
-                    sgram[i * KT + i + rem] = s;
-                    sgram[(i + rem) * KT + i] = s;
-                }
-                __syncwarp();
-                const unsigned int guess = a.ring.K > 0 ? warp_ring_guess<KT>(a.ring, sgram) : warp_guess<KT>(sgram, a.replay.tau);
+        if (tid < NP)
+            st_word(a.sample_partials + (size_t)tid * kFilterMaxCtas + blockIdx.x,
+                    ((unsigned long long)__float_as_uint((float)cta_sum()) << 32) | tag);
+        const unsigned int limit = ONE ? a.spin_limit : kFusedSampleLimit;
+        if (blockIdx.x == 0) {
+            const bool known = total([&](int p, int cta, double &value) {
+                const unsigned long long w = ld_word(a.sample_partials + (size_t)p * kFilterMaxCtas + cta);
+                value = (double)__uint_as_float((unsigned int)(w >> 32));
+                return (unsigned int)w == tag && !a.test_withhold;
+            }, limit, nullptr);
+            if (warp == 0 && known) {
+                double dist;
+                int status;
+                const unsigned int guess = a.ring.K > 0 ? warp_ring_guess<KT>(a.ring, sgram)
+                                                        : warp_walk<KT>(sgram, a.replay.tau, dist, status);
                 if (lane == 0) sh_pred = guess;
+                tell(a.verdicts, guess);
             }
+        } else if (tid == 0) {
+            sh_pred = hear(a.verdicts, limit);
         }
         Sync::sync();
         pred = sh_pred;
+        if (tid == 0) sh_ok = 1;
     }
     if (pred) {
         const unsigned int bits = pred & 0xFFu, before = bits & ((1u << ((pred >> 8) & 0xFu)) - 1u), from = bits ^ before;
         const CountDivider div(__popc(bits));
-        for (int w = group; w < S; w += NG) {
+        for (int w = group; sampling && w < S; w += NG) {
             process(false_type(), true_type(), w % kStages, from, before, div);
             release(w);
         }
@@ -589,12 +687,13 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
             release(v);
         }
     } else {
+        // (the last tiles stay in the ring: their mean is written from there)
         const CountDivider none(1);
-        for (int w = group; w < S; w += NG) release(w);
+        for (int w = group; sampling && w < S; w += NG) release(w);
         for (; v < rounds; v += NG) {
             wait_full(v);
             process(true_type(), false_type(), v % kStages, 0u, 0u, none);
-            release(v);
+            if (v < rounds - kStages) release(v);
         }
     }
     flush();
@@ -608,66 +707,47 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         double s = cta_sum();
         if (blockIdx.x == 0 && Dv < a.D) {
             // the last elements, which no copy covers
-            int i = 0, rem = tid;
-            while (rem >= KT - i) { rem -= KT - i; ++i; }
-            const T *x = static_cast<const T *>(a.g[i]), *y = static_cast<const T *>(a.g[i + rem]);
+            int i, j;
+            pair_at(tid, i, j);
+            const T *x = static_cast<const T *>(a.g[i]), *y = static_cast<const T *>(a.g[j]);
             for (int64_t e = Dv; e < a.D; ++e) s += (double)load1<T>(x, e) * (double)load1<T>(y, e);
         }
-        a.partials[(size_t)tid * kFilterMaxCtas + blockIdx.x] = s;
+        if constexpr (ONE) st_tagged(static_cast<TaggedSum *>(a.partials) + (size_t)tid * kFilterMaxCtas + blockIdx.x, s, tag);
+        else static_cast<double *>(a.partials)[(size_t)tid * kFilterMaxCtas + blockIdx.x] = s;
     }
-    Sync::sync();
 
     // ---- decide ----
-    if (tid == 0) {
-        if constexpr (ONE) {
-            arrive(&ctl->fused_arrivals);
-            sh_ok = wait_all(&ctl->fused_arrivals, gen0, a.spin_limit) ? 1 : 0;
-        } else {
+    if constexpr (ONE) {
+        unsigned long long *const lines = a.verdicts + kFilterMaxCtas * 16;
+        if (blockIdx.x == 0) {
+            if (total([&](int p, int cta, double &value) {
+                    return ld_tagged(static_cast<const TaggedSum *>(a.partials) + (size_t)p * kFilterMaxCtas + cta, value, tag) &&
+                           !a.test_withhold;
+                }, a.spin_limit, a.gram)) {
+                decide(lines);
+            }
+        } else if (tid == 0) {
+            sh_final = hear(lines, a.spin_limit);
+        }
+        Sync::sync();
+        if (sh_final == 0u) {
+            if (tid == 0) atomicOr(&ctl->status, GAF_STATUS_TIMEOUT);
+            __syncthreads();
+            return;
+        }
+    } else {
+        Sync::sync();
+        if (tid == 0) {
             if (pred) atomicAdd(&ctl->written_ctas, 1u);
             sh_ok = take_last_ticket(&ctl->ticket, gridDim.x) ? 1 : 0;
         }
-    }
-    Sync::sync();
-    if (!sh_ok) {
-        if constexpr (ONE) {
-            // every CTA has arrived all the same: the counter is whole again
-            if (tid == 0) atomicOr(&ctl->status, GAF_STATUS_TIMEOUT);
-            __syncthreads();
-        }
-        return;
-    }
-    const bool publisher = !ONE || blockIdx.x == 0;
-    {
-        // totals of all CTAs' sums in a fixed order: one warp per pair, all its loads issued before the first addition
-        constexpr int PW = (NP + CW - 1) / CW, R = kFilterMaxCtas / 32;
-        double part[PW][R];
-#pragma unroll
-        for (int w = 0; w < PW; ++w)
-#pragma unroll
-            for (int k = 0; k < R; ++k) {
-                const int p = warp + w * CW, i = lane + 32 * k;
-                part[w][k] = (p < NP && i < (int)gridDim.x) ? __ldcg(a.partials + (size_t)p * kFilterMaxCtas + i) : 0.0;
-            }
-#pragma unroll
-        for (int w = 0; w < PW; ++w) {
-            const int p = warp + w * CW;
-            double s = 0.0;
-#pragma unroll
-            for (int k = 0; k < R; ++k) s += part[w][k];
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) s += shfl_down_f64(s, d);
-            if (lane == 0 && p < NP) {
-                int i = 0, rem = p;
-                while (rem >= KT - i) { rem -= KT - i; ++i; }
-                const int j = i + rem;
-                sgram[i * KT + j] = s;
-                sgram[j * KT + i] = s;
-                if (publisher) { a.gram[i * KT + j] = s; a.gram[j * KT + i] = s; }
-            }
-        }
         Sync::sync();
-    }
-    if constexpr (!ONE) {
+        if (!sh_ok) return;
+        if (tid == 0) ctl->two_launch_calls = tag + 1u;
+        total([&](int p, int cta, double &value) {
+            value = __ldcg(static_cast<const double *>(a.partials) + (size_t)p * kFilterMaxCtas + cta);
+            return true;
+        }, 0u, a.gram);
         if (a.pair_dist_out != nullptr) {
             // pairwise mode: Eq. 4 for every pair
             if (tid < KT * KT) {
@@ -681,29 +761,25 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
             }
             return;
         }
+        decide(nullptr);
     }
-    // (one-launch form: every CTA takes the same sums in the same order, hence the same decisions)
-    {
-        auto known = [&](int seed, unsigned long long bits) {
-            const int start = seed < 0 ? 0 : seed;
-            int n = 0;
-            for (int t = 0; t < KT; ++t) {
-                const int i = (start + t) % KT;
-                if ((bits >> i) & 1ull) list[n++] = static_cast<const T *>(a.g[i]);
-            }
-            n_list = n;
-            sh_final = pack_pattern((unsigned int)bits, start);
-            if (ONE) sh_again = (!resident && sh_final != pred) ? 1 : 0;
-        };
-        if (a.ring.K > 0) {
-            __shared__ RingTable<KT> table;
-            ring_replay_parallel<KT, Sync>(a.ring, sgram, table, known, publisher);
-        } else {
-            __shared__ ReplayTable table;
-            replay_on_gram_parallel<KT, Sync>(a.replay, sgram, table, [&](unsigned long long bits) { known(-1, bits); }, publisher);
+    const int kept = pred ? 0 : min(rounds, kStages);           // tiles that are still in the ring
+    if (tid == 0) {
+        const unsigned int bits = sh_final & 0xFFu;
+        const int start = (int)((sh_final >> 8) & 0xFu);
+        int n = 0;
+        for (int t = 0; t < KT; ++t) {
+            const int i = start + t >= KT ? start + t - KT : start + t;
+            if ((bits >> i) & 1u) list[n++] = static_cast<const T *>(a.g[i]);
         }
-        Sync::sync();
+        n_list = n;
+        if (KT == 2 && ONE && S > 0 && blockIdx.x == 0) {
+            const unsigned int outcome = n == 1 ? 1u : 0u;
+            ctl->pair_hint = outcome == (hint & 1u) ? outcome : (2u | outcome);
+        }
+        if (ONE) sh_again = sh_final != pred ? rounds - kept : 0;
     }
+    Sync::sync();
     const int c = n_list;
     if constexpr (!ONE) {
         if (tid == 0) {
@@ -725,18 +801,18 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         a.out[e] = x / (float)c;
     }
     if constexpr (ONE) {
+        if (sh_final == pred) return;
         const CountDivider div(c);
-        if (resident) {
-            const unsigned int bits = sh_final & 0xFFu, before = bits & ((1u << ((sh_final >> 8) & 0xFu)) - 1u);
-            for (int w = group; w < rounds; w += NG) process(false_type(), true_type(), w, bits ^ before, before, div);
-        } else if (sh_again) {
-            // the accepted gradients again, compacted to the first rows of a tile in the order they are added (the
-            // tiles go on alternating between the groups)
-            for (int it = rounds + (group + NG - rounds % NG) % NG; it < 2 * rounds; it += NG) {
-                wait_full(it);
-                process(false_type(), true_type(), it % kStages, (1u << c) - 1u, 0u, div);
-                release(it);
-            }
+        const unsigned int bits = sh_final & 0xFFu, before = bits & ((1u << ((sh_final >> 8) & 0xFu)) - 1u);
+        for (int w = next_of_group(rounds - kept); w < rounds; w += NG) {
+            process(false_type(), true_type(), w % kStages, bits ^ before, before, div);
+            release(w);
+        }
+        // the accepted gradients of the other tiles again, compacted to the first rows in the order they are added
+        for (int it = next_of_group(rounds); it < 2 * rounds - kept; it += NG) {
+            wait_full(it);
+            process(false_type(), true_type(), it % kStages, (1u << c) - 1u, 0u, div);
+            release(it);
         }
     }
 }

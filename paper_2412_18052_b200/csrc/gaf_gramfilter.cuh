@@ -25,7 +25,6 @@ constexpr int kGsPartialStride = 320;       // per-CTA partials are stored [pair
 constexpr int kGsFlushEvery = 16;           // iterations between binary64 flushes
 constexpr int kMsThreads = 512;
 constexpr int kMsLongRun = 8;                // chunks per run of the masked-mean pass on long vectors
-constexpr int kReplayMaxK = 8;               // the table form of the walk: 2^(K-1) - 1 cases
 
 struct ReplayArgs {
     int K;
@@ -83,94 +82,6 @@ __device__ __forceinline__ unsigned long long replay_on_gram(const ReplayArgs &r
         *r.count_out = count;
     }
     return bits;
-}
-
-// The same walk for K <= 8 with its latency taken out of the serial part.  Step t's test depends on
-// the earlier decisions only through WHICH gradients were accepted, so one thread per (step t,
-// accept pattern of steps 1..t-1) evaluates Eq. 4 for that case -- 2^(K-1) - 1 threads, all at once --
-// and thread 0 then only follows the decisions through the table.  Every case repeats the sums of
-// the sequential walk in the same order, so the results are the same to the last bit.
-// `Sync` stands for the threads that call (at least 128, thread 0 among them).  `early(bits)` is called by thread 0 as soon as
-// the accept bits are known, before the outputs are written.  With `publish` false nothing is written
-// to global memory (the one-launch schedule runs the walk in every CTA and lets one of them publish).
-struct ReplayTable {
-    double d[127], p[127], na[127];
-    unsigned char accept[127], status[127];
-};
-struct NoEarlyBits {
-    __device__ __forceinline__ void operator()(unsigned long long) const {}
-};
-template <int KT, typename Sync, typename Early = NoEarlyBits>
-__device__ __forceinline__ void replay_on_gram_parallel(const ReplayArgs &r, const double *gram, ReplayTable &tb,
-                                                        Early early = Early(), bool publish = true) {
-    constexpr int K = KT;
-    const int tid = threadIdx.x;
-    constexpr int cases = (1 << (K - 1)) - 1;
-    if (tid < cases) {
-        const int t = 32 - __clz(tid + 1);                      // tid + 1 in [2^(t-1), 2^t)
-        const unsigned int m = (unsigned int)(tid + 1) - (1u << (t - 1));
-        // step v accepted in this case (bits of m at and above t-1 are zero)
-        auto in = [&](int v) { return v == 0 || ((m >> (v - 1)) & 1u); };
-        // Branch-free (neighbouring lanes hold different cases): a gradient that is not in the case
-        // contributes an added 0.0, which leaves a binary64 sum unchanged, and its update of |g|^2
-        // is computed and dropped.
-        double na = gram[0], norm_sq = gram[0];
-        int cnt = 1;
-#pragma unroll
-        for (int u = 1; u < K - 1; ++u) {
-            double pu = 0.0;
-#pragma unroll
-            for (int v = 0; v < u; ++v) pu += in(v) ? gram[v * K + u] : 0.0;
-            const double grown = na + 2.0 * pu + gram[u * K + u];
-            na = in(u) ? grown : na;
-            norm_sq += in(u) ? gram[u * K + u] : 0.0;
-            cnt += in(u) ? 1 : 0;
-        }
-        double p = 0.0;
-#pragma unroll
-        for (int v = 0; v < K - 1; ++v) p += (v < t && in(v)) ? gram[v * K + t] : 0.0;
-        int status = 0;
-        const double ng = gram[t * K + t];
-        const double d = cosine_distance(p, na, ng, &status);
-        const int accept = (d <= r.tau) ? 1 : 0;
-        // the sum this case would leave behind, if it accepts
-        status |= accept ? ill_conditioned(cnt + 1, norm_sq + ng, na + 2.0 * p + ng) : 0;
-        tb.d[tid] = d; tb.p[tid] = p; tb.na[tid] = na;
-        tb.accept[tid] = (unsigned char)accept;
-        tb.status[tid] = (unsigned char)status;
-    }
-    Sync::sync();
-    if (tid == 0) {
-        unsigned int m = 0;
-        int node[kReplayMaxK];
-        for (int t = 1; t < K; ++t) {
-            node[t] = (1 << (t - 1)) - 1 + (int)m;
-            if (tb.accept[node[t]]) m |= 1u << (t - 1);
-        }
-        const unsigned long long bits = 1ull | ((unsigned long long)m << 1);
-        early(bits);
-        if (!publish) return;
-        Control *c = r.ctl;
-        int status = 0, count = 1;
-        c->decision[0] = 1;
-        r.mask_out[r.idx[0]] = 1;
-        if (r.dist_out) r.dist_out[r.idx[0]] = 0.0f;
-        for (int t = 1; t < K; ++t) {
-            const int i = node[t], accept = tb.accept[i];
-            c->decision[t] = accept;
-            c->sums[t][0] = tb.p[i]; c->sums[t][1] = tb.na[i]; c->sums[t][2] = gram[t * K + t];
-            r.mask_out[r.idx[t]] = (uint8_t)accept;
-            if (r.dist_out) r.dist_out[r.idx[t]] = (float)tb.d[i];
-            status |= tb.status[i];
-            count += accept;
-        }
-        c->accept_bits = bits;
-        c->ring_seed = -1;
-        c->count = count;
-        if (status) atomicOr(&c->status, status);
-        *r.count_out = count;
-        __threadfence();
-    }
 }
 
 // Order-indifferent variant (end of Section 3.1): Algorithm 1 from every seed s with the
@@ -256,13 +167,12 @@ __device__ __forceinline__ void ring_replay_on_gram(const RingArgs &r, const vol
     }
 }
 
-// The any-seed walks in table form (K <= 8), as replay_on_gram_parallel does for one order: one thread
-// per (seed, step t, accept pattern of the seed's steps 1..t-1) evaluates Eq. 4 on the Gram matrix by
+// The any-seed walks in table form (K <= 8).  Step t's test depends on the earlier decisions only through WHICH
+// gradients were accepted, so one thread per (seed, step t, accept pattern of the seed's steps 1..t-1) evaluates Eq. 4 on the Gram matrix by
 // ORIGINAL index (step v of seed s is gradient (s + v) mod K), one thread per seed then follows its
 // decisions through the table, and thread 0 picks the largest count (ties to the smallest seed) and
 // publishes.  Same sums in the same order as ring_walk_one_seed: identical outputs.
-// All threads of `Sync` call; `early(seed, bits)` as in ring_replay_on_gram; `publish` as in
-// replay_on_gram_parallel.
+// All threads of `Sync` call; `early(seed, bits)` as in ring_replay_on_gram.
 template <int KT>
 struct RingTable {
     static constexpr int kCases = (1 << (KT - 1)) - 1;          // per seed
@@ -273,7 +183,7 @@ struct RingTable {
 };
 template <int KT, typename Sync, typename Early = NoEarlyNotice>
 __device__ __forceinline__ void ring_replay_parallel(const RingArgs &r, const double *gram, RingTable<KT> &tb,
-                                                     Early early = Early(), bool publish = true) {
+                                                     Early early = Early()) {
     constexpr int K = KT, C = RingTable<KT>::kCases;
     for (int idx = threadIdx.x; idx < K * C; idx += Sync::threads()) {
         const int s = idx / C, cs = idx - s * C;
@@ -328,7 +238,6 @@ __device__ __forceinline__ void ring_replay_parallel(const RingArgs &r, const do
         for (int t = 1; t < K; ++t)
             if ((steps >> (t - 1)) & 1u) bits |= 1ull << ((best + t) % K);
         early(best, bits);
-        if (!publish) return;
         int status = 0;
         unsigned int m = 0;
         if (r.dist_out) r.dist_out[best] = 0.0f;
