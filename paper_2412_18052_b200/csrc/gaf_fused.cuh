@@ -69,21 +69,25 @@ constexpr int kFilterConsumers = kFilterWarps * 32;
 constexpr int kFilterThreads = kFilterConsumers + 32;
 constexpr int kFilterMaxStages = 24;
 constexpr int kFilterMaxCtas = 160;
+// Two gradients: a shorter ring of smaller tiles, 112 KB in flight (2 x 30 M fp32: 63.3 us with 28 KB tiles in 172 KB, 62.1 with
+// 14 KB tiles, 58.8 in the shorter ring as well; a third of the traffic are writes there).
 constexpr int kFilterRingBytes = 206 << 10;
+constexpr int kFilterPairRingBytes = 130 << 10;
 
 // Tile of K gradients: kVecs groups of 4 elements per thread of a group and gradient, about 28 KB in all.
 template <typename T, int KT> struct FilterTile {
     static constexpr bool kMma = std::is_same<T, __nv_bfloat16>::value && KT >= 7;
-    static constexpr int kVecs = KT == 2 ? 16 / int(sizeof(T)) : (KT <= 4 ? 8 / int(sizeof(T)) : 4 / int(sizeof(T)));
+    static constexpr int kVecs = KT == 2 ? 8 / int(sizeof(T)) : (KT <= 4 ? 8 / int(sizeof(T)) : 4 / int(sizeof(T)));
     static constexpr int kElems = kVecs * 4 * kFilterGroupThreads;
     // (the MMA fragments of eight rows are read together: 64 bytes between rows keep them apart in the banks)
     static constexpr int kPitch = kElems * int(sizeof(T)) + (kMma ? 64 : 0);
     static constexpr int kBytes = KT * kPitch;
     // A multiple of the groups: a stage then always belongs to the same group, which has seen its previous tile land
     // before it waits for the next one (copies complete in any order; a barrier's parity tells only two phases apart).
-    static constexpr int kFit = kFilterRingBytes / kBytes < kFilterMaxStages ? kFilterRingBytes / kBytes : kFilterMaxStages;
+    static constexpr int kRing = KT == 2 ? kFilterPairRingBytes : kFilterRingBytes;
+    static constexpr int kFit = kRing / kBytes < kFilterMaxStages ? kRing / kBytes : kFilterMaxStages;
     static constexpr int kStages = kFit / kFilterGroups * kFilterGroups;
-    static constexpr int kBatch = KT == 2 ? 4 : (KT <= 4 ? 2 : 1);  // groups of 4 elements a thread loads together
+    static constexpr int kBatch = KT <= 4 ? 2 : 1;  // groups of 4 elements a thread loads together
 };
 
 struct GramFusedArgs {
