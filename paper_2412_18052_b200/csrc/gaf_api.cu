@@ -259,10 +259,14 @@ bool stacked_tensor_maps(const void *const *grads, int K, int Kp, int R, int box
 
 // Tiled Gram matrix of K gradients (by original index) into the workspace; optional
 // distance matrix.  Two launches.
+// `replay` or `ring` given: Algorithm 1 on the matrix instead.
 int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, float *dist_out,
-                      double *gram_out, unsigned char *base, const DeviceInfo &di, cudaStream_t st) {
+                      double *gram_out, const ReplayArgs *replay, const RingArgs *ring, unsigned char *base,
+                      const DeviceInfo &di, cudaStream_t st) {
     const int sms = di.sms;
     GramArgs a{};
+    if (replay) a.replay = *replay;
+    if (ring) a.ring = *ring;
     for (int i = 0; i < K; ++i) a.g[i] = grads[i];
     a.K = K; a.D = D;
     a.tiles = (K + kGramTile - 1) / kGramTile;
@@ -570,7 +574,6 @@ int launch_gram_first(const void *const *g, int K, int64_t D, int dtype, double 
     ReplayArgs r{};
     r.K = K; r.tau = tau; r.mask_out = mask_out; r.dist_out = dist_out; r.count_out = count_out; r.ctl = ctl;
     for (int t = 0; t < K; ++t) r.idx[t] = ord[t];
-    double *gram_by_index = reinterpret_cast<double *>(base + kExtraOffset + gram_partials_bytes(K));
     double *gram_by_step = reinterpret_cast<double *>(base + kExtraOffset + gram_partials_bytes(K) +
                                                       gram_matrix_bytes(K));
     if (one_launch && (K < 2 || K > kGsMaxK)) return GAF_ERR_UNSUPPORTED;
@@ -588,10 +591,9 @@ int launch_gram_first(const void *const *g, int K, int64_t D, int dtype, double 
         if (one_launch) return launch_gram_fused<T>(f, K, di, st);
         if (int rc = launch_gram_filter<T>(f, K, di, st)) return rc;
     } else {
-        if (int rc = launch_gram_tiles(g, K, D, dtype, nullptr, nullptr, base, di, st)) return rc;
-        if (seed_out) gram_ring_replay_kernel<<<1, GAF_MAX_K, 0, st>>>(ring, gram_by_index);
-        else gram_replay_kernel<<<1, 256, 0, st>>>(r, gram_by_index, gram_by_step);
-        ++g_launches;
+        if (int rc = launch_gram_tiles(g, K, D, dtype, nullptr, nullptr, seed_out ? nullptr : &r, seed_out ? &ring : nullptr,
+                                       base, di, st))
+            return rc;
     }
     MaskedMeanArgs m{};
     for (int t = 0; t < K; ++t) m.g[t] = g[ord[t]];
@@ -1102,7 +1104,7 @@ int gaf_pairwise_cosdist(const void *const *grads, int K, int64_t D, int dtype, 
         return dtype == GAF_F32 ? launch_gram_filter<float>(a, K, di, st)
                                 : launch_gram_filter<__nv_bfloat16>(a, K, di, st);
     }
-    return launch_gram_tiles(grads, K, D, dtype, dist_out, gram_out, base, di, st);
+    return launch_gram_tiles(grads, K, D, dtype, dist_out, gram_out, nullptr, nullptr, base, di, st);
 }
 
 int gaf_read_status(const void *workspace, void *cuda_stream, int *status_out) {

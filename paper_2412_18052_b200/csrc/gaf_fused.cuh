@@ -148,7 +148,7 @@ struct FilterConsumers {
     static __device__ __forceinline__ void sync() {
         asm volatile("barrier.cta.sync 1, %0;" ::"n"(kFilterConsumers) : "memory");
     }
-    static __device__ __forceinline__ int threads() { return kFilterConsumers; }
+    static __device__ __forceinline__ constexpr int threads() { return kFilterConsumers; }
 };
 
 // Two binary32 values in one register pair, and the two-wide instructions on them (each half rounds as the scalar
@@ -242,47 +242,6 @@ __device__ __forceinline__ int round_of_visit(int v, int S, int seg, int phase) 
     return b * seg + i + (i >= phase ? 1 : 0);
 }
 
-// Algorithm 1 on a Gram matrix in shared memory by one warp.  Lane j carries <g_j, running sum>, its sums taken in
-// processing order; every lane takes every decision, lane t keeps the distance of step t.  Returns the packed pattern in every lane.
-template <int KT>
-__device__ __forceinline__ unsigned int warp_walk(const double *gram, double tau, double &dist, int &status) {
-    const int lane = threadIdx.x & 31, j = lane < KT ? lane : 0;
-    double pj = gram[j], na = gram[0], norm_sq = na;
-    const double ng_j = gram[j * KT + j], root_j = sqrt(ng_j);
-    unsigned int bits = 1u;
-    int count = 1;
-    dist = 0.0;
-    status = 0;
-#pragma unroll 1
-    for (int t = 1; t < KT; ++t) {
-        const double p = __shfl_sync(0xFFFFFFFFu, pj, t), ng = __shfl_sync(0xFFFFFFFFu, ng_j, t);
-        const double root = __shfl_sync(0xFFFFFFFFu, root_j, t);
-        const double d = cosine_distance(p, na, ng, sqrt(na), root, &status);
-        if (lane == t) dist = d;
-        if (d <= tau) {
-            bits |= 1u << t;
-            na = na + 2.0 * p + ng;
-            norm_sq += ng;
-            ++count;
-            status |= ill_conditioned(count, norm_sq, na);
-            pj += gram[t * KT + j];
-        }
-    }
-    return pack_pattern(bits, 0);
-}
-// ... and of its order-indifferent variant: lane s walks seed s, the largest count wins, ties to the smallest seed.
-template <int KT>
-__device__ __forceinline__ unsigned int warp_ring_guess(const RingArgs &r, const double *gram) {
-    const int lane = threadIdx.x & 31;
-    int count = 0, status = 0;
-    unsigned long long bits = 0;
-    if (lane < KT) ring_walk_one_seed(r, gram, lane, count, bits, status, nullptr);
-    const unsigned int key = lane < KT ? ((unsigned int)count << 8) | (unsigned int)(KT - 1 - lane) : 0u;
-    const unsigned int best = __reduce_max_sync(0xFFFFFFFFu, key);
-    const int seed = KT - 1 - (int)(best & 0xFFu);
-    return pack_pattern(__shfl_sync(0xFFFFFFFFu, (unsigned int)bits, seed), seed);
-}
-
 // Warp-wide sums of NP per-lane values by recursive halving, added to dst: in each round a lane keeps the half of its
 // values chosen by one bit of its number, adding its partner's copy of that half, so about NP shuffles (not 5 NP)
 // leave every sum in one lane.  A fixed tree.
@@ -323,6 +282,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     __shared__ int stage_n[kStages];
     __shared__ double ssum[CW][NP];         // per-warp sums
     __shared__ double sgram[KT * KT];
+    __shared__ int seed_counts[KT];
     __shared__ const T *list[kGsMaxK];      // accepted gradients in the order they are added
     __shared__ int n_list;                  // c
     __shared__ int sh_ok, sh_again;         // outcome of a wait; how many tiles are fetched a second time
@@ -607,29 +567,21 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     // Algorithm 1 (or its order-indifferent variant) on sgram, by all consumers: decided pattern into sh_final and, if
     // there are lines, to every CTA; mask, distances and count to their places.
     auto decide = [&](unsigned long long *lines) {
-        if (a.ring.K > 0) {
-            __shared__ RingTable<KT> table;
-            ring_replay_parallel<KT, Sync>(a.ring, sgram, table,
-                                           [&](int seed, unsigned long long bits) { sh_final = pack_pattern((unsigned int)bits, seed); });
-            if (lines != nullptr && warp == 0) { __syncwarp(); tell(lines, sh_final); }
-        } else if (warp == 0) {
-            double dist;
-            int status;
-            const unsigned int final = warp_walk<KT>(sgram, a.replay.tau, dist, status);
+        const bool any_seed = a.ring.K > 0;
+        const double tau = any_seed ? a.ring.tau : a.replay.tau;
+        const int seed = any_seed ? best_seed<1, Sync>(sgram, KT, tau, seed_counts) : 0;
+        if (warp == 0) {
+            WalkSteps<1> st;
+            const WalkResult r = warp_walk<1>(sgram, KT, seed, tau, st);
+            const unsigned int final = pack_pattern((unsigned int)r.bits, seed);
             if (lines != nullptr) tell(lines, final);
-            const unsigned int bits = final & 0xFFu;
-            if (lane < KT) {
-                a.replay.mask_out[a.replay.idx[lane]] = (uint8_t)((bits >> lane) & 1u);
-                if (a.replay.dist_out) a.replay.dist_out[a.replay.idx[lane]] = (float)dist;
-            }
             if (lane == 0) {
                 sh_final = final;
-                ctl->accept_bits = bits;
-                ctl->ring_seed = -1;
-                ctl->count = __popc(bits);
-                *a.replay.count_out = __popc(bits);
-                if (status) atomicOr(&ctl->status, status);
+                ctl->ring_seed = any_seed ? seed : -1;
+                if (any_seed) *a.ring.seed_out = seed;
             }
+            if (any_seed) walk_outputs<1>(sgram, KT, seed, r, st, nullptr, a.ring.mask_out, a.ring.dist_out, a.ring.count_out, ctl);
+            else walk_outputs<1>(sgram, KT, seed, r, st, a.replay.idx, a.replay.mask_out, a.replay.dist_out, a.replay.count_out, ctl);
         }
         Sync::sync();
     };
@@ -663,11 +615,12 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
                 value = (double)__uint_as_float((unsigned int)(w >> 32));
                 return (unsigned int)w == tag && !a.test_withhold;
             }, limit, nullptr);
+            const bool any_seed = a.ring.K > 0;
+            const double tau = any_seed ? a.ring.tau : a.replay.tau;
+            const int seed = known && any_seed ? best_seed<1, Sync>(sgram, KT, tau, seed_counts) : 0;
             if (warp == 0 && known) {
-                double dist;
-                int status;
-                const unsigned int guess = a.ring.K > 0 ? warp_ring_guess<KT>(a.ring, sgram)
-                                                        : warp_walk<KT>(sgram, a.replay.tau, dist, status);
+                WalkSteps<1> st;
+                const unsigned int guess = pack_pattern((unsigned int)warp_walk<1>(sgram, KT, seed, tau, st).bits, seed);
                 if (lane == 0) sh_pred = guess;
                 tell(a.verdicts, guess);
             }

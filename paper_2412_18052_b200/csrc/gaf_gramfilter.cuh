@@ -5,7 +5,7 @@
 // the K x K Gram matrix G_ij = <g_i, g_j> of the raw micro-gradients:
 //     <g_i, sum_A g_j> = sum_{j in A} G_ji,     |sum_A g_j|^2 = sum_{j,l in A} G_jl.
 // The schedule therefore reads every gradient ONCE to build G (binary64 sums), walks
-// the K-1 sequential decisions of Algorithm 1 on K^2 scalars in a single thread, and
+// the K-1 sequential decisions of Algorithm 1 on K^2 scalars in one warp, and
 // then reads only the accepted gradients once more to write g/c (Eq. 5):
 // ((K + c) b + 4) D bytes instead of one pass over the running sum per step, and no
 // grid-wide serialisation per step.  The accepted gradients are added in processing
@@ -20,8 +20,6 @@ namespace gaf {
 
 constexpr int kGsThreads = 512;
 constexpr int kGsMaxK = 8;                  // gradients the one-pass register-tiled Gram handles
-constexpr int kGsMaxCtas = 296;
-constexpr int kGsPartialStride = 320;       // per-CTA partials are stored [pair][CTA]: the totalling loads coalesce
 constexpr int kGsFlushEvery = 16;           // iterations between binary64 flushes
 constexpr int kMsThreads = 512;
 constexpr int kMsLongRun = 8;                // chunks per run of the masked-mean pass on long vectors
@@ -36,59 +34,8 @@ struct ReplayArgs {
     Control *ctl;
 };
 
-// Algorithm 1 on the Gram matrix (indexed by processing step): one thread.
-// gram is K x K row-major in binary64.  With `publish` the decisions, distances and count go
-// to the outputs and the control block; the accept bits (bit t = step t) are returned either way.
-__device__ __forceinline__ unsigned long long replay_on_gram(const ReplayArgs &r, const volatile double *gram,
-                                                             bool publish) {
-    const int K = r.K;
-    Control *c = r.ctl;
-    int status = 0, count = 1;
-    unsigned long long bits = 1ull;         // step 0 is the seed
-    double na = gram[0];                    // |g|^2 of the running sum
-    double norm_sq = gram[0];               // sum of |g_i|^2 over the accepted gradients
-    if (publish) {
-        c->decision[0] = 1;
-        r.mask_out[r.idx[0]] = 1;
-        if (r.dist_out) r.dist_out[r.idx[0]] = 0.0f;
-    }
-    for (int t = 1; t < K; ++t) {
-        double p = 0.0;                     // <g_t, running sum>
-        for (int u = 0; u < t; ++u)
-            if ((bits >> u) & 1ull) p += gram[(size_t)u * K + t];
-        const double ng = gram[(size_t)t * K + t];
-        const double d = cosine_distance(p, na, ng, &status);
-        const int accept = (d <= r.tau) ? 1 : 0;
-        if (publish) {
-            c->decision[t] = accept;
-            c->sums[t][0] = p; c->sums[t][1] = na; c->sums[t][2] = ng;
-            r.mask_out[r.idx[t]] = (uint8_t)accept;
-            if (r.dist_out) r.dist_out[r.idx[t]] = (float)d;
-        }
-        if (accept) {
-            bits |= 1ull << t;
-            na = na + 2.0 * p + ng;         // |g + g_t|^2
-            norm_sq += ng;
-            ++count;
-            status |= ill_conditioned(count, norm_sq, na);
-        }
-    }
-    if (publish) {
-        c->accept_bits = bits;
-        c->ring_seed = -1;
-        c->count = count;
-        // (OR, not store: an earlier kernel of the operation may have raised a bit; the first kernel cleared the word)
-        if (status) atomicOr(&c->status, status);
-        *r.count_out = count;
-    }
-    return bits;
-}
-
-// Order-indifferent variant (end of Section 3.1): Algorithm 1 from every seed s with the
-// others following in ring order s, s+1, ..., K-1, 0, ..., s-1; the seed with the largest
-// accepted count wins, ties to the smallest s.  Threads 0..K-1 of the calling block each walk
-// one seed on the Gram matrix (by ORIGINAL index); thread 0 then publishes the winner.
-// `scratch` holds K ints + K unsigned long longs in shared memory.  All threads must call.
+// Order-indifferent variant (end of Section 3.1): Algorithm 1 from every seed s with the others following in ring
+// order s, s+1, ..., K-1, 0, ..., s-1; the seed with the largest accepted count wins, ties to the smallest s.
 struct RingArgs {
     int K;
     double tau;
@@ -99,164 +46,114 @@ struct RingArgs {
     Control *ctl;
 };
 
-__device__ __forceinline__ void ring_walk_one_seed(const RingArgs &r, const volatile double *gram, int s,
-                                                   int &count_out, unsigned long long &bits_out, int &status_out,
-                                                   float *dist_by_index) {
-    const int K = r.K;
-    unsigned long long bits = 1ull << s;    // bit i set = gradient i (original index) accepted
-    int count = 1, status = 0;
-    double na = gram[(size_t)s * K + s], norm_sq = na;
-    if (dist_by_index) dist_by_index[s] = 0.0f;
+// ---- Algorithm 1 on a K x K Gram matrix in shared memory, by one warp ----
+// The order is the ring order from `seed` (seed 0: 0, 1, ..., K-1).  Lane l carries <g_j, running sum> for j = l, l + 32, ...
+// (JW values), each summed in processing order; every lane takes every decision.  A step's distance needs a square
+// root and a division, 350 cycles when the steps wait for one another; but the decision alone needs the cosine to the
+// accuracy of its distance from 1 - tau, so it is taken on a binary32 estimate (error below 1e-6) where that is 1e-5 or more away
+// and on Eq. 4 itself otherwise.  The distances are Eq. 4 for all steps at once, afterwards.  (One thread that walked the
+// matrix in global memory took 17 us with 16 gradients, 60 with 32 and 150 with 64; this takes 1, 2 and 4.)
+template <int JW> struct WalkSteps {        // what lane l knows of the steps of its gradients j
+    double p[JW], na[JW], norm_sq[JW];      // <g_j, g>, |g|^2 before the step, sum of |g_i|^2 with g_j
+    int count[JW];                          // c if g_j is accepted
+};
+struct WalkResult {
+    unsigned long long bits;                // bit j = gradient j accepted
+    int count;
+};
+template <int JW>
+__device__ __forceinline__ WalkResult warp_walk(const double *gram, int K, int seed, double tau, WalkSteps<JW> &st) {
+    const int lane = threadIdx.x & 31;
+    double pj[JW];
+#pragma unroll
+    for (int w = 0; w < JW; ++w) {
+        pj[w] = lane + 32 * w < K ? gram[seed * K + lane + 32 * w] : 0.0;
+        st.p[w] = st.na[w] = st.norm_sq[w] = 0.0;
+        st.count[w] = 1;
+    }
+    double na = gram[seed * K + seed], norm_sq = na;
+    const float bound = (float)(1.0 - tau);
+    WalkResult r = {1ull << seed, 1};
+#pragma unroll 1
     for (int t = 1; t < K; ++t) {
-        const int i = (s + t) % K;
-        double p = 0.0;
-        for (int u = 0; u < t; ++u) {       // accepted gradients in processing order
-            const int j = (s + u) % K;
-            if ((bits >> j) & 1ull) p += gram[(size_t)j * K + i];
+        const int i = seed + t < K ? seed + t : seed + t - K;
+        double mine = pj[0];
+#pragma unroll
+        for (int w = 1; w < JW; ++w) mine = i >= 32 * w ? pj[w] : mine;
+        const double p = __shfl_sync(0xFFFFFFFFu, mine, i & 31), ng = gram[i * K + i];
+        const float fp = (float)p, fa = (float)na, fg = (float)ng;
+        const float margin = fp * (rsqrtf(fa) * rsqrtf(fg)) - bound;
+        bool accept = margin >= 0.0f;
+        const bool safe = fa > 1e-30f && fa < 1e30f && fg > 1e-30f && fg < 1e30f && fabsf(fp) < 1e30f && fabsf(margin) > 1e-5f;
+        if (!safe) {
+            int ignored = 0;
+            accept = cosine_distance(p, na, ng, &ignored) <= tau;
         }
-        const double ng = gram[(size_t)i * K + i];
-        const double d = cosine_distance(p, na, ng, &status);
-        if (dist_by_index) dist_by_index[i] = (float)d;
-        if (d <= r.tau) {
-            bits |= 1ull << i;
-            na = na + 2.0 * p + ng;
+#pragma unroll
+        for (int w = 0; w < JW; ++w)
+            if (lane + 32 * w == i) { st.p[w] = p; st.na[w] = na; st.norm_sq[w] = norm_sq + ng; st.count[w] = r.count + 1; }
+        if (accept) {
+            r.bits |= 1ull << i;
+            ++r.count;
+            na = na + 2.0 * p + ng;         // |g + g_i|^2
             norm_sq += ng;
-            ++count;
-            status |= ill_conditioned(count, norm_sq, na);
+#pragma unroll
+            for (int w = 0; w < JW; ++w)
+                if (lane + 32 * w < K) pj[w] += gram[i * K + lane + 32 * w];
         }
     }
-    count_out = count; bits_out = bits; status_out = status;
+    return r;
 }
-
-// `early`, when given, is called by thread 0 with (winning seed, its accept bits) as soon as they are
-// known, before the outputs are written.
-struct NoEarlyNotice {
-    __device__ __forceinline__ void operator()(int, unsigned long long) const {}
-};
-template <typename Early = NoEarlyNotice>
-__device__ __forceinline__ void ring_replay_on_gram(const RingArgs &r, const volatile double *gram,
-                                                    int *sh_count, unsigned long long *sh_bits,
-                                                    Early early = Early()) {
-    const int K = r.K;
-    if ((int)threadIdx.x < K) {
-        int c, st;
-        unsigned long long b;
-        ring_walk_one_seed(r, gram, threadIdx.x, c, b, st, nullptr);
-        sh_count[threadIdx.x] = c;
-        sh_bits[threadIdx.x] = b;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int best = 0;
-        for (int s = 1; s < K; ++s)
-            if (sh_count[s] > sh_count[best]) best = s;
-        early(best, sh_bits[best]);
-        // walk the winner once more to write its distances and status
-        int c, st;
-        unsigned long long b;
-        ring_walk_one_seed(r, gram, best, c, b, st, r.dist_out);
-        for (int i = 0; i < K; ++i) r.mask_out[i] = (uint8_t)((b >> i) & 1ull);
-        Control *ctl = r.ctl;
-        ctl->accept_bits = b;
-        ctl->ring_seed = best;
-        ctl->count = c;
-        if (st) atomicOr(&ctl->status, st);
-        *r.count_out = c;
-        *r.seed_out = best;
-        __threadfence();
-    }
-}
-
-// The any-seed walks in table form (K <= 8).  Step t's test depends on the earlier decisions only through WHICH
-// gradients were accepted, so one thread per (seed, step t, accept pattern of the seed's steps 1..t-1) evaluates Eq. 4 on the Gram matrix by
-// ORIGINAL index (step v of seed s is gradient (s + v) mod K), one thread per seed then follows its
-// decisions through the table, and thread 0 picks the largest count (ties to the smallest seed) and
-// publishes.  Same sums in the same order as ring_walk_one_seed: identical outputs.
-// All threads of `Sync` call; `early(seed, bits)` as in ring_replay_on_gram.
-template <int KT>
-struct RingTable {
-    static constexpr int kCases = (1 << (KT - 1)) - 1;          // per seed
-    float d[KT * kCases + 1];
-    unsigned char accept[KT * kCases + 1], status[KT * kCases + 1];
-    int count[KT];
-    unsigned int steps[KT];                                     // bit t-1 = step t of this seed accepted
-};
-template <int KT, typename Sync, typename Early = NoEarlyNotice>
-__device__ __forceinline__ void ring_replay_parallel(const RingArgs &r, const double *gram, RingTable<KT> &tb,
-                                                     Early early = Early()) {
-    constexpr int K = KT, C = RingTable<KT>::kCases;
-    for (int idx = threadIdx.x; idx < K * C; idx += Sync::threads()) {
-        const int s = idx / C, cs = idx - s * C;
-        const int t = 32 - __clz(cs + 1);
-        const unsigned int m = (unsigned int)(cs + 1) - (1u << (t - 1));
-        auto in = [&](int v) { return v == 0 || ((m >> (v - 1)) & 1u); };
-        auto gi = [&](int v) { const int i = s + v; return i >= K ? i - K : i; };      // gradient of step v
-        double na = gram[s * K + s], norm_sq = na;
-        int cnt = 1;
+// Mask, distances and count of a walk to their places, by the warp that walked.  Gradient j of the matrix is gradient
+// idx[j] of the caller (idx null: the same).
+template <int JW>
+__device__ __forceinline__ void walk_outputs(const double *gram, int K, int seed, const WalkResult &r, const WalkSteps<JW> &st,
+                                             const int *idx, uint8_t *mask_out, float *dist_out, int32_t *count_out,
+                                             Control *ctl) {
+    const int lane = threadIdx.x & 31;
+    int status = 0;
 #pragma unroll
-        for (int u = 1; u < K - 1; ++u) {
-            double pu = 0.0;
-#pragma unroll
-            for (int v = 0; v < u; ++v) pu += in(v) ? gram[gi(v) * K + gi(u)] : 0.0;
-            const double guu = gram[gi(u) * K + gi(u)];
-            const double grown = na + 2.0 * pu + guu;
-            na = in(u) ? grown : na;
-            norm_sq += in(u) ? guu : 0.0;
-            cnt += in(u) ? 1 : 0;
+    for (int w = 0; w < JW; ++w) {
+        const int j = lane + 32 * w;
+        if (j >= K) continue;
+        const bool accepted = (r.bits >> j) & 1ull;
+        double d = 0.0;
+        if (j != seed) {
+            const double ng = gram[j * K + j];
+            d = cosine_distance(st.p[w], st.na[w], ng, &status);
+            // the conditioning of the sum that an accept leaves behind
+            if (accepted) status |= ill_conditioned(st.count[w], st.norm_sq[w], st.na[w] + 2.0 * st.p[w] + ng);
         }
-        double p = 0.0;
-#pragma unroll
-        for (int v = 0; v < K - 1; ++v) p += (v < t && in(v)) ? gram[gi(v) * K + gi(t)] : 0.0;
-        int status = 0;
-        const double ng = gram[gi(t) * K + gi(t)];
-        const double d = cosine_distance(p, na, ng, &status);
-        const int accept = (d <= r.tau) ? 1 : 0;
-        status |= accept ? ill_conditioned(cnt + 1, norm_sq + ng, na + 2.0 * p + ng) : 0;
-        tb.d[idx] = (float)d;
-        tb.accept[idx] = (unsigned char)accept;
-        tb.status[idx] = (unsigned char)status;
+        const int o = idx ? idx[j] : j;
+        mask_out[o] = accepted ? 1 : 0;
+        if (dist_out) dist_out[o] = (float)d;
     }
-    Sync::sync();
-    if ((int)threadIdx.x < K) {
-        const int s = threadIdx.x;
-        unsigned int m = 0;
-        int count = 1;
-        for (int t = 1; t < K; ++t) {
-            const int node = s * C + (1 << (t - 1)) - 1 + (int)m;
-            if (tb.accept[node]) { m |= 1u << (t - 1); ++count; }
-        }
-        tb.count[s] = count;
-        tb.steps[s] = m;
-    }
-    Sync::sync();
-    if (threadIdx.x == 0) {
-        int best = 0;
-        for (int s = 1; s < K; ++s)
-            if (tb.count[s] > tb.count[best]) best = s;
-        const unsigned int steps = tb.steps[best];
-        unsigned long long bits = 1ull << best;                 // by original index
-        for (int t = 1; t < K; ++t)
-            if ((steps >> (t - 1)) & 1u) bits |= 1ull << ((best + t) % K);
-        early(best, bits);
-        int status = 0;
-        unsigned int m = 0;
-        if (r.dist_out) r.dist_out[best] = 0.0f;
-        for (int t = 1; t < K; ++t) {
-            const int node = best * C + (1 << (t - 1)) - 1 + (int)m;
-            if (r.dist_out) r.dist_out[(best + t) % K] = tb.d[node];
-            status |= tb.status[node];
-            if (tb.accept[node]) m |= 1u << (t - 1);
-        }
-        for (int i = 0; i < K; ++i) r.mask_out[i] = (uint8_t)((bits >> i) & 1ull);
-        Control *ctl = r.ctl;
-        ctl->accept_bits = bits;
-        ctl->ring_seed = best;
-        ctl->count = tb.count[best];
+    status = __reduce_or_sync(0xFFFFFFFFu, status);
+    if (lane == 0) {
+        *count_out = r.count;
+        ctl->accept_bits = r.bits;
+        ctl->count = r.count;
+        // (OR, not store: an earlier kernel of the operation may have raised a bit; the first kernel cleared the word)
         if (status) atomicOr(&ctl->status, status);
-        *r.count_out = tb.count[best];
-        *r.seed_out = best;
-        __threadfence();
     }
+}
+// The seed with the largest accepted count; the warps of `Sync` share the walks.  `counts`: K ints in shared memory.
+template <int JW, typename Sync>
+__device__ __forceinline__ int best_seed(const double *gram, int K, double tau, int *counts) {
+    const int lane = threadIdx.x & 31;
+    for (int s = threadIdx.x >> 5; s < K; s += Sync::threads() / 32) {
+        WalkSteps<JW> st;
+        const WalkResult r = warp_walk<JW>(gram, K, s, tau, st);
+        if (lane == 0) counts[s] = r.count;
+    }
+    Sync::sync();
+    unsigned int key = 0;
+#pragma unroll
+    for (int w = 0; w < JW; ++w) {
+        const int s = lane + 32 * w;
+        if (s < K) key = max(key, ((unsigned int)counts[s] << 8) | (unsigned int)(GAF_MAX_K - 1 - s));
+    }
+    return GAF_MAX_K - 1 - (int)(__reduce_max_sync(0xFFFFFFFFu, key) & 0xFFu);
 }
 
 // 16-byte read-only load with an explicit L2 eviction policy.
@@ -319,27 +216,6 @@ template <> struct GsAcc<float, 3> { using type = double; static constexpr bool 
 template <> struct GsAcc<float, 4> { using type = double; static constexpr bool kPeriodicFlush = false; };
 __device__ __forceinline__ float gs_fma(float a, float b, float s) { return fmaf(a, b, s); }
 __device__ __forceinline__ double gs_fma(float a, float b, double s) { return fma((double)a, (double)b, s); }
-
-// Scalar walk as its own launch (Gram matrix produced by the tiled pairwise kernels).
-// `perm` maps processing step -> row of `gram_by_index` (K x K by original index).
-__global__ void gram_replay_kernel(ReplayArgs r, const double *gram_by_index, double *gram_by_step) {
-    const int K = r.K;
-    for (int i = threadIdx.x; i < K * K; i += blockDim.x) {
-        const int t = i / K, u = i % K;
-        gram_by_step[i] = gram_by_index[(size_t)r.idx[t] * K + r.idx[u]];
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) { replay_on_gram(r, gram_by_step, true); __threadfence(); }
-}
-
-// Any-seed walk as its own launch (Gram matrix by original index from the tiled or
-// tensor-core kernels).  One block of at least K threads.
-__global__ void gram_ring_replay_kernel(RingArgs r, const double *gram_by_index) {
-    __shared__ int ring_count[GAF_MAX_K];
-    __shared__ unsigned long long ring_bits[GAF_MAX_K];
-    ring_replay_on_gram(r, gram_by_index, ring_count, ring_bits);
-}
 
 // ------------------------------------------------------- masked mean (Eq. 5) --
 

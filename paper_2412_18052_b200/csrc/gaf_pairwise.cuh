@@ -4,10 +4,11 @@
 // What the Gram kernels for more than 8 gradients share (gaf_gram_panel.cuh on CUDA cores,
 // gaf_gram_tc.cuh on tensor cores): the K x K matrix cut into 8 x 8 tiles of pairs, per-CTA
 // binary64 partial sums in a [tile pair][slice][64] layout, and the finishing kernel that totals
-// the slices in a fixed order and whose last CTA derives the distances.
+// the slices in a fixed order and whose last CTA derives the distances, or walks Algorithm 1 on the matrix.
 #pragma once
 
 #include "gaf_device.cuh"
+#include "gaf_gramfilter.cuh"
 
 namespace gaf {
 
@@ -25,6 +26,8 @@ struct GramArgs {
     double *gram_out;       // [K][K] or null
     Control *ctl;
     int slices;
+    ReplayArgs replay;      // replay.K > 0: Algorithm 1 on the matrix instead of the distances of all pairs
+    RingArgs ring;          // ring.K > 0: its order-indifferent variant
 };
 
 // Decode the linear upper-triangle tile index into (ti, tj), ti <= tj.
@@ -34,11 +37,16 @@ __device__ __forceinline__ void tile_pair(int idx, int tiles, int &ti, int &tj) 
     tj = ti + idx;
 }
 
-// One CTA per tile pair: sums the slices in a fixed order, writes both triangles of
-// the Gram matrix; the last CTA to finish turns the Gram matrix into distances.
+// One CTA per tile pair: sums the slices in a fixed order, writes both triangles of the Gram matrix; the last CTA to
+// finish turns the Gram matrix into distances, or takes the filter's decisions on it.
 constexpr int kFinishParts = 16;        // each entry's slices are summed in 16 independent chains
-__global__ void __launch_bounds__(64 * kFinishParts) gram_finish_kernel(GramArgs a) {
+struct FinishBlock {
+    static __device__ __forceinline__ void sync() { __syncthreads(); }
+    static __device__ __forceinline__ constexpr int threads() { return 64 * kFinishParts; }
+};
+__global__ void __launch_bounds__(64 * kFinishParts) gram_finish_kernel(const __grid_constant__ GramArgs a) {
     __shared__ double part[kFinishParts][64];
+    __shared__ double sgram[GAF_MAX_K * GAF_MAX_K];
     __shared__ bool is_last;
     int ti, tj;
     tile_pair(blockIdx.x, a.tiles, ti, tj);
@@ -73,11 +81,36 @@ __global__ void __launch_bounds__(64 * kFinishParts) gram_finish_kernel(GramArgs
     if (threadIdx.x == 0) is_last = take_last_ticket(&a.ctl->ticket, gridDim.x);
     __syncthreads();
     if (!is_last) return;
-    const volatile double *G = a.gram;
+    const int K = a.K;
+    if (a.replay.K > 0 || a.ring.K > 0) {
+        const bool any_seed = a.ring.K > 0;
+        // by processing step, or by original index (the ring orders start anywhere)
+        for (int e = threadIdx.x; e < K * K; e += blockDim.x) {
+            const int t = e / K, u = e % K;
+            const int i = any_seed ? t : a.replay.idx[t], j = any_seed ? u : a.replay.idx[u];
+            sgram[e] = __ldcg(a.gram + (size_t)i * K + j);
+        }
+        __syncthreads();
+        const double tau = any_seed ? a.ring.tau : a.replay.tau;
+        int *counts = reinterpret_cast<int *>(&part[0][0]);
+        const int seed = any_seed ? best_seed<2, FinishBlock>(sgram, K, tau, counts) : 0;
+        if (threadIdx.x < 32) {
+            WalkSteps<2> st;
+            const WalkResult r = warp_walk<2>(sgram, K, seed, tau, st);
+            if (any_seed) walk_outputs<2>(sgram, K, seed, r, st, nullptr, a.ring.mask_out, a.ring.dist_out, a.ring.count_out, a.ctl);
+            else walk_outputs<2>(sgram, K, seed, r, st, a.replay.idx, a.replay.mask_out, a.replay.dist_out, a.replay.count_out, a.ctl);
+            if (threadIdx.x == 0) {
+                a.ctl->ring_seed = any_seed ? seed : -1;
+                if (any_seed) *a.ring.seed_out = seed;
+            }
+        }
+        return;
+    }
+    const double *G = a.gram;
     int status = 0;
     for (int idx = threadIdx.x; idx < a.K * a.K; idx += blockDim.x) {
         int i = idx / a.K, j = idx % a.K;
-        double gii = G[(size_t)i * a.K + i], gjj = G[(size_t)j * a.K + j], gij = G[idx];
+        double gii = __ldcg(G + (size_t)i * a.K + i), gjj = __ldcg(G + (size_t)j * a.K + j), gij = __ldcg(G + idx);
         double d;
         if (i == j && gii > 0.0) d = 0.0;
         else d = cosine_distance(gij, gii, gjj, &status);
