@@ -637,12 +637,16 @@ int launch_stepwise(const void *const *g, int K, int64_t D, double tau, const in
     a.seed_index = ord[0];
     a.g_seed = g[ord[0]];
     if (K == 1) {
-        step_kernel<T, kOnly><<<grid, kStepThreads, 0, st>>>(a);
+        const cudaError_t err = launch_dependent(step_kernel<T, kOnly>, grid, kStepThreads, st, a);
         ++g_launches;
-        return cudaGetLastError() == cudaSuccess ? GAF_OK : GAF_ERR_CUDA;
+        if (err != cudaSuccess) { cudaGetLastError(); return GAF_ERR_CUDA; }
+        return GAF_OK;
     }
     a.t = 0; a.g_next = g[ord[1]]; a.i_next = ord[1];
-    step_kernel<T, kFirst><<<grid, kStepThreads, 0, st>>>(a);
+    if (launch_dependent(step_kernel<T, kFirst>, grid, kStepThreads, st, a) != cudaSuccess) {
+        cudaGetLastError();
+        return GAF_ERR_CUDA;
+    }
     ++g_launches;
     for (int t = 1; t <= K - 2; ++t) {
         a.t = t; a.g_cur = g[ord[t]]; a.g_next = g[ord[t + 1]]; a.i_next = ord[t + 1];
@@ -974,10 +978,11 @@ int gaf_stream_begin(const void *seed, int64_t D, int dtype, float *acc, void *w
     a.mask_out = ctl->stream_mask; a.dist_out = ctl->stream_dist; a.count_out = &ctl->count;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int grid = stream_grid(D, kStepThreads, di.sms);
-    if (dtype == GAF_F32) step_kernel<float, kOnly><<<grid, kStepThreads, 0, st>>>(a);
-    else step_kernel<__nv_bfloat16, kOnly><<<grid, kStepThreads, 0, st>>>(a);
+    const cudaError_t err = dtype == GAF_F32 ? launch_dependent(step_kernel<float, kOnly>, grid, kStepThreads, st, a)
+                                             : launch_dependent(step_kernel<__nv_bfloat16, kOnly>, grid, kStepThreads, st, a);
     ++g_launches;
-    return cudaGetLastError() == cudaSuccess ? GAF_OK : GAF_ERR_CUDA;
+    if (err != cudaSuccess) { cudaGetLastError(); return GAF_ERR_CUDA; }
+    return GAF_OK;
 }
 
 int gaf_stream_push(const void *g, int t, int64_t D, int dtype, double tau, float *acc, void *workspace,
@@ -999,19 +1004,13 @@ int gaf_stream_push(const void *g, int t, int64_t D, int dtype, double tau, floa
                  reinterpret_cast<double *>(base + kPartialsOffset), tau, t};
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int grid = stream_grid(D, kStreamThreads, di.sms);
-    if (dtype == GAF_F32) {
-        stream_test_kernel<float><<<grid, kStreamThreads, 0, st>>>(a);
-        if (launch_dependent(stream_add_kernel<float>, grid, kStreamThreads, st, a) != cudaSuccess) {
-            cudaGetLastError();
-            return GAF_ERR_CUDA;
-        }
-    } else {
-        stream_test_kernel<__nv_bfloat16><<<grid, kStreamThreads, 0, st>>>(a);
-        if (launch_dependent(stream_add_kernel<__nv_bfloat16>, grid, kStreamThreads, st, a) != cudaSuccess) {
-            cudaGetLastError();
-            return GAF_ERR_CUDA;
-        }
-    }
+    auto launch = [&](auto test, auto add) {
+        return launch_dependent(test, grid, kStreamThreads, st, a) == cudaSuccess &&
+               launch_dependent(add, grid, kStreamThreads, st, a) == cudaSuccess;
+    };
+    const bool ok = dtype == GAF_F32 ? launch(stream_test_kernel<float>, stream_add_kernel<float>)
+                                     : launch(stream_test_kernel<__nv_bfloat16>, stream_add_kernel<__nv_bfloat16>);
+    if (!ok) { cudaGetLastError(); return GAF_ERR_CUDA; }
     g_launches += 2;
     return cudaGetLastError() == cudaSuccess ? GAF_OK : GAF_ERR_CUDA;
 }
@@ -1026,9 +1025,10 @@ int gaf_stream_end(int K, int64_t D, float *acc, uint8_t *mask_out, float *dist_
     if (!device_info(&di)) return GAF_ERR_CUDA;
     StreamEndArgs a{acc, D, K, static_cast<const Control *>(workspace), mask_out, dist_out, count_out};
     const int grid = stream_grid(D, kStreamThreads, di.sms);
-    stream_end_kernel<<<grid, kStreamThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(a);
+    const cudaError_t err = launch_dependent(stream_end_kernel, grid, kStreamThreads, static_cast<cudaStream_t>(cuda_stream), a);
     ++g_launches;
-    return cudaGetLastError() == cudaSuccess ? GAF_OK : GAF_ERR_CUDA;
+    if (err != cudaSuccess) { cudaGetLastError(); return GAF_ERR_CUDA; }
+    return GAF_OK;
 }
 
 int gaf_host_staging_bytes(int K, int64_t D, int dtype, size_t *bytes_out) {

@@ -75,10 +75,10 @@ __global__ void __launch_bounds__(kStepThreads, 2) step_kernel(StepArgs a) {
     float *acc = a.acc;
 
     int accept = 0, count = 1;
+    // launched as a programmatic dependent of what precedes it on the stream (the previous step's launch): its blocks are
+    // placed while that grid winds down, and wait here until it has completed and its decision is visible
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (MODE == kMid || MODE == kLast) {
-        // launched as a programmatic dependent of the previous step's launch: its blocks are placed
-        // while that grid winds down, and wait here until it has completed and its decision is visible
-        asm volatile("griddepcontrol.wait;" ::: "memory");
         accept = *reinterpret_cast<volatile int *>(&a.ctl->decision[a.t]);
         count = *reinterpret_cast<volatile int *>(&a.ctl->count);
     }
@@ -98,7 +98,10 @@ __global__ void __launch_bounds__(kStepThreads, 2) step_kernel(StepArgs a) {
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
     const int64_t n_oct = a.D / kOct;
 
-    for (int64_t o = tid; o < n_oct; o += nthreads) {
+    for (int64_t q = tid; q < n_oct; q += nthreads) {
+        // (one gradient, the start of the streaming form: from the end, so that the first test, which starts at the
+        // start, finds that part of the running sum in L2)
+        const int64_t o = MODE == kOnly ? n_oct - 1 - q : q;
         const int64_t e = o * kOct;
         float v[8], gc[8], gn[8];
         if (MODE == kFirst || MODE == kOnly) load8_stream<T>(g_seed, e, v);
@@ -114,7 +117,7 @@ __global__ void __launch_bounds__(kStepThreads, 2) step_kernel(StepArgs a) {
             for (int k = 0; k < 8; ++k) v[k] = v[k] / inv_note;
             store8(acc, e, v, true);
         } else if (MODE == kFirst || MODE == kOnly || accept) {
-            store8(acc, e, v, MODE == kOnly);
+            store8(acc, e, v, false);
         }
         if (MODE == kFirst || MODE == kMid) {
             s.p += (double)dot8(v, gn);
@@ -143,7 +146,11 @@ __global__ void __launch_bounds__(kStepThreads, 2) step_kernel(StepArgs a) {
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         Sums3 blk = block_reduce(s, scratch);
         finalize_step(a, blk, a.t + 1);
-    } else if (MODE == kLast) {
+    } else {
+        // (a dependent of this launch waits for this grid itself)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
+    if (MODE == kLast) {
         if (blockIdx.x == 0 && threadIdx.x == 0) *a.count_out = count;
     }
 }
