@@ -1,8 +1,8 @@
-"""Thin ctypes binding of the C ABI in ``include/gaf.h``.
+"""Thin binding of the C ABI in ``include/gaf.h``.
 
-Argument marshalling only: every step of the path runs in the CUDA library.
-PyTorch supplies device memory and the stream.  There is no fallback: if the
-shared library has not been built, or a call fails, an exception is raised.
+Argument marshalling only: every step of the path runs in the CUDA library.  The calls of a training step go through
+the CPython extension ``csrc/gaf_native.cpp``, the others through ctypes.  PyTorch supplies device memory and the
+stream.  There is no fallback: if the shared libraries have not been built, or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
@@ -77,6 +77,24 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_native_module = None
+
+
+def _native():
+    """The extension module over the library.  Raises if it has not been built."""
+    global _native_module
+    if _native_module is None:
+        lib()
+        try:
+            from . import _gaf_native
+        except ImportError as e:
+            raise RuntimeError("_gaf_native.so is missing or does not load: build it with "
+                               f"`python -m paper_2412_18052_b200.build` ({e})") from e
+        _gaf_native.register_error(GafError)
+        _native_module = _gaf_native
+    return _native_module
+
+
 def _check(code: int, where: str) -> None:
     if code != 0:
         raise GafError(code, where)
@@ -133,15 +151,7 @@ def gaf_cosdist(x: torch.Tensor, y: torch.Tensor, workspace: torch.Tensor,
                 dist_out: Optional[torch.Tensor] = None,
                 stats_out: Optional[torch.Tensor] = None) -> Tuple[torch.Tensor, torch.Tensor]:
     """Eq. 4 between two device tensors.  Returns (dist[1] float32, stats[3] float64)."""
-    assert x.numel() == y.numel() and x.dtype == y.dtype
-    if dist_out is None:
-        dist_out = torch.empty(1, dtype=torch.float32, device=x.device)
-    if stats_out is None:
-        stats_out = torch.empty(3, dtype=torch.float64, device=x.device)
-    _check(lib().gaf_cosdist(x.data_ptr(), y.data_ptr(), x.numel(), _dtype_code(x),
-                             dist_out.data_ptr(), stats_out.data_ptr(),
-                             workspace.data_ptr(), workspace.numel(), _stream()), "gaf_cosdist")
-    return dist_out, stats_out
+    return _native().cosdist(x, y, workspace, dist_out, stats_out)
 
 
 def gaf_cosdist_static(x: torch.Tensor, y: torch.Tensor, dist_out: torch.Tensor,
@@ -165,27 +175,7 @@ def gaf_filter_accumulate(grads: Sequence[torch.Tensor], tau: float, workspace: 
                           count_out: Optional[torch.Tensor] = None,
                           schedule: int = GAF_SCHED_AUTO):
     """Algorithm 1 + Eq. 5 on device tensors.  Returns (macro, mask, dist, count) device tensors."""
-    K, D = len(grads), grads[0].numel()
-    dev = grads[0].device
-    code = _dtype_code(grads[0])
-    for g in grads:
-        assert g.numel() == D and g.dtype == grads[0].dtype and g.is_contiguous()
-    if macro_out is None:
-        macro_out = torch.empty(D, dtype=torch.float32, device=dev)
-    if mask_out is None:
-        mask_out = torch.empty(K, dtype=torch.uint8, device=dev)
-    if dist_out is None:
-        dist_out = torch.empty(K, dtype=torch.float32, device=dev)
-    if count_out is None:
-        count_out = torch.empty(1, dtype=torch.int32, device=dev)
-    ptrs = _ptr_array(grads)
-    ordp = _order_array(order)
-    _check(lib().gaf_filter_accumulate(ctypes.cast(ptrs, ctypes.c_void_p), K, D, code, float(tau),
-                                       ordp and ctypes.cast(ordp, ctypes.c_void_p),
-                                       macro_out.data_ptr(), mask_out.data_ptr(), dist_out.data_ptr(),
-                                       count_out.data_ptr(), workspace.data_ptr(), workspace.numel(),
-                                       int(schedule), _stream()), "gaf_filter_accumulate")
-    return macro_out, mask_out, dist_out, count_out
+    return _native().filter_accumulate(grads, tau, workspace, order, macro_out, mask_out, dist_out, count_out, schedule)
 
 
 def gaf_filter_accumulate_repeat(repeats: int, sets: Sequence[Sequence[torch.Tensor]], tau: float,
@@ -209,21 +199,7 @@ def gaf_filter_accumulate_any_seed(grads: Sequence[torch.Tensor], tau: float, wo
                                    macro_out: Optional[torch.Tensor] = None):
     """Order-indifferent variant (end of Section 3.1): every gradient in turn is the seed, ring
     order, largest accepted count wins.  Returns (macro, mask, dist, count, seed) device tensors."""
-    K, D = len(grads), grads[0].numel()
-    dev = grads[0].device
-    if macro_out is None:
-        macro_out = torch.empty(D, dtype=torch.float32, device=dev)
-    mask_out = torch.empty(K, dtype=torch.uint8, device=dev)
-    dist_out = torch.empty(K, dtype=torch.float32, device=dev)
-    count_out = torch.empty(1, dtype=torch.int32, device=dev)
-    seed_out = torch.empty(1, dtype=torch.int32, device=dev)
-    ptrs = _ptr_array(grads)
-    _check(lib().gaf_filter_accumulate_any_seed(
-        ctypes.cast(ptrs, ctypes.c_void_p), K, D, _dtype_code(grads[0]), float(tau),
-        macro_out.data_ptr(), mask_out.data_ptr(), dist_out.data_ptr(), count_out.data_ptr(),
-        seed_out.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream()),
-        "gaf_filter_accumulate_any_seed")
-    return macro_out, mask_out, dist_out, count_out, seed_out
+    return _native().filter_accumulate_any_seed(grads, tau, workspace, macro_out)
 
 
 def gaf_filter_accumulate_bucketed(grads: Sequence[torch.Tensor], tau: float, offsets: Sequence[int],
@@ -231,47 +207,22 @@ def gaf_filter_accumulate_bucketed(grads: Sequence[torch.Tensor], tau: float, of
                                    macro_out: Optional[torch.Tensor] = None):
     """Bucketed variant: Algorithm 1 + Eq. 5 independently on every bucket [offsets[b], offsets[b+1]).
     Returns (macro[D], mask[S,K], dist[S,K], count[S]) device tensors."""
-    K, D = len(grads), grads[0].numel()
-    S = len(offsets) - 1
-    dev = grads[0].device
-    if macro_out is None:
-        macro_out = torch.empty(D, dtype=torch.float32, device=dev)
-    mask_out = torch.empty(S, K, dtype=torch.uint8, device=dev)
-    dist_out = torch.empty(S, K, dtype=torch.float32, device=dev)
-    count_out = torch.empty(S, dtype=torch.int32, device=dev)
-    ptrs = _ptr_array(grads)
-    ordp = _order_array(order)
-    offs = (ctypes.c_int64 * (S + 1))(*[int(o) for o in offsets])
-    _check(lib().gaf_filter_accumulate_bucketed(
-        ctypes.cast(ptrs, ctypes.c_void_p), K, D, _dtype_code(grads[0]), float(tau),
-        ordp and ctypes.cast(ordp, ctypes.c_void_p), S, ctypes.cast(offs, ctypes.c_void_p),
-        macro_out.data_ptr(), mask_out.data_ptr(), dist_out.data_ptr(), count_out.data_ptr(),
-        workspace.data_ptr(), workspace.numel(), _stream()), "gaf_filter_accumulate_bucketed")
-    return macro_out, mask_out, dist_out, count_out
+    return _native().filter_accumulate_bucketed(grads, tau, offsets, workspace, order, macro_out)
 
 
 def gaf_stream_begin(seed: torch.Tensor, acc: torch.Tensor, workspace: torch.Tensor) -> None:
     """Streaming form: g <- seed, c <- 1 (``acc`` is the caller's float32 running sum)."""
-    _check(lib().gaf_stream_begin(seed.data_ptr(), seed.numel(), _dtype_code(seed), acc.data_ptr(),
-                                  workspace.data_ptr(), workspace.numel(), _stream()), "gaf_stream_begin")
+    _native().stream_begin(seed, acc, workspace)
 
 
 def gaf_stream_push(g: torch.Tensor, t: int, tau: float, acc: torch.Tensor, workspace: torch.Tensor) -> None:
     """Streaming form: test gradient number t (arrival order, from 1) and add it if accepted."""
-    _check(lib().gaf_stream_push(g.data_ptr(), int(t), g.numel(), _dtype_code(g), float(tau), acc.data_ptr(),
-                                 workspace.data_ptr(), workspace.numel(), _stream()), "gaf_stream_push")
+    _native().stream_push(g, t, tau, acc, workspace)
 
 
 def gaf_stream_end(K: int, acc: torch.Tensor, workspace: torch.Tensor):
     """Streaming form: acc <- g / c.  Returns (mask[K], dist[K], count) in arrival order."""
-    dev = acc.device
-    mask = torch.empty(K, dtype=torch.uint8, device=dev)
-    dist = torch.empty(K, dtype=torch.float32, device=dev)
-    count = torch.empty(1, dtype=torch.int32, device=dev)
-    _check(lib().gaf_stream_end(int(K), acc.numel(), acc.data_ptr(), mask.data_ptr(), dist.data_ptr(),
-                                count.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream()),
-           "gaf_stream_end")
-    return mask, dist, count
+    return _native().stream_end(K, acc, workspace)
 
 
 def gaf_filter_accumulate_host(grads_host: Sequence[torch.Tensor], tau: float,
@@ -298,18 +249,7 @@ def gaf_pairwise_cosdist(grads: Sequence[torch.Tensor], workspace: torch.Tensor,
                          dist_out: Optional[torch.Tensor] = None,
                          gram_out: Optional[torch.Tensor] = None):
     """K x K cosine-distance matrix (float32) and Gram matrix (float64) on the device."""
-    K, D = len(grads), grads[0].numel()
-    dev = grads[0].device
-    if dist_out is None:
-        dist_out = torch.empty(K, K, dtype=torch.float32, device=dev)
-    if gram_out is None:
-        gram_out = torch.empty(K, K, dtype=torch.float64, device=dev)
-    ptrs = _ptr_array(grads)
-    _check(lib().gaf_pairwise_cosdist(ctypes.cast(ptrs, ctypes.c_void_p), K, D, _dtype_code(grads[0]),
-                                      dist_out.data_ptr(), gram_out.data_ptr(),
-                                      workspace.data_ptr(), workspace.numel(), _stream()),
-           "gaf_pairwise_cosdist")
-    return dist_out, gram_out
+    return _native().pairwise_cosdist(grads, workspace, dist_out, gram_out)
 
 
 def gaf_read_status(workspace: torch.Tensor) -> int:
