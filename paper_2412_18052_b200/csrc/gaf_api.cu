@@ -294,8 +294,9 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
         w.run = D >= int64_t(32) * kMmaLongRun * per_cta * grid ? kMmaLongRun : 1;
         void (*kernel)(GramWideArgs) = gram_mma_wide_kernel;
         const int dyn = (kWideThreads / 32) * 2 * 128 * int(sizeof(double));       // [warp][tile][lane][4] doubles: 32 KB
-        kernel<<<int(grid), kWideThreads, dyn, st>>>(w);
+        const cudaError_t err = launch_dependent_smem(kernel, int(grid), kWideThreads, size_t(dyn), st, w);
         ++g_launches;
+        if (err != cudaSuccess) { cudaGetLastError(); return GAF_ERR_CUDA; }
     } else if (use_tensor_gram(K, D, dtype)) {
         // tensor cores: one CTA per SM, each with a contiguous slice of D
         GramTcArgs t{};
@@ -356,9 +357,9 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
         // A panel is at most 32 KB: 2 KB of every row up to 16 (padded) rows, 1 KB up to 32, 512 bytes
         // beyond.  With 3 or 6 tile pairs, 4 or 2 warps share a pair.
         const int shift = a.tiles <= 2 ? 7 : (a.tiles <= 4 ? 6 : 5);
-        const int wpp = a.tiles <= 2 ? 4 : (a.tiles == 3 ? 2 : 1);
+        const int wpp = a.tiles <= 2 ? 4 : (a.tiles == 3 ? 2 : (a.tiles == 4 ? 0 : 1));     // 0: 10 pairs on 12 warps
         pa.partials = a.partials; pa.ctl = a.ctl;
-        const int threads = 32 * pa.pairs_per_cta * wpp;
+        const int threads = wpp == 0 ? 32 * kPanelMaxWarps : 32 * pa.pairs_per_cta * wpp;
         const int row_bytes = 16 << shift;
         const int dyn = kPanelStages * a.tiles * 8 * row_bytes;
         // (bfloat16 comes here with a single gradient only: 2 to 8 take the register-tiled kernel, up to 64
@@ -366,11 +367,11 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
         void (*kernel)(GramPanelArgs) = nullptr;
         if (dtype == GAF_F32)
             kernel = shift == 7 ? gram_panel_kernel<float, 7, 4>
-                   : (shift == 6 ? (wpp == 2 ? gram_panel_kernel<float, 6, 2> : gram_panel_kernel<float, 6, 1>)
+                   : (shift == 6 ? (wpp == 2 ? gram_panel_kernel<float, 6, 2> : gram_panel_kernel<float, 6, 0>)
                                  : gram_panel_kernel<float, 5, 1>);
         else
             kernel = shift == 7 ? gram_panel_kernel<__nv_bfloat16, 7, 4>
-                   : (shift == 6 ? (wpp == 2 ? gram_panel_kernel<__nv_bfloat16, 6, 2> : gram_panel_kernel<__nv_bfloat16, 6, 1>)
+                   : (shift == 6 ? (wpp == 2 ? gram_panel_kernel<__nv_bfloat16, 6, 2> : gram_panel_kernel<__nv_bfloat16, 6, 0>)
                                  : gram_panel_kernel<__nv_bfloat16, 5, 1>);
         {
             // (the kernel pointer is the key: six instantiations per input type)
@@ -391,8 +392,16 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
         if (slices > work) slices = work;
         if (slices < 1) slices = 1;
         a.slices = int(slices);
-        kernel<<<dim3(a.slices, groups), threads, dyn, st>>>(pa);
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(unsigned(a.slices), unsigned(groups)); cfg.blockDim = dim3(unsigned(threads));
+        cfg.dynamicSmemBytes = size_t(dyn); cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, pa);
         ++g_launches;
+        if (err != cudaSuccess) { cudaGetLastError(); return GAF_ERR_CUDA; }
     }
     {
         // the finishing blocks are placed while the Gram kernel winds down

@@ -74,6 +74,8 @@ __global__ void __launch_bounds__(kWideThreads, 2) gram_mma_wide_kernel(const __
     extern __shared__ double wide_red[];            // [warp][tile][lane][4] at the end
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
+    // a programmatic dependent of what precedes it on the stream (a no-op after an ordinary launch)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->status = 0;            // first kernel of the operation
 
     const unsigned short *rowp[NB];

@@ -20,6 +20,8 @@
 // the FMA pipes.
 #pragma once
 
+#include <type_traits>
+
 #include "gaf_device.cuh"
 #include "gaf_pairwise.cuh"
 
@@ -66,7 +68,12 @@ template <> struct PanelLane<__nv_bfloat16> {
     }
 };
 
-// SHIFT: bytes of one gradient in one panel = 16 << SHIFT; WPP: warps that share a tile pair.  Both
+// 25 to 32 gradients: 10 tile pairs on 12 warps.  Hex digit w = tile pair of warp w: the four diagonal ones (0, 4, 7 and 9: 36
+// multiply-adds against 64) have a warp each, 5 and 6 two, so that the warps of every scheduler (w mod 4) add up to
+// 64 + 32 + 36.  One warp per pair in order left one scheduler 164 of 528 (32 x 3 M: 133 us, now 124).
+constexpr unsigned long long kPanelOwners10 = 0x974066558321ull;
+
+// SHIFT: bytes of one gradient in one panel = 16 << SHIFT; WPP: warps that share a tile pair (0: by the table above).  Both
 // are compile-time so that shared-memory addresses are immediates and a warp's steps unroll.
 template <typename T, int SHIFT, int WPP>
 __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(const __grid_constant__ GramPanelArgs a) {
@@ -79,7 +86,6 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
     const size_t stage_bytes = (size_t)rows_padded * RB;
     unsigned char *smem = reinterpret_cast<unsigned char *>(panel_smem);
 
-    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) a.ctl->status = 0;          // first kernel of the operation
     for (int i = tid; i < a.K; i += nthreads) rowp[i] = static_cast<const unsigned char *>(a.g[i]);
     for (int p = lane; p < 64; p += 32) wsum[warp][p] = 0.0;
     // rows of absent gradients (K not a multiple of 8) stay zero in every stage
@@ -90,15 +96,21 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
                 panel_smem[(size_t)s * per_stage + i] = make_uint4(0, 0, 0, 0);
     }
     __syncthreads();
+    // a programmatic dependent of what precedes it on the stream: nothing global is touched before that has completed
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) a.ctl->status = 0;          // first kernel of the operation
 
     // this warp's tile pair, and which of the pair's warps it is
-    constexpr int wpp = WPP;
-    const int pair_local = warp / wpp, sub = warp - pair_local * wpp;
+    int wpp = WPP, pair_local = warp / (WPP ? WPP : 1), sub = warp - pair_local * WPP;
+    if (WPP == 0) {
+        pair_local = int((kPanelOwners10 >> (4 * warp)) & 15u);
+        wpp = pair_local == 5 || pair_local == 6 ? 2 : 1;
+        sub = wpp == 2 ? warp & 1 : 0;
+    }
     const int pair = blockIdx.y * a.pairs_per_cta + pair_local;
     const bool active = pair_local < a.pairs_per_cta && pair < a.pairs;
     int ti = 0, tj = 0;
     if (active) tile_pair(pair, a.tiles, ti, tj);
-    const bool diag = ti == tj;
 
     float acc[8][8];
 #pragma unroll
@@ -183,24 +195,30 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
 
     constexpr int LB = PanelLane<T>::kBytes;
     constexpr int steps = RB / (32 * LB);
-    static_assert(steps % WPP == 0, "a panel's steps divide evenly between the warps of a pair");
+    static_assert(steps % (WPP ? WPP : 2) == 0, "a panel's steps divide evenly between the warps of a pair");
+    // (one copy of the loop for diagonal tiles and one for the others: with the choice inside, its two sides keep the
+    // accumulators in different registers and every step ends with 64 moves)
+    auto consume = [&](auto diag_tag) {
+    constexpr bool DIAG = decltype(diag_tag)::value;
     int since_flush = 0;
     for (int it = 0; it < kPanelStages - 1; ++it) issue(it);
     for (int it = 0; it < n_mine; ++it) {
         panel_cp_async_wait<kPanelStages - 2>();        // this thread's copies of panel `it` have landed
-        __syncthreads();                                // ... everybody's have, and panel it-1 is no longer read
+        // ... everybody's have, and panel it-1 is no longer read (one barrier, whichever copy of the loop a warp is in)
+        asm volatile("barrier.cta.sync 0;" ::: "memory");
         issue(it + kPanelStages - 1);                   // refills the stage of panel it-1
         if (active) {
             const unsigned char *stage = smem + (size_t)(it % kPanelStages) * stage_bytes;
             const unsigned char *bi = stage + (size_t)(ti * 8) * RB + lane * LB;
             const unsigned char *bj = stage + (size_t)(tj * 8) * RB + lane * LB;
 #pragma unroll
-            for (int s0 = 0; s0 < steps; s0 += wpp) {
-                const int s = s0 + sub;
+            for (int s0 = 0; s0 < steps; s0 += (WPP ? WPP : 1)) {
+                if (WPP == 0 && wpp == 2 && (s0 & 1) != sub) continue;
+                const int s = WPP ? s0 + sub : s0;
                 float xi[8][2];
 #pragma unroll
                 for (int r = 0; r < 8; ++r) PanelLane<T>::load(bi + (size_t)r * RB + s * (32 * LB), xi[r]);
-                if (diag) {
+                if constexpr (DIAG) {
 #pragma unroll
                     for (int r = 0; r < 8; ++r)
 #pragma unroll
@@ -220,6 +238,9 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
             }
         }
     }
+    };
+    if (ti == tj) consume(std::true_type());
+    else consume(std::false_type());
     panel_cp_async_wait<0>();
     // the streaming part of this CTA is over: the finishing kernel may start placing its blocks
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
