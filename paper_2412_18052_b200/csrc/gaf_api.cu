@@ -154,6 +154,7 @@ int stream_grid(int64_t D, int threads, int sms) {
 // kernels for few gradients are faster at every length: with exactly 8, where the 128 x 128 product keeps 1/16 of
 // its work, the warp-level MMA kernel streams 16 GB of inputs at 6.6 TB/s against 5.2 TB/s (measured).
 constexpr int kPanelAutoMaxK = 32;
+constexpr int64_t kPanelAutoMinD = 32768;
 bool use_tensor_gram(int K, int64_t D, int dtype) {
     (void)D;
     return dtype == GAF_BF16 && K > kGsMaxK && K <= kTcMaxK;
@@ -685,23 +686,24 @@ int check_grads(const void *const *grads, int K, int64_t D, int dtype) {
 }
 
 template <typename T, int KT>
-void launch_bucket_gram_kt(const BucketGramArgs &a, const BucketTable &bt, int grid, cudaStream_t st) {
-    bucket_gram_kernel<T, KT><<<grid, kBkThreads, 0, st>>>(a, bt);
+int launch_bucket_gram_kt(const BucketGramArgs &a, const BucketTable &bt, int grid, cudaStream_t st) {
+    if (launch_dependent(bucket_gram_kernel<T, KT>, grid, kBkThreads, st, a, bt) == cudaSuccess) return GAF_OK;
+    cudaGetLastError();
+    return GAF_ERR_CUDA;
 }
 template <typename T>
 int launch_bucket_gram(const BucketGramArgs &a, const BucketTable &bt, int K, int grid, cudaStream_t st) {
     switch (K) {
-        case 1: launch_bucket_gram_kt<T, 1>(a, bt, grid, st); break;
-        case 2: launch_bucket_gram_kt<T, 2>(a, bt, grid, st); break;
-        case 3: launch_bucket_gram_kt<T, 3>(a, bt, grid, st); break;
-        case 4: launch_bucket_gram_kt<T, 4>(a, bt, grid, st); break;
-        case 5: launch_bucket_gram_kt<T, 5>(a, bt, grid, st); break;
-        case 6: launch_bucket_gram_kt<T, 6>(a, bt, grid, st); break;
-        case 7: launch_bucket_gram_kt<T, 7>(a, bt, grid, st); break;
-        case 8: launch_bucket_gram_kt<T, 8>(a, bt, grid, st); break;
+        case 1: return launch_bucket_gram_kt<T, 1>(a, bt, grid, st);
+        case 2: return launch_bucket_gram_kt<T, 2>(a, bt, grid, st);
+        case 3: return launch_bucket_gram_kt<T, 3>(a, bt, grid, st);
+        case 4: return launch_bucket_gram_kt<T, 4>(a, bt, grid, st);
+        case 5: return launch_bucket_gram_kt<T, 5>(a, bt, grid, st);
+        case 6: return launch_bucket_gram_kt<T, 6>(a, bt, grid, st);
+        case 7: return launch_bucket_gram_kt<T, 7>(a, bt, grid, st);
+        case 8: return launch_bucket_gram_kt<T, 8>(a, bt, grid, st);
         default: return GAF_ERR_ARG;
     }
-    return GAF_OK;
 }
 
 }  // namespace
@@ -797,9 +799,11 @@ int gaf_filter_accumulate(const void *const *grads, int K, int64_t D, int dtype,
     if (schedule == GAF_SCHED_AUTO) {
         // Gram-first moves fewer bytes whenever its one-pass Gram kernel applies
         const bool ws_ok = workspace_bytes >= kExtraOffset + pairwise_extra_bytes(K);
-        // (the general CUDA-core Gram kernel beats the stepwise schedule up to 32 binary32 gradients)
+        // The general CUDA-core Gram kernel beats the stepwise schedule at any number of binary32 gradients (40 / 64 of
+        // 3 M: 312 / 617 us against 423 / 694; 40 / 64 of 100 k: 39 / 62 against 185 / 290); beyond 32 gradients tiny
+        // vectors keep the stepwise schedule.
         const bool fast_gram = K >= 2 && (K <= kGsMaxK || use_tensor_gram(K, D, dtype) ||
-                                          (dtype == GAF_F32 && K <= kPanelAutoMaxK));
+                                          (dtype == GAF_F32 && (K <= kPanelAutoMaxK || D >= kPanelAutoMinD)));
         schedule = (fast_gram && ws_ok) ? (auto_one_launch(K, D, dtype) ? GAF_SCHED_GRAM_FUSED : GAF_SCHED_GRAM)
                                         : GAF_SCHED_STEPWISE;
     }

@@ -3,10 +3,14 @@
 // bucket independently.  Gram-first, as for the whole vector: one pass builds a K x K Gram matrix
 // PER BUCKET, a small kernel walks Algorithm 1 per bucket, one pass writes every bucket's g/c.
 //
-// Work split: every CTA owns one contiguous range of the D elements (equal shares), and inside
-// it handles the part of every bucket that intersects the range.  A (CTA c, bucket b) intersection
-// writes its partial Gram sums to slot c + b, which is unique because both indices only grow along
-// the vector.  The per-bucket totals are taken over the CTAs in ascending order (fixed order).
+// Work split: every CTA owns one contiguous range of the D elements, and inside it handles the part of every bucket
+// that intersects the range.  A (CTA c, bucket b) intersection writes its partial Gram sums to slot c + b, which is
+// unique because both indices only grow along the vector.  The per-bucket totals are taken over the CTAs in
+// ascending order (fixed order).  Every further bucket costs a CTA a reduction and a memory latency, and two thirds of a network's
+// tensors have a few hundred elements, so a bucket counts as kBkBucketCost elements when the ranges are cut (62 tensors of
+// ResNet18, 4 fp32 gradients, whole call: 75.0 us with equal shares, 74.0 / 72.3 / 71.6 with a bucket counted as 1024 / 2048 / 5000
+// elements; 200 buckets of 3 M: 34.9, 30.0, 28.6, 29.2.  Before, with a walk that recomputed every range in every thread and a
+// mean pass with two barriers a bucket: 78.6 and 47.4 us; 20 buckets of 100 k: 28.1, now 12.8).
 #pragma once
 
 #include "gaf_device.cuh"
@@ -33,12 +37,24 @@ __device__ __forceinline__ int bucket_of(const BucketTable &bt, int64_t e) {
     return lo;
 }
 
-// Element range of CTA c out of G: equal shares in units of 8 elements; the last CTA also takes
-// the D mod 8 leftover.
-__device__ __forceinline__ void cta_range(int64_t D, int c, int G, int64_t &lo, int64_t &hi) {
-    const int64_t n_oct = D / kOct;
-    lo = (n_oct * c / G) * kOct;
-    hi = (c == G - 1) ? D : (n_oct * (c + 1) / G) * kOct;
+// Where CTA c's range starts, out of G equal shares of (elements + kBkBucketCost per bucket): a multiple of 8.
+constexpr int kBkBucketCost = 3072;
+__device__ __forceinline__ int64_t cta_start(const BucketTable &bt, int64_t D, int c, int G) {
+    if (c <= 0) return 0;
+    if (c >= G) return D;
+    const int64_t x = (D + (int64_t)kBkBucketCost * bt.S) * c / G;
+    int lo = 0, hi = bt.S;                  // largest b with off[b] + cost b <= x
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (bt.off[mid] + (int64_t)kBkBucketCost * mid <= x) lo = mid; else hi = mid;
+    }
+    const int64_t into = x - (bt.off[lo] + (int64_t)kBkBucketCost * (lo + 1));
+    const int64_t e = bt.off[lo] + (into > 0 ? into : 0), end = bt.off[lo + 1];
+    return (e < end ? e : end) / kOct * kOct;
+}
+__device__ __forceinline__ void cta_range(const BucketTable &bt, int64_t D, int c, int G, int64_t &lo, int64_t &hi) {
+    lo = cta_start(bt, D, c, G);
+    hi = cta_start(bt, D, c + 1, G);
 }
 
 struct BucketGramArgs {
@@ -61,10 +77,11 @@ bucket_gram_kernel(const __grid_constant__ BucketGramArgs a, const __grid_consta
     for (int r = 0; r < KT; ++r) row[r] = static_cast<const T *>(a.g[r]);
     // the mean pass walks every CTA's range from its end: the end of the range is asked to stay in L2
     const uint64_t pol_first = l2_policy_evict_first(), pol_last = l2_policy_evict_last();
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->status = 0;     // first kernel of the operation
-
     int64_t lo, hi;
-    cta_range(a.D, blockIdx.x, gridDim.x, lo, hi);
+    cta_range(bt, a.D, blockIdx.x, gridDim.x, lo, hi);
+    // a programmatic dependent of what precedes it on the stream (a no-op after an ordinary launch)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->status = 0;     // first kernel of the operation
     if (lo >= hi) return;
     int b = bucket_of(bt, lo);
     while (true) {
@@ -153,51 +170,42 @@ struct BucketWalkArgs {
 };
 
 // One CTA per bucket (64 pairs x 16 chains of threads): totals over the intersecting CTAs in
-// ascending order, then the walk.
+// ascending order, then the walk by one warp.
 constexpr int kWalkChains = 16;
 __global__ void __launch_bounds__(64 * kWalkChains)
 bucket_walk_kernel(const __grid_constant__ BucketWalkArgs a, const __grid_constant__ BucketTable bt) {
     __shared__ double sgram[kGsMaxK * kGsMaxK];
     __shared__ double part[kWalkChains][64];
+    __shared__ int first, last;
+    __shared__ unsigned char meets[kBkMaxCtas];
     const int b = blockIdx.x, K = a.K, NP = K * (K + 1) / 2;
     const int64_t b0 = bt.off[b], b1 = bt.off[b + 1];
-    // CTAs of the Gram pass whose range meets [b0, b1)
-    int c_first = 0, c_last = -1;
-    if (b1 > b0) {
-        int lo = 0, hi = a.ctas - 1;            // first CTA with range end > b0
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            int64_t l, h;
-            cta_range(a.D, mid, a.ctas, l, h);
-            if (h > b0) hi = mid; else lo = mid + 1;
-        }
-        c_first = lo;
-        lo = c_first; hi = a.ctas - 1;          // last CTA with range start < b1
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            int64_t l, h;
-            cta_range(a.D, mid, a.ctas, l, h);
-            if (l < b1) lo = mid; else hi = mid - 1;
-        }
-        c_last = lo;
+    if (threadIdx.x == 0) { first = a.ctas; last = -1; }
+    __syncthreads();
+    // CTAs of the Gram pass whose range meets [b0, b1): one thread per CTA looks
+    if ((int)threadIdx.x < a.ctas) {
+        int64_t lo, hi;
+        cta_range(bt, a.D, threadIdx.x, a.ctas, lo, hi);
+        const bool m = (lo > b0 ? lo : b0) < (hi < b1 ? hi : b1);
+        meets[threadIdx.x] = m ? 1 : 0;
+        if (m) { atomicMin(&first, (int)threadIdx.x); atomicMax(&last, (int)threadIdx.x); }
     }
+    static_assert(kBkMaxCtas <= 64 * kWalkChains, "one thread per CTA");
+    __syncthreads();
     const int p = threadIdx.x & 63, chain = threadIdx.x >> 6;
     // programmatic dependent of the Gram pass: wait for that grid and its partial sums; the mean pass
     // behind this kernel may be placed at once (it waits for this grid in turn)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     {
-        const int n = c_last - c_first + 1;
+        const int n = last - first + 1;
         const int per = (n + kWalkChains - 1) / kWalkChains;
-        const int c0 = c_first + chain * per, c1 = min(c_last + 1, c0 + per);
+        const int c0 = first + chain * per, c1 = min(last + 1, c0 + per);
         double s = 0.0;
         if (p < NP) {
-            for (int c = c0; c < c1; ++c) {
-                int64_t l, h;
-                cta_range(a.D, c, a.ctas, l, h);
-                const int64_t s0 = l > b0 ? l : b0, s1 = h < b1 ? h : b1;
-                if (s1 > s0) s += __ldcg(a.partials + (size_t)(c + b) * 64 + p);
-            }
+#pragma unroll 4
+            for (int c = c0; c < c1; ++c)
+                if (meets[c]) s += __ldcg(a.partials + (size_t)(c + b) * 64 + p);
         }
         part[chain][p] = s;
     }
@@ -213,31 +221,12 @@ bucket_walk_kernel(const __grid_constant__ BucketWalkArgs a, const __grid_consta
         sgram[cc * K + r] = s;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int status = 0, count = 1;
-        unsigned long long bits = 1ull;
-        double na = sgram[0], norm_sq = sgram[0];
-        uint8_t *mask = a.mask_out + (size_t)b * K;
-        float *dist = a.dist_out ? a.dist_out + (size_t)b * K : nullptr;
-        mask[a.idx[0]] = 1;
-        if (dist) dist[a.idx[0]] = 0.0f;
-        for (int t = 1; t < K; ++t) {
-            double p = 0.0;
-            for (int u = 0; u < t; ++u)
-                if ((bits >> u) & 1ull) p += sgram[u * K + t];
-            const double ng = sgram[t * K + t];
-            const double d = cosine_distance(p, na, ng, &status);
-            const int accept = (d <= a.tau) ? 1 : 0;
-            mask[a.idx[t]] = (uint8_t)accept;
-            if (dist) dist[a.idx[t]] = (float)d;
-            if (accept) {
-                bits |= 1ull << t; na = na + 2.0 * p + ng; norm_sq += ng; ++count;
-                status |= ill_conditioned(count, norm_sq, na);
-            }
-        }
-        a.bits[b] = bits;
-        a.count_out[b] = count;
-        if (status) atomicOr(&a.ctl->status, status);
+    if (threadIdx.x < 32) {
+        WalkSteps<1> st;
+        const WalkResult r = warp_walk<1>(sgram, K, 0, a.tau, st);
+        if (threadIdx.x == 0) a.bits[b] = r.bits;
+        walk_outputs<1>(sgram, K, 0, r, st, a.idx, a.mask_out + (size_t)b * K, a.dist_out ? a.dist_out + (size_t)b * K : nullptr,
+                        a.count_out + b, a.ctl);
     }
 }
 
@@ -252,59 +241,61 @@ struct BucketMeanArgs {
 template <typename T>
 __global__ void __launch_bounds__(kBkThreads, 2)
 bucket_mean_kernel(const __grid_constant__ BucketMeanArgs a, const __grid_constant__ BucketTable bt) {
-    __shared__ const T *list[kGsMaxK];
-    __shared__ int n_list;
+    constexpr int N = GsVec<T>::N;          // elements of a 16-byte load
     int64_t lo, hi;
-    cta_range(a.D, blockIdx.x, gridDim.x, lo, hi);
+    cta_range(bt, a.D, blockIdx.x, gridDim.x, lo, hi);
     // programmatic dependent of the per-bucket walk: wait for its accept bits
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (lo >= hi) return;
-    // the range is walked from its END (buckets last to first, each from its end): the Gram pass
-    // walked it from the start, so its last-read lines are the ones still in L2
+    // The range is walked from its END (buckets last to first, each from its end): the Gram pass walked it from the start,
+    // so its last-read lines are the ones still in L2.  Every thread looks at the bucket's bits itself: no barriers.
     int b = bucket_of(bt, hi - 1);
     while (true) {
         const int64_t s0 = lo > bt.off[b] ? lo : bt.off[b];
         const int64_t s1 = hi < bt.off[b + 1] ? hi : bt.off[b + 1];
         if (s1 > s0) {
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                const unsigned long long bits = __ldcg(a.bits + b);
-                int n = 0;
-                for (int t = 0; t < a.K; ++t)
-                    if ((bits >> t) & 1ull) list[n++] = static_cast<const T *>(a.g[t]);
-                n_list = n;
-            }
-            __syncthreads();
-            const int n = n_list;
-            const float cdiv = (float)n;
-            const int64_t n_oct = (s1 - s0) / kOct;
-            for (int64_t o = threadIdx.x; o < n_oct; o += kBkThreads) {
-                const int64_t e = s0 + (n_oct - 1 - o) * kOct;
-                float v[8];
-                RawOct<T>::load(list[0], e).widen(v);
-                for (int i = 1; i < n; i += 3) {
-                    RawOct<T> w[3];
+            const unsigned int bits = (unsigned int)__ldcg(a.bits + b);
+            const float cdiv = (float)__popc(bits);
+            const int64_t n_vec = (s1 - s0) / N;
+            for (int64_t o = threadIdx.x; o < n_vec; o += kBkThreads) {
+                const int64_t e = s0 + (n_vec - 1 - o) * N;
+                uint4 w[kGsMaxK];
 #pragma unroll
-                    for (int j = 0; j < 3; ++j)
-                        if (i + j < n) w[j] = RawOct<T>::load(list[i + j], e);
+                for (int t = 0; t < kGsMaxK; ++t)
+                    if ((bits >> t) & 1u) w[t] = __ldcs(reinterpret_cast<const uint4 *>(static_cast<const T *>(a.g[t]) + e));
+                float v[N];
 #pragma unroll
-                    for (int j = 0; j < 3; ++j)
-                        if (i + j < n) {
-                            float x[8];
-                            w[j].widen(x);
+                for (int k = 0; k < N; ++k) v[k] = -0.0f;           // (-0 + x = x for every x)
 #pragma unroll
-                            for (int k = 0; k < 8; ++k) v[k] += x[k];
+                for (int t = 0; t < kGsMaxK; ++t)
+                    if ((bits >> t) & 1u) {
+                        float x[N];
+                        if constexpr (sizeof(T) == 4) {
+                            x[0] = __uint_as_float(w[t].x); x[1] = __uint_as_float(w[t].y);
+                            x[2] = __uint_as_float(w[t].z); x[3] = __uint_as_float(w[t].w);
+                        } else {
+                            const unsigned int q[4] = {w[t].x, w[t].y, w[t].z, w[t].w};
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                x[2 * k] = bf16_bits_to_float(q[k] & 0xFFFFu);
+                                x[2 * k + 1] = __uint_as_float(q[k] & 0xFFFF0000u);
+                            }
                         }
-                }
 #pragma unroll
-                for (int k = 0; k < 8; ++k) v[k] = v[k] / cdiv;
-                store8(a.out, e, v, true);
+                        for (int k = 0; k < N; ++k) v[k] += x[k];
+                    }
+#pragma unroll
+                for (int h = 0; h < N / 4; ++h)
+                    __stcs(reinterpret_cast<float4 *>(a.out + e) + h,
+                           make_float4(v[4 * h] / cdiv, v[4 * h + 1] / cdiv, v[4 * h + 2] / cdiv, v[4 * h + 3] / cdiv));
             }
-            const int64_t t0 = s0 + n_oct * kOct;
+            const int64_t t0 = s0 + n_vec * N;
             if (t0 + threadIdx.x < s1) {
                 const int64_t e = t0 + threadIdx.x;
-                float v = load1<T>(list[0], e);
-                for (int i = 1; i < n; ++i) v += load1<T>(list[i], e);
+                float v = -0.0f;
+                for (int t = 0; t < a.K; ++t)
+                    if ((bits >> t) & 1u) v += load1<T>(static_cast<const T *>(a.g[t]), e);
                 a.out[e] = v / cdiv;
             }
         }
