@@ -81,6 +81,9 @@ __device__ __forceinline__ WalkResult warp_walk(const double *gram, int K, int s
 #pragma unroll
         for (int w = 1; w < JW; ++w) mine = i >= 32 * w ? pj[w] : mine;
         const double p = __shfl_sync(0xFFFFFFFFu, mine, i & 31), ng = gram[i * K + i];
+        double row[JW];                     // (loaded before the decision is known)
+#pragma unroll
+        for (int w = 0; w < JW; ++w) row[w] = lane + 32 * w < K ? gram[i * K + lane + 32 * w] : 0.0;
         const float fp = (float)p, fa = (float)na, fg = (float)ng;
         const float margin = fp * (rsqrtf(fa) * rsqrtf(fg)) - bound;
         bool accept = margin >= 0.0f;
@@ -98,8 +101,7 @@ __device__ __forceinline__ WalkResult warp_walk(const double *gram, int K, int s
             na = na + 2.0 * p + ng;         // |g + g_i|^2
             norm_sq += ng;
 #pragma unroll
-            for (int w = 0; w < JW; ++w)
-                if (lane + 32 * w < K) pj[w] += gram[i * K + lane + 32 * w];
+            for (int w = 0; w < JW; ++w) pj[w] += row[w];
         }
     }
     return r;
@@ -266,6 +268,83 @@ struct MaskedMeanArgs {
 // keep an SM inside the same pages for several trips, which the address translation needs
 // (12 GB through this pass: 5.5 TB/s with run = U, measured, against the 6.5 TB/s it reaches
 // on shorter vectors).
+template <typename T>
+struct MeanVec;
+template <> struct MeanVec<float> {
+    static constexpr int N = 4;
+    static __device__ __forceinline__ void widen(const uint4 &r, float (&v)[4]) {
+        v[0] = __uint_as_float(r.x); v[1] = __uint_as_float(r.y); v[2] = __uint_as_float(r.z); v[3] = __uint_as_float(r.w);
+    }
+};
+template <> struct MeanVec<__nv_bfloat16> {
+    static constexpr int N = 8;
+    static __device__ __forceinline__ void widen(const uint4 &r, float (&v)[8]) {
+        const unsigned int w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[2 * k] = bf16_bits_to_float(w[k] & 0xFFFFu);
+            v[2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u);
+        }
+    }
+};
+
+// masked_mean_kernel for short vectors of many gradients, where a call waits for memory latencies and not for bytes: one
+// 16-byte vector per thread and sixteen gradients in flight instead of three, the list made by 128 threads instead of one.
+// Whole filter calls: 64 bf16 gradients of 20 k / 500 k elements 55.1 -> 40.8 / 68.1 -> 53.5 us, 32 bf16 of 100 k
+// 34.5 -> 26.7, 16 fp32 of 100 k 17.7 -> 15.5.
+constexpr int kMsShortThreads = 128;
+constexpr int kMsShortGrads = 16;
+template <typename T>
+__global__ void __launch_bounds__(kMsShortThreads) masked_mean_short_kernel(const __grid_constant__ MaskedMeanArgs a) {
+    constexpr int N = MeanVec<T>::N;
+    __shared__ const T *list[GAF_MAX_K + kMsShortGrads];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const unsigned long long bits = __ldcg(&a.ctl->accept_bits);
+    const int seed = __ldcg(&a.ctl->ring_seed), start = seed < 0 ? 0 : seed;
+    const int n = __popcll(bits);
+    // accepted gradients in processing order: the ring order from `start`
+    for (int i = threadIdx.x; i < a.K; i += kMsShortThreads)
+        if ((bits >> i) & 1ull) {
+            const unsigned long long below = bits & ((1ull << i) - 1ull), from = bits & ~((1ull << start) - 1ull);
+            const int rank = i >= start ? __popcll(below & from) : __popcll(from) + __popcll(below);
+            list[rank] = static_cast<const T *>(a.g[i]);
+        }
+    __syncthreads();
+    const float cdiv = (float)n;
+    const int64_t n_vec = a.D / N, q = (int64_t)blockIdx.x * kMsShortThreads + threadIdx.x;
+    if (q < n_vec) {
+        const int64_t e = q * N;
+        float v[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) v[k] = -0.0f;                       // (-0 + x = x for every x)
+        for (int i = 0; i < n; i += kMsShortGrads) {
+            uint4 w[kMsShortGrads];
+#pragma unroll
+            for (int g = 0; g < kMsShortGrads; ++g)
+                if (i + g < n) w[g] = __ldcs(reinterpret_cast<const uint4 *>(list[i + g] + e));
+#pragma unroll
+            for (int g = 0; g < kMsShortGrads; ++g)
+                if (i + g < n) {
+                    float x[N];
+                    MeanVec<T>::widen(w[g], x);
+#pragma unroll
+                    for (int k = 0; k < N; ++k) v[k] += x[k];
+                }
+        }
+#pragma unroll
+        for (int h = 0; h < N / 4; ++h)
+            *(reinterpret_cast<float4 *>(a.out + e) + h) =
+                make_float4(v[4 * h] / cdiv, v[4 * h + 1] / cdiv, v[4 * h + 2] / cdiv, v[4 * h + 3] / cdiv);
+    }
+    const int64_t tail0 = n_vec * N;
+    if (blockIdx.x == 0 && tail0 + threadIdx.x < a.D) {
+        const int64_t e = tail0 + threadIdx.x;
+        float v = -0.0f;
+        for (int i = 0; i < n; ++i) v += load1<T>(list[i], e);
+        a.out[e] = v / cdiv;
+    }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kMsThreads, 2) masked_mean_kernel(const __grid_constant__ MaskedMeanArgs a) {
     __shared__ const T *list[GAF_MAX_K];

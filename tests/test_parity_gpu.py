@@ -711,6 +711,29 @@ def test_predicted_accept_pattern_right_and_wrong(ws, K, dtype):
                 check_any_seed(grads, 0.9, ws)
 
 
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("K", [9, 16, 33, 64])
+def test_many_gradients_mean_of_short_vectors(ws, K, dtype):
+    """More gradients than the one-launch form takes: no whole 16-byte vector, one CTA and a remainder, and both sides of
+    the length up to which the mean gives every thread one vector.  Mask, distances and mean against the oracle, and the
+    mean bit for bit against the stepwise schedule (the same additions in the same order)."""
+    n = 4 if dtype == "f32" else 8
+    limit = torch.cuda.get_device_properties(0).multi_processor_count * 8 * 128 * n
+    for D in (3, 128 * n - 1, 32_768 + n + 1, limit, limit + 1):
+        w = _mix(K, D, dtype, seed=K + D, rho=([0.8] + [0.7, -0.6, 0.5, 0.0, 0.6, -0.2, 0.4] * 9)[:K])
+        for tau in (0.9, 2.0):
+            plain = [t.clone() for t in gaf.gaf_filter_accumulate(w.grads, tau, ws, schedule=gaf.GAF_SCHED_STEPWISE)]
+            got = gaf.gaf_filter_accumulate(w.grads, tau, ws, schedule=gaf.GAF_SCHED_GRAM)
+            if torch.equal(got[1], plain[1]):                        # (masks may differ on a tie only)
+                assert torch.equal(got[0], plain[0]), (K, D, tau)
+        check_filter(w.grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM)
+        if D < limit:
+            check_any_seed(w.grads, 0.9, ws)
+        if K > 32 and D == limit:                                    # the library's own choice for long vectors
+            check_filter(w.grads, 0.9, ws)
+            assert gaf.gaf_last_schedule() == gaf.GAF_SCHED_GRAM
+
+
 def test_division_by_the_count_is_correctly_rounded(ws):
     """The mean's division by c (3, 5, 6, 7: two multiply-adds; powers of two: a multiplication) against the division
     itself: significands across the range, zeros, subnormal and huge values, infinities."""
