@@ -717,6 +717,12 @@ int launch_bucket_gram(const BucketGramArgs &a, const BucketTable &bt, int K, in
         default: return GAF_ERR_ARG;
     }
 }
+template <typename T>
+cudaError_t launch_bucket_mean(const BucketMeanArgs &a, const BucketTable &bt, int grid, cudaStream_t st) {
+    if (a.K <= 2) return launch_dependent(bucket_mean_kernel<T, 2>, grid, kBkThreads, st, a, bt);
+    if (a.K <= 4) return launch_dependent(bucket_mean_kernel<T, 4>, grid, kBkThreads, st, a, bt);
+    return launch_dependent(bucket_mean_kernel<T, 8>, grid, kBkThreads, st, a, bt);
+}
 
 }  // namespace
 
@@ -976,8 +982,7 @@ int gaf_filter_accumulate_bucketed(const void *const *grads, int K, int64_t D, i
         if (mean_grid > kBkMaxCtas) mean_grid = kBkMaxCtas;
         if (n_oct < mean_grid) mean_grid = n_oct > 0 ? int(n_oct) : 1;
         const cudaError_t err = dtype == GAF_F32
-            ? launch_dependent(bucket_mean_kernel<float>, mean_grid, kBkThreads, st, ma, bt)
-            : launch_dependent(bucket_mean_kernel<__nv_bfloat16>, mean_grid, kBkThreads, st, ma, bt);
+            ? launch_bucket_mean<float>(ma, bt, mean_grid, st) : launch_bucket_mean<__nv_bfloat16>(ma, bt, mean_grid, st);
         if (err != cudaSuccess) { cudaGetLastError(); return GAF_ERR_CUDA; }
     }
     ++g_launches;

@@ -70,6 +70,8 @@ __global__ void __launch_bounds__(kBkThreads, (KT <= 4 ? 2 : 1))
 bucket_gram_kernel(const __grid_constant__ BucketGramArgs a, const __grid_constant__ BucketTable bt) {
     constexpr int NP = KT * (KT + 1) / 2;
     constexpr int N = GsVec<T>::N;
+    constexpr int U = KT <= 2 ? 4 / KT : 1; // vectors of a gradient a thread has in flight
+    static_assert(kGsFlushEvery % U == 0, "the sums are flushed between rounds");
     __shared__ double sacc[kBkThreads / 32][NP];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const T *row[KT];
@@ -108,13 +110,20 @@ bucket_gram_kernel(const __grid_constant__ BucketGramArgs a, const __grid_consta
             const int64_t n_vec = (s1 - s0) / N;
             int since_flush = 0;
             // warp-uniform trip count: the flush shuffles across the whole warp
-            for (int64_t qw = threadIdx.x & ~31; qw < n_vec; qw += kBkThreads) {
-                const int64_t q = qw + lane;
-                if (q < n_vec) {
-                    float x[KT][N];
-                    const uint64_t pol = (s0 + q * N >= hi - a.keep_elems) ? pol_last : pol_first;
+            for (int64_t qw = threadIdx.x & ~31; qw < n_vec; qw += U * kBkThreads) {
+                float x[U][KT][N];
 #pragma unroll
-                    for (int r = 0; r < KT; ++r) GsVec<T>::load(row[r], s0 + q * N, pol, x[r]);
+                for (int u = 0; u < U; ++u) {
+                    const int64_t q = qw + u * kBkThreads + lane;
+                    const uint64_t pol = (s0 + q * N >= hi - a.keep_elems) ? pol_last : pol_first;
+                    if (q < n_vec) {
+#pragma unroll
+                        for (int r = 0; r < KT; ++r) GsVec<T>::load(row[r], s0 + q * N, pol, x[u][r]);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (qw + u * kBkThreads + lane >= n_vec) break;
                     int p = 0;
 #pragma unroll
                     for (int r = 0; r < KT; ++r)
@@ -122,11 +131,11 @@ bucket_gram_kernel(const __grid_constant__ BucketGramArgs a, const __grid_consta
                         for (int c = r; c < KT; ++c, ++p) {
                             Acc s = acc[p];
 #pragma unroll
-                            for (int k = 0; k < N; ++k) s = gs_fma(x[r][k], x[c][k], s);
+                            for (int k = 0; k < N; ++k) s = gs_fma(x[u][r][k], x[u][c][k], s);
                             acc[p] = s;
                         }
                 }
-                if (GsAcc<T, KT>::kPeriodicFlush && ++since_flush == kGsFlushEvery) { flush(); since_flush = 0; }
+                if (GsAcc<T, KT>::kPeriodicFlush && (since_flush += U) == kGsFlushEvery) { flush(); since_flush = 0; }
             }
             const int64_t t0 = s0 + n_vec * N;          // fewer than N leftover elements
             if (t0 + threadIdx.x < s1) {
@@ -238,10 +247,11 @@ struct BucketMeanArgs {
     const unsigned long long *bits;         // [S]
 };
 
-template <typename T>
+template <typename T, int KM>               // KM: at most so many gradients
 __global__ void __launch_bounds__(kBkThreads, 2)
 bucket_mean_kernel(const __grid_constant__ BucketMeanArgs a, const __grid_constant__ BucketTable bt) {
-    constexpr int N = GsVec<T>::N;          // elements of a 16-byte load
+    constexpr int N = MeanVec<T>::N;        // elements of a 16-byte load
+    constexpr int U = 8 / KM;               // vectors of a gradient a thread has in flight
     int64_t lo, hi;
     cta_range(bt, a.D, blockIdx.x, gridDim.x, lo, hi);
     // programmatic dependent of the per-bucket walk: wait for its accept bits
@@ -258,37 +268,34 @@ bucket_mean_kernel(const __grid_constant__ BucketMeanArgs a, const __grid_consta
             const unsigned int bits = (unsigned int)__ldcg(a.bits + b);
             const float cdiv = (float)__popc(bits);
             const int64_t n_vec = (s1 - s0) / N;
-            for (int64_t o = threadIdx.x; o < n_vec; o += kBkThreads) {
-                const int64_t e = s0 + (n_vec - 1 - o) * N;
-                uint4 w[kGsMaxK];
+            for (int64_t o = threadIdx.x; o < n_vec; o += U * kBkThreads) {
+                uint4 w[U][KM];
 #pragma unroll
-                for (int t = 0; t < kGsMaxK; ++t)
-                    if ((bits >> t) & 1u) w[t] = __ldcs(reinterpret_cast<const uint4 *>(static_cast<const T *>(a.g[t]) + e));
-                float v[N];
+                for (int u = 0; u < U; ++u)
 #pragma unroll
-                for (int k = 0; k < N; ++k) v[k] = -0.0f;           // (-0 + x = x for every x)
+                    for (int t = 0; t < KM; ++t)
+                        if (((bits >> t) & 1u) && o + u * kBkThreads < n_vec)
+                            w[u][t] = __ldcs(reinterpret_cast<const uint4 *>(static_cast<const T *>(a.g[t]) + s0 + (n_vec - 1 - o - u * kBkThreads) * N));
 #pragma unroll
-                for (int t = 0; t < kGsMaxK; ++t)
-                    if ((bits >> t) & 1u) {
-                        float x[N];
-                        if constexpr (sizeof(T) == 4) {
-                            x[0] = __uint_as_float(w[t].x); x[1] = __uint_as_float(w[t].y);
-                            x[2] = __uint_as_float(w[t].z); x[3] = __uint_as_float(w[t].w);
-                        } else {
-                            const unsigned int q[4] = {w[t].x, w[t].y, w[t].z, w[t].w};
+                for (int u = 0; u < U; ++u) {
+                    if (o + u * kBkThreads >= n_vec) break;
+                    const int64_t e = s0 + (n_vec - 1 - o - u * kBkThreads) * N;
+                    float v[N];
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                x[2 * k] = bf16_bits_to_float(q[k] & 0xFFFFu);
-                                x[2 * k + 1] = __uint_as_float(q[k] & 0xFFFF0000u);
-                            }
+                    for (int k = 0; k < N; ++k) v[k] = -0.0f;       // (-0 + x = x for every x)
+#pragma unroll
+                    for (int t = 0; t < KM; ++t)
+                        if ((bits >> t) & 1u) {
+                            float x[N];
+                            MeanVec<T>::widen(w[u][t], x);
+#pragma unroll
+                            for (int k = 0; k < N; ++k) v[k] += x[k];
                         }
 #pragma unroll
-                        for (int k = 0; k < N; ++k) v[k] += x[k];
-                    }
-#pragma unroll
-                for (int h = 0; h < N / 4; ++h)
-                    __stcs(reinterpret_cast<float4 *>(a.out + e) + h,
-                           make_float4(v[4 * h] / cdiv, v[4 * h + 1] / cdiv, v[4 * h + 2] / cdiv, v[4 * h + 3] / cdiv));
+                    for (int h = 0; h < N / 4; ++h)
+                        __stcs(reinterpret_cast<float4 *>(a.out + e) + h,
+                               make_float4(v[4 * h] / cdiv, v[4 * h + 1] / cdiv, v[4 * h + 2] / cdiv, v[4 * h + 3] / cdiv));
+                }
             }
             const int64_t t0 = s0 + n_vec * N;
             if (t0 + threadIdx.x < s1) {
