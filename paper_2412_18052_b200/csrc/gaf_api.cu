@@ -447,9 +447,16 @@ std::atomic<unsigned int> g_fused_tag{1};               // tags the sums that th
 constexpr int kPredictRings = 2;
 constexpr int kSampleTiles = 2;
 constexpr int kLongRounds = 64;
-template <typename T, int KT>
+// (bf16, 5 and 6 gradients: large tiles from here on; 5 x 12 M 39.8 us with small ones, 40.7 with large ones, 5 x 60 M 153, 136)
+constexpr int64_t kLongTileBytes = 300'000'000;
+// Gradients of 4/3 of L2 and more: the copies of up to six rows are better off without an eviction hint (4 x 11.2 M fp32 45.5 us
+// with evict-first, 44.0 without; 4 / 6 x 60 M 198.5 / 268.8, 190.0 / 252.9; bf16 5 x 60 M 140.5, 136.1), those of eight with
+// it (8 x 124 M fp32 720, 742; 8 x 60 M 355, 366; bf16 2 / 4 x 60 M 85.8 / 128.1, 90.2 / 132.4), and so are smaller inputs, of
+// which more is found in L2 by the next call (4 x 3 M fp32 18.0, 19.6; 8 x 5 M 43.2, 45.7).
+constexpr int kNormalMaxK = 6, kNormalMinKBf16 = 5;
+template <typename T, int KT, bool LONG>
 int filter_shape(GramFusedArgs &a, const DeviceInfo &di, bool predict) {
-    using Tile = FilterTile<T, KT>;
+    using Tile = FilterTile<T, KT, LONG>;
     // at least 256 elements per CTA; tiles cut so that all CTAs get the same number of equally long ones
     int64_t grid = (a.D + 255) / 256;
     if (grid > di.sms) grid = di.sms;
@@ -462,19 +469,22 @@ int filter_shape(GramFusedArgs &a, const DeviceInfo &di, bool predict) {
     if (a.tile_elems < 64) a.tile_elems = 64;
     a.rounds = int(rounds);
     a.sample = 0;
+    const bool stays = KT <= kNormalMaxK && (sizeof(T) == 4 || KT >= kNormalMinKBf16);
+    a.evict_first = !stays || int64_t(KT) * a.D * int64_t(sizeof(T)) * 3 < int64_t(di.l2_bytes) * 4;
     // (two gradients: the kernel has a guess without a sample most of the time)
     if (predict && rounds > (KT == 2 ? 1 : kPredictRings) * Tile::kStages)
-        a.sample = rounds < kLongRounds ? kSampleTiles : Tile::kStages / 2;
+        // (four stages of large tiles: as many elements in the sample)
+        a.sample = rounds >= kLongRounds ? Tile::kStages / 2 : (Tile::kStages > 4 ? kSampleTiles : kSampleTiles / 2);
     return int(grid);
 }
 
 // Shared-memory attributes of one instantiation, once per device; GAF_ERR_UNSUPPORTED when no CTA of it fits an SM.
-template <typename T, int KT, bool ONE>
+template <typename T, int KT, bool ONE, bool LONG>
 int filter_plan(const DeviceInfo &di) {
     static PerDevice<DynSmemPlan> table;
     return plan_once(table.plan[di.dev], table.ready[di.dev], [&](DynSmemPlan &pl) {
-        auto kernel = gram_filter_kernel<T, KT, ONE>;
-        pl.dyn = FilterTile<T, KT>::kStages * FilterTile<T, KT>::kBytes;
+        auto kernel = gram_filter_kernel<T, KT, ONE, LONG>;
+        pl.dyn = FilterTile<T, KT, LONG>::kStages * FilterTile<T, KT, LONG>::kBytes;
         if (pl.dyn > di.smem_per_cta_max) return GAF_ERR_UNSUPPORTED;
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.dyn) != cudaSuccess) return GAF_ERR_CUDA;
         int occ = 0;
@@ -484,11 +494,11 @@ int filter_plan(const DeviceInfo &di) {
     });
 }
 
-template <typename T, int KT>
+template <typename T, int KT, bool LONG = false>
 int launch_gram_fused_kt(GramFusedArgs &a, const DeviceInfo &di, cudaStream_t st) {
-    if (int rc = filter_plan<T, KT, true>(di)) return rc;
-    auto kernel = gram_filter_kernel<T, KT, true>;
-    const int grid = filter_shape<T, KT>(a, di, true);
+    if (int rc = filter_plan<T, KT, true, LONG>(di)) return rc;
+    auto kernel = gram_filter_kernel<T, KT, true, LONG>;
+    const int grid = filter_shape<T, KT, LONG>(a, di, true);
     a.spin_limit = g_test_wait_limit ? g_test_wait_limit : kFusedSpinLimit;
     a.test_withhold = g_test_withhold;
     a.tag = g_fused_tag.fetch_add(1, std::memory_order_relaxed);
@@ -512,7 +522,7 @@ int launch_gram_fused_kt(GramFusedArgs &a, const DeviceInfo &di, cudaStream_t st
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kFilterThreads);
-    cfg.dynamicSmemBytes = size_t(FilterTile<T, KT>::kStages * FilterTile<T, KT>::kBytes); cfg.stream = st;
+    cfg.dynamicSmemBytes = size_t(FilterTile<T, KT, LONG>::kStages * FilterTile<T, KT, LONG>::kBytes); cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -531,8 +541,12 @@ int launch_gram_fused(GramFusedArgs &a, int K, const DeviceInfo &di, cudaStream_
         case 2: return launch_gram_fused_kt<T, 2>(a, di, st);
         case 3: return launch_gram_fused_kt<T, 3>(a, di, st);
         case 4: return launch_gram_fused_kt<T, 4>(a, di, st);
-        case 5: return launch_gram_fused_kt<T, 5>(a, di, st);
-        case 6: return launch_gram_fused_kt<T, 6>(a, di, st);
+        case 5:
+            return kTwoTileForms<T, 5> && K * 2 * a.D >= kLongTileBytes ? launch_gram_fused_kt<T, 5, kTwoTileForms<T, 5>>(a, di, st)
+                                                                        : launch_gram_fused_kt<T, 5>(a, di, st);
+        case 6:
+            return kTwoTileForms<T, 6> && K * 2 * a.D >= kLongTileBytes ? launch_gram_fused_kt<T, 6, kTwoTileForms<T, 6>>(a, di, st)
+                                                                        : launch_gram_fused_kt<T, 6>(a, di, st);
         case 7: return launch_gram_fused_kt<T, 7>(a, di, st);
         case 8: return launch_gram_fused_kt<T, 8>(a, di, st);
         default: return GAF_ERR_UNSUPPORTED;
@@ -543,12 +557,13 @@ int launch_gram_fused(GramFusedArgs &a, int K, const DeviceInfo &di, cudaStream_
 // distances of up to 8 gradients (no mean, nothing behind it).
 template <typename T, int KT>
 int launch_gram_filter_kt(GramFusedArgs &a, const DeviceInfo &di, cudaStream_t st) {
-    if (int rc = filter_plan<T, KT, false>(di)) return rc;
-    const int grid = filter_shape<T, KT>(a, di, a.pair_dist_out == nullptr);
+    constexpr bool LONG = kTwoTileForms<T, KT>;
+    if (int rc = filter_plan<T, KT, false, LONG>(di)) return rc;
+    const int grid = filter_shape<T, KT, LONG>(a, di, a.pair_dist_out == nullptr);
     a.spin_limit = kFusedSpinLimit;
     a.test_withhold = 0;
-    const cudaError_t err = launch_dependent_smem(gram_filter_kernel<T, KT, false>, grid, kFilterThreads,
-                                                  size_t(FilterTile<T, KT>::kStages * FilterTile<T, KT>::kBytes), st, a);
+    const cudaError_t err = launch_dependent_smem(gram_filter_kernel<T, KT, false, LONG>, grid, kFilterThreads,
+                                                  size_t(FilterTile<T, KT, LONG>::kStages * FilterTile<T, KT, LONG>::kBytes), st, a);
     ++g_launches;
     if (err != cudaSuccess) { cudaGetLastError(); return GAF_ERR_CUDA; }
     return GAF_OK;

@@ -74,10 +74,15 @@ constexpr int kFilterMaxCtas = 160;
 constexpr int kFilterRingBytes = 206 << 10;
 constexpr int kFilterPairRingBytes = 130 << 10;
 
-// Tile of K gradients: kVecs groups of 4 elements per thread of a group and gradient, about 28 KB in all.
-template <typename T, int KT> struct FilterTile {
+// Tile of K gradients: kVecs groups of 4 elements per thread of a group and gradient, 20 to 43 KB in all.  Five and six gradients
+// (50 M elements fp32): tiles of 18 and 21 KB in ten and eight stages took 167 and 190 us for all pairs, 222 and 239 for the
+// filter, of twice that in four 141 and 170, 192 and 227; bfloat16 (60 M) 113 -> 88 and 127 -> 106, 153 -> 136 and 165 -> 160.
+// But a filter call on a shorter bfloat16 input waits longer for its prediction behind large tiles (5 x 5.5 M 24.6 us with
+// small ones, 26.8 with large ones; 6 x 8 M 33.9, 36.5): there the large ones are a form of their own (LONG).
+template <typename T, int KT> constexpr bool kTwoTileForms = std::is_same<T, __nv_bfloat16>::value && (KT == 5 || KT == 6);
+template <typename T, int KT, bool LONG = false> struct FilterTile {
     static constexpr bool kMma = std::is_same<T, __nv_bfloat16>::value && KT >= 7;
-    static constexpr int kVecs = KT == 2 ? 8 / int(sizeof(T)) : (KT <= 4 ? 8 / int(sizeof(T)) : 4 / int(sizeof(T)));
+    static constexpr int kVecs = KT == 2 ? 8 / int(sizeof(T)) : (KT <= 4 || (KT <= 6 && (LONG || !kTwoTileForms<T, KT>)) ? 8 / int(sizeof(T)) : 4 / int(sizeof(T)));
     static constexpr int kElems = kVecs * 4 * kFilterGroupThreads;
     // (the MMA fragments of eight rows are read together: 64 bytes between rows keep them apart in the banks)
     static constexpr int kPitch = kElems * int(sizeof(T)) + (kMma ? 64 : 0);
@@ -96,6 +101,7 @@ struct GramFusedArgs {
     int tile_elems;                         // elements of a tile per gradient (a multiple of 64, at most FilterTile::kElems)
     int rounds;                             // tiles per CTA
     int sample;                             // tiles per CTA in the sample; 0 = no prediction
+    int evict_first;                        // what is read once gives way in L2 first
     void *partials;                         // [pair][kFilterMaxCtas]: TaggedSum (ONE) or double
     unsigned long long *sample_partials;    // [pair][kFilterMaxCtas]: binary32 sum and tag
     unsigned long long *verdicts;           // [2][kFilterMaxCtas][16]: a line per CTA, predicted and decided pattern and tag
@@ -130,11 +136,14 @@ __device__ __forceinline__ void st_tagged(TaggedSum *p, double v, unsigned int t
     const unsigned long long lo = (b << 32) | tag, hi = (b & 0xFFFFFFFF00000000ull) | (unsigned int)~tag;
     asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(lo), "l"(hi) : "memory");
 }
-__device__ __forceinline__ bool ld_tagged(const TaggedSum *p, double &v, unsigned int tag) {
-    unsigned long long lo, hi;
-    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
-    v = __longlong_as_double((long long)((lo >> 32) | (hi & 0xFFFFFFFF00000000ull)));
-    return (unsigned int)lo == tag && (unsigned int)hi == (unsigned int)~tag;
+__device__ __forceinline__ TaggedSum ld_tagged(const TaggedSum *p) {
+    TaggedSum t;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(t.w[0]), "=l"(t.w[1]) : "l"(p) : "memory");
+    return t;
+}
+__device__ __forceinline__ bool tagged_value(const TaggedSum &t, double &v, unsigned int tag) {
+    v = __longlong_as_double((long long)((t.w[0] >> 32) | (t.w[1] & 0xFFFFFFFF00000000ull)));
+    return (unsigned int)t.w[0] == tag && (unsigned int)t.w[1] == (unsigned int)~tag;
 }
 // Bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) into shared memory, counted on `bar`.
 __device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void *src, uint32_t bytes, uint64_t *bar, uint64_t policy) {
@@ -269,10 +278,10 @@ struct HalvingSums<NP, 0, Acc> {
     }
 };
 
-template <typename T, int KT, bool ONE>
+template <typename T, int KT, bool ONE, bool LONG>
 __global__ void __launch_bounds__(kFilterThreads, 1)
 gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
-    using Tile = FilterTile<T, KT>;
+    using Tile = FilterTile<T, KT, LONG>;
     using Sync = FilterConsumers;
     constexpr int NP = KT * (KT + 1) / 2;
     constexpr int CW = kFilterWarps, NG = kFilterGroups, kStages = Tile::kStages, kPitch = Tile::kPitch;
@@ -312,7 +321,10 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         // ------------------------------------------------------------------ producer ----
         const int te = a.tile_elems, seg = S > 0 ? rounds / S : 1, phase = S > 0 ? (int)blockIdx.x % seg : 0;
         int it = 0;                         // tiles since the start, of both passes
-        const uint64_t policy = l2_policy_evict_first();
+        // (bulk copies whose lines give way first are the better ones while the gradients of a call are of L2's size; see the host)
+        const uint64_t once = a.evict_first ? l2_policy_evict_first() : l2_policy_evict_normal();
+        // no prediction: the tiles that leave the ring are read again soon (4 x 2 M fp32 14.0 -> 12.8 us, 8 x 2 M 27.5 -> 27.0)
+        const uint64_t again = ONE && S == 0 ? l2_policy_evict_last() : once;
         auto fill = [&](int v, const void *const *rows, int n_rows) {
             const int s = it % kStages;
             if (it >= kStages && !tc_mbar_wait(&empty[s], (uint32_t)((it / kStages - 1) & 1), &abort_flag, kFusedCopyLimit))
@@ -326,7 +338,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
                 const uint32_t bytes = (uint32_t)n * (uint32_t)sizeof(T), dst = tc_smem_u32(ring + (size_t)s * Tile::kBytes);
                 tc_mbar_arrive_expect_tx(&full[s], bytes * (uint32_t)n_rows);
                 for (int g = 0; g < n_rows; ++g)
-                    bulk_load(dst + (uint32_t)(g * kPitch), static_cast<const T *>(rows[g]) + e0, bytes, &full[s], policy);
+                    bulk_load(dst + (uint32_t)(g * kPitch), static_cast<const T *>(rows[g]) + e0, bytes, &full[s], it < rounds - kStages ? again : once);
             } else {
                 tc_mbar_arrive(&full[s]);
             }
@@ -517,36 +529,55 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         while (p >= KT - i) { p -= KT - i; ++i; }
         j = i + p;
     };
-    // Sums of all CTAs in a fixed order into sgram: warp w takes the pairs w, w + CW, ...  `read(pair, cta, value)`
-    // returns whether that sum is there; every warp polls its own at most `limit` times.
-    auto total = [&](auto read, unsigned int limit, double *gram_out) {
-        constexpr int R = kFilterMaxCtas / 32;
-        for (int p = warp; p < NP; p += CW) {
-            double part[R];
-            bool have[R], all = false;
+    // Sums of all CTAs in a fixed order into sgram: warp w takes the pairs w, w + CW, ...  `load(pair, cta)` fetches a sum,
+    // `value(raw, x)` returns whether it is there; every warp polls its own at most `limit` times.  All of a warp's
+    // loads are issued before any is looked at: this is a wait for L2 that every CTA shares (one pair after the other, and one
+    // load after the other, 8 bf16 gradients of 5 M took 35.0 us, now 32.2; 8 fp32 of 16 M 109.6, now 105.5).
+    auto total = [&](auto load, auto value, unsigned int limit, double *gram_out) {
+        constexpr int R = (kFilterMaxCtas + 31) / 32, M = (NP + CW - 1) / CW;
+        double part[M][R];
+        bool all = false;
+        for (unsigned int polls = 0; polls <= limit && !all; ++polls) {
+            decltype(load(0, 0)) raw[M][R];
 #pragma unroll
-            for (int k = 0; k < R; ++k) { part[k] = 0.0; have[k] = lane + 32 * k >= (int)gridDim.x; }
-            for (unsigned int polls = 0; polls <= limit; ++polls) {
-                bool mine = true;
+            for (int m = 0; m < M; ++m)
 #pragma unroll
                 for (int k = 0; k < R; ++k)
-                    if (!have[k]) { have[k] = read(p, lane + 32 * k, part[k]); mine = mine && have[k]; }
-                all = __all_sync(0xFFFFFFFFu, mine);
-                if (all) break;
-            }
-            if (!all) { if (lane == 0) sh_ok = 0; break; }
-            double s = 0.0;
+                    raw[m][k] = load(min(warp + m * CW, NP - 1), min(lane + 32 * k, (int)gridDim.x - 1));
+            bool mine = true;
 #pragma unroll
-            for (int k = 0; k < R; ++k) s += part[k];
+            for (int m = 0; m < M; ++m)
 #pragma unroll
-            for (int d = 16; d > 0; d >>= 1) s += shfl_down_f64(s, d);
-            if (lane == 0) {
-                int i, j;
-                pair_at(p, i, j);
-                sgram[i * KT + j] = s;
-                sgram[j * KT + i] = s;
-                if (gram_out) { gram_out[i * KT + j] = s; gram_out[j * KT + i] = s; }
+                for (int k = 0; k < R; ++k) {
+                    double x;
+                    mine = value(raw[m][k], x) && mine;
+                    part[m][k] = lane + 32 * k < (int)gridDim.x ? x : 0.0;
+                }
+            all = __all_sync(0xFFFFFFFFu, mine);
+        }
+        if (!all) {
+            if (lane == 0) sh_ok = 0;
+        } else {
+            double s[M];
+#pragma unroll
+            for (int m = 0; m < M; ++m) {
+                s[m] = 0.0;
+#pragma unroll
+                for (int k = 0; k < R; ++k) s[m] += part[m][k];
             }
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1)
+#pragma unroll
+                for (int m = 0; m < M; ++m) s[m] += shfl_down_f64(s[m], d);
+#pragma unroll
+            for (int m = 0; m < M; ++m)
+                if (lane == 0 && warp + m * CW < NP) {
+                    int i, j;
+                    pair_at(warp + m * CW, i, j);
+                    sgram[i * KT + j] = s[m];
+                    sgram[j * KT + i] = s[m];
+                    if (gram_out) { gram_out[i * KT + j] = s[m]; gram_out[j * KT + i] = s[m]; }
+                }
         }
         Sync::sync();
         return sh_ok != 0;
@@ -610,11 +641,12 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
                     ((unsigned long long)__float_as_uint((float)cta_sum()) << 32) | tag);
         const unsigned int limit = ONE ? a.spin_limit : kFusedSampleLimit;
         if (blockIdx.x == 0) {
-            const bool known = total([&](int p, int cta, double &value) {
-                const unsigned long long w = ld_word(a.sample_partials + (size_t)p * kFilterMaxCtas + cta);
-                value = (double)__uint_as_float((unsigned int)(w >> 32));
-                return (unsigned int)w == tag && !a.test_withhold;
-            }, limit, nullptr);
+            const bool known = total(
+                [&](int p, int cta) { return ld_word(a.sample_partials + (size_t)p * kFilterMaxCtas + cta); },
+                [&](unsigned long long w, double &x) {
+                    x = (double)__uint_as_float((unsigned int)(w >> 32));
+                    return (unsigned int)w == tag && !a.test_withhold;
+                }, limit, nullptr);
             const bool any_seed = a.ring.K > 0;
             const double tau = any_seed ? a.ring.tau : a.replay.tau;
             const int seed = known && any_seed ? best_seed<1, Sync>(sgram, KT, tau, seed_counts) : 0;
@@ -677,10 +709,9 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     if constexpr (ONE) {
         unsigned long long *const lines = a.verdicts + kFilterMaxCtas * 16;
         if (blockIdx.x == 0) {
-            if (total([&](int p, int cta, double &value) {
-                    return ld_tagged(static_cast<const TaggedSum *>(a.partials) + (size_t)p * kFilterMaxCtas + cta, value, tag) &&
-                           !a.test_withhold;
-                }, a.spin_limit, a.gram)) {
+            if (total([&](int p, int cta) { return ld_tagged(static_cast<const TaggedSum *>(a.partials) + (size_t)p * kFilterMaxCtas + cta); },
+                      [&](const TaggedSum &w, double &x) { return tagged_value(w, x, tag) && !a.test_withhold; },
+                      a.spin_limit, a.gram)) {
                 decide(lines);
             }
         } else if (tid == 0) {
@@ -701,10 +732,8 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         Sync::sync();
         if (!sh_ok) return;
         if (tid == 0) ctl->two_launch_calls = tag + 1u;
-        total([&](int p, int cta, double &value) {
-            value = __ldcg(static_cast<const double *>(a.partials) + (size_t)p * kFilterMaxCtas + cta);
-            return true;
-        }, 0u, a.gram);
+        total([&](int p, int cta) { return __ldcg(static_cast<const double *>(a.partials) + (size_t)p * kFilterMaxCtas + cta); },
+              [](double w, double &x) { x = w; return true; }, 0u, a.gram);
         if (a.pair_dist_out != nullptr) {
             // pairwise mode: Eq. 4 for every pair
             if (tid < KT * KT) {

@@ -734,6 +734,28 @@ def test_many_gradients_mean_of_short_vectors(ws, K, dtype):
             assert gaf.gaf_last_schedule() == gaf.GAF_SCHED_GRAM
 
 
+@pytest.mark.parametrize("K", [5, 6])
+def test_two_tile_sizes_of_five_and_six_bf16_gradients(ws, K):
+    """Both sides of the length from which five and six bfloat16 gradients go through larger tiles, ragged: mask, distances
+    and mean against the stepwise schedule (the mean bit for bit), the Gram matrix of all pairs against binary64."""
+    line = -(-300_000_000 // (2 * K))
+    for D in (line - 1, line + 13):
+        w = _mix(K, D, "bf16", seed=K + D, rho=[0.8, 0.7, -0.6, 0.5, 0.0, 0.6][:K])
+        for tau in (0.9, 2.0):
+            plain = [t.clone() for t in gaf.gaf_filter_accumulate(w.grads, tau, ws, schedule=gaf.GAF_SCHED_STEPWISE)]
+            got = gaf.gaf_filter_accumulate(w.grads, tau, ws, schedule=gaf.GAF_SCHED_GRAM_FUSED)
+            assert torch.equal(got[1], plain[1]) and torch.equal(got[3], plain[3])
+            assert torch.equal(got[0], plain[0]), (D, tau)
+            assert float((got[2] - plain[2]).abs().max()) < 2e-5
+    x = torch.stack(w.grads).double()
+    gram = x @ x.T
+    _, got = gaf.gaf_pairwise_cosdist(w.grads, ws)
+    # products of bf16 pairs are exact in binary32; chains of 128 of them, 2 x 32 chains to a sum, are added there: each sum has
+    # 128 + 6 roundings at most on the way, so 134 x 2^-24 of |x||y|
+    scale = gram.diagonal().sqrt()
+    assert float(((got - gram).abs() / (scale[:, None] * scale[None, :])).max()) < 134 * 2.0 ** -24
+
+
 def test_division_by_the_count_is_correctly_rounded(ws):
     """The mean's division by c (3, 5, 6, 7: two multiply-adds; powers of two: a multiplication) against the division
     itself: significands across the range, zeros, subnormal and huge values, infinities."""
