@@ -973,6 +973,12 @@ int gaf_filter_accumulate_bucketed(const void *const *grads, int K, int64_t D, i
     // the end of every CTA's range, kKeepL2Pct of L2 in all, is asked to stay in L2 for the mean pass
     ga.keep_elems = int64_t(di.l2_bytes) * kKeepL2Pct / 100 / (int64_t(K) * int64_t(elem_bytes(dtype))) / grid;
     ga.keep_elems = (ga.keep_elems + 7) / 8 * 8;
+    // gradients of 4/3 of L2 and more: the mean pass reads without the hint that its lines leave L2 first (2 / 4 / 8 fp32 gradients of
+    // 39 / 100 / 20 M 123.6 -> 120.7, 491 with the hint in the Gram pass, 475 without in both, 199.8 -> 185.5 us), and so does the
+    // Gram pass of four fp32 gradients and more (3 x 30 M 127.1 without, 124.4 with; bf16 4 x 30 M 103.5, 101.7).  Shorter
+    // ones are better off with it (4 x 3 M in 20 buckets 22.4, 24.1 without).
+    const bool beyond_l2 = int64_t(K) * D * int64_t(elem_bytes(dtype)) * 3 >= int64_t(di.l2_bytes) * 4;
+    ga.evict_first = !(beyond_l2 && dtype == GAF_F32 && K >= 4);
     int rc = dtype == GAF_F32 ? launch_bucket_gram<float>(ga, bt, K, grid, st)
                               : launch_bucket_gram<__nv_bfloat16>(ga, bt, K, grid, st);
     if (rc != GAF_OK) return rc;
@@ -991,6 +997,7 @@ int gaf_filter_accumulate_bucketed(const void *const *grads, int K, int64_t D, i
     BucketMeanArgs ma{};
     for (int t = 0; t < K; ++t) ma.g[t] = grads[ord[t]];
     ma.K = K; ma.D = D; ma.out = macro_out; ma.bits = bits;
+    ma.evict_first = !beyond_l2;
     {
         // (its own grid, two CTAs per SM: the ranges need not be those of the Gram pass)
         int mean_grid = di.sms * 2;

@@ -10,7 +10,8 @@
 // tensors have a few hundred elements, so a bucket counts as kBkBucketCost elements when the ranges are cut (62 tensors of
 // ResNet18, 4 fp32 gradients, whole call: 75.0 us with equal shares, 74.0 / 72.3 / 71.6 with a bucket counted as 1024 / 2048 / 5000
 // elements; 200 buckets of 3 M: 34.9, 30.0, 28.6, 29.2.  Before, with a walk that recomputed every range in every thread and a
-// mean pass with two barriers a bucket: 78.6 and 47.4 us; 20 buckets of 100 k: 28.1, now 12.8).
+// mean pass with two barriers a bucket: 78.6 and 47.4 us; 20 buckets of 100 k: 28.1, now 12.8).  Eight 16-byte vectors in flight per
+// thread of the mean pass, whatever the number of gradients, and no eviction hint beyond L2: 71.6 -> 63.7.
 #pragma once
 
 #include "gaf_device.cuh"
@@ -61,6 +62,7 @@ struct BucketGramArgs {
     const void *g[kGsMaxK];                 // processing order
     int64_t D;
     int64_t keep_elems;                     // the last so many elements of every CTA's range are loaded "keep in L2"
+    int evict_first;                        // the others are the first to leave it
     double *partials;                       // [slot][64], slot = cta + bucket
     Control *ctl;
 };
@@ -78,7 +80,7 @@ bucket_gram_kernel(const __grid_constant__ BucketGramArgs a, const __grid_consta
 #pragma unroll
     for (int r = 0; r < KT; ++r) row[r] = static_cast<const T *>(a.g[r]);
     // the mean pass walks every CTA's range from its end: the end of the range is asked to stay in L2
-    const uint64_t pol_first = l2_policy_evict_first(), pol_last = l2_policy_evict_last();
+    const uint64_t pol_first = a.evict_first ? l2_policy_evict_first() : l2_policy_evict_normal(), pol_last = l2_policy_evict_last();
     int64_t lo, hi;
     cta_range(bt, a.D, blockIdx.x, gridDim.x, lo, hi);
     // a programmatic dependent of what precedes it on the stream (a no-op after an ordinary launch)
@@ -244,6 +246,7 @@ struct BucketMeanArgs {
     int K;
     int64_t D;
     float *out;
+    int evict_first;                        // what is read leaves L2 first
     const unsigned long long *bits;         // [S]
 };
 
@@ -252,6 +255,7 @@ __global__ void __launch_bounds__(kBkThreads, 2)
 bucket_mean_kernel(const __grid_constant__ BucketMeanArgs a, const __grid_constant__ BucketTable bt) {
     constexpr int N = MeanVec<T>::N;        // elements of a 16-byte load
     constexpr int U = 8 / KM;               // vectors of a gradient a thread has in flight
+    const uint64_t policy = a.evict_first ? l2_policy_evict_first() : l2_policy_evict_normal();
     int64_t lo, hi;
     cta_range(bt, a.D, blockIdx.x, gridDim.x, lo, hi);
     // programmatic dependent of the per-bucket walk: wait for its accept bits
@@ -275,7 +279,7 @@ bucket_mean_kernel(const __grid_constant__ BucketMeanArgs a, const __grid_consta
 #pragma unroll
                     for (int t = 0; t < KM; ++t)
                         if (((bits >> t) & 1u) && o + u * kBkThreads < n_vec)
-                            w[u][t] = __ldcs(reinterpret_cast<const uint4 *>(static_cast<const T *>(a.g[t]) + s0 + (n_vec - 1 - o - u * kBkThreads) * N));
+                            w[u][t] = ld16_policy(static_cast<const T *>(a.g[t]) + s0 + (n_vec - 1 - o - u * kBkThreads) * N, policy);
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     if (o + u * kBkThreads >= n_vec) break;
