@@ -127,25 +127,9 @@ def min_bytes(K, D, b):
 #   "steady"   caches left as the previous call left them (ncu --cache-control none): what crosses HBM while
 #              calls run back to back, as they do in the timed region -- this is `traffic`;
 #   "flushed"  ncu's default, caches flushed before every launch: a call that starts with a cold L2.
-# At configuration 2 they differ: back to back, about 32 MB of L2 hold the previous call's output (dirty lines
-# that the next call overwrites in place, so they never reach HBM) and fewer of the second pass's re-reads hit.
-# Captures on a shorter vector of the same recipe scale in proportion (both passes stream; inputs far beyond
-# L2).  An entry is used only while the listed kernel sources hash to what was profiled; otherwise null.
-NCU_TRAFFIC = {
-    # gram_fused_kernel<float,4> at configuration 2 itself (D = 11,227,812)
-    (2, 3): {"sources": ["gaf_fused.cuh", "gaf_gramfilter.cuh", "gaf_device.cuh"],
-             "sha256": "c818aa29bb0ab3cfd20979d4de48b461b64f5638d0d403cbeae6950f4970cd2f",
-             "steady": {2: 262.6e6 / 11227812, 3: 296.4e6 / 11227812},
-             "flushed": {2: 230.3e6 / 11227812, 3: 257.8e6 / 11227812}},
-    # gram_small_kernel<float,8> + masked_mean_kernel<float>, captured at D = 80,000,000
-    (4, 2): {"sources": ["gaf_gramfilter.cuh", "gaf_device.cuh"],
-             "sha256": "707df4a1adb38d5c23a4b0a9334cb7ee98408cb34984959ae16d9bc13231b65d",
-             "steady": {4: (2563.4e6 + 1573.5e6) / 80e6, 1: (2563.9e6 + 591.2e6) / 80e6}},
-    # gram_mma_kernel<8> + masked_mean_kernel<bf16>, captured at D = 100,000,000
-    (5, 2): {"sources": ["gaf_gram_mma.cuh", "gaf_gramfilter.cuh", "gaf_device.cuh"],
-             "sha256": "9e4d0496b3660411997f70119a65ea597629d6649e27b79cad70329530722984",
-             "steady": {4: (1604.5e6 + 1169.0e6) / 100e6}},
-}
+# Captures on a shorter vector of the same recipe scale in proportion (inputs far beyond L2).  An entry is used
+# only while the listed kernel sources hash to what was profiled; otherwise null.
+NCU_TRAFFIC = {}
 
 
 def kernel_sources_hash(names):
@@ -550,7 +534,7 @@ def measure_pairwise(torch, gaf, workloads, dev, steps, warmup, nvml, K=None, D=
             "gram_loader": {0: None, 1: "16-byte asynchronous copies", 2: "tensor copies (TMA)"}[loader],
             "kernel": ("gram_tc_kernel" if (not fp32 and 16 < K <= 64) else
                        "gram_mma_wide_kernel" if (not fp32 and 8 < K <= 16) else
-                       "gram_panel_kernel" if K > 8 else "gram_small_kernel") + " + finishing (whole call)"}
+                       "gram_panel_kernel" if K > 8 else "gram_filter_kernel") + " + finishing (whole call)"}
 
 
 def measure_cosdist(torch, gaf, workloads, dev, D, steps, nvml, peak, peak_kind):
@@ -859,8 +843,8 @@ def run_ours(args):
                 "dram_frac": fr["dram_frac"], "dram_frac_flushed_caches": fr["dram_frac_flushed_caches"], "min_bytes_frac": fr["min_bytes_frac"], "model_frac": fr["model_frac"],
                 "dram_gbs": fr["dram_gbs"], "min_bytes_gbs": fr["min_bytes_gbs"], "model_gbs": fr["model_gbs"],
                 "frac_of_nominal_8000": achieved / 8000.0,
-                "kernel": {3: "gram_fused_kernel (the whole call is this one launch)",
-                           2: "Gram kernel + masked_mean_kernel (whole call, both HBM-streaming)",
+                "kernel": {3: "gram_filter_kernel (the whole call is this one launch)",
+                           2: "Gram kernel + mean kernel (whole call; up to 8 gradients the mean is written by the first)",
                            1: "step_kernel x%d (whole call)" % m["launches_per_step"]}[sched_used],
                 "byte_model": ("Gram-first: ((K + c) b + 4) D; part of it is served by shared memory and L2, "
                                "so model_frac is an effective rate, not HBM utilisation" if sched_used in (2, 3)
@@ -911,7 +895,7 @@ def run_two_gradients(args):
                                "experiments); headline = the stream of calls that all accept"},
         "roofline": {"bound": "hbm", "achieved": head["min_bytes_frac"] * peak, "peak": peak, "unit": "GB/s",
                      "frac": head["min_bytes_frac"], "basis": "min_bytes: (2 b + 4) D", "traffic": None,
-                     "peak_kind": peak_kind, "kernel": "gram_fused_kernel<float, 2>",
+                     "peak_kind": peak_kind, "kernel": "gram_filter_kernel<float, 2>",
                      "algorithmic_bytes_per_launch": m["min_bytes_per_call"]},
         "two_gradients": m, "e2e": None, "gpu_launches": head["launches_per_call"] * args.steps,
         "clocks": head["clocks"], "cpu_baseline": None,

@@ -93,7 +93,6 @@ struct PerDevice {
 };
 struct DynSmemPlan { int dyn = 0; };    // "the dynamic shared memory limit of this kernel has been raised"
 struct OccPlan { int occ = 1; };
-struct FusedPlan { int occ = 0, park = 0, dyn = 0; };
 
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline size_t elem_bytes(int dtype) { return dtype == GAF_F32 ? 4 : 2; }
