@@ -129,7 +129,12 @@ def min_bytes(K, D, b):
 #   "flushed"  ncu's default, caches flushed before every launch: a call that starts with a cold L2.
 # Captures on a shorter vector of the same recipe scale in proportion (inputs far beyond L2).  An entry is used
 # only while the listed kernel sources hash to what was profiled; otherwise null.
-NCU_TRAFFIC = {}
+NCU_TRAFFIC = {
+    # gram_filter_kernel<float,4> at configuration 2 itself (D = 11,227,812): the minimum, whatever is accepted
+    (2, 3): {"sources": ["gaf_fused.cuh", "gaf_gramfilter.cuh", "gaf_device.cuh"],
+             "sha256": "b5b8d90ddd01b8c3af9a16659c4342c08c3f8197724f7060755890876350aecb",
+             "steady": {2: 225.2e6 / 11227812, 3: 225.2e6 / 11227812}},
+}
 
 
 def kernel_sources_hash(names):

@@ -417,10 +417,10 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
 constexpr int kKeepL2Pct = 10;          // share of L2 the Gram pass asks to keep for the second pass
                                         // ("evict last" lines live in the persisting part of L2, 24.9 MB by
                                         // default on this GPU; larger shares slow both passes down)
-// AUTO takes the one-launch form for binary32 inputs up to this many bytes in all: beyond, what stays
-// on chip between the passes is a negligible share and the two-launch form is as fast or slightly
-// faster.  For bfloat16 with up to 6 gradients the one-launch form stays ahead at every length measured;
-// with 7 or 8 the two-launch form on the warp-level MMA Gram kernel overtakes it near 1 GB of inputs.
+// AUTO takes the one-launch form up to these many bytes of inputs in all (the header states them; two gradients, and up to 6 of
+// bfloat16: at every length).  Beyond, the launch of a mean kernel that finds its work done is 1 to 3 % of the call (8 fp32 gradients of
+// 30 M 182 us in one launch, 188 in two; 8 of 124 M 707 to 770, 711 to 730; 8 bf16 of 600 M 2290 to 2360, 2370), and two launches
+// do not need the whole device to themselves for that long.
 constexpr int64_t kFusedMaxInputBytesF32 = int64_t(512) << 20;
 constexpr int64_t kFusedMaxInputBytesBf16Mma = int64_t(1) << 30;
 
