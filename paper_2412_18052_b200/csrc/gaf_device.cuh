@@ -18,7 +18,7 @@ constexpr int kOct = 8;                 // elements handled per inner step
 struct Control {
     unsigned int ticket;                // last-block election, wraps to 0 by itself
     unsigned int pair_hint;             // one-launch schedule with two gradients: what the latest two calls kept (0 both, 1 the seed alone, 2 | latest: they differed)
-    unsigned int written_ctas;          // two-launch form: CTAs that wrote the predicted mean of all their elements
+    unsigned int reserved1;
     int mean_done;                      // two-launch form: 1 = the first launch has written the result
     int status;                         // GAF_STATUS_* bits of the latest call
     int count;                          // running c of Algorithm 1

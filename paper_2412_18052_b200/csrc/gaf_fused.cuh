@@ -295,6 +295,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     __shared__ const T *list[kGsMaxK];      // accepted gradients in the order they are added
     __shared__ int n_list;                  // c
     __shared__ int sh_ok, sh_again;         // outcome of a wait; how many tiles are fetched a second time
+    __shared__ int sh_done;                 // two launches: every CTA has written the decided mean
     __shared__ unsigned int sh_pred;        // predicted and decided pattern
     __shared__ volatile unsigned int sh_final;
     __shared__ volatile int abort_flag;
@@ -303,7 +304,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
 
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) { tc_mbar_init(&full[s], 1); tc_mbar_init(&empty[s], kFilterGroupWarps); }
-        sh_pred = 0u; sh_final = 0u; sh_ok = 1; sh_again = 0; abort_flag = 0;
+        sh_pred = 0u; sh_final = 0u; sh_ok = 1; sh_again = 0; sh_done = 1; abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     for (int i = tid; i < CW * NP; i += kFilterThreads) (&ssum[0][0])[i] = 0.0;
@@ -704,6 +705,12 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         if constexpr (ONE) st_tagged(static_cast<TaggedSum *>(a.partials) + (size_t)tid * kFilterMaxCtas + blockIdx.x, s, tag);
         else static_cast<double *>(a.partials)[(size_t)tid * kFilterMaxCtas + blockIdx.x] = s;
     }
+    // two launches: the pattern under which this CTA wrote its share of the mean, for the CTA that decides (the words that tell
+    // the decision, which this form does not use)
+    unsigned int *const written = reinterpret_cast<unsigned int *>(a.verdicts + kFilterMaxCtas * 16);
+    if constexpr (!ONE) {
+        if (tid == 0 && a.pair_dist_out == nullptr) written[blockIdx.x] = pred;
+    }
 
     // ---- decide ----
     if constexpr (ONE) {
@@ -725,13 +732,11 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         }
     } else {
         Sync::sync();
-        if (tid == 0) {
-            if (pred) atomicAdd(&ctl->written_ctas, 1u);
-            sh_ok = take_last_ticket(&ctl->ticket, gridDim.x) ? 1 : 0;
-        }
+        if (tid == 0) sh_ok = take_last_ticket(&ctl->ticket, gridDim.x) ? 1 : 0;
         Sync::sync();
         if (!sh_ok) return;
         if (tid == 0) ctl->two_launch_calls = tag + 1u;
+        const unsigned int share = a.pair_dist_out == nullptr && tid < (int)gridDim.x ? __ldcg(written + tid) : 0u;
         total([&](int p, int cta) { return __ldcg(static_cast<const double *>(a.partials) + (size_t)p * kFilterMaxCtas + cta); },
               [](double w, double &x) { x = w; return true; }, 0u, a.gram);
         if (a.pair_dist_out != nullptr) {
@@ -748,6 +753,8 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
             return;
         }
         decide(nullptr);
+        // the result is complete if EVERY CTA wrote its share under the decided pattern, wherever it had the pattern from
+        if (tid < (int)gridDim.x && share != sh_final) sh_done = 0;
     }
     const int kept = pred ? 0 : min(rounds, kStages);           // tiles that are still in the ring
     if (tid == 0) {
@@ -768,12 +775,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     Sync::sync();
     const int c = n_list;
     if constexpr (!ONE) {
-        if (tid == 0) {
-            // (the ticket ordered every CTA's count before this read)
-            const unsigned int written = __ldcg(&ctl->written_ctas);
-            ctl->written_ctas = 0u;
-            ctl->mean_done = (written == gridDim.x && pred == sh_final) ? 1 : 0;
-        }
+        if (tid == 0) ctl->mean_done = sh_done;
     } else {
         // the launch behind this one on the stream may be placed from here on (it waits for this grid itself)
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -1,0 +1,86 @@
+"""The Gram-first forms of the filter from every state a workspace can be in: GPU tests, results against the stepwise
+schedule bit for bit."""
+import pytest
+import torch
+
+import paper_2412_18052_b200 as gaf
+from paper_2412_18052_b200 import workloads
+
+pytestmark = pytest.mark.gpu
+
+CODE = {"f32": gaf.GAF_F32, "bf16": gaf.GAF_BF16}
+
+
+def _mix(K, D, dtype, seed, rho, stacked=False):
+    return workloads.mixture(K, D, dtype, rho, seed, device="cuda", stacked=stacked).grads
+
+
+def _predicted_length(K, dtype):
+    """A length from which the one-pass kernel predicts the accept pattern: four times what the SMs' shared memory holds."""
+    return 4 * 200_000 // (K * (4 if dtype == "f32" else 2)) * 148
+
+
+def _stepwise(grads, tau, ws):
+    return [t.clone() for t in gaf.gaf_filter_accumulate(grads, tau, ws, schedule=gaf.GAF_SCHED_STEPWISE)]
+
+
+def _same(got, want):
+    assert torch.equal(got[1], want[1]) and torch.equal(got[3], want[3])
+    assert torch.equal(got[0], want[0])
+
+
+@pytest.mark.parametrize("K,dtype", [(3, "f32"), (4, "f32"), (8, "f32"), (8, "bf16")])
+def test_two_launches_on_a_workspace_initialised_for_every_call(K, dtype):
+    """One buffer, initialised anew for every call, as a workspace per step at one address is; the accept patterns alternate, so
+    that what the memory still holds from the call before is always the wrong one."""
+    D = _predicted_length(K, dtype)
+    both = [_mix(K, D, dtype, 3, [0.8] * K), _mix(K, D, dtype, 4, ([0.8] + [0.7, -0.6] * K)[:K])]
+    other = gaf.new_workspace(K, D, CODE[dtype])
+    want = [_stepwise(g, 0.9, other) for g in both]
+    assert not torch.equal(want[0][1], want[1][1])
+    ws = gaf.new_workspace(K, D, CODE[dtype])
+    for call in range(12):
+        gaf.gaf_workspace_init(ws)
+        _same(gaf.gaf_filter_accumulate(both[call % 2], 0.9, ws, schedule=gaf.GAF_SCHED_GRAM), want[call % 2])
+
+
+@pytest.mark.parametrize("before", ["cosdist", "stepwise", "stream", "bucketed", "pairwise16"])
+def test_two_launches_first_after_another_operation(before):
+    """Whole-numbered gradients: the partial sums that other operations leave in the workspace have empty low words.  The first
+    two-launch call behind them."""
+    K, D = 4, _predicted_length(4, "f32")
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    grads = [torch.randint(0, 2, (D,), generator=gen, device="cuda").float() + 1.0 for _ in range(K)]
+    grads[2] = -grads[2]
+    want = _stepwise(grads, 0.9, gaf.new_workspace(K, D, gaf.GAF_F32))
+    assert want[1].tolist() == [1, 1, 0, 1]
+    for _ in range(3):
+        ws = gaf.new_workspace(16, D, gaf.GAF_F32)
+        if before == "cosdist":
+            gaf.gaf_cosdist(grads[0], grads[2], ws)
+        elif before == "stepwise":
+            _stepwise(grads, 0.9, ws)
+        elif before == "stream":
+            acc = torch.empty(D, device="cuda")
+            gaf.gaf_stream_begin(grads[0], acc, ws)
+            gaf.gaf_stream_push(grads[1], 1, 0.9, acc, ws)
+            gaf.gaf_stream_end(2, acc, ws)
+        elif before == "bucketed":
+            gaf.gaf_filter_accumulate_bucketed(grads, 0.9, [0, D // 16 * 8, D], ws)
+        else:
+            gaf.gaf_pairwise_cosdist([g[:100_000].contiguous() for g in grads * 4], ws)
+        _same(gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM), want)
+
+
+@pytest.mark.parametrize("fill", [0.0, 1.0, -3.0, 1e-3])
+def test_two_launches_on_memory_that_held_other_data(fill):
+    """A workspace whose memory was a binary64 tensor before: zeros, values with an empty low word, any others."""
+    K, D = 4, _predicted_length(4, "f32")
+    grads = _mix(K, D, "f32", 5, [0.8, 0.7, -0.6, 0.5])
+    want = _stepwise(grads, 0.9, gaf.new_workspace(K, D, gaf.GAF_F32))
+    ws = gaf.new_workspace(K, D, gaf.GAF_F32)
+    for _ in range(3):
+        ws.view(torch.float64).fill_(fill)
+        gaf.gaf_workspace_init(ws)
+        for _ in range(2):
+            _same(gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM), want)
