@@ -149,8 +149,8 @@ const char *gaf_error_string(int code);
 int gaf_workspace_bytes(int K, int64_t D, int dtype, size_t *bytes_out);
 
 /*
- * Prepare a workspace: clears its control block (asynchronous memset on the
- * stream).  Needed once after allocation; every call leaves the workspace ready
+ * Prepare a workspace: clears its control block and the words through which
+ * kernels exchange sums (one asynchronous memset on the stream).  Needed once after allocation; every call leaves the workspace ready
  * for the next one.  A workspace serves one call at a time: calls that share a
  * workspace must be ordered on one stream.
  *   workspace        device, 256-byte aligned, >= gaf_workspace_bytes(...)

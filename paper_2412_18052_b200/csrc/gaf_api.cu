@@ -175,7 +175,8 @@ size_t gram_matrix_bytes(int K) { return round_up(size_t(K) * K * sizeof(double)
 // what gram_partials_bytes reserves).
 // (the CTAs' lines lie where the stepwise schedule has its partial sums)
 constexpr size_t kFilterSumsBytes = size_t(36) * kFilterMaxCtas * sizeof(TaggedSum);
-static_assert(kFilterSumsBytes + size_t(36) * kFilterMaxCtas * 8 <= size_t(kGramMaxSlices) * 64 * sizeof(double), "workspace layout");
+constexpr size_t kFilterExchangeBytes = kFilterSumsBytes + size_t(36) * kFilterMaxCtas * 8;
+static_assert(kFilterExchangeBytes <= size_t(kGramMaxSlices) * 64 * sizeof(double), "workspace layout");
 static_assert(size_t(2) * kFilterMaxCtas * 128 <= kPartialsBytes, "workspace layout");
 // Bucketed variant: partial slots [ctas + buckets][64] doubles and one bit mask per bucket.
 size_t bucketed_extra_bytes() {
@@ -779,7 +780,10 @@ int gaf_workspace_bytes(int K, int64_t D, int dtype, size_t *bytes_out) {
 int gaf_workspace_init(void *workspace, size_t workspace_bytes, void *cuda_stream) {
     if (int rc = check_workspace(workspace, workspace_bytes, kExtraOffset)) return rc;
     g_launches = 0; g_gram_loader = 0;
-    if (cudaMemsetAsync(workspace, 0, kControlBytes, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
+    // the control block, and what CTAs of the one-pass kernel tell one another: the memory may hold another workspace's words,
+    // whose call numbers start at the same value
+    const size_t all = kExtraOffset + kFilterExchangeBytes, clear = workspace_bytes < all ? workspace_bytes : all;
+    if (cudaMemsetAsync(workspace, 0, clear, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
         return GAF_ERR_CUDA;
     return GAF_OK;
 }

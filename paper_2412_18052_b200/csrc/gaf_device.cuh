@@ -29,7 +29,7 @@ struct Control {
     float stream_dist[GAF_MAX_K];       // streaming form: distance of arrival t
     uint8_t stream_mask[GAF_MAX_K];     // streaming form: decision of arrival t
     double norm_sq_sum;                 // stepwise and streaming forms: sum of |g_i|^2 over the accepted gradients
-    unsigned int two_launch_calls;      // calls of the two-launch form of gaf_fused.cuh so far: the tag of their sample sums
+    unsigned int two_launch_calls;      // calls of the two-launch form of gaf_fused.cuh so far: the next one's tag is one more
 };
 constexpr size_t kControlBytes = 4096;  // sizeof(Control) rounded up
 static_assert(sizeof(Control) <= kControlBytes, "control block");

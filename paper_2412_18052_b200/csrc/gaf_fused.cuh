@@ -104,7 +104,7 @@ struct GramFusedArgs {
     int evict_first;                        // what is read once gives way in L2 first
     void *partials;                         // [pair][kFilterMaxCtas]: TaggedSum (ONE) or double
     unsigned long long *sample_partials;    // [pair][kFilterMaxCtas]: binary32 sum and tag
-    unsigned long long *verdicts;           // [2][kFilterMaxCtas][16]: a line per CTA, predicted and decided pattern and tag
+    unsigned long long *verdicts;           // [2][kFilterMaxCtas][16]: a line per CTA for the predicted and one for the decided pattern
     unsigned int tag;                       // ONE: a number no other launch has
     double *gram;                           // [K][K]
     float *out;                             // D floats
@@ -119,9 +119,11 @@ struct GramFusedArgs {
 
 // What CTAs tell one another carries the call's tag in every word, so that the reader polls the data itself: one
 // trip to L2 and back after the last store, where an arrival counter (stores, release, counter, poll, then the
-// loads) took three.  A binary64 sum travels as two words, half a sum and the tag each; every word is written and
-// read as a whole.  What an earlier call or another kernel left in the place carries another tag.  Every word
+// loads) took three.  A binary64 sum travels as two words, half a sum and the tag or its complement each; a pattern as two
+// words as well, whole in both; every word is written and read as a whole.  What an earlier call left in the place
+// carries another tag, and 64 bits of a number that another operation left there would have to agree.  Every word
 // has ONE reader: 148 CTAs that read the same lines at the same time wait 3 to 6 us for them.
+// (The sample's sums travel as one word each, binary32 and the tag: all that can come of a stale one is a wrong prediction.)
 __device__ __forceinline__ void st_word(unsigned long long *p, unsigned long long v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
@@ -144,6 +146,16 @@ __device__ __forceinline__ TaggedSum ld_tagged(const TaggedSum *p) {
 __device__ __forceinline__ bool tagged_value(const TaggedSum &t, double &v, unsigned int tag) {
     v = __longlong_as_double((long long)((t.w[0] >> 32) | (t.w[1] & 0xFFFFFFFF00000000ull)));
     return (unsigned int)t.w[0] == tag && (unsigned int)t.w[1] == (unsigned int)~tag;
+}
+__device__ __forceinline__ void st_pattern(unsigned long long *p, unsigned int pattern, unsigned int tag) {
+    const unsigned long long hi = (unsigned long long)pattern << 32;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(hi | tag), "l"(hi | (unsigned int)~tag) : "memory");
+}
+__device__ __forceinline__ bool ld_pattern(const unsigned long long *p, unsigned int &pattern, unsigned int tag) {
+    unsigned long long a, b;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+    pattern = (unsigned int)(a >> 32);
+    return (unsigned int)a == tag && (unsigned int)b == (unsigned int)~tag && (unsigned int)(b >> 32) == pattern;
 }
 // Bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned) into shared memory, counted on `bar`.
 __device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void *src, uint32_t bytes, uint64_t *bar, uint64_t policy) {
@@ -365,9 +377,10 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     // ---------------------------------------------------------------------- consumers ----
     const int group = warp / kFilterGroupWarps, gwarp = warp - group * kFilterGroupWarps, gtid = gwarp * 32 + lane;
     if (blockIdx.x == 0 && tid == 0) ctl->status = 0;
-    // Two launches may be replayed from a graph: their tag is a count of such calls in the workspace, which moves on
-    // when every CTA of the call has taken its ticket.  (The tags of the one-launch form have the upper bit set.)
-    const unsigned int tag = ONE ? a.tag | 0x80000000u : __ldcg(&ctl->two_launch_calls) & 0x7FFFFFFFu;
+    // Two launches may be replayed from a graph: their tag is the number of the call among such calls on the workspace, from 1 on
+    // (gaf_workspace_init clears the words that carry it); the count moves on when every CTA of the call has taken its ticket.
+    // (The tags of the one-launch form have the upper bit set.)
+    const unsigned int tag = ONE ? a.tag | 0x80000000u : (__ldcg(&ctl->two_launch_calls) + 1u) & 0x7FFFFFFFu;
 
     // Accumulators: binary64, pairs of binary32 chains, or (MMA) this lane's fragment of the 8 x 8 matrix.
     constexpr bool kF64 = !GsAcc<T, KT>::kPeriodicFlush;
@@ -586,12 +599,12 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
 
     // CTA 0, one warp: a pattern to every CTA's line; the other CTAs, one thread: wait for it (0 = it did not come).
     auto tell = [&](unsigned long long *lines, unsigned int pattern) {
-        for (int cta = lane; cta < (int)gridDim.x; cta += 32) st_word(lines + cta * 16, ((unsigned long long)pattern << 32) | tag);
+        for (int cta = lane; cta < (int)gridDim.x; cta += 32) st_pattern(lines + cta * 16, pattern, tag);
     };
     auto hear = [&](const unsigned long long *lines, unsigned int limit) {
         for (unsigned int polls = 0; polls <= limit; ++polls) {
-            const unsigned long long w = ld_word(lines + blockIdx.x * 16);
-            if ((unsigned int)w == tag && !a.test_withhold) return (unsigned int)(w >> 32);
+            unsigned int pattern;
+            if (ld_pattern(lines + blockIdx.x * 16, pattern, tag) && !a.test_withhold) return pattern;
         }
         return 0u;
     };
@@ -705,11 +718,10 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         if constexpr (ONE) st_tagged(static_cast<TaggedSum *>(a.partials) + (size_t)tid * kFilterMaxCtas + blockIdx.x, s, tag);
         else static_cast<double *>(a.partials)[(size_t)tid * kFilterMaxCtas + blockIdx.x] = s;
     }
-    // two launches: the pattern under which this CTA wrote its share of the mean, for the CTA that decides (the words that tell
-    // the decision, which this form does not use)
-    unsigned int *const written = reinterpret_cast<unsigned int *>(a.verdicts + kFilterMaxCtas * 16);
+    // two launches: the pattern under which this CTA wrote its share of the mean, for the CTA that decides (in the CTA's line,
+    // behind the words that carry a tag)
     if constexpr (!ONE) {
-        if (tid == 0 && a.pair_dist_out == nullptr) written[blockIdx.x] = pred;
+        if (tid == 0 && a.pair_dist_out == nullptr) a.verdicts[blockIdx.x * 16 + 8] = pred;
     }
 
     // ---- decide ----
@@ -735,8 +747,8 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         if (tid == 0) sh_ok = take_last_ticket(&ctl->ticket, gridDim.x) ? 1 : 0;
         Sync::sync();
         if (!sh_ok) return;
-        if (tid == 0) ctl->two_launch_calls = tag + 1u;
-        const unsigned int share = a.pair_dist_out == nullptr && tid < (int)gridDim.x ? __ldcg(written + tid) : 0u;
+        if (tid == 0) ctl->two_launch_calls = tag;
+        const unsigned int share = a.pair_dist_out == nullptr && tid < (int)gridDim.x ? (unsigned int)__ldcg(a.verdicts + tid * 16 + 8) : 0u;
         total([&](int p, int cta) { return __ldcg(static_cast<const double *>(a.partials) + (size_t)p * kFilterMaxCtas + cta); },
               [](double w, double &x) { x = w; return true; }, 0u, a.gram);
         if (a.pair_dist_out != nullptr) {

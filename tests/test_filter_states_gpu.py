@@ -84,3 +84,47 @@ def test_two_launches_on_memory_that_held_other_data(fill):
         gaf.gaf_workspace_init(ws)
         for _ in range(2):
             _same(gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM), want)
+
+
+def _lines(ws, table):
+    """The lines of 16 words through which the CTAs of the one-pass kernel are told the predicted (0) or decided (1) pattern."""
+    return ws[4096 + table * 160 * 128:4096 + (table + 1) * 160 * 128].view(torch.int64).view(160, 16)
+
+
+@pytest.mark.parametrize("K,dtype", [(4, "f32"), (8, "f32"), (8, "bf16")])
+def test_first_call_on_a_workspace_predicts(K, dtype):
+    """The first two-launch call on memory that was zero, or held another workspace, writes the result in its first launch
+    (word 3 of the workspace says so) like every later one.  A prediction is given up after some tens of microseconds, so one call
+    of several counts."""
+    D = _predicted_length(K, dtype)
+    grads = _mix(K, D, dtype, 5, ([0.8, 0.7, -0.6, 0.5] * 2)[:K])
+    ws = gaf.new_workspace(K, D, CODE[dtype])
+    for zeroed in (True, False):
+        done = 0
+        for _ in range(5):
+            if zeroed:
+                ws.zero_()
+            gaf.gaf_workspace_init(ws)
+            gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM)
+            done += int(ws[:16].view(torch.int32)[3])
+        assert done >= 1, zeroed
+
+
+def test_words_that_only_look_like_a_pattern():
+    """Lines that hold a whole valid word of the call's tag with the wrong pattern (two launches: only the comparison of what the
+    CTAs wrote can tell), and words whose low half alone is the tag of the call (either form)."""
+    K, D = 4, _predicted_length(4, "f32")
+    grads = _mix(K, D, "f32", 5, [0.8, 0.7, -0.6, 0.5])
+    ws = gaf.new_workspace(K, D, gaf.GAF_F32)
+    want = _stepwise(grads, 0.9, ws)
+    wrong = (0x80000004 - (1 << 32)) << 32                      # the third gradient alone
+    for whole in (True, False):
+        gaf.gaf_workspace_init(ws)
+        _lines(ws, 0)[:, 0] = wrong | 1
+        _lines(ws, 0)[:, 1] = wrong | 0xFFFFFFFE if whole else 0
+        _same(gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM), want)
+    for _ in range(3):
+        _same(gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM_FUSED), want)
+        tag = (int(_lines(ws, 1)[1, 0]) + 1) & 0xFFFFFFFF        # the next call's
+        _lines(ws, 1)[:, 0] = wrong | tag
+        _lines(ws, 1)[:, 1] = 0
