@@ -85,7 +85,8 @@ __device__ __forceinline__ WalkResult warp_walk(const double *gram, int K, int s
 #pragma unroll
         for (int w = 0; w < JW; ++w) row[w] = lane + 32 * w < K ? gram[i * K + lane + 32 * w] : 0.0;
         const float fp = (float)p, fa = (float)na, fg = (float)ng;
-        const float margin = fp * (rsqrtf(fa) * rsqrtf(fg)) - bound;
+        // (clamped like Eq. 4's cosine: where accepted gradients have nearly cancelled, the sums' rounding can put it outside)
+        const float margin = fminf(fmaxf(fp * (rsqrtf(fa) * rsqrtf(fg)), -1.0f), 1.0f) - bound;
         bool accept = margin >= 0.0f;
         const bool safe = fa > 1e-30f && fa < 1e30f && fg > 1e-30f && fg < 1e30f && fabsf(fp) < 1e30f && fabsf(margin) > 1e-5f;
         if (!safe) {

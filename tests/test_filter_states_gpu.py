@@ -1,5 +1,5 @@
-"""The Gram-first forms of the filter from every state a workspace can be in: GPU tests, results against the stepwise
-schedule bit for bit."""
+"""The Gram-first forms of the filter from every state a workspace can be in, and decisions and sums that must not depend on the
+form or on what ran before: GPU tests, results against the stepwise schedule bit for bit."""
 import pytest
 import torch
 
@@ -128,3 +128,27 @@ def test_words_that_only_look_like_a_pattern():
         tag = (int(_lines(ws, 1)[1, 0]) + 1) & 0xFFFFFFFF        # the next call's
         _lines(ws, 1)[:, 0] = wrong | tag
         _lines(ws, 1)[:, 1] = 0
+
+
+@pytest.mark.parametrize("K,dtype", [(3, "f32"), (5, "f32"), (8, "f32"), (6, "bf16"), (8, "bf16"), (12, "f32"), (12, "bf16")])
+def test_everything_is_accepted_from_tau_two_on(K, dtype):
+    """tau >= 2 accepts everything, also a gradient that points exactly against a running sum most of which has cancelled: the
+    sums' rounding puts that cosine below -1 in about every other case, and Eq. 4 takes it as -1."""
+    ws = gaf.new_workspace(16, 1 << 20, gaf.GAF_F32)
+    torch.manual_seed(17)
+    tdtype = torch.float32 if dtype == "f32" else torch.bfloat16
+    for D in (4_001, 60_007):
+        for trial in range(24):
+            a = torch.randn(D, device="cuda").to(tdtype)
+            b = (-a.float() + 4e-3 * torch.randn(D, device="cuda")).to(tdtype)
+            c = ((a.double() + b.double()) * -100.0).to(tdtype)
+            grads = [a, b, c] + [torch.randn(D, device="cuda").to(tdtype) for _ in range(K - 3)]
+            for tau in (2.0, 2.5):
+                for schedule in (gaf.GAF_SCHED_STEPWISE, gaf.GAF_SCHED_GRAM, gaf.GAF_SCHED_AUTO):
+                    _, mask, _, count = gaf.gaf_filter_accumulate(grads, tau, ws, schedule=schedule)
+                    assert mask.tolist() == [1] * K and int(count) == K, (D, trial, tau, schedule)
+                if K <= 8:
+                    got = gaf.gaf_filter_accumulate_bucketed(grads, tau, [0, D // 16 * 8, D], ws)
+                    assert bool((got[1] == 1).all()), (D, trial, tau)
+                got = gaf.gaf_filter_accumulate_any_seed(grads, tau, ws)
+                assert bool((got[1] == 1).all()) and int(got[4]) == 0, (D, trial, tau)
