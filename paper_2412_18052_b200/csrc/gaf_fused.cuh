@@ -688,6 +688,8 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
             wait_full(v);
             process(true_type(), true_type(), v % kStages, from, before, div);
             release(v);
+            // the sums are cut where a call that samples cuts them: same bits whatever the calls before it left
+            if (KT == 2 && ONE && !sampling && v < S && v + NG >= S) flush();
         }
     } else {
         // (the last tiles stay in the ring: their mean is written from there)

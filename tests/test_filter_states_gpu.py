@@ -8,6 +8,7 @@ from paper_2412_18052_b200 import workloads
 
 pytestmark = pytest.mark.gpu
 
+DTYPES = ["f32", "bf16"]
 CODE = {"f32": gaf.GAF_F32, "bf16": gaf.GAF_BF16}
 
 
@@ -152,3 +153,31 @@ def test_everything_is_accepted_from_tau_two_on(K, dtype):
                     assert bool((got[1] == 1).all()), (D, trial, tau)
                 got = gaf.gaf_filter_accumulate_any_seed(grads, tau, ws)
                 assert bool((got[1] == 1).all()) and int(got[4]) == 0, (D, trial, tau)
+
+
+def _nearly_equal(K, D, dtype, seed):
+    """Gradients so close to one another that their distances show the last bits of the sums."""
+    torch.manual_seed(seed)
+    x = torch.randn(D, device="cuda")
+    tdtype = torch.float32 if dtype == "f32" else torch.bfloat16
+    return [(x + (1e-5 if dtype == "f32" else 4e-3) * torch.randn(D, device="cuda")).to(tdtype) for _ in range(K)]
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+def test_two_gradients_same_bits_after_every_history(dtype):
+    """What a call of two gradients gives does not depend on how the calls before it on the workspace ended."""
+    for D in (_predicted_length(2, dtype) // 4 + 12_345, _predicted_length(2, dtype) + 5):
+        ws = gaf.new_workspace(2, D, CODE[dtype])
+        for seed in range(4):
+            grads = _nearly_equal(2, D, dtype, seed)
+            yes, no = grads, [grads[0], -grads[1]]
+            seen = []
+            for history in ((), (yes, yes), (no, no), (yes, no), (no, yes)):
+                gaf.gaf_workspace_init(ws)
+                for h in history:
+                    gaf.gaf_filter_accumulate(h, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM_FUSED)
+                seen.append([t.clone() for t in gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM_FUSED)])
+            seen.append([t.clone() for t in gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM)])
+            for other in seen[1:]:
+                for a, b in zip(seen[0], other):
+                    assert torch.equal(a, b), (D, seed)
