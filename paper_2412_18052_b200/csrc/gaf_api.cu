@@ -535,6 +535,10 @@ int launch_gram_fused_kt(GramFusedArgs &a, const DeviceInfo &di, cudaStream_t st
     return GAF_OK;
 }
 
+// Whether a filter call takes the large tiles of a pair of tile sizes; both forms ask, so that they take the same sums.
+template <typename T, int KT>
+bool long_tiles(int64_t D) { return kTwoTileForms<T, KT> && int64_t(KT) * int64_t(sizeof(T)) * D >= kLongTileBytes; }
+
 template <typename T>
 int launch_gram_fused(GramFusedArgs &a, int K, const DeviceInfo &di, cudaStream_t st) {
     switch (K) {
@@ -542,11 +546,11 @@ int launch_gram_fused(GramFusedArgs &a, int K, const DeviceInfo &di, cudaStream_
         case 3: return launch_gram_fused_kt<T, 3>(a, di, st);
         case 4: return launch_gram_fused_kt<T, 4>(a, di, st);
         case 5:
-            return kTwoTileForms<T, 5> && K * 2 * a.D >= kLongTileBytes ? launch_gram_fused_kt<T, 5, kTwoTileForms<T, 5>>(a, di, st)
-                                                                        : launch_gram_fused_kt<T, 5>(a, di, st);
+            return long_tiles<T, 5>(a.D) ? launch_gram_fused_kt<T, 5, kTwoTileForms<T, 5>>(a, di, st)
+                                         : launch_gram_fused_kt<T, 5>(a, di, st);
         case 6:
-            return kTwoTileForms<T, 6> && K * 2 * a.D >= kLongTileBytes ? launch_gram_fused_kt<T, 6, kTwoTileForms<T, 6>>(a, di, st)
-                                                                        : launch_gram_fused_kt<T, 6>(a, di, st);
+            return long_tiles<T, 6>(a.D) ? launch_gram_fused_kt<T, 6, kTwoTileForms<T, 6>>(a, di, st)
+                                         : launch_gram_fused_kt<T, 6>(a, di, st);
         case 7: return launch_gram_fused_kt<T, 7>(a, di, st);
         case 8: return launch_gram_fused_kt<T, 8>(a, di, st);
         default: return GAF_ERR_UNSUPPORTED;
@@ -555,9 +559,8 @@ int launch_gram_fused(GramFusedArgs &a, int K, const DeviceInfo &di, cudaStream_
 
 // Two-launch form: the same kernel without the wait at its end; masked_mean_kernel behind it.  Also the pairwise
 // distances of up to 8 gradients (no mean, nothing behind it).
-template <typename T, int KT>
+template <typename T, int KT, bool LONG = false>
 int launch_gram_filter_kt(GramFusedArgs &a, const DeviceInfo &di, cudaStream_t st) {
-    constexpr bool LONG = kTwoTileForms<T, KT>;
     if (int rc = filter_plan<T, KT, false, LONG>(di)) return rc;
     const int grid = filter_shape<T, KT, LONG>(a, di, a.pair_dist_out == nullptr);
     a.spin_limit = kFusedSpinLimit;
@@ -574,8 +577,13 @@ int launch_gram_filter(GramFusedArgs &a, int K, const DeviceInfo &di, cudaStream
         case 2: return launch_gram_filter_kt<T, 2>(a, di, st);
         case 3: return launch_gram_filter_kt<T, 3>(a, di, st);
         case 4: return launch_gram_filter_kt<T, 4>(a, di, st);
-        case 5: return launch_gram_filter_kt<T, 5>(a, di, st);
-        case 6: return launch_gram_filter_kt<T, 6>(a, di, st);
+        // (the pairwise distances wait for no prediction: large tiles at every length)
+        case 5:
+            return a.pair_dist_out != nullptr || long_tiles<T, 5>(a.D) ? launch_gram_filter_kt<T, 5, kTwoTileForms<T, 5>>(a, di, st)
+                                                                       : launch_gram_filter_kt<T, 5>(a, di, st);
+        case 6:
+            return a.pair_dist_out != nullptr || long_tiles<T, 6>(a.D) ? launch_gram_filter_kt<T, 6, kTwoTileForms<T, 6>>(a, di, st)
+                                                                       : launch_gram_filter_kt<T, 6>(a, di, st);
         case 7: return launch_gram_filter_kt<T, 7>(a, di, st);
         case 8: return launch_gram_filter_kt<T, 8>(a, di, st);
         default: return GAF_ERR_ARG;

@@ -181,3 +181,17 @@ def test_two_gradients_same_bits_after_every_history(dtype):
             for other in seen[1:]:
                 for a, b in zip(seen[0], other):
                     assert torch.equal(a, b), (D, seed)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("K", [3, 4, 5, 6, 7, 8])
+def test_one_and_two_launches_same_bits(K, dtype):
+    """Both Gram-first forms take the same sums in the same order, short vectors (no prediction) and longer ones."""
+    for D in (_predicted_length(K, dtype) // 8 + 12_345, _predicted_length(K, dtype) + 5):
+        ws = gaf.new_workspace(K, D, CODE[dtype])
+        for seed in range(3):
+            grads = _nearly_equal(K, D, dtype, seed)
+            one = [t.clone() for t in gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM_FUSED)]
+            two = gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM)
+            for a, b in zip(one, two):
+                assert torch.equal(a, b), (D, seed)
