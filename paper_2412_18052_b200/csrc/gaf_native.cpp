@@ -68,11 +68,23 @@ int64_t integer(PyObject *o) {
     return v;
 }
 
-// A list or tuple, kept alive while its items are read.
+// The items of anything that has a length and, where `indexed`, can be indexed (a generator has neither: its items would be
+// used up by one call).  They stay alive as long as this object does.
 struct Sequence {
     PyObject *fast;
     Py_ssize_t n;
-    explicit Sequence(PyObject *o) : fast(PySequence_Fast(o, "expected a sequence")), n(0) {
+    explicit Sequence(PyObject *o, bool indexed = false) : fast(nullptr), n(0) {
+        if (!PyList_Check(o) && !PyTuple_Check(o)) {
+            const Py_ssize_t len = PyObject_Size(o);
+            if (len < 0) throw Failed();
+            if (indexed && len > 0) {
+                PyObject *zero = PyLong_FromLong(0), *item = zero ? PyObject_GetItem(o, zero) : nullptr;
+                Py_XDECREF(zero);
+                if (!item) throw Failed();
+                Py_DECREF(item);
+            }
+        }
+        fast = PySequence_Fast(o, "expected a sequence");
         if (!fast) throw Failed();
         n = PySequence_Fast_GET_SIZE(fast);
     }
@@ -81,14 +93,15 @@ struct Sequence {
     PyObject *operator[](Py_ssize_t i) const { return PySequence_Fast_GET_ITEM(fast, i); }
 };
 
-// The gradients of a call: pointers, length, type, device.
+// The gradients of a call: pointers, length, type, device.  It holds the tensors until the call has been made: a sequence may make
+// them as they are asked for, and memory that is freed before the outputs are allocated becomes the outputs.
 struct Gradients {
+    const Sequence seq;
     std::vector<const void *> ptr;
     int64_t D = 0;
     int dtype = 0;
     at::Device device = at::kCPU;
-    Gradients(PyObject *o, bool must_match) {
-        const Sequence seq(o);
+    Gradients(PyObject *o, bool must_match) : seq(o, true) {
         if (seq.n == 0) fail(PyExc_IndexError, "no gradients");
         ptr.reserve(seq.n);
         const at::Tensor &first = tensor(seq[0]);

@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 from paper_2412_18052_b200 import binding
 from paper_2412_18052_b200.build import build
@@ -124,3 +125,23 @@ def test_binding_fails_loudly_without_library(monkeypatch):
     monkeypatch.setattr(binding, "_LIB_PATH", "/nonexistent/libgaf.so")
     with pytest.raises(RuntimeError, match="no CPU or PyTorch fallback"):
         binding.lib()
+
+
+def test_gradients_must_have_a_length_and_an_order(L):
+    """An iterator of gradients is refused before anything is read from it: the tensors it makes would be gone by the launch."""
+    g = [torch.zeros(64) for _ in range(3)]
+    ws = torch.zeros(16, dtype=torch.uint8)
+    calls = [lambda x: binding.gaf_filter_accumulate(x, 0.9, ws), lambda x: binding.gaf_filter_accumulate_any_seed(x, 0.9, ws),
+             lambda x: binding.gaf_filter_accumulate_bucketed(x, 0.9, [0, 64], ws), lambda x: binding.gaf_pairwise_cosdist(x, ws)]
+    for call in calls:
+        for bad in ((t.clone() for t in g), map(torch.clone, g), iter(g), set(g)):
+            with pytest.raises(TypeError):
+                call(bad)
+        with pytest.raises(KeyError):
+            call({"a": g[0]})
+        with pytest.raises(IndexError):
+            call([])
+    with pytest.raises(TypeError):
+        binding.gaf_filter_accumulate_bucketed(g, 0.9, (o for o in (0, 64)), ws)
+    with pytest.raises(TypeError):
+        binding.gaf_filter_accumulate(g, 0.9, ws, order=(o for o in (0, 1, 2)))

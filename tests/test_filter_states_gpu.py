@@ -195,3 +195,31 @@ def test_one_and_two_launches_same_bits(K, dtype):
             two = gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM)
             for a, b in zip(one, two):
                 assert torch.equal(a, b), (D, seed)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+def test_gradients_made_as_they_are_asked_for(dtype):
+    """A sequence that makes its tensors on request, and the rows of one tensor: the call holds them until it has been launched,
+    so that none of the outputs it allocates lies in their memory."""
+    K, D = 4, 300_000
+    kept = _mix(K, D, "f32", 3, [0.8, 0.7, -0.6, 0.5])
+    tdtype = torch.float32 if dtype == "f32" else torch.bfloat16
+
+    class Made:
+        def __len__(self):
+            return K
+
+        def __getitem__(self, i):
+            if i >= K:
+                raise IndexError
+            return kept[i].clone().to(tdtype)
+
+    grads = [Made()[i] for i in range(K)]
+    ws = gaf.new_workspace(K, D, CODE[dtype])
+    want = [t.clone() for t in gaf.gaf_filter_accumulate(grads, 0.9, ws)]
+    want_pairs = gaf.gaf_pairwise_cosdist(grads, ws)[0].clone()
+    for _ in range(3):
+        for given in (Made(), torch.stack(grads)):
+            for a, b in zip(gaf.gaf_filter_accumulate(given, 0.9, ws), want):
+                assert torch.equal(a, b)
+            assert torch.equal(gaf.gaf_pairwise_cosdist(given, ws)[0], want_pairs)
