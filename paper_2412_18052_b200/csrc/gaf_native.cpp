@@ -13,6 +13,7 @@
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <cstdint>
 #include <vector>
 
 #include "../../include/gaf.h"
@@ -118,20 +119,20 @@ struct Gradients {
     int K() const { return static_cast<int>(ptr.size()); }
 };
 
-// A step order, or null for the identity.
+// A step order for K gradients, or null for the identity.  What is missing from one that is too short, and a number that no int32
+// holds, become -1, which the library refuses; what a longer one has beyond K is not looked at.
 struct Order {
     std::vector<int32_t> v;
-    explicit Order(PyObject *o) {
+    const int32_t *ptr = nullptr;
+    Order(PyObject *o, int K) {
         if (o == Py_None) return;
         const Sequence seq(o);
-        v.reserve(seq.n);
-        for (Py_ssize_t i = 0; i < seq.n; ++i) v.push_back(static_cast<int32_t>(integer(seq[i])));
-    }
-    // (a wrong length is an invalid order)
-    const int32_t *get(int K) {
-        if (v.empty()) return nullptr;
-        if (static_cast<int>(v.size()) < K) v.resize(K, -1);
-        return v.data();
+        v.assign(K, -1);
+        for (Py_ssize_t i = 0; i < seq.n && i < K; ++i) {
+            const int64_t x = integer(seq[i]);
+            if (x >= 0 && x <= INT32_MAX) v[i] = static_cast<int32_t>(x);
+        }
+        ptr = v.data();
     }
 };
 
@@ -201,13 +202,13 @@ PyObject *py_filter_accumulate(PyObject *, PyObject *const *a, Py_ssize_t n) {
         const Gradients g(a[0], true);
         const double tau = number(a[1]);
         const Workspace ws(a[2]);
-        Order order(a[3]);
+        const Order order(a[3], g.K());
         Output macro(a[4], {g.D}, at::kFloat, g.device), mask(a[5], {g.K()}, at::kByte, g.device),
             dist(a[6], {g.K()}, at::kFloat, g.device), count(a[7], {1}, at::kInt, g.device);
         const int schedule = static_cast<int>(integer(a[8]));
         void *const st = stream();
         check(without_gil([&] {
-            return gaf_filter_accumulate(g.ptr.data(), g.K(), g.D, g.dtype, tau, order.get(g.K()), as<float>(macro), as<uint8_t>(mask),
+            return gaf_filter_accumulate(g.ptr.data(), g.K(), g.D, g.dtype, tau, order.ptr, as<float>(macro), as<uint8_t>(mask),
                                          as<float>(dist), as<int32_t>(count), ws.ptr, ws.bytes, schedule, st);
         }), "gaf_filter_accumulate");
         return tuple_of(macro, mask, dist, count);
@@ -244,12 +245,12 @@ PyObject *py_filter_accumulate_bucketed(PyObject *, PyObject *const *a, Py_ssize
         const int64_t S = static_cast<int64_t>(offsets.size()) - 1;
         if (S < 0) fail(PyExc_ValueError, "no bucket offsets");
         const Workspace ws(a[3]);
-        Order order(a[4]);
+        const Order order(a[4], g.K());
         Output macro(a[5], {g.D}, at::kFloat, g.device), mask(Py_None, {S, g.K()}, at::kByte, g.device),
             dist(Py_None, {S, g.K()}, at::kFloat, g.device), count(Py_None, {S}, at::kInt, g.device);
         void *const st = stream();
         check(without_gil([&] {
-            return gaf_filter_accumulate_bucketed(g.ptr.data(), g.K(), g.D, g.dtype, tau, order.get(g.K()), static_cast<int>(S),
+            return gaf_filter_accumulate_bucketed(g.ptr.data(), g.K(), g.D, g.dtype, tau, order.ptr, static_cast<int>(S),
                                                   offsets.data(), as<float>(macro), as<uint8_t>(mask), as<float>(dist),
                                                   as<int32_t>(count), ws.ptr, ws.bytes, st);
         }), "gaf_filter_accumulate_bucketed");

@@ -1,5 +1,6 @@
 """The Gram-first forms of the filter from every state a workspace can be in, and decisions and sums that must not depend on the
 form or on what ran before: GPU tests, results against the stepwise schedule bit for bit."""
+import numpy as np
 import pytest
 import torch
 
@@ -223,3 +224,19 @@ def test_gradients_made_as_they_are_asked_for(dtype):
             for a, b in zip(gaf.gaf_filter_accumulate(given, 0.9, ws), want):
                 assert torch.equal(a, b)
             assert torch.equal(gaf.gaf_pairwise_cosdist(given, ws)[0], want_pairs)
+
+
+def test_orders_that_are_no_permutation_are_refused():
+    K, D = 3, 1000
+    grads = _mix(K, D, "f32", 3, [0.8, 0.7, -0.6])
+    ws = gaf.new_workspace(K, D, gaf.GAF_F32)
+    want = [t.clone() for t in gaf.gaf_filter_accumulate(grads, 0.9, ws, order=[2, 0, 1])]
+    for bad in ([], [0], [0, 1], [0, 1, 3], [0, 1, -1], [0, 1, 2 + 2 ** 32], [2 ** 31, 1, 2], [0, 1, 1]):
+        for call in (lambda: gaf.gaf_filter_accumulate(grads, 0.9, ws, order=bad),
+                     lambda: gaf.gaf_filter_accumulate_bucketed(grads, 0.9, [0, D], ws, order=bad)):
+            with pytest.raises(gaf.GafError) as e:
+                call()
+            assert e.value.code == 1, bad
+    for good in ([2, 0, 1], (2, 0, 1), np.array([2, 0, 1]), torch.tensor([2, 0, 1]), [2, 0, 1, 7]):
+        for a, b in zip(gaf.gaf_filter_accumulate(grads, 0.9, ws, order=good), want):
+            assert torch.equal(a, b)
