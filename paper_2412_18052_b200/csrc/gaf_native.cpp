@@ -51,8 +51,11 @@ int dtype_code(const at::Tensor &t) {
 void *stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
 double number(PyObject *o) {
-    const double v = PyFloat_AsDouble(o);
-    if (v == -1.0 && PyErr_Occurred()) throw Failed();
+    if (PyFloat_Check(o)) return PyFloat_AS_DOUBLE(o);
+    PyObject *f = PyNumber_Float(o);    // what float() takes: numpy and torch scalars, texts
+    if (!f) throw Failed();
+    const double v = PyFloat_AS_DOUBLE(f);
+    Py_DECREF(f);
     return v;
 }
 int64_t integer(PyObject *o) {

@@ -240,3 +240,15 @@ def test_orders_that_are_no_permutation_are_refused():
     for good in ([2, 0, 1], (2, 0, 1), np.array([2, 0, 1]), torch.tensor([2, 0, 1]), [2, 0, 1, 7]):
         for a, b in zip(gaf.gaf_filter_accumulate(grads, 0.9, ws, order=good), want):
             assert torch.equal(a, b)
+
+
+def test_thresholds_that_float_takes():
+    grads = _mix(3, 1000, "f32", 3, [0.8, 0.7, -0.6])
+    ws = gaf.new_workspace(3, 1000, gaf.GAF_F32)
+    want = [t.clone() for t in gaf.gaf_filter_accumulate(grads, 0.5, ws)]
+    for tau in (np.float32(0.5), torch.tensor(0.5), "0.5"):
+        for a, b in zip(gaf.gaf_filter_accumulate(grads, tau, ws), want):
+            assert torch.equal(a, b)
+    for bad in ("half", None, [0.5]):
+        with pytest.raises((TypeError, ValueError)):
+            gaf.gaf_filter_accumulate(grads, bad, ws)
