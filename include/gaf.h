@@ -382,18 +382,22 @@ int gaf_last_gram_loader(void);
 
 /*
  * Test hook for the bounded waits inside the kernels (failure detection without a faulted GPU).
- * Two kernels wait on something another part of the same launch produces: the one-launch
- * Gram-first schedule (its CTAs poll one word for the decisions) and the tensor-core Gram
- * pipeline (mbarrier waits between loaders, MMA issuer and epilogue).  Every such wait gives up
- * after a fixed number of attempts -- seconds in normal use, never reached -- raises
- * GAF_STATUS_TIMEOUT and lets the kernel return in an orderly way (copies in flight are awaited,
- * tensor memory is freed).  This call lets a test see that path run, for the following launches of
- * the calling thread:
+ * Kernels that wait on something another part of the same launch produces: the one-pass
+ * kernel of the Gram-first schedules (its warps wait for tiles, its CTAs for the predicted
+ * pattern and, in the one-launch form, for the decision) and the tensor-core Gram pipeline
+ * (mbarrier waits between loaders, MMA issuer and epilogue).  Every such wait gives up after a
+ * fixed number of attempts -- seconds in normal use, never reached -- raises GAF_STATUS_TIMEOUT
+ * and lets the kernel return in an orderly way (copies in flight are awaited, tensor memory is
+ * freed, no tile is touched whose copy was not seen to land).  A prediction that does not come
+ * is no failure: the call goes on without.  This call lets a test see those paths run, for the
+ * following launches of the calling thread:
  *   wait_limit   attempts before a wait gives up; 0 restores the built-in limits
- *   withhold     non-zero: the awaited signal is never given (the deciding CTA does not publish the
- *                decision word; the first tile's barrier expects one arrival more than will come),
- *                so that every wait runs out.  Nothing traps and nothing waits without a limit.
- * The outputs of a call made with `withhold` set are not valid; the workspace stays usable: the next
+ *   withhold     bits: 1 the awaited signal is never given (no CTA is shown sums or patterns; the
+ *                first tile's barrier of the tensor-core pipeline expects one arrival more than
+ *                will come); 2 only the prediction is never given; 4 the one-pass kernel copies
+ *                no tile, 8 none from the second lap of its ring on.  Nothing traps and nothing
+ *                waits without a limit.
+ * The outputs of a call made with bit 1, 4 or 8 set are not valid; the workspace stays usable: the next
  * ordinary call on it is correct.  Always returns GAF_OK.  Off by default; not for production use.
  */
 int gaf_test_set_wait_fault(unsigned int wait_limit, int withhold);

@@ -274,7 +274,7 @@ def gaf_last_gram_loader() -> int:
     return lib().gaf_last_gram_loader()
 
 
-def gaf_test_set_wait_fault(wait_limit: int, withhold: bool) -> None:
-    """Test hook: poll limit of the kernels' bounded waits and whether the awaited signal is withheld,
-    for the following launches of this thread.  ``(0, False)`` restores normal operation."""
-    _check(lib().gaf_test_set_wait_fault(int(wait_limit), 1 if withhold else 0), "gaf_test_set_wait_fault")
+def gaf_test_set_wait_fault(wait_limit: int, withhold: int) -> None:
+    """Test hook: poll limit of the kernels' bounded waits and what is withheld from them (the bits of gaf.h; True: every
+    awaited signal), for the following launches of this thread.  ``(0, False)`` restores normal operation."""
+    _check(lib().gaf_test_set_wait_fault(int(wait_limit), int(withhold)), "gaf_test_set_wait_fault")

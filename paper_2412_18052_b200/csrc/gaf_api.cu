@@ -341,7 +341,7 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
                 return rc;
         }
         t.spin_limit = g_test_wait_limit ? g_test_wait_limit : kTcSpinLimit;
-        t.test_extra_arrival = g_test_withhold;
+        t.test_extra_arrival = g_test_withhold & 1;
         // (a programmatic dependent of whatever precedes it on the stream: barriers and tensor memory are set up
         // while that grid winds down, and the kernel waits for it before it touches global memory)
         const cudaError_t err = launch_dependent_smem(kernel, a.slices, tc_threads(t.Kp == 64, tma), size_t(dyn), st,
@@ -500,6 +500,7 @@ int launch_gram_fused_kt(GramFusedArgs &a, const DeviceInfo &di, cudaStream_t st
     auto kernel = gram_filter_kernel<T, KT, true, LONG>;
     const int grid = filter_shape<T, KT, LONG>(a, di, true);
     a.spin_limit = g_test_wait_limit ? g_test_wait_limit : kFusedSpinLimit;
+    a.copy_limit = g_test_wait_limit ? g_test_wait_limit : kFusedCopyLimit;
     a.test_withhold = g_test_withhold;
     a.tag = g_fused_tag.fetch_add(1, std::memory_order_relaxed);
     // The grid is no larger than what the device holds at once (occupancy above), so all its CTAs become
@@ -564,7 +565,8 @@ int launch_gram_filter_kt(GramFusedArgs &a, const DeviceInfo &di, cudaStream_t s
     if (int rc = filter_plan<T, KT, false, LONG>(di)) return rc;
     const int grid = filter_shape<T, KT, LONG>(a, di, a.pair_dist_out == nullptr);
     a.spin_limit = kFusedSpinLimit;
-    a.test_withhold = 0;
+    a.copy_limit = g_test_wait_limit ? g_test_wait_limit : kFusedCopyLimit;
+    a.test_withhold = g_test_withhold & ~kWithholdAll;      // (this form waits for no decision)
     const cudaError_t err = launch_dependent_smem(gram_filter_kernel<T, KT, false, LONG>, grid, kFilterThreads,
                                                   size_t(FilterTile<T, KT, LONG>::kStages * FilterTile<T, KT, LONG>::kBytes), st, a);
     ++g_launches;
@@ -774,7 +776,7 @@ int gaf_last_gram_loader(void) { return g_gram_loader; }
 
 int gaf_test_set_wait_fault(unsigned int wait_limit, int withhold) {
     g_test_wait_limit = wait_limit;
-    g_test_withhold = withhold ? 1 : 0;
+    g_test_withhold = withhold;
     return GAF_OK;
 }
 

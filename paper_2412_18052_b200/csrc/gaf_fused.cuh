@@ -59,6 +59,9 @@ constexpr unsigned int kFusedSpinLimit = 1u << 22;   // polls of an L2 round tri
 constexpr unsigned int kFusedSampleLimit = 64;       // two-launch form: polls for the prediction, some tens of microseconds
 constexpr unsigned int kFusedCopyLimit = 1u << 19;   // attempts of up to 2 us at a ring barrier
 
+// Test hook: no CTA is shown sums or patterns; none of the sample; no tile is copied; none from the second lap of the ring on.
+constexpr int kWithholdAll = 1, kWithholdSample = 2, kWithholdTiles = 4, kWithholdLaterTiles = 8;
+
 // Consumer warps work in groups; a tile belongs to one group, the groups take the tiles in turn.  One more warp
 // produces.  15 warps of at most 128 registers.
 constexpr int kFilterGroups = 2;
@@ -113,8 +116,8 @@ struct GramFusedArgs {
     float *pair_dist_out;                   // pairwise mode: K x K distances instead of the walk and the mean
     double *pair_gram_out;                  // pairwise mode: optional copy of the Gram matrix
     unsigned int spin_limit;                // polls a waiting CTA makes before it gives up
-    int test_withhold;                      // test hook, normally 0: the waiting CTAs are never shown the full
-                                            // counter, so that every wait runs out
+    unsigned int copy_limit;                // attempts at a ring barrier before a wait gives up
+    int test_withhold;                      // test hook, normally 0: what is never given or shown (kWithhold...)
 };
 
 // What CTAs tell one another carries the call's tag in every word, so that the reader polls the data itself: one
@@ -340,7 +343,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         const uint64_t again = ONE && S == 0 ? l2_policy_evict_last() : once;
         auto fill = [&](int v, const void *const *rows, int n_rows) {
             const int s = it % kStages;
-            if (it >= kStages && !tc_mbar_wait(&empty[s], (uint32_t)((it / kStages - 1) & 1), &abort_flag, kFusedCopyLimit))
+            if (it >= kStages && !tc_mbar_wait(&empty[s], (uint32_t)((it / kStages - 1) & 1), &abort_flag, a.copy_limit))
                 return false;
             const int r = round_of_visit(v, S, seg, phase);
             const int64_t e0 = ((int64_t)r * gridDim.x + blockIdx.x) * te, left = Dv - e0;
@@ -359,15 +362,18 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
             return true;
         };
         if (lane == 0)
-            for (int v = 0; v < rounds; ++v)
+            for (int v = 0; v < rounds; ++v) {
+                if ((a.test_withhold & kWithholdTiles) || ((a.test_withhold & kWithholdLaterTiles) && v == kStages)) break;
                 if (!fill(v, a.g, KT)) break;
+            }
         __syncwarp();
         __syncthreads();                    // the consumers have decided whether there is a second pass
-        if (ONE && lane == 0)
+        if (ONE && lane == 0 && !abort_flag)
             for (int v = sh_again - 1; v >= 0; --v)
                 if (!fill(v, reinterpret_cast<const void *const *>(list), n_list)) break;
-        // after a wait that gave up: the copies in flight must land before the CTA leaves its shared memory
-        if (lane == 0 && abort_flag)
+        // after a wait that gave up, which may be one of the second pass: the copies in flight must land before the CTA leaves
+        // its shared memory
+        if (lane == 0 && (abort_flag || sh_again > 0))
             for (int i = it > kStages ? it - kStages : 0; i < it; ++i)
                 for (unsigned int spin = 0; spin < kFusedCopyLimit; ++spin)
                     if (tc_mbar_try(&full[i % kStages], (uint32_t)((i / kStages) & 1), 2000u)) break;
@@ -519,12 +525,15 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     };
     using std::false_type;
     using std::true_type;
+    // Whether the tile has landed.  After a wait that ran out the warp touches no tile any more: what stands in stage_e0 and
+    // stage_n may be another tile's, half of it, or nothing yet.
     auto wait_full = [&](int it) {
         const uint32_t parity = (uint32_t)((it / kStages) & 1);
-        if (!tc_mbar_try(&full[it % kStages], parity, 2000u) &&
-            !tc_mbar_wait(&full[it % kStages], parity, &abort_flag, kFusedCopyLimit) && lane == 0)
-            atomicOr(&ctl->status, GAF_STATUS_TIMEOUT);
-        __syncwarp();
+        const bool mine = tc_mbar_try(&full[it % kStages], parity, 2000u) ||
+                          tc_mbar_wait(&full[it % kStages], parity, &abort_flag, a.copy_limit);
+        const bool ok = __all_sync(0xFFFFFFFFu, mine);
+        if (!ok && lane == 0) atomicOr(&ctl->status, GAF_STATUS_TIMEOUT);
+        return ok;
     };
     auto release = [&](int it) {
         __syncwarp();
@@ -601,10 +610,10 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     auto tell = [&](unsigned long long *lines, unsigned int pattern) {
         for (int cta = lane; cta < (int)gridDim.x; cta += 32) st_pattern(lines + cta * 16, pattern, tag);
     };
-    auto hear = [&](const unsigned long long *lines, unsigned int limit) {
+    auto hear = [&](const unsigned long long *lines, unsigned int limit, bool withheld) {
         for (unsigned int polls = 0; polls <= limit; ++polls) {
             unsigned int pattern;
-            if (ld_pattern(lines + blockIdx.x * 16, pattern, tag) && !a.test_withhold) return pattern;
+            if (ld_pattern(lines + blockIdx.x * 16, pattern, tag) && !withheld) return pattern;
         }
         return 0u;
     };
@@ -640,12 +649,10 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     auto next_of_group = [&](int it) { return it + (group + NG - it % NG) % NG; };
     unsigned int pred = hint < 2u ? pack_pattern(hint == 1u ? 1u : 3u, 0) : 0u;
     int v = group;
+    bool good = true;                       // no wait for a tile has run out
     if (sampling) {
         const CountDivider none(1);
-        for (; v < S; v += NG) {
-            wait_full(v);
-            process(true_type(), false_type(), v % kStages, 0u, 0u, none);
-        }
+        for (; v < S && (good = wait_full(v)); v += NG) process(true_type(), false_type(), v % kStages, 0u, 0u, none);
     }
     if (sampling) {
         flush();
@@ -654,12 +661,13 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
             st_word(a.sample_partials + (size_t)tid * kFilterMaxCtas + blockIdx.x,
                     ((unsigned long long)__float_as_uint((float)cta_sum()) << 32) | tag);
         const unsigned int limit = ONE ? a.spin_limit : kFusedSampleLimit;
+        const bool withheld = (a.test_withhold & (kWithholdAll | kWithholdSample)) != 0;
         if (blockIdx.x == 0) {
             const bool known = total(
                 [&](int p, int cta) { return ld_word(a.sample_partials + (size_t)p * kFilterMaxCtas + cta); },
                 [&](unsigned long long w, double &x) {
                     x = (double)__uint_as_float((unsigned int)(w >> 32));
-                    return (unsigned int)w == tag && !a.test_withhold;
+                    return (unsigned int)w == tag && !withheld;
                 }, limit, nullptr);
             const bool any_seed = a.ring.K > 0;
             const double tau = any_seed ? a.ring.tau : a.replay.tau;
@@ -671,7 +679,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
                 tell(a.verdicts, guess);
             }
         } else if (tid == 0) {
-            sh_pred = hear(a.verdicts, limit);
+            sh_pred = hear(a.verdicts, limit, withheld);
         }
         Sync::sync();
         pred = sh_pred;
@@ -680,12 +688,11 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     if (pred) {
         const unsigned int bits = pred & 0xFFu, before = bits & ((1u << ((pred >> 8) & 0xFu)) - 1u), from = bits ^ before;
         const CountDivider div(__popc(bits));
-        for (int w = group; sampling && w < S; w += NG) {
+        for (int w = group; sampling && good && w < S; w += NG) {
             process(false_type(), true_type(), w % kStages, from, before, div);
             release(w);
         }
-        for (; v < rounds; v += NG) {
-            wait_full(v);
+        for (; good && v < rounds && (good = wait_full(v)); v += NG) {
             process(true_type(), true_type(), v % kStages, from, before, div);
             release(v);
             // the sums are cut where a call that samples cuts them: same bits whatever the calls before it left
@@ -694,9 +701,8 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     } else {
         // (the last tiles stay in the ring: their mean is written from there)
         const CountDivider none(1);
-        for (int w = group; sampling && w < S; w += NG) release(w);
-        for (; v < rounds; v += NG) {
-            wait_full(v);
+        for (int w = group; sampling && good && w < S; w += NG) release(w);
+        for (; good && v < rounds && (good = wait_full(v)); v += NG) {
             process(true_type(), false_type(), v % kStages, 0u, 0u, none);
             if (v < rounds - kStages) release(v);
         }
@@ -731,12 +737,12 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         unsigned long long *const lines = a.verdicts + kFilterMaxCtas * 16;
         if (blockIdx.x == 0) {
             if (total([&](int p, int cta) { return ld_tagged(static_cast<const TaggedSum *>(a.partials) + (size_t)p * kFilterMaxCtas + cta); },
-                      [&](const TaggedSum &w, double &x) { return tagged_value(w, x, tag) && !a.test_withhold; },
+                      [&](const TaggedSum &w, double &x) { return tagged_value(w, x, tag) && !(a.test_withhold & kWithholdAll); },
                       a.spin_limit, a.gram)) {
                 decide(lines);
             }
         } else if (tid == 0) {
-            sh_final = hear(lines, a.spin_limit);
+            sh_final = hear(lines, a.spin_limit, (a.test_withhold & kWithholdAll) != 0);
         }
         Sync::sync();
         if (sh_final == 0u) {
@@ -806,13 +812,12 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         if (sh_final == pred) return;
         const CountDivider div(c);
         const unsigned int bits = sh_final & 0xFFu, before = bits & ((1u << ((sh_final >> 8) & 0xFu)) - 1u);
-        for (int w = next_of_group(rounds - kept); w < rounds; w += NG) {
+        for (int w = next_of_group(rounds - kept); good && w < rounds; w += NG) {
             process(false_type(), true_type(), w % kStages, bits ^ before, before, div);
             release(w);
         }
         // the accepted gradients of the other tiles again, compacted to the first rows in the order they are added
-        for (int it = next_of_group(rounds); it < 2 * rounds - kept; it += NG) {
-            wait_full(it);
+        for (int it = next_of_group(rounds); good && it < 2 * rounds - kept && (good = wait_full(it)); it += NG) {
             process(false_type(), true_type(), it % kStages, (1u << c) - 1u, 0u, div);
             release(it);
         }

@@ -252,3 +252,51 @@ def test_thresholds_that_float_takes():
     for bad in ("half", None, [0.5]):
         with pytest.raises((TypeError, ValueError)):
             gaf.gaf_filter_accumulate(grads, bad, ws)
+
+
+class _Fault:
+    """Limit and withheld signals of the bounded waits, for the calls inside."""
+
+    def __init__(self, limit, withhold):
+        self.args = (limit, withhold)
+
+    def __enter__(self):
+        gaf.gaf_test_set_wait_fault(*self.args)
+
+    def __exit__(self, *_):
+        gaf.gaf_test_set_wait_fault(0, 0)
+
+
+@pytest.mark.parametrize("tiles", [4, 8])
+@pytest.mark.parametrize("K,dtype", [(2, "f32"), (4, "f32"), (5, "bf16"), (8, "f32"), (8, "bf16")])
+def test_tiles_that_never_land(K, dtype, tiles):
+    """No copy at all, and none from the second lap of the ring on: every warp gives up, touches no tile that it has not seen land,
+    and the call ends with GAF_STATUS_TIMEOUT.  Nothing outside the outputs is written, and the next call is right."""
+    for D in (_predicted_length(K, dtype) + 5, _predicted_length(K, dtype) // 2 + 64):
+        grads = _mix(K, D, dtype, 5, ([0.8, 0.7, -0.6, 0.5] * 2)[:K])
+        ws = gaf.new_workspace(K, D, CODE[dtype])
+        want = _stepwise(grads, 0.9, ws)
+        guarded = torch.full((D + 8192,), 777.0, device="cuda")
+        for schedule in (gaf.GAF_SCHED_GRAM, gaf.GAF_SCHED_GRAM_FUSED):
+            with _Fault(200, tiles):
+                gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=schedule, macro_out=guarded[4096:4096 + D])
+                status = gaf.gaf_read_status(ws)
+            assert status & gaf.GAF_STATUS_TIMEOUT
+            assert bool((guarded[:4096] == 777.0).all()) and bool((guarded[4096 + D:] == 777.0).all())
+            _same(gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=schedule), want)
+            assert gaf.gaf_read_status(ws) == 0
+
+
+@pytest.mark.parametrize("K,dtype", [(3, "f32"), (6, "bf16"), (8, "f32"), (8, "bf16")])
+def test_prediction_that_does_not_come(K, dtype):
+    """The wait for the predicted pattern runs out and nothing else does: a valid call, written after the decision."""
+    for D in (_predicted_length(K, dtype) + 5, _predicted_length(K, dtype) // 2 + 64):
+        ws = gaf.new_workspace(K, D, CODE[dtype])
+        for rho in ([0.8] * K, ([0.8, 0.7, -0.6, 0.5] * 2)[:K]):
+            grads = _mix(K, D, dtype, 5, rho)
+            want = _stepwise(grads, 0.9, ws)
+            for schedule in (gaf.GAF_SCHED_GRAM, gaf.GAF_SCHED_GRAM_FUSED):
+                with _Fault(1000, 2):
+                    got = gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=schedule)
+                    assert gaf.gaf_read_status(ws) == 0
+                _same(got, want)
