@@ -701,7 +701,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     } else {
         // (the last tiles stay in the ring: their mean is written from there)
         const CountDivider none(1);
-        for (int w = group; sampling && good && w < S; w += NG) release(w);
+        for (int w = group; sampling && good && w < S && w < rounds - kStages; w += NG) release(w);
         for (; good && v < rounds && (good = wait_full(v)); v += NG) {
             process(true_type(), false_type(), v % kStages, 0u, 0u, none);
             if (v < rounds - kStages) release(v);

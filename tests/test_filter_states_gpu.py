@@ -300,3 +300,24 @@ def test_prediction_that_does_not_come(K, dtype):
                     got = gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=schedule)
                     assert gaf.gaf_read_status(ws) == 0
                 _same(got, want)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+def test_two_gradients_prediction_that_does_not_come(dtype):
+    """The shortest vectors that two gradients predict on (one tile more than the ring holds), where a sample's tile is among those
+    that stay in the ring; the pattern of the calls before is no help, since they ended differently."""
+    tile = 1792 if dtype == "f32" else 3584
+    ring = 8 * tile * torch.cuda.get_device_properties(0).multi_processor_count
+    for D in (ring + 1000, ring + ring // 8, ring + ring // 8 + 1000):
+        ws = gaf.new_workspace(2, D, CODE[dtype])
+        yes = _mix(2, D, dtype, 5, [0.8, 0.7])
+        no = [yes[0], -yes[1]]
+        for grads in (yes, no):
+            want = _stepwise(grads, 0.9, ws)
+            for _ in range(3):
+                for h in (yes, no):
+                    gaf.gaf_filter_accumulate(h, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM_FUSED)
+                with _Fault(1000, 2):
+                    got = gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM_FUSED)
+                    assert gaf.gaf_read_status(ws) == 0
+                _same(got, want)
