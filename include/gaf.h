@@ -388,7 +388,7 @@ int gaf_last_gram_loader(void);
  * (mbarrier waits between loaders, MMA issuer and epilogue).  Every such wait gives up after a
  * fixed number of attempts -- seconds in normal use, never reached -- raises GAF_STATUS_TIMEOUT
  * and lets the kernel return in an orderly way (copies in flight are awaited, tensor memory is
- * freed, no tile is touched whose copy was not seen to land).  A prediction that does not come
+ * freed, nothing is read or written outside the kernel's own buffers).  A prediction that does not come
  * is no failure: the call goes on without.  This call lets a test see those paths run, for the
  * following launches of the calling thread:
  *   wait_limit   attempts before a wait gives up; 0 restores the built-in limits

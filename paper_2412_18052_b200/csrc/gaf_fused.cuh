@@ -302,8 +302,11 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     constexpr int CW = kFilterWarps, NG = kFilterGroups, kStages = Tile::kStages, kPitch = Tile::kPitch;
     extern __shared__ __align__(128) unsigned char ring[];      // [stage][gradient][pitch]
     __shared__ uint64_t full[kStages], empty[kStages];
-    __shared__ int64_t stage_e0[kStages];   // first element and length of the tile in a stage (written by the producer)
-    __shared__ int stage_n[kStages];
+    // the tile in a stage, written by the producer: first element, and from kTileShift on its length.  One word, so that a consumer
+    // that stopped waiting for it sees one tile or another (at the start: none), never the start of one and the length of another.
+    __shared__ unsigned long long stage_tile[kStages];
+    constexpr int kTileShift = 48;
+    static_assert(Tile::kElems < 1 << (64 - kTileShift), "a tile's length fits above its first element");
     __shared__ double ssum[CW][NP];         // per-warp sums
     __shared__ double sgram[KT * KT];
     __shared__ int seed_counts[KT];
@@ -318,7 +321,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     Control *ctl = a.replay.ctl;
 
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) { tc_mbar_init(&full[s], 1); tc_mbar_init(&empty[s], kFilterGroupWarps); }
+        for (int s = 0; s < kStages; ++s) { tc_mbar_init(&full[s], 1); tc_mbar_init(&empty[s], kFilterGroupWarps); stage_tile[s] = 0ull; }
         sh_pred = 0u; sh_final = 0u; sh_ok = 1; sh_again = 0; sh_done = 1; abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -336,6 +339,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     if (warp == CW) {
         // ------------------------------------------------------------------ producer ----
         const int te = a.tile_elems, seg = S > 0 ? rounds / S : 1, phase = S > 0 ? (int)blockIdx.x % seg : 0;
+        const int given = a.test_withhold & kWithholdTiles ? 0 : (a.test_withhold & kWithholdLaterTiles ? min(rounds, kStages) : rounds);
         int it = 0;                         // tiles since the start, of both passes
         // (bulk copies whose lines give way first are the better ones while the gradients of a call are of L2's size; see the host)
         const uint64_t once = a.evict_first ? l2_policy_evict_first() : l2_policy_evict_normal();
@@ -348,8 +352,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
             const int r = round_of_visit(v, S, seg, phase);
             const int64_t e0 = ((int64_t)r * gridDim.x + blockIdx.x) * te, left = Dv - e0;
             const int n = left >= te ? te : (left > 0 ? (int)left : 0);
-            stage_e0[s] = e0;
-            stage_n[s] = n;
+            *reinterpret_cast<volatile unsigned long long *>(&stage_tile[s]) = (unsigned long long)e0 | (unsigned long long)n << kTileShift;
             if (n > 0) {
                 const uint32_t bytes = (uint32_t)n * (uint32_t)sizeof(T), dst = tc_smem_u32(ring + (size_t)s * Tile::kBytes);
                 tc_mbar_arrive_expect_tx(&full[s], bytes * (uint32_t)n_rows);
@@ -362,10 +365,8 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
             return true;
         };
         if (lane == 0)
-            for (int v = 0; v < rounds; ++v) {
-                if ((a.test_withhold & kWithholdTiles) || ((a.test_withhold & kWithholdLaterTiles) && v == kStages)) break;
+            for (int v = 0; v < given; ++v)
                 if (!fill(v, a.g, KT)) break;
-            }
         __syncwarp();
         __syncthreads();                    // the consumers have decided whether there is a second pass
         if (ONE && lane == 0 && !abort_flag)
@@ -431,8 +432,9 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         constexpr bool GRAM = decltype(gram_tag)::value, MEAN = decltype(mean_tag)::value;
         constexpr int B = Tile::kBatch;
         const unsigned char *tile = ring + (size_t)s * Tile::kBytes;
-        const int n = stage_n[s];
-        float *out = a.out + stage_e0[s];
+        const unsigned long long where = *reinterpret_cast<volatile unsigned long long *>(&stage_tile[s]);
+        const int n = (int)(where >> kTileShift);
+        float *out = a.out + (where & ((1ull << kTileShift) - 1ull));
         if constexpr (GRAM && Tile::kMma) {
             const int g = lane >> 2, t = lane & 3;
             const unsigned char *row = tile + (g < KT ? g : 0) * kPitch;
@@ -525,15 +527,14 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     };
     using std::false_type;
     using std::true_type;
-    // Whether the tile has landed.  After a wait that ran out the warp touches no tile any more: what stands in stage_e0 and
-    // stage_n may be another tile's, half of it, or nothing yet.
+    // (After a wait that ran out the warp goes on with whatever the stage holds: the call is not valid, but every word that stage_tile
+    // can hold lies inside the output.)
     auto wait_full = [&](int it) {
         const uint32_t parity = (uint32_t)((it / kStages) & 1);
-        const bool mine = tc_mbar_try(&full[it % kStages], parity, 2000u) ||
-                          tc_mbar_wait(&full[it % kStages], parity, &abort_flag, a.copy_limit);
-        const bool ok = __all_sync(0xFFFFFFFFu, mine);
-        if (!ok && lane == 0) atomicOr(&ctl->status, GAF_STATUS_TIMEOUT);
-        return ok;
+        if (!tc_mbar_try(&full[it % kStages], parity, 2000u) &&
+            !tc_mbar_wait(&full[it % kStages], parity, &abort_flag, a.copy_limit) && lane == 0)
+            atomicOr(&ctl->status, GAF_STATUS_TIMEOUT);
+        __syncwarp();
     };
     auto release = [&](int it) {
         __syncwarp();
@@ -649,10 +650,12 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     auto next_of_group = [&](int it) { return it + (group + NG - it % NG) % NG; };
     unsigned int pred = hint < 2u ? pack_pattern(hint == 1u ? 1u : 3u, 0) : 0u;
     int v = group;
-    bool good = true;                       // no wait for a tile has run out
     if (sampling) {
         const CountDivider none(1);
-        for (; v < S && (good = wait_full(v)); v += NG) process(true_type(), false_type(), v % kStages, 0u, 0u, none);
+        for (; v < S; v += NG) {
+            wait_full(v);
+            process(true_type(), false_type(), v % kStages, 0u, 0u, none);
+        }
     }
     if (sampling) {
         flush();
@@ -688,11 +691,12 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     if (pred) {
         const unsigned int bits = pred & 0xFFu, before = bits & ((1u << ((pred >> 8) & 0xFu)) - 1u), from = bits ^ before;
         const CountDivider div(__popc(bits));
-        for (int w = group; sampling && good && w < S; w += NG) {
+        for (int w = group; sampling && w < S; w += NG) {
             process(false_type(), true_type(), w % kStages, from, before, div);
             release(w);
         }
-        for (; good && v < rounds && (good = wait_full(v)); v += NG) {
+        for (; v < rounds; v += NG) {
+            wait_full(v);
             process(true_type(), true_type(), v % kStages, from, before, div);
             release(v);
             // the sums are cut where a call that samples cuts them: same bits whatever the calls before it left
@@ -701,8 +705,9 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     } else {
         // (the last tiles stay in the ring: their mean is written from there)
         const CountDivider none(1);
-        for (int w = group; sampling && good && w < S && w < rounds - kStages; w += NG) release(w);
-        for (; good && v < rounds && (good = wait_full(v)); v += NG) {
+        for (int w = group; sampling && w < S && w < rounds - kStages; w += NG) release(w);
+        for (; v < rounds; v += NG) {
+            wait_full(v);
             process(true_type(), false_type(), v % kStages, 0u, 0u, none);
             if (v < rounds - kStages) release(v);
         }
@@ -812,12 +817,13 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         if (sh_final == pred) return;
         const CountDivider div(c);
         const unsigned int bits = sh_final & 0xFFu, before = bits & ((1u << ((sh_final >> 8) & 0xFu)) - 1u);
-        for (int w = next_of_group(rounds - kept); good && w < rounds; w += NG) {
+        for (int w = next_of_group(rounds - kept); w < rounds; w += NG) {
             process(false_type(), true_type(), w % kStages, bits ^ before, before, div);
             release(w);
         }
         // the accepted gradients of the other tiles again, compacted to the first rows in the order they are added
-        for (int it = next_of_group(rounds); good && it < 2 * rounds - kept && (good = wait_full(it)); it += NG) {
+        for (int it = next_of_group(rounds); it < 2 * rounds - kept; it += NG) {
+            wait_full(it);
             process(false_type(), true_type(), it % kStages, (1u << c) - 1u, 0u, div);
             release(it);
         }
