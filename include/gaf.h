@@ -394,7 +394,7 @@ int gaf_last_gram_loader(void);
  *   wait_limit   attempts before a wait gives up; 0 restores the built-in limits
  *   withhold     bits: 1 the awaited signal is never given (no CTA is shown sums or patterns; the
  *                first tile's barrier of the tensor-core pipeline expects one arrival more than
- *                will come); 2 only the prediction is never given; 4 the one-pass kernel copies
+ *                will come); 2 only the prediction is never given (given up after some polls); 4 the one-pass kernel copies
  *                no tile, 8 none from the second lap of its ring on.  Nothing traps and nothing
  *                waits without a limit.
  * The outputs of a call made with bit 1, 4 or 8 set are not valid; the workspace stays usable: the next

@@ -663,7 +663,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         if (tid < NP)
             st_word(a.sample_partials + (size_t)tid * kFilterMaxCtas + blockIdx.x,
                     ((unsigned long long)__float_as_uint((float)cta_sum()) << 32) | tag);
-        const unsigned int limit = ONE ? a.spin_limit : kFusedSampleLimit;
+        const unsigned int limit = ONE && !(a.test_withhold & kWithholdSample) ? a.spin_limit : kFusedSampleLimit;
         const bool withheld = (a.test_withhold & (kWithholdAll | kWithholdSample)) != 0;
         if (blockIdx.x == 0) {
             const bool known = total(

@@ -296,7 +296,7 @@ def test_prediction_that_does_not_come(K, dtype):
             grads = _mix(K, D, dtype, 5, rho)
             want = _stepwise(grads, 0.9, ws)
             for schedule in (gaf.GAF_SCHED_GRAM, gaf.GAF_SCHED_GRAM_FUSED):
-                with _Fault(1000, 2):
+                with _Fault(0, 2):
                     got = gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=schedule)
                     assert gaf.gaf_read_status(ws) == 0
                 _same(got, want)
@@ -317,7 +317,7 @@ def test_two_gradients_prediction_that_does_not_come(dtype):
             for _ in range(3):
                 for h in (yes, no):
                     gaf.gaf_filter_accumulate(h, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM_FUSED)
-                with _Fault(1000, 2):
+                with _Fault(0, 2):
                     got = gaf.gaf_filter_accumulate(grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM_FUSED)
                     assert gaf.gaf_read_status(ws) == 0
                 _same(got, want)
