@@ -92,7 +92,6 @@ struct PerDevice {
     PerDevice() { for (auto &r : ready) r.store(0, std::memory_order_relaxed); }
 };
 struct DynSmemPlan { int dyn = 0; };    // "the dynamic shared memory limit of this kernel has been raised"
-struct OccPlan { int occ = 1; };
 
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline size_t elem_bytes(int dtype) { return dtype == GAF_F32 ? 4 : 2; }
@@ -163,8 +162,8 @@ bool use_small_gram(int K, int64_t D, int dtype) {
 }
 
 // Layout after the per-CTA triples: Gram partials [tile pair][slice][64] doubles, the
-// Gram matrix by original index, the Gram matrix by processing step, a K x K float
-// scratch for distances nobody asked for.
+// Gram matrix by original index, room for another, a K x K float scratch for
+// distances nobody asked for.
 size_t gram_partials_bytes(int K) {
     const int tiles = (K + kGramTile - 1) / kGramTile;
     const size_t pairs = size_t(tiles) * (tiles + 1) / 2;
@@ -283,7 +282,7 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
         // 9..16 bfloat16 gradients: warp-level MMAs fed straight from the global loads, two CTAs per SM
         GramWideArgs w{};
         for (int i = 0; i < K; ++i) w.g[i] = grads[i];
-        w.K = K; w.D = D; w.keep_from = D; w.partials = a.partials; w.ctl = a.ctl;
+        w.K = K; w.D = D; w.partials = a.partials; w.ctl = a.ctl;
         const int64_t per_cta = int64_t(kWideThreads / 32) * kMmaTileElems;      // elements per trip of one CTA
         int64_t grid = int64_t(sms) * 2;
         if (grid > kGramMaxSlices) grid = kGramMaxSlices;
@@ -363,8 +362,7 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
         const int threads = wpp == 0 ? 32 * kPanelMaxWarps : 32 * pa.pairs_per_cta * wpp;
         const int row_bytes = 16 << shift;
         const int dyn = kPanelStages * a.tiles * 8 * row_bytes;
-        // (bfloat16 comes here with a single gradient only: 2 to 8 take the register-tiled kernel, up to 64
-        // the tensor cores)
+        // (bfloat16 comes here with a single gradient only: 2 to 8 take the one-pass kernel, up to 64 the tensor cores)
         void (*kernel)(GramPanelArgs) = nullptr;
         if (dtype == GAF_F32)
             kernel = shift == 7 ? gram_panel_kernel<float, 7, 4>
@@ -614,8 +612,6 @@ int launch_gram_first(const void *const *g, int K, int64_t D, int dtype, double 
     ReplayArgs r{};
     r.K = K; r.tau = tau; r.mask_out = mask_out; r.dist_out = dist_out; r.count_out = count_out; r.ctl = ctl;
     for (int t = 0; t < K; ++t) r.idx[t] = ord[t];
-    double *gram_by_step = reinterpret_cast<double *>(base + kExtraOffset + gram_partials_bytes(K) +
-                                                      gram_matrix_bytes(K));
     if (one_launch && (K < 2 || K > kGsMaxK)) return GAF_ERR_UNSUPPORTED;
     const bool filter_pass = K >= 2 && K <= kGsMaxK;
     if (filter_pass) {
@@ -625,7 +621,6 @@ int launch_gram_first(const void *const *g, int K, int64_t D, int dtype, double 
         f.partials = base + kExtraOffset;
         f.sample_partials = reinterpret_cast<unsigned long long *>(base + kExtraOffset + kFilterSumsBytes);
         f.verdicts = reinterpret_cast<unsigned long long *>(base + kPartialsOffset);
-        f.gram = gram_by_step;
         f.replay = r;
         f.ring = ring;
         if (one_launch) return launch_gram_fused<T>(f, K, di, st);
@@ -1162,7 +1157,6 @@ int gaf_pairwise_cosdist(const void *const *grads, int K, int64_t D, int dtype, 
         for (int i = 0; i < K; ++i) a.g[i] = grads[i];
         a.D = D;
         a.partials = base + kExtraOffset;
-        a.gram = reinterpret_cast<double *>(base + kExtraOffset + gram_partials_bytes(K));
         a.replay.ctl = reinterpret_cast<Control *>(base);
         a.pair_dist_out = dist_out;
         a.pair_gram_out = gram_out;

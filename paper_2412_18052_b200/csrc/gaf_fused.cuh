@@ -109,7 +109,6 @@ struct GramFusedArgs {
     unsigned long long *sample_partials;    // [pair][kFilterMaxCtas]: binary32 sum and tag
     unsigned long long *verdicts;           // [2][kFilterMaxCtas][16]: a line per CTA for the predicted and one for the decided pattern
     unsigned int tag;                       // ONE: a number no other launch has
-    double *gram;                           // [K][K]
     float *out;                             // D floats
     ReplayArgs replay;                      // used when ring.K == 0
     RingArgs ring;                          // any-seed mode when ring.K > 0
@@ -557,7 +556,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
     // `value(raw, x)` returns whether it is there; every warp polls its own at most `limit` times.  All of a warp's
     // loads are issued before any is looked at: this is a wait for L2 that every CTA shares (one pair after the other, and one
     // load after the other, 8 bf16 gradients of 5 M took 35.0 us, now 32.2; 8 fp32 of 16 M 109.6, now 105.5).
-    auto total = [&](auto load, auto value, unsigned int limit, double *gram_out) {
+    auto total = [&](auto load, auto value, unsigned int limit) {
         constexpr int R = (kFilterMaxCtas + 31) / 32, M = (NP + CW - 1) / CW;
         double part[M][R];
         bool all = false;
@@ -600,7 +599,6 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
                     pair_at(warp + m * CW, i, j);
                     sgram[i * KT + j] = s[m];
                     sgram[j * KT + i] = s[m];
-                    if (gram_out) { gram_out[i * KT + j] = s[m]; gram_out[j * KT + i] = s[m]; }
                 }
         }
         Sync::sync();
@@ -671,7 +669,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
                 [&](unsigned long long w, double &x) {
                     x = (double)__uint_as_float((unsigned int)(w >> 32));
                     return (unsigned int)w == tag && !withheld;
-                }, limit, nullptr);
+                }, limit);
             const bool any_seed = a.ring.K > 0;
             const double tau = any_seed ? a.ring.tau : a.replay.tau;
             const int seed = known && any_seed ? best_seed<1, Sync>(sgram, KT, tau, seed_counts) : 0;
@@ -753,7 +751,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         if (blockIdx.x == 0) {
             if (total([&](int p, int cta) { return ld_tagged(static_cast<const TaggedSum *>(a.partials) + (size_t)p * kFilterMaxCtas + cta); },
                       [&](const TaggedSum &w, double &x) { return tagged_value(w, x, tag) && !(a.test_withhold & kWithholdAll); },
-                      a.spin_limit, a.gram)) {
+                      a.spin_limit)) {
                 decide(lines);
             }
         } else if (tid == 0) {
@@ -773,7 +771,7 @@ gram_filter_kernel(const __grid_constant__ GramFusedArgs a) {
         if (tid == 0) ctl->two_launch_calls = tag;
         const unsigned int share = a.pair_dist_out == nullptr && tid < (int)gridDim.x ? (unsigned int)__ldcg(a.verdicts + tid * 16 + 8) : 0u;
         total([&](int p, int cta) { return __ldcg(static_cast<const double *>(a.partials) + (size_t)p * kFilterMaxCtas + cta); },
-              [](double w, double &x) { x = w; return true; }, 0u, a.gram);
+              [](double w, double &x) { x = w; return true; }, 0u);
         if (a.pair_dist_out != nullptr) {
             // pairwise mode: Eq. 4 for every pair
             if (tid < KT * KT) {

@@ -51,7 +51,6 @@ struct GramWideArgs {
     const void *g[16];
     int K;
     int64_t D;
-    int64_t keep_from;
     double *partials;           // [tile pair][slice][64]
     Control *ctl;
     int run;                    // tiles per warp a CTA takes in a row (even)
@@ -85,7 +84,7 @@ __global__ void __launch_bounds__(kWideThreads, 2) gram_mma_wide_kernel(const __
         have[m] = g + 8 * m < a.K;
         rowp[m] = static_cast<const unsigned short *>(a.g[have[m] ? g + 8 * m : 0]);
     }
-    const uint64_t pol_first = l2_policy_evict_first(), pol_last = l2_policy_evict_last();
+    const uint64_t pol = l2_policy_evict_first();
     const int64_t n_tiles = a.D / kMmaTileElems;
     float c[NT][4];
     double d[NT][4];
@@ -103,7 +102,6 @@ __global__ void __launch_bounds__(kWideThreads, 2) gram_mma_wide_kernel(const __
             if (tile >= n_tiles) break;
             // one tile of 64 elements: two chunks of 32, all 2 NB loads issued before the first MMA
             const int64_t e0 = tile * kMmaTileElems + t * 8;
-            const uint64_t pol = (e0 >= a.keep_from) ? pol_last : pol_first;
             uint4 r[2][NB];
 #pragma unroll
             for (int h = 0; h < 2; ++h)
