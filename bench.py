@@ -152,7 +152,9 @@ def ncu_traffic(cfg, sched_used, masks, D, n_sets, steps, which="steady"):
     entry = NCU_TRAFFIC.get((cfg, sched_used))
     if not entry or kernel_sources_hash(entry["sources"]) != entry["sha256"]:
         return None
-    table = entry.get(which) or entry["steady"]
+    table = entry.get(which)
+    if not table:                       # no such capture on record
+        return None
     per_set = []
     for m in masks:
         c = sum(int(x) for x in m)

@@ -719,19 +719,26 @@ def test_many_gradients_mean_of_short_vectors(ws, K, dtype):
     mean bit for bit against the stepwise schedule (the same additions in the same order)."""
     n = 4 if dtype == "f32" else 8
     limit = torch.cuda.get_device_properties(0).multi_processor_count * 8 * 128 * n
+    compared = 0
     for D in (3, 128 * n - 1, 32_768 + n + 1, limit, limit + 1):
         w = _mix(K, D, dtype, seed=K + D, rho=([0.8] + [0.7, -0.6, 0.5, 0.0, 0.6, -0.2, 0.4] * 9)[:K])
         for tau in (0.9, 2.0):
             plain = [t.clone() for t in gaf.gaf_filter_accumulate(w.grads, tau, ws, schedule=gaf.GAF_SCHED_STEPWISE)]
             got = gaf.gaf_filter_accumulate(w.grads, tau, ws, schedule=gaf.GAF_SCHED_GRAM)
-            if torch.equal(got[1], plain[1]):                        # (masks may differ on a tie only)
+            # (masks may differ on a tie only, and after accepted gradients have cancelled: three elements at tau = 2)
+            tie = bool(((plain[2] - tau).abs() < 1e-5).any()) or gaf.gaf_read_status(ws) & gaf.GAF_STATUS_ILL_CONDITIONED
+            assert torch.equal(got[1], plain[1]) or tie, (K, D, tau)
+            if torch.equal(got[1], plain[1]):
                 assert torch.equal(got[0], plain[0]), (K, D, tau)
+            if D > 1000:
+                compared += torch.equal(got[1], plain[1])
         check_filter(w.grads, 0.9, ws, schedule=gaf.GAF_SCHED_GRAM)
         if D < limit:
             check_any_seed(w.grads, 0.9, ws)
         if K > 32 and D == limit:                                    # the library's own choice for long vectors
             check_filter(w.grads, 0.9, ws)
             assert gaf.gaf_last_schedule() == gaf.GAF_SCHED_GRAM
+    assert compared >= 4                                             # of six calls longer than a thousand elements
 
 
 @pytest.mark.parametrize("K", [5, 6])
