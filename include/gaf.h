@@ -29,7 +29,8 @@
  *     aligned (else GAF_ERR_ALIGN).  D need not be a multiple of anything; with
  *     D == 0 the element buffers may be NULL.
  *   - dtype: GAF_F32 = IEEE binary32, GAF_BF16 = bfloat16.  Arithmetic on
- *     elements is binary32: products of at most 64 pairs are summed in binary32
+ *     elements is binary32: products of at most 64 pairs (bfloat16: 128, whose
+ *     products are exact) are summed in binary32, and the chains of a warp once more,
  *     before they are widened (on the tensor-core paths that bfloat16 gradients
  *     take from 7 gradients on: binary32 accumulators over at most 512 products);
  *     the Gram sums of up to 4 binary32 gradients are taken in binary64
@@ -82,7 +83,7 @@ enum {
                                    stepwise.
                                    For K <= 8 the one-launch form is taken for K = 2, for binary32
                                    inputs of at most 512 MB in all, and for bfloat16 inputs except 7
-                                   or 8 gradients of more than 1 GB in all (tensor-core Gram then);
+                                   or 8 gradients of more than 1 GB in all (two launches then);
                                    if the device refuses that launch, two launches. */
     GAF_SCHED_STEPWISE = 1,     /* streaming: one launch per step; each launch adds the
                                    gradient accepted at step t to the running sum and, in
@@ -92,20 +93,23 @@ enum {
     GAF_SCHED_GRAM = 2,         /* Gram-first: every gradient is read once to build the
                                    K x K Gram matrix, the K-1 decisions are taken on it (dot
                                    products are bilinear), then the accepted gradients are
-                                   read once more to write g/c.  The distances agree with
-                                   the stepwise schedule to rounding.  Two launches. */
+                                   read once more to write g/c; with K <= 8 g/c is written in
+                                   the first pass already, under a predicted accept pattern
+                                   (below), and the second is left out when that proved right.
+                                   The distances agree with the stepwise schedule to rounding.
+                                   Two launches (K <= 8), else three. */
     GAF_SCHED_GRAM_FUSED = 3    /* Gram-first as ONE launch (K <= 8) of a grid sized to what the device
-                                   holds at once: the same two passes, every CTA taking the decisions
-                                   itself from the partial sums all CTAs left in the workspace, so that
-                                   part of what the first pass read (shared memory, L2) need not cross
-                                   HBM again.  Identical outputs to GAF_SCHED_GRAM.  GAF_ERR_UNSUPPORTED
+                                   holds at once.  Its first CTA totals the partial sums that all CTAs
+                                   leave in the workspace, takes the decisions and tells the others, which
+                                   write what is still missing of g/c from what shared memory and L2 hold.
+                                   Identical outputs to GAF_SCHED_GRAM.  GAF_ERR_UNSUPPORTED
                                    for K > 8.  Such a call needs the whole device for its CTAs to meet:
                                    calls on one stream are ordered and fine; a second one on ANOTHER
                                    stream while the first stream still has work pending returns
                                    GAF_ERR_UNSUPPORTED (GAF_SCHED_AUTO takes two launches then), and so
                                    does a call on a stream that is being captured into a graph (what
-                                   runs beside the node is decided at replay).  The one
-                                   wait on other CTAs is bounded: GAF_STATUS_TIMEOUT if it ever runs out
+                                   runs beside the node is decided at replay).  The waits on other CTAs
+                                   are bounded: GAF_STATUS_TIMEOUT if one ever runs out
                                    (only when something else, another process say, keeps part of the
                                    device busy for seconds).
                                    Which gradients will be accepted is predicted inside the call from the
@@ -116,7 +120,8 @@ enum {
                                    values never depend on the prediction.  With K = 2, where the result
                                    can only be the mean of both or the seed alone, a call takes the
                                    pattern that the latest two such calls on the workspace both ended
-                                   with, if they did, instead of a sample's.  (GAF_SCHED_GRAM with K <= 8
+                                   with, if they did, instead of a sample's (a new workspace counts as
+                                   one whose calls kept both).  (GAF_SCHED_GRAM with K <= 8
                                    predicts too; its second launch then has nothing to do.)
                                    GAF_SCHED_AUTO takes this form for K = 2 at every length. */
 };
@@ -226,8 +231,7 @@ int gaf_filter_accumulate_repeat(int repeats, int n_sets, const void *const *gra
  * with the largest agreement is kept.  Where the paper leaves it open: agreement
  * is the accepted count c; ties go to the smallest s.  All K walks run on one
  * K x K Gram matrix (dot products are bilinear), so the cost is that of
- * gaf_filter_accumulate with GAF_SCHED_GRAM: every gradient read once, the
- * accepted ones once more.
+ * gaf_filter_accumulate with GAF_SCHED_AUTO.
  *   mask_out, dist_out, count_out, macro_out   as in gaf_filter_accumulate, for
  *               the winning seed (dist[seed] = 0); the accepted gradients are added
  *               in the winning ring order

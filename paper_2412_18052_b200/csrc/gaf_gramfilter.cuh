@@ -8,7 +8,8 @@
 // the K-1 sequential decisions of Algorithm 1 on K^2 scalars in one warp, and
 // then reads only the accepted gradients once more to write g/c (Eq. 5):
 // ((K + c) b + 4) D bytes instead of one pass over the running sum per step, and no
-// grid-wide serialisation per step.  The accepted gradients are added in processing
+// grid-wide serialisation per step.  (Up to 8 gradients gaf_fused.cuh writes g/c in the
+// first pass, under a predicted accept pattern.)  The accepted gradients are added in processing
 // order in binary32, so the macro-gradient is bit-identical to the streaming
 // schedules'; the distances differ from theirs only by rounding (the running sum is
 // never rounded to binary32 here).
@@ -18,8 +19,7 @@
 
 namespace gaf {
 
-constexpr int kGsThreads = 512;
-constexpr int kGsMaxK = 8;                  // gradients the one-pass register-tiled Gram handles
+constexpr int kGsMaxK = 8;                  // gradients the one-pass kernel (gaf_fused.cuh) and the bucketed form handle
 constexpr int kGsFlushEvery = 16;           // iterations between binary64 flushes
 constexpr int kMsThreads = 512;
 constexpr int kMsLongRun = 8;                // chunks per run of the masked-mean pass on long vectors
@@ -206,7 +206,7 @@ template <> struct GsVec<__nv_bfloat16> {
     }
 };
 
-// Accumulator of the register-tiled Gram kernels (K <= 8).
+// Accumulator of the Gram sums of up to 8 gradients on CUDA cores (gaf_fused.cuh, gaf_bucketed.cuh).
 // binary32 inputs, up to 4 gradients: binary64.  A product of two binary32 values is exact in binary64, so
 // the Gram sums are exact up to binary64 rounding and need no periodic flush; binary64 FMAs (half the
 // binary32 rate on this GPU) keep up with HBM here (measured: the same pass time, and a shorter call because
