@@ -16,8 +16,9 @@
 // binary64 in shared memory; at the end the warps of a pair are added in a fixed order and the
 // tile's 64 binary64 partials are written in the [tile pair][slice][64] layout that
 // gram_finish_kernel totals in a fixed order.
-// Shared-memory reads bound this kernel (8 x 8 tiles give 4 multiply-adds per word read), not
-// the FMA pipes.
+// No pipe bounds this kernel (fp32 pipe 40 % busy, 60 % of the issue slots taken, HBM 0.42 to 0.66 of the
+// copy rate with 32 and 16 gradients): twelve warps wait for fixed latencies, for operands read from shared
+// memory in the step that uses them (4 multiply-adds per word read) and for one barrier per panel.
 #pragma once
 
 #include <type_traits>
@@ -70,7 +71,7 @@ template <> struct PanelLane<__nv_bfloat16> {
 
 // 25 to 32 gradients: 10 tile pairs on 12 warps.  Hex digit w = tile pair of warp w: the four diagonal ones (0, 4, 7 and 9: 36
 // multiply-adds against 64) have a warp each, 5 and 6 two, so that the warps of every scheduler (w mod 4) add up to
-// 64 + 32 + 36.  One warp per pair in order left one scheduler 164 of 528 (32 x 3 M: 133 us, now 124).
+// 64 + 32 + 36.  One warp per pair in order left one scheduler 164 of 528 (32 x 3 M: 142 us for all pairs, now 131).
 constexpr unsigned long long kPanelOwners10 = 0x974066558321ull;
 
 // SHIFT: bytes of one gradient in one panel = 16 << SHIFT; WPP: warps that share a tile pair (0: by the table above).  Both
