@@ -541,7 +541,7 @@ def measure_pairwise(torch, gaf, workloads, dev, steps, warmup, nvml, K=None, D=
             "gram_loader": {0: None, 1: "16-byte asynchronous copies", 2: "tensor copies (TMA)"}[loader],
             "kernel": ("gram_tc_kernel" if (not fp32 and 16 < K <= 64) else
                        "gram_mma_wide_kernel" if (not fp32 and 8 < K <= 16) else
-                       "gram_panel_kernel" if K > 8 else "gram_filter_kernel") + " + finishing (whole call)"}
+                       "gram_digits_kernel or gram_panel_kernel" if K > 8 else "gram_filter_kernel") + " + finishing (whole call)"}
 
 
 def measure_cosdist(torch, gaf, workloads, dev, D, steps, nvml, peak, peak_kind):

@@ -12,6 +12,7 @@
 #include "gaf_bucketed.cuh"
 #include "gaf_device.cuh"
 #include "gaf_fused.cuh"
+#include "gaf_gram_digits.cuh"
 #include "gaf_gram_mma.cuh"
 #include "gaf_gram_panel.cuh"
 #include "gaf_gram_tc.cuh"
@@ -151,8 +152,14 @@ int stream_grid(int64_t D, int threads, int sms) {
 // Which Gram kernel.  The 128-row tcgen05 tile pays off from 9 bfloat16 gradients on.  Up to 8 the one-pass
 // kernels for few gradients are faster at every length: with exactly 8, where the 128 x 128 product keeps 1/16 of
 // its work, the warp-level MMA kernel streams 16 GB of inputs at 6.6 TB/s against 5.2 TB/s (measured).
-constexpr int kPanelAutoMaxK = 32;
-constexpr int64_t kPanelAutoMinD = 32768;
+// Binary32 with one gradient, or more than 8: digits on the tensor cores, except for few gradients of short vectors, where the kernel on the
+// CUDA cores starts and ends 2 us sooner (all pairs, panels / digits, us: 16 gradients of 100 k / 400 k / 800 k / 1.2 M / 2.4 M elements 7.7 /
+// 11.4 / 16.9 / 22.0 / 36.9 against 9.3 / 13.3 / 18.5 / 22.3 / 33.9; 24 of 100 k / 300 k / 400 k / 1.2 M 8.9 / 13.9 / 17.5 / 39.6 against
+// 10.9 / 14.6 / 16.8 / 29.0; 32 of 100 k 12.6 against 12.7).
+constexpr int kGramAutoMaxK = 32;
+constexpr int64_t kGramAutoMinD = 32768;
+constexpr int64_t kPanelMaxD16 = int64_t(1) << 20, kPanelMaxD24 = 5 * 65536;
+bool use_panel_gram(int K, int64_t D) { return K <= 16 ? D < kPanelMaxD16 : (K <= 24 && D < kPanelMaxD24); }
 bool use_tensor_gram(int K, int64_t D, int dtype) {
     (void)D;
     return dtype == GAF_BF16 && K > kGsMaxK && K <= kTcMaxK;
@@ -257,6 +264,34 @@ bool stacked_tensor_maps(const void *const *grads, int K, int Kp, int R, int box
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+template <int KP>
+int launch_gram_digits_kp(const GramDigitsArgs &d, int slices, const DeviceInfo &di, cudaStream_t st) {
+    using S = DigitsShape<KP>;
+    static PerDevice<DynSmemPlan> table;
+    if (int rc = plan_once(table.plan[di.dev], table.ready[di.dev], [&](DynSmemPlan &pl) {
+            pl.dyn = S::kDyn;
+            return cudaFuncSetAttribute(gram_digits_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.dyn) == cudaSuccess
+                ? GAF_OK : GAF_ERR_CUDA;
+        }))
+        return rc;
+    const cudaError_t err = launch_dependent_smem(gram_digits_kernel<KP>, slices, S::kThreads, size_t(S::kDyn), st, d);
+    ++g_launches;
+    if (err != cudaSuccess) { cudaGetLastError(); return GAF_ERR_CUDA; }
+    return GAF_OK;
+}
+int launch_gram_digits(const GramDigitsArgs &d, int slices, const DeviceInfo &di, cudaStream_t st) {
+    switch ((d.K + 7) / 8) {
+        case 1: case 2: return launch_gram_digits_kp<16>(d, slices, di, st);
+        case 3: return launch_gram_digits_kp<24>(d, slices, di, st);
+        case 4: return launch_gram_digits_kp<32>(d, slices, di, st);
+        case 5: return launch_gram_digits_kp<40>(d, slices, di, st);
+        case 6: return launch_gram_digits_kp<48>(d, slices, di, st);
+        case 7: return launch_gram_digits_kp<56>(d, slices, di, st);
+        case 8: return launch_gram_digits_kp<64>(d, slices, di, st);
+        default: return GAF_ERR_ARG;
+    }
+}
+
 // Tiled Gram matrix of K gradients (by original index) into the workspace; optional
 // distance matrix.  Two launches.
 // `replay` or `ring` given: Algorithm 1 on the matrix instead.
@@ -278,8 +313,8 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
                                                       2 * gram_matrix_bytes(K));
     a.gram_out = gram_out;
     a.ctl = reinterpret_cast<Control *>(base);
-    if (use_tensor_gram(K, D, dtype) && K <= kWideMaxK) {
-        // 9..16 bfloat16 gradients: warp-level MMAs fed straight from the global loads, two CTAs per SM
+    if (dtype == GAF_BF16 && K <= kWideMaxK) {
+        // 9..16 bfloat16 gradients (or a single one, alone in its block): warp-level MMAs fed straight from the global loads, two CTAs per SM
         GramWideArgs w{};
         for (int i = 0; i < K; ++i) w.g[i] = grads[i];
         w.K = K; w.D = D; w.partials = a.partials; w.ctl = a.ctl;
@@ -347,60 +382,51 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
                                                       t, tmap, tmap_row);
         ++g_launches;
         if (err != cudaSuccess) { cudaGetLastError(); return GAF_ERR_CUDA; }
-    } else {
+    } else if (use_panel_gram(K, D)) {
         // CUDA cores, every gradient read once: one warp per tile pair, panels of D through shared memory
         GramPanelArgs pa{};
-        for (int i = 0; i < K; ++i) pa.g[i] = grads[i];
+        for (int i = 0; i < K; ++i) pa.g[i] = static_cast<const float *>(grads[i]);
         pa.K = K; pa.D = D; pa.tiles = a.tiles; pa.pairs = pairs;
-        const int groups = (pairs + kPanelMaxWarps - 1) / kPanelMaxWarps;
-        pa.pairs_per_cta = (pairs + groups - 1) / groups;
-        // A panel is at most 32 KB: 2 KB of every row up to 16 (padded) rows, 1 KB up to 32, 512 bytes
-        // beyond.  With 3 or 6 tile pairs, 4 or 2 warps share a pair.
-        const int shift = a.tiles <= 2 ? 7 : (a.tiles <= 4 ? 6 : 5);
-        const int wpp = a.tiles <= 2 ? 4 : (a.tiles == 3 ? 2 : (a.tiles == 4 ? 0 : 1));     // 0: 10 pairs on 12 warps
+        // A panel is at most 32 KB: 2 KB of every row up to 16 (padded) rows, 1 KB up to 24.  4 or 2 warps share a tile pair.
+        const int shift = a.tiles <= 2 ? 7 : 6, wpp = a.tiles <= 2 ? 4 : 2;
         pa.partials = a.partials; pa.ctl = a.ctl;
-        const int threads = wpp == 0 ? 32 * kPanelMaxWarps : 32 * pa.pairs_per_cta * wpp;
+        const int threads = 32 * pairs * wpp;
         const int row_bytes = 16 << shift;
         const int dyn = kPanelStages * a.tiles * 8 * row_bytes;
-        // (bfloat16 comes here with a single gradient only: 2 to 8 take the one-pass kernel, up to 64 the tensor cores)
-        void (*kernel)(GramPanelArgs) = nullptr;
-        if (dtype == GAF_F32)
-            kernel = shift == 7 ? gram_panel_kernel<float, 7, 4>
-                   : (shift == 6 ? (wpp == 2 ? gram_panel_kernel<float, 6, 2> : gram_panel_kernel<float, 6, 0>)
-                                 : gram_panel_kernel<float, 5, 1>);
-        else
-            kernel = shift == 7 ? gram_panel_kernel<__nv_bfloat16, 7, 4>
-                   : (shift == 6 ? (wpp == 2 ? gram_panel_kernel<__nv_bfloat16, 6, 2> : gram_panel_kernel<__nv_bfloat16, 6, 0>)
-                                 : gram_panel_kernel<__nv_bfloat16, 5, 1>);
+        void (*kernel)(GramPanelArgs) = shift == 7 ? gram_panel_kernel<7, 4> : gram_panel_kernel<6, 2>;
         {
-            // (the kernel pointer is the key: six instantiations per input type)
-            static PerDevice<DynSmemPlan> table[2][4];
-            const int v = shift == 7 ? 0 : (shift == 6 ? (wpp == 2 ? 1 : 2) : 3);
-            auto &tb = table[dtype == GAF_F32 ? 0 : 1][v];
+            static PerDevice<DynSmemPlan> table[2];
+            auto &tb = table[shift == 7 ? 0 : 1];
             if (int rc = plan_once(tb.plan[di.dev], tb.ready[di.dev], [&](DynSmemPlan &pl) {
                     // the largest panel this instantiation is ever launched with
-                    pl.dyn = kPanelStages * (shift == 7 ? 2 : (shift == 6 ? 4 : 8)) * 8 * row_bytes;
+                    pl.dyn = kPanelStages * (shift == 7 ? 2 : 3) * 8 * row_bytes;
                     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.dyn) == cudaSuccess
                         ? GAF_OK : GAF_ERR_CUDA;
                 }))
                 return rc;
         }
-        const int64_t chunk_elems = row_bytes / int64_t(elem_bytes(dtype));
+        const int64_t chunk_elems = row_bytes / 4;
         const int64_t work = (D + chunk_elems - 1) / chunk_elems;
         int64_t slices = sms < kGramMaxSlices ? sms : kGramMaxSlices;      // one CTA per SM
         if (slices > work) slices = work;
         if (slices < 1) slices = 1;
         a.slices = int(slices);
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(unsigned(a.slices), unsigned(groups)); cfg.blockDim = dim3(unsigned(threads));
-        cfg.dynamicSmemBytes = size_t(dyn); cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
-        const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, pa);
+        const cudaError_t err = launch_dependent_smem(kernel, a.slices, threads, size_t(dyn), st, pa);
         ++g_launches;
         if (err != cudaSuccess) { cudaGetLastError(); return GAF_ERR_CUDA; }
+    } else {
+        // binary32: 8-bit digits on the tensor cores, one CTA per SM
+        GramDigitsArgs d{};
+        for (int i = 0; i < K; ++i) d.g[i] = static_cast<const float *>(grads[i]);
+        d.K = K; d.D = D; d.tiles = a.tiles; d.pairs = pairs; d.partials = a.partials; d.ctl = a.ctl;
+        d.wait_limit = g_test_wait_limit ? g_test_wait_limit : kDgPollLimit;
+        d.test_extra_arrival = g_test_withhold & 1;
+        const int64_t tile = kDgChunk * (K <= 16 ? DigitsShape<16>::kChunks : 1), work = (D + tile - 1) / tile;
+        int64_t slices = sms < kGramMaxSlices ? sms : kGramMaxSlices;
+        if (slices > work) slices = work;
+        if (slices < 1) slices = 1;
+        a.slices = int(slices);
+        if (int rc = launch_gram_digits(d, a.slices, di, st)) return rc;
     }
     {
         // the finishing blocks are placed while the Gram kernel winds down
@@ -840,11 +866,9 @@ int gaf_filter_accumulate(const void *const *grads, int K, int64_t D, int dtype,
     if (schedule == GAF_SCHED_AUTO) {
         // Gram-first moves fewer bytes whenever its one-pass Gram kernel applies
         const bool ws_ok = workspace_bytes >= kExtraOffset + pairwise_extra_bytes(K);
-        // The general CUDA-core Gram kernel beats the stepwise schedule at any number of binary32 gradients (40 / 64 of
-        // 3 M: 312 / 617 us against 423 / 694; 40 / 64 of 100 k: 39 / 62 against 185 / 290); beyond 32 gradients tiny
-        // vectors keep the stepwise schedule.
+        // (more than 32 binary32 gradients of fewer elements than this keep the streaming passes)
         const bool fast_gram = K >= 2 && (K <= kGsMaxK || use_tensor_gram(K, D, dtype) ||
-                                          (dtype == GAF_F32 && (K <= kPanelAutoMaxK || D >= kPanelAutoMinD)));
+                                          (dtype == GAF_F32 && (K <= kGramAutoMaxK || D >= kGramAutoMinD)));
         schedule = (fast_gram && ws_ok) ? (auto_one_launch(K, D, dtype) ? GAF_SCHED_GRAM_FUSED : GAF_SCHED_GRAM)
                                         : GAF_SCHED_STEPWISE;
     }

@@ -1,0 +1,499 @@
+// Gram matrix G = X X^T of binary32 gradients (one, or 9 to 64 of them; 2 to 8 go to the one-pass kernel of gaf_fused.cuh)
+// on the 5th-generation tensor cores, every gradient read ONCE, with sums that are exact integers.
+//
+// A binary32 value is brought to 31-bit fixed point under a power of two of its gradient and cut into four signed
+// base-256 digits, x 2^k = d0 2^24 + d1 2^16 + d2 2^8 + d3.  The digits of all K gradients are the rows of ONE 8-bit
+// matrix, row s KP + i = digit s of gradient i (KP = K rounded up to 8, 16 at least), so that its product with itself
+// (tcgen05.mma.kind::i8, 8-bit x 8-bit -> 32-bit integers) holds every product of digits of every pair.  Integer sums
+// are exact and do not depend on their order, up to 2^17 products a sum; they are put together in 64-bit integers and
+// binary64 at the end.  What is rounded at all is the value to fixed point: half a unit of 2^-k, about 2^-23 of the
+// gradient's root mean square, at random over the vector: less than the chains of 64 rounded products of a kernel on the
+// binary32 pipes left (24 x 3 M: 2e-10 of the norms' product against 4e-9).
+//
+// The power of two.  A CTA looks at the first tile of each of its teams and allows for elements 2^5 times as
+// large.  Anything beyond that (or an infinity or a NaN) is noticed in
+// the conversion; the CTA then takes the largest finite magnitude of its share and does its share again.
+// Infinities and NaNs count as zero there; their products with the other gradients, whose sums do not depend on an order
+// either, are added at the end.
+//
+// Work split.  One CTA per SM.  A tile is 128 consecutive elements of all K gradients (256 up to 16); tiles are dealt round-robin to the
+// CTAs, and inside a CTA to teams of KP / 8 warps.  Every warp of a team has eight gradients for the whole kernel (their
+// addresses and scales stay in registers); it reads 512 consecutive bytes of each, writes their digits into the team's tile
+// buffer in shared memory (128-byte swizzle, K-major: the operand format; 192 KB in all), and the team hands the tile to the one
+// thread that issues the MMAs, in whatever order the tiles come:
+// 4 MMAs of 128 rows x 4 KP columns x 32 elements, and beyond 32 gradients 4 more for the products of d2 and d3
+// among themselves (what is missing of the 4 KP x 4 KP products then is the mirror image of something present).
+// Rows of absent gradients, and the rows of the 128 beyond 4 KP, hold whatever the memory holds: their sums are not read.
+//
+// Bound by HBM in short runs, by the power cap in long ones (tensor pipe 36 % busy, issue slots 55 %).  All pairs, D = 11.2 M, against the
+// kernel on the binary32 pipes (bound by these and by shared memory): 9 / 16 / 24 / 32 / 40 / 64 gradients 142 / 140 / 307 / 459 / 903 / 1954 us, now
+// 98 / 120 / 205 / 245 / 325 / 508; a second of calls on end 16 / 24 x 3 M / 32 gradients 153 / 88 / 459, now 148 / 64 / 287 (the SM
+// clock falls to 1.1 to 1.5 GHz).  What decided the shape: loads under a condition, or in a ring of single registers, wait for one another
+// (32 gradients: 900 us); eight gradients for the whole kernel per warp, 20 warps and more (300 -> 265); the MMAs issued by a converged warp with
+// an elected lane (their operands are scalars then; 16 gradients 147 -> 118 with two chunks a product).  Products of 64 rows, which waste less, cost the
+// same time and no less power.  The mean written meanwhile under the pattern of a sample: 16 x 11.2 M 199 us, 179 with a pass of its own.
+#pragma once
+
+#include "gaf_device.cuh"
+#include "gaf_fused.cuh"
+#include "gaf_gram_tc.cuh"
+#include "gaf_gramfilter.cuh"
+#include "gaf_pairwise.cuh"
+
+namespace gaf {
+
+constexpr int kDgChunk = 128;                   // elements of a digit row in one swizzle block
+constexpr int kDgHeadroom = 5;                  // bits between the largest sampled magnitude and the bound
+constexpr unsigned int kDgPollLimit = 1u << 23; // looks at all barriers without a tile: a second
+constexpr int kDgMaxChain = 1023;               // chunks: 1023 x 128 products of at most 2^14 fit a 32-bit sum
+
+template <int KP> struct DigitsShape {
+    // Chunks of 128 elements of a tile.  Up to 16 gradients two of them lie one above the other in the 128 rows of a product, each
+    // a diagonal block of it (the thread that issues cannot keep up with products of 64 columns: 16 x 11.2 M 147 us, 118).
+    static constexpr int kChunks = KP <= 16 ? 2 : 1;
+    static constexpr int kTeam = KP / 8;                        // warps of a team
+    static constexpr int kTeams = KP == 64 ? 3 : 23 / kTeam;
+    static constexpr int kTeamBuffers = 2 / kChunks;
+    static constexpr int kWarps = kTeams * kTeam;
+    static constexpr int kThreads = (kWarps + 1) * 32;
+    static constexpr bool kTwo = KP > 32;                       // two products
+    static constexpr int kColumns = kChunks * 4 * KP;           // of a product
+    static constexpr int kRowsValid = kTwo ? 2 * KP : kColumns;
+    static constexpr int kChunkBytes = 4 * KP * kDgChunk;
+    static constexpr int kTileBytes = kChunks * kChunkBytes;
+    static constexpr int kBuffers = kTeams * kTeamBuffers;
+    // an operand of 128 rows read from the last tile may reach past it
+    static constexpr int kRowsRead = kTwo ? 2 * KP + 128 : 128;
+    static constexpr int kPad = kRowsRead > kColumns ? (kRowsRead - kColumns) * 128 : 0;
+    static constexpr int kDyn = kBuffers * kTileBytes + kPad + 1024;
+    static constexpr int kCols = kTwo ? 512 : 128;              // tensor memory
+    static constexpr int kPeriodTiles = kDgMaxChain / kChunks / kTeams * kTeams;
+    static_assert(kBuffers <= 32, "a lane of the issuing warp per buffer");
+    static_assert(4 * KP * (KP + 1) * 8 <= kBuffers * kTileBytes, "the tile buffers hold the sums at the end");
+};
+
+struct GramDigitsArgs {
+    const float *g[GAF_MAX_K];
+    int K;
+    int64_t D;
+    int tiles;                  // T = ceil(K / 8)
+    int pairs;                  // T (T + 1) / 2
+    double *partials;           // [tile pair][slice][64]
+    Control *ctl;
+    unsigned int wait_limit;
+    int test_extra_arrival;     // test hook, normally 0: warp 0's barrier expects an arrival that never comes
+};
+
+// One attempt at waiting for the phase with the given parity, for as long as the hardware suspends a thread by itself.
+__device__ __forceinline__ bool dg_mbar_try(uint64_t *bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(tc_smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool dg_mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag, unsigned int limit) {
+    for (unsigned int spin = 0; spin < limit; ++spin) {
+        if (dg_mbar_try(bar, parity)) return true;
+        if (*abort_flag) return false;
+    }
+    *abort_flag = 1;
+    return false;
+}
+// True in one lane of a whole warp, the same one every time.
+__device__ __forceinline__ bool dg_elect() {
+    uint32_t is;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(is)::"memory");
+    return is != 0;
+}
+__device__ __forceinline__ bool dg_mbar_test(uint64_t *bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(tc_smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// 8-bit signed x 8-bit signed -> 32-bit integer, both operands K-major, M = 128.
+__device__ __forceinline__ void dg_mma(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+__host__ __device__ constexpr uint32_t dg_idesc(int n) {
+    return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24);
+}
+// 32 lanes x 4 columns of 32-bit accumulators.
+__device__ __forceinline__ void dg_tmem_ld4(uint32_t taddr, int (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(taddr)
+                 : "memory");
+}
+template <int OFFSET> __device__ __forceinline__ void dg_st(uint32_t addr, unsigned int v) {
+    asm volatile("st.shared.b32 [%0 + %2], %1;" ::"r"(addr), "r"(v), "n"(OFFSET) : "memory");
+}
+// The largest of m and the magnitudes of a pair; NaN if any is one.
+__device__ __forceinline__ float dg_max_abs(float m, float a, float b) {
+    float r;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ double dg_pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }   // |k| <= 1022
+
+// 2^k under which a magnitude of 2^headroom times the given one is at most 2^30 (all zeros: the largest such power there is).
+__device__ __forceinline__ int dg_exponent(unsigned int max_bits, int headroom) {
+    const int e = (int)(max_bits >> 23) - 126;          // the magnitude is below 2^e
+    return max_bits == 0u ? 126 : min(30 - e - headroom, 126);
+}
+
+template <int KP>
+__global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kernel(const __grid_constant__ GramDigitsArgs a) {
+    using S = DigitsShape<KP>;
+    constexpr int W = S::kWarps, TEAMS = S::kTeams, TEAM = S::kTeam, NB = S::kBuffers, TB = S::kTeamBuffers, CH = S::kChunks;
+    extern __shared__ unsigned char dg_smem[];
+    __shared__ uint64_t full[NB], empty[NB], drained;
+    __shared__ uint32_t tmem_base_s;
+    __shared__ int abort_s, over_s, nonfinite_s;
+    __shared__ int expo[KP];                            // value = fixed point x 2^-expo
+    __shared__ unsigned int rowmax[KP];
+    // (the warp's number from a shuffle: known to be the same in all lanes, so that a row's address is a scalar and the lane's part 32 bits)
+    const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;
+    unsigned char *tiles = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(dg_smem) + 1023) & ~uintptr_t(1023));
+    const uint32_t tiles_u32 = tc_smem_u32(tiles);
+    volatile int *const abort_flag = &abort_s;
+
+    for (int r = tid; r < KP; r += S::kThreads) rowmax[r] = 0u;
+    if (tid == 0) {
+        for (int b = 0; b < NB; ++b) {
+            tc_mbar_init(&full[b], TEAM + (b == 0 && a.test_extra_arrival ? 1 : 0));
+            tc_mbar_init(&empty[b], 1);
+        }
+        tc_mbar_init(&drained, 1);
+        abort_s = 0; over_s = 0; nonfinite_s = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == W) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem_u32(&tmem_base_s)),
+                     "r"(S::kCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem = tmem_base_s;
+    // a programmatic dependent of what precedes it on the stream: nothing global is touched before that has completed
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (blockIdx.x == 0 && tid == 0) a.ctl->status = 0;          // first kernel of the operation
+
+    const int K = a.K;
+    const int64_t n_quads = a.D / 4, G = gridDim.x;
+    const int64_t n_tiles = (n_quads + CH * 32 - 1) / (CH * 32);
+    const int n_mine = blockIdx.x < n_tiles ? (int)((n_tiles - blockIdx.x + G - 1) / G) : 0;
+    const uint64_t policy = l2_policy_evict_first();
+    auto quad_of = [&](int n) { return ((int64_t)n * G + blockIdx.x) * (CH * 32); };      // first four elements of the CTA's tile n
+    // this warp's eight gradients (absent ones: never read)
+    const int team = warp / TEAM, row0 = (warp - team * TEAM) * 8;
+    auto row = [&](int u) { return reinterpret_cast<const unsigned char *>(a.g[row0 + u]); };
+    auto finite_max = [&](const uint4 &x) {
+        unsigned int m = 0u;
+        const unsigned int v[4] = {x.x & 0x7FFFFFFFu, x.y & 0x7FFFFFFFu, x.z & 0x7FFFFFFFu, x.w & 0x7FFFFFFFu};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) m = v[i] < 0x7F800000u ? max(m, v[i]) : m;
+        return m;
+    };
+
+    // The team takes its tiles of a period [n0, n1) (n0 a multiple of the teams) in ascending order, but for one that changes places
+    // with its first: the first tiles of all teams, from which the scales are taken, are spread over the CTA's share.
+    auto tiles_of = [&](int n0, int n1) { return n1 - n0 > team ? (n1 - n0 - team + TEAMS - 1) / TEAMS : 0; };
+    auto visit = [&](int v, int count) {
+        const int first = (int)((int64_t)count * team / TEAMS);
+        return v == 0 ? first : (v == first ? 0 : v);
+    };
+    uint4 x[8];
+    auto fetch = [&](auto full_tag, int n, int chunk) {
+        const int64_t q = quad_of(n) + chunk * 32, left = n_quads - q;
+        // lanes past the end of the vectors read the last four elements and count them as zeros
+        const bool inside = lane < left;
+        const int mine = inside ? lane * 16 : ((int)left - 1) * 16;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (decltype(full_tag)::value || row0 + u < K) x[u] = ld16_policy(row(u) + q * 16 + mine, policy);
+        if (left < 32) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = inside ? x[u] : make_uint4(0u, 0u, 0u, 0u);
+        }
+    };
+    if (warp < W && n_mine > team) {
+        const int n = visit(0, tiles_of(0, min(n_mine, S::kPeriodTiles))) * TEAMS + team;
+        if (row0 + 8 <= K) fetch(std::true_type(), n, 0);
+        else fetch(std::false_type(), n, 0);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const unsigned int top = __reduce_max_sync(0xFFFFFFFFu, finite_max(x[u]));
+            if (lane == 0 && row0 + u < K) atomicMax(&rowmax[row0 + u], top);
+        }
+    }
+    __syncthreads();
+    if (tid < KP) expo[tid] = dg_exponent(rowmax[tid], kDgHeadroom);        // (read behind the next barrier)
+
+    uint32_t done_tiles = 0;                            // tiles this warp's team has handed over so far
+    uint32_t phase = 0, n_drained = 0;                  // issuing warp: parity of the next tile in buffer `lane`; periods so far
+    // This warp's digits of the team's tiles of [n0, n1), into the team's buffers in turn.
+    auto convert_tiles = [&](auto exact_tag, auto full_tag, int n0, int n1, bool fetched) {
+        constexpr bool EXACT = decltype(exact_tag)::value, FULL = decltype(full_tag)::value;
+        float scale[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) scale[u] = __uint_as_float((unsigned int)(dg_exponent(rowmax[row0 + u], EXACT ? 0 : kDgHeadroom) + 127) << 23);
+        float most = 0.0f;
+        bool odd = false;
+        const int count = tiles_of(n0, n1);
+        if (count > 0 && !fetched) fetch(full_tag, n0 + team + visit(0, count) * TEAMS, 0);
+        for (int v = 0, chunk = 0; v < count;) {
+            const int buffer = team * TB + (int)(done_tiles % TB);
+            // the MMAs on what this buffer held before are complete
+            if (chunk == 0 && done_tiles >= TB && !__all_sync(0xFFFFFFFFu, dg_mbar_wait(&empty[buffer], (done_tiles / TB - 1) & 1u, abort_flag, kDgPollLimit))) break;
+            const uint32_t block = tiles_u32 + (uint32_t)(buffer * S::kTileBytes + chunk * S::kChunkBytes + row0 * 128);
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (FULL || row0 + u < K) {
+                    float f[4] = {__uint_as_float(x[u].x), __uint_as_float(x[u].y), __uint_as_float(x[u].z), __uint_as_float(x[u].w)};
+                    if constexpr (EXACT) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const bool finite = fabsf(f[i]) <= 3.402823466e+38f;
+                            f[i] = finite ? f[i] : 0.0f;
+                            odd |= !finite;
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) f[i] *= scale[u];
+                    if constexpr (!EXACT) most = dg_max_abs(dg_max_abs(most, f[0], f[1]), f[2], f[3]);
+                    // signed digits: carries by an addition, then the lower three bytes without their bias
+                    unsigned int d[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) d[i] = (unsigned int)__float2int_rn(f[i]) + 0x00808080u;
+                    // 4 x 4 bytes turned: word s = digit s of the four elements
+                    const unsigned int t0 = __byte_perm(d[0], d[1], 0x5140), t1 = __byte_perm(d[0], d[1], 0x7362);
+                    const unsigned int t2 = __byte_perm(d[2], d[3], 0x5140), t3 = __byte_perm(d[2], d[3], 0x7362);
+                    const uint32_t dst = block + (uint32_t)(u * 128) + (uint32_t)((lane * 4) ^ (u << 4));
+                    dg_st<0>(dst, __byte_perm(t1, t3, 0x7632));
+                    dg_st<KP * 128>(dst, __byte_perm(t1, t3, 0x5410) ^ 0x80808080u);
+                    dg_st<2 * KP * 128>(dst, __byte_perm(t0, t2, 0x7632) ^ 0x80808080u);
+                    dg_st<3 * KP * 128>(dst, __byte_perm(t0, t2, 0x5410) ^ 0x80808080u);
+                }
+            if (++chunk == CH) {
+                tc_fence_async_smem();
+                __syncwarp();
+                if (lane == 0) tc_mbar_arrive(&full[buffer]);
+                ++done_tiles;
+                chunk = 0;
+                ++v;
+            }
+            if (v < count) fetch(full_tag, n0 + team + visit(v, count) * TEAMS, chunk);
+        }
+        odd |= !(most <= 1073741824.0f);
+        if (__any_sync(0xFFFFFFFFu, odd) && lane == 0) {
+            if (EXACT) nonfinite_s = 1;
+            else over_s = 1;
+        }
+    };
+    // MMAs of `total` tiles in the order they come, by lane 0 of the issuing warp; back when all are complete (or a wait gave
+    // up).  Lane b looks at buffer b's barrier.  (In a fixed order the teams wait for one another: 32 x 2 M 69 us for 59.)
+    auto issue_tiles = [&](int total) {
+        uint32_t accumulate = 0;
+        while (total > 0) {
+            unsigned int ready = 0;
+            for (unsigned int idle = 0; idle <= a.wait_limit; ++idle) {
+                ready = __ballot_sync(0xFFFFFFFFu, dg_mbar_test(&full[lane < NB ? lane : 0], phase) && lane < NB);
+                if (ready || __any_sync(0xFFFFFFFFu, *abort_flag)) break;
+                __nanosleep(32);                        // (without it the polls take issue slots from the conversion: 3 us on short calls)
+            }
+            if (!ready) {
+                *abort_flag = 1;
+                break;
+            }
+            phase ^= (ready >> lane) & 1u;
+            total -= __popc(ready);
+            __syncwarp();
+            tc_fence_after_sync();
+            for (; ready; ready &= ready - 1u) {
+                // (everything but the instructions themselves by the whole warp: scalars, which they want their operands to be)
+                const int b = __ffs(ready) - 1;
+                const uint32_t tile = tiles_u32 + (uint32_t)(b * S::kTileBytes);
+                const uint64_t d0 = tc_smem_desc(tile), d2 = tc_smem_desc(tile + 2 * KP * 128);
+                if (dg_elect()) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        // 32 elements = 32 bytes further along K inside the swizzle atom
+                        dg_mma(tmem, d0 + (uint64_t)(2 * k), d0 + (uint64_t)(2 * k), dg_idesc(S::kColumns), k == 0 ? accumulate : 1u);
+                        if (S::kTwo) dg_mma(tmem + 4 * KP, d2 + (uint64_t)(2 * k), d2 + (uint64_t)(2 * k), dg_idesc(2 * KP), k == 0 ? accumulate : 1u);
+                    }
+                    tc_commit(&empty[b]);
+                }
+                accumulate = 1;
+                __syncwarp();
+            }
+        }
+        if (dg_elect()) tc_commit(&drained);            // (the lane that issued the MMAs)
+        __syncwarp();
+        if (lane == 0) {
+            // (this last commit arrives when everything issued so far has completed: also before tensor memory is freed after a
+            // wait that gave up)
+            bool complete = false;
+            for (unsigned int spin = 0; spin < kTcSpinLimit && !complete; ++spin) complete = tc_mbar_try(&drained, n_drained & 1u, 2000u);
+            if (!complete) *abort_flag = 1;
+        }
+        ++n_drained;
+    };
+
+    // The sums of a period out of tensor memory, put together and added to what the periods before it left.
+    auto collect = [&](bool first) {
+        constexpr int P = KP + 1;                       // (a pitch of 2 banks between rows)
+        double *red = reinterpret_cast<double *>(tiles);
+        if (n_mine > 0 && warp < W) {
+            const int row = (warp & 3) * 32 + lane, s = row / KP % 4;
+            const bool valid = row < S::kRowsValid;
+            const double weight = dg_pow2(24 - 8 * s), weight2 = dg_pow2(8 - 8 * s);
+            // (of the rows' own chunk: a warp's rows are of one)
+            const uint32_t lanes = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(CH > 1 ? (warp & 3) * 32 / (4 * KP) * (4 * KP) : 0);
+            for (int jb = warp >> 2; jb < KP / 4; jb += (W - (warp & 3) + 3) / 4) {
+                int d[4][4], d2[2][4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) dg_tmem_ld4(lanes + (uint32_t)(t * KP + jb * 4), d[t]);
+                if (S::kTwo) {
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) dg_tmem_ld4(lanes + (uint32_t)((4 + t) * KP + jb * 4), d2[t]);
+                }
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (valid) {
+#pragma unroll
+                    for (int jj = 0; jj < 4; ++jj) {
+                        const long long hi = (long long)d[0][jj] * 16777216ll + (long long)d[1][jj] * 65536ll;
+                        const long long lo = (long long)d[2][jj] * 256ll + (long long)d[3][jj];
+                        double *const at = red + (size_t)row * P + jb * 4 + jj;
+                        if constexpr (S::kTwo) {
+                            // rows of d0, d1 against all columns (the upper two digits' columns, the lower two's), and rows of
+                            // d2, d3 against columns of d2, d3
+                            const long long lo2 = (long long)d2[0][jj] * 256ll + (long long)d2[1][jj];
+                            at[0] = (double)hi * weight + (double)lo2 * weight2;
+                            at[(size_t)2 * KP * P] = (double)lo * weight;
+                        } else {
+                            at[0] = (double)(hi + lo) * weight;
+                        }
+                    }
+                }
+            }
+        }
+        tc_fence_before_sync();
+        __syncthreads();
+        tc_fence_after_sync();
+        for (int e = tid; e < a.pairs * 64; e += S::kThreads) {
+            int ti, tj;
+            tile_pair(e >> 6, a.tiles, ti, tj);
+            const int i = ti * 8 + ((e >> 3) & 7), j = tj * 8 + (e & 7);
+            if (i > j || j >= K) continue;
+            double v = 0.0;
+            if (n_mine > 0) {
+                if constexpr (S::kTwo) {
+                    const double *const low = red + (size_t)2 * KP * P;
+#pragma unroll
+                    for (int s = 0; s < 2; ++s)
+                        v += red[(s * KP + i) * P + j] + (low[(s * KP + i) * P + j] + low[(s * KP + j) * P + i]);
+                } else {
+#pragma unroll
+                    for (int s = 0; s < 4 * CH; ++s) v += red[(s * KP + i) * P + j];
+                }
+                v *= dg_pow2(-(expo[i] + expo[j]));
+            }
+            double *const dst = a.partials + ((size_t)(e >> 6) * gridDim.x + blockIdx.x) * 64 + (e & 63);
+            if (first) {
+                // fewer than 4 leftover elements: plain binary64 products
+                if (blockIdx.x == 0)
+                    for (int64_t el = n_quads * 4; el < a.D; ++el) v += (double)a.g[i][el] * (double)a.g[j][el];
+                *dst = v;
+            } else {
+                *dst += v;
+            }
+        }
+        __syncthreads();
+    };
+
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        for (int n0 = 0; n0 == 0 || n0 < n_mine; n0 += S::kPeriodTiles) {
+            const int n1 = min(n_mine, n0 + S::kPeriodTiles);
+            if (warp < W) {
+                if (attempt == 1) convert_tiles(std::true_type(), std::false_type(), n0, n1, false);
+                else if (row0 + 8 <= K) convert_tiles(std::false_type(), std::true_type(), n0, n1, n0 == 0);
+                else convert_tiles(std::false_type(), std::false_type(), n0, n1, n0 == 0);
+            } else {
+                issue_tiles(n1 - n0);
+            }
+            __syncwarp();
+            tc_fence_before_sync();
+            __syncthreads();
+            tc_fence_after_sync();
+            if (abort_s || (attempt == 0 && over_s)) break;     // (the same for every thread)
+            collect(n0 == 0);
+        }
+        if (abort_s || !over_s || attempt == 1) break;
+        // a sum of four beyond its bound: the largest finite magnitude of every gradient's share, and again
+        for (int r = tid; r < KP; r += S::kThreads) rowmax[r] = 0u;
+        __syncthreads();
+        if (warp < W)
+            for (int n = team * CH; n < n_mine * CH; n += (n + 1) % CH == 0 ? (TEAMS - 1) * CH + 1 : 1) {
+                const int64_t q = min(quad_of(n / CH) + (n % CH) * 32 + lane, n_quads - 1);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const unsigned int top = __reduce_max_sync(0xFFFFFFFFu, finite_max(ld16_policy(row(row0 + u < K ? u : -row0) + q * 16, policy)));
+                    if (lane == 0) atomicMax(&rowmax[row0 + u], top);
+                }
+            }
+        __syncthreads();
+        for (int r = tid; r < K; r += S::kThreads) expo[r] = dg_exponent(rowmax[r], 0);
+        __syncthreads();
+    }
+    // the streaming part of this CTA is over: the finishing kernel may be placed (it waits for this grid)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    __syncthreads();
+    if (warp == W) {
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(S::kCols) : "memory");
+    }
+    if (abort_s) {
+        if (tid == 0) atomicOr(&a.ctl->status, kStatusTimeoutBit);
+        return;
+    }
+    if (nonfinite_s && warp < W) {
+        auto slot_of = [&](int i, int j) {
+            const int ti = i >> 3, tj = j >> 3, tp = ti * a.tiles - ti * (ti - 1) / 2 + (tj - ti);
+            return a.partials + ((size_t)tp * gridDim.x + blockIdx.x) * 64 + (i & 7) * 8 + (j & 7);
+        };
+        // the products of infinities and NaNs, element by element: infinite or NaN, whatever the order
+        for (int n = warp; n < n_mine * CH; n += W) {
+            const int64_t off = (quad_of(n / CH) + (n % CH) * 32 + lane) * 16;
+            if (off >= n_quads * 16) continue;
+            for (int r = 0; r < K; ++r)
+                for (int i = 0; i < 4; ++i) {
+                    const float v = *reinterpret_cast<const float *>(reinterpret_cast<const unsigned char *>(a.g[r]) + off + 4 * i);
+                    if (fabsf(v) <= 3.402823466e+38f) continue;
+                    for (int j = 0; j < K; ++j) {
+                        const float y = *reinterpret_cast<const float *>(reinterpret_cast<const unsigned char *>(a.g[j]) + off + 4 * i);
+                        atomicAdd(slot_of(min(r, j), max(r, j)), (double)v * (double)y);
+                    }
+                }
+        }
+    }
+}
+
+}  // namespace gaf

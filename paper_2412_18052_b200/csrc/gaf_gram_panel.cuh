@@ -1,24 +1,20 @@
-// Gram matrix G = X X^T for any number of gradients up to GAF_MAX_K and both input types, on
-// CUDA cores, reading every gradient ONCE from HBM (the general path: binary32 with more than 8
-// gradients; fewer go to the one-pass kernel of gaf_fused.cuh, bfloat16 with 9 to 64 to the tensor
-// cores).
+// Gram matrix G = X X^T of one, or 9 to 24, binary32 gradients of short vectors on CUDA cores, reading every gradient ONCE
+// (longer vectors and more gradients: the digits of gaf_gram_digits.cuh, which take about 1 us longer to start and end;
+// the rule is beside use_panel_gram in gaf_api.cu).
 //
 // The K x K matrix is cut into 8 x 8 tiles of pairs (upper triangle: P = T(T+1)/2 tile pairs for
 // T = ceil(K/8)).  One CTA per SM streams panels of the D axis -- all K rows x one chunk of
 // consecutive elements, at most 32 KB -- through a ring of five shared-memory stages filled by
-// 16-byte cp.async copies (four panels, up to 128 KB, in flight per SM).  Every warp owns ONE tile
-// pair for the whole kernel; with few tile pairs several warps share a pair and split each panel's
+// 16-byte cp.async copies (four panels, up to 128 KB, in flight per SM).  Several warps share a tile
+// pair for the whole kernel and split each panel's
 // steps between them.  Per step a lane reads two consecutive elements of the 8 + 8 rows of its pair
 // out of shared memory (conflict-free) and updates the 64 partial dot products of the tile, kept in
-// registers (36 on a diagonal tile).  With more than 12 tile pairs (K > 32) the pairs are split
-// over gridDim.y groups of CTAs, each of which streams the whole panel.
+// registers (36 on a diagonal tile).
 // Binary32 accumulation runs over 64 products per accumulator, then the warp's sums go to
 // binary64 in shared memory; at the end the warps of a pair are added in a fixed order and the
 // tile's 64 binary64 partials are written in the [tile pair][slice][64] layout that
 // gram_finish_kernel totals in a fixed order.
-// No pipe bounds this kernel (fp32 pipe 40 % busy, 60 % of the issue slots taken, HBM 0.42 to 0.66 of the
-// copy rate with 32 and 16 gradients): twelve warps wait for fixed latencies, for operands read from shared
-// memory in the step that uses them (4 multiply-adds per word read) and for one barrier per panel.
+// Bound by latencies at the sizes it is for: 16 gradients of 30 k elements 7.1 us with the finishing kernel, 8.5 as digits.
 #pragma once
 
 #include <type_traits>
@@ -33,12 +29,11 @@ constexpr int kPanelMaxWarps = 12;          // warps per CTA (384 threads leave 
 constexpr int kPanelFlushEvery = 32;        // steps of two products per accumulator between binary64 flushes
 
 struct GramPanelArgs {
-    const void *g[GAF_MAX_K];
+    const float *g[GAF_MAX_K];
     int K;
     int64_t D;
     int tiles;              // T = ceil(K / 8)
     int pairs;              // T (T + 1) / 2
-    int pairs_per_cta;      // gridDim.y = ceil(pairs / pairs_per_cta)
     double *partials;       // [tile pair][slice][64]
     Control *ctl;
 };
@@ -53,30 +48,9 @@ __device__ __forceinline__ void panel_cp_async_commit() { asm volatile("cp.async
 template <int N>
 __device__ __forceinline__ void panel_cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <typename T> struct PanelLane;     // two consecutive elements of one row, as a lane reads them
-template <> struct PanelLane<float> {
-    static constexpr int kBytes = 8;
-    static __device__ __forceinline__ void load(const unsigned char *p, float (&v)[2]) {
-        const float2 x = *reinterpret_cast<const float2 *>(p);
-        v[0] = x.x; v[1] = x.y;
-    }
-};
-template <> struct PanelLane<__nv_bfloat16> {
-    static constexpr int kBytes = 4;
-    static __device__ __forceinline__ void load(const unsigned char *p, float (&v)[2]) {
-        const unsigned int w = *reinterpret_cast<const unsigned int *>(p);
-        v[0] = bf16_bits_to_float(w & 0xFFFFu); v[1] = __uint_as_float(w & 0xFFFF0000u);
-    }
-};
-
-// 25 to 32 gradients: 10 tile pairs on 12 warps.  Hex digit w = tile pair of warp w: the four diagonal ones (0, 4, 7 and 9: 36
-// multiply-adds against 64) have a warp each, 5 and 6 two, so that the warps of every scheduler (w mod 4) add up to
-// 64 + 32 + 36.  One warp per pair in order left one scheduler 164 of 528 (32 x 3 M: 142 us for all pairs, now 131).
-constexpr unsigned long long kPanelOwners10 = 0x974066558321ull;
-
-// SHIFT: bytes of one gradient in one panel = 16 << SHIFT; WPP: warps that share a tile pair (0: by the table above).  Both
+// SHIFT: bytes of one gradient in one panel = 16 << SHIFT; WPP: warps that share a tile pair.  Both
 // are compile-time so that shared-memory addresses are immediates and a warp's steps unroll.
-template <typename T, int SHIFT, int WPP>
+template <int SHIFT, int WPP>
 __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(const __grid_constant__ GramPanelArgs a) {
     extern __shared__ uint4 panel_smem[];                       // [stage][8 T rows][row_bytes]
     __shared__ double wsum[kPanelMaxWarps][64];
@@ -87,7 +61,7 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
     const size_t stage_bytes = (size_t)rows_padded * RB;
     unsigned char *smem = reinterpret_cast<unsigned char *>(panel_smem);
 
-    for (int i = tid; i < a.K; i += nthreads) rowp[i] = static_cast<const unsigned char *>(a.g[i]);
+    for (int i = tid; i < a.K; i += nthreads) rowp[i] = reinterpret_cast<const unsigned char *>(a.g[i]);
     for (int p = lane; p < 64; p += 32) wsum[warp][p] = 0.0;
     // rows of absent gradients (K not a multiple of 8) stay zero in every stage
     {
@@ -99,17 +73,11 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
     __syncthreads();
     // a programmatic dependent of what precedes it on the stream: nothing global is touched before that has completed
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) a.ctl->status = 0;          // first kernel of the operation
+    if (blockIdx.x == 0 && tid == 0) a.ctl->status = 0;          // first kernel of the operation
 
     // this warp's tile pair, and which of the pair's warps it is
-    int wpp = WPP, pair_local = warp / (WPP ? WPP : 1), sub = warp - pair_local * WPP;
-    if (WPP == 0) {
-        pair_local = int((kPanelOwners10 >> (4 * warp)) & 15u);
-        wpp = pair_local == 5 || pair_local == 6 ? 2 : 1;
-        sub = wpp == 2 ? warp & 1 : 0;
-    }
-    const int pair = blockIdx.y * a.pairs_per_cta + pair_local;
-    const bool active = pair_local < a.pairs_per_cta && pair < a.pairs;
+    const int pair = warp / WPP, sub = warp - pair * WPP;
+    const bool active = pair < a.pairs;
     int ti = 0, tj = 0;
     if (active) tile_pair(pair, a.tiles, ti, tj);
 
@@ -147,13 +115,13 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
 
     // panels are dealt round-robin to the CTAs of a group: at any moment the grid reads one
     // compact window of every gradient
-    const int64_t chunk_elems = RB / (int)sizeof(T);
+    const int64_t chunk_elems = RB / 4;
     const int64_t n_chunks = (a.D + chunk_elems - 1) / chunk_elems;
     const int64_t G = gridDim.x;
     const int n_mine = blockIdx.x < n_chunks ? (int)((n_chunks - blockIdx.x + G - 1) / G) : 0;
     constexpr int pieces_per_row = RB / 16;
     const int pieces = a.K * pieces_per_row;
-    const int64_t total_bytes = a.D * (int64_t)sizeof(T);
+    const int64_t total_bytes = a.D * 4;
 
     // Every panel has the same shape: which 16-byte pieces this thread copies, from where (relative to
     // the panel's first byte in the row) and to where (relative to the stage) is worked out once.
@@ -194,9 +162,13 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
         panel_cp_async_commit();                                                    // (an empty group keeps the count in step)
     };
 
-    constexpr int LB = PanelLane<T>::kBytes;
+    constexpr int LB = 8;                               // two consecutive elements of a row, as a lane reads them
     constexpr int steps = RB / (32 * LB);
-    static_assert(steps % (WPP ? WPP : 2) == 0, "a panel's steps divide evenly between the warps of a pair");
+    auto pair_at = [](const unsigned char *p, float (&v)[2]) {
+        const float2 x = *reinterpret_cast<const float2 *>(p);
+        v[0] = x.x; v[1] = x.y;
+    };
+    static_assert(steps % WPP == 0, "a panel's steps divide evenly between the warps of a pair");
     // (one copy of the loop for diagonal tiles and one for the others: with the choice inside, its two sides keep the
     // accumulators in different registers and every step ends with 64 moves)
     auto consume = [&](auto diag_tag) {
@@ -213,12 +185,11 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
             const unsigned char *bi = stage + (size_t)(ti * 8) * RB + lane * LB;
             const unsigned char *bj = stage + (size_t)(tj * 8) * RB + lane * LB;
 #pragma unroll
-            for (int s0 = 0; s0 < steps; s0 += (WPP ? WPP : 1)) {
-                if (WPP == 0 && wpp == 2 && (s0 & 1) != sub) continue;
-                const int s = WPP ? s0 + sub : s0;
+            for (int s0 = 0; s0 < steps; s0 += WPP) {
+                const int s = s0 + sub;
                 float xi[8][2];
 #pragma unroll
-                for (int r = 0; r < 8; ++r) PanelLane<T>::load(bi + (size_t)r * RB + s * (32 * LB), xi[r]);
+                for (int r = 0; r < 8; ++r) pair_at(bi + (size_t)r * RB + s * (32 * LB), xi[r]);
                 if constexpr (DIAG) {
 #pragma unroll
                     for (int r = 0; r < 8; ++r)
@@ -228,7 +199,7 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
                 } else {
                     float xj[8][2];
 #pragma unroll
-                    for (int r = 0; r < 8; ++r) PanelLane<T>::load(bj + (size_t)r * RB + s * (32 * LB), xj[r]);
+                    for (int r = 0; r < 8; ++r) pair_at(bj + (size_t)r * RB + s * (32 * LB), xj[r]);
 #pragma unroll
                     for (int r = 0; r < 8; ++r)
 #pragma unroll
@@ -250,7 +221,7 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
     if (active && sub == 0) {
         // the pair's warps in a fixed order
         double v0 = 0.0, v1 = 0.0;
-        for (int k = 0; k < wpp; ++k) { v0 += wsum[warp + k][lane]; v1 += wsum[warp + k][lane + 32]; }
+        for (int k = 0; k < WPP; ++k) { v0 += wsum[warp + k][lane]; v1 += wsum[warp + k][lane + 32]; }
         double *dst = a.partials + ((size_t)pair * gridDim.x + blockIdx.x) * 64;
         dst[lane] = v0;
         dst[lane + 32] = v1;

@@ -1,0 +1,106 @@
+"""Gram matrix of binary32 gradients as 8-bit digits on the tensor cores: against binary64 products of the same values.
+
+A value is rounded to fixed point of at most 2^-24 of the largest magnitude of the gradient, half a unit off; by Cauchy-Schwarz
+    |G_ij - exact| <= 2^-25 sqrt(D) (max|x_i| |x_j| + max|x_j| |x_i|),
+and the sums themselves are exact integers, put together in binary64."""
+import pytest
+import torch
+
+import paper_2412_18052_b200 as gaf
+
+pytestmark = pytest.mark.gpu
+
+
+def _grads(K, D, kind, seed):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    shared = torch.randn(D, generator=gen, device="cuda")
+    out = []
+    for i in range(K):
+        x = 0.5 * shared + torch.randn(D, generator=gen, device="cuda")
+        if kind == "scales":
+            x *= 10.0 ** (i % 7 - 3)
+        elif kind == "outlier":                     # far beyond what the sample lets expect
+            x[(i * 37) % D] *= 1e6
+        elif kind == "segments":
+            x *= torch.exp(2.5 * torch.randn((D + 999) // 1000, generator=gen, device="cuda")).repeat_interleave(1000)[:D]
+        elif kind == "sparse":                      # most samples see nothing but zeros
+            x *= torch.rand(D, generator=gen, device="cuda") < 0.001
+        elif kind == "tiny":
+            x *= 1e-30
+        elif kind == "huge":
+            x *= 1e17
+        out.append(x.contiguous())
+    return out
+
+
+def _exact(grads):
+    G = torch.zeros(len(grads), len(grads), dtype=torch.float64, device="cuda")
+    for s in range(0, grads[0].numel(), 1 << 20):
+        m = torch.stack([g[s:s + (1 << 20)].double() for g in grads])
+        G += m @ m.T
+    return G
+
+
+def _gram(grads, ws):
+    K = len(grads)
+    return gaf.gaf_pairwise_cosdist(grads, ws, gram_out=torch.empty(K, K, dtype=torch.float64, device="cuda"))[1]
+
+
+def _check(grads):
+    K, D = len(grads), grads[0].numel()
+    ws = gaf.new_workspace(K, D, gaf.GAF_F32)
+    G = _gram(grads, ws)
+    assert gaf.gaf_read_status(ws) & ~gaf.GAF_STATUS_ZERO_NORM == 0
+    assert torch.equal(G, _gram(grads, ws))         # integer sums do not depend on the order the tiles come in
+    E = _exact(grads)
+    norm, top = E.diagonal().sqrt(), torch.stack([g.abs().max() for g in grads]).double()
+    bound = 2.0 ** -25 * D ** 0.5 * (torch.outer(top, norm) + torch.outer(norm, top)) + 1e-12 * torch.outer(norm, norm)
+    assert bool(((G - E).abs() <= bound).all()), (K, D, ((G - E).abs() / bound).max().item())
+
+
+# (up to 16 gradients of fewer than 2^20 elements, and up to 24 of fewer than 327680, go to another kernel)
+@pytest.mark.parametrize("K", [9, 16, 17, 24, 25, 32, 33, 40, 41, 48, 49, 56, 57, 64])
+def test_tiles_and_remainders(K):
+    short = (1, 3, 5, 127, 128, 129, 10_007, 148 * 128 * 3 + 130) if K > 24 else ()
+    for D in short + ((1 << 20, (1 << 20) + 3, 148 * 256 * 30 + 130) if K <= 16 else (327_680, 327_683, 148 * 128 * 23 + 130)):
+        _check(_grads(K, D, "", K + D))
+
+
+@pytest.mark.parametrize("kind", ["scales", "outlier", "segments", "sparse", "tiny", "huge"])
+@pytest.mark.parametrize("K, D", [(12, 1_100_001), (40, 300_001)])
+def test_ranges_of_values(K, D, kind):
+    _check(_grads(K, D, kind, 3))
+
+
+def test_more_products_than_one_integer_sum_holds():
+    _check(_grads(9, 2 * 148 * 1023 * 128 + 77, "", 4))
+    _check(_grads(1, 148 * 1023 * 128 + 5, "outlier", 4))
+
+
+@pytest.mark.parametrize("K, D", [(9, 1_100_003), (40, 70_003)])
+def test_infinities_and_nans(K, D):
+    grads = _grads(K, D, "", 5)
+    grads[1][77], grads[3][77], grads[4][4001] = float("inf"), -float("inf"), float("nan")
+    grads[5][D - 1], grads[6][10], grads[6][11] = float("inf"), float("inf"), -float("inf")
+    ws = gaf.new_workspace(K, D, gaf.GAF_F32)
+    G = _gram(grads, ws)
+    assert gaf.gaf_read_status(ws) & gaf.GAF_STATUS_NONFINITE
+    E = torch.stack([torch.stack([(x.double() * y.double()).sum() for y in grads]) for x in grads])
+    finite = torch.isfinite(E)
+    assert torch.equal(torch.isfinite(G), finite) and torch.equal(torch.isnan(G), torch.isnan(E))
+    assert torch.equal(G[torch.isinf(E)], E[torch.isinf(E)])
+    assert bool(((G - E)[finite].abs() <= 1e-7 * D).all())
+
+
+def test_bounded_wait_runs_out():
+    grads = _grads(24, 400_000, "", 6)
+    ws = gaf.new_workspace(24, 400_000, gaf.GAF_F32)
+    want = _gram(grads, ws)
+    try:
+        gaf.gaf_test_set_wait_fault(2000, 1)
+        _gram(grads, ws)
+        torch.cuda.synchronize()
+        assert gaf.gaf_read_status(ws) & gaf.GAF_STATUS_TIMEOUT
+    finally:
+        gaf.gaf_test_set_wait_fault(0, 0)
+    assert torch.equal(_gram(grads, ws), want) and gaf.gaf_read_status(ws) == 0
