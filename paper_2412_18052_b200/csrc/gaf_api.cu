@@ -159,7 +159,10 @@ int stream_grid(int64_t D, int threads, int sms) {
 constexpr int kGramAutoMaxK = 32;
 constexpr int64_t kGramAutoMinD = 32768;
 constexpr int64_t kPanelMaxD16 = int64_t(1) << 20, kPanelMaxD24 = 5 * 65536;
-bool use_panel_gram(int K, int64_t D) { return K <= 16 ? D < kPanelMaxD16 : (K <= 24 && D < kPanelMaxD24); }
+// (one bfloat16 gradient at every length: the MMAs' accumulators cut off, which adds up where all products are positive)
+bool use_panel_gram(int K, int64_t D, int dtype) {
+    return dtype == GAF_BF16 || (K <= 16 ? D < kPanelMaxD16 : (K <= 24 && D < kPanelMaxD24));
+}
 bool use_tensor_gram(int K, int64_t D, int dtype) {
     (void)D;
     return dtype == GAF_BF16 && K > kGsMaxK && K <= kTcMaxK;
@@ -313,8 +316,8 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
                                                       2 * gram_matrix_bytes(K));
     a.gram_out = gram_out;
     a.ctl = reinterpret_cast<Control *>(base);
-    if (dtype == GAF_BF16 && K <= kWideMaxK) {
-        // 9..16 bfloat16 gradients (or a single one, alone in its block): warp-level MMAs fed straight from the global loads, two CTAs per SM
+    if (use_tensor_gram(K, D, dtype) && K <= kWideMaxK) {
+        // 9..16 bfloat16 gradients: warp-level MMAs fed straight from the global loads, two CTAs per SM
         GramWideArgs w{};
         for (int i = 0; i < K; ++i) w.g[i] = grads[i];
         w.K = K; w.D = D; w.partials = a.partials; w.ctl = a.ctl;
@@ -382,10 +385,10 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
                                                       t, tmap, tmap_row);
         ++g_launches;
         if (err != cudaSuccess) { cudaGetLastError(); return GAF_ERR_CUDA; }
-    } else if (use_panel_gram(K, D)) {
+    } else if (use_panel_gram(K, D, dtype)) {
         // CUDA cores, every gradient read once: one warp per tile pair, panels of D through shared memory
         GramPanelArgs pa{};
-        for (int i = 0; i < K; ++i) pa.g[i] = static_cast<const float *>(grads[i]);
+        for (int i = 0; i < K; ++i) pa.g[i] = grads[i];
         pa.K = K; pa.D = D; pa.tiles = a.tiles; pa.pairs = pairs;
         // A panel is at most 32 KB: 2 KB of every row up to 16 (padded) rows, 1 KB up to 24.  4 or 2 warps share a tile pair.
         const int shift = a.tiles <= 2 ? 7 : 6, wpp = a.tiles <= 2 ? 4 : 2;
@@ -393,10 +396,12 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
         const int threads = 32 * pairs * wpp;
         const int row_bytes = 16 << shift;
         const int dyn = kPanelStages * a.tiles * 8 * row_bytes;
-        void (*kernel)(GramPanelArgs) = shift == 7 ? gram_panel_kernel<7, 4> : gram_panel_kernel<6, 2>;
+        // (bfloat16 comes here with a single gradient only: 2 to 8 take the one-pass kernel, up to 64 the tensor cores)
+        void (*kernel)(GramPanelArgs) = dtype == GAF_BF16 ? gram_panel_kernel<__nv_bfloat16, 7, 4>
+                                      : (shift == 7 ? gram_panel_kernel<float, 7, 4> : gram_panel_kernel<float, 6, 2>);
         {
-            static PerDevice<DynSmemPlan> table[2];
-            auto &tb = table[shift == 7 ? 0 : 1];
+            static PerDevice<DynSmemPlan> table[3];
+            auto &tb = table[dtype == GAF_BF16 ? 2 : (shift == 7 ? 0 : 1)];
             if (int rc = plan_once(tb.plan[di.dev], tb.ready[di.dev], [&](DynSmemPlan &pl) {
                     // the largest panel this instantiation is ever launched with
                     pl.dyn = kPanelStages * (shift == 7 ? 2 : 3) * 8 * row_bytes;
@@ -405,7 +410,7 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
                 }))
                 return rc;
         }
-        const int64_t chunk_elems = row_bytes / 4;
+        const int64_t chunk_elems = row_bytes / int64_t(elem_bytes(dtype));
         const int64_t work = (D + chunk_elems - 1) / chunk_elems;
         int64_t slices = sms < kGramMaxSlices ? sms : kGramMaxSlices;      // one CTA per SM
         if (slices > work) slices = work;

@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kWideThreads, 2) gram_mma_wide_kernel(const __
 #pragma unroll
         for (int k = 0; k < 4; ++k) wide_red[((size_t)(warp * NT + i) * 32 + lane) * 4 + k] = d[i][k] + (double)c[i][k];
     __syncthreads();
-    const int tiles8 = (a.K + 7) / 8;                // 8 x 8 blocks per side
+    const int tiles8 = NB;                           // 8 x 8 blocks per side
     for (int e = threadIdx.x; e < NT * 128; e += kWideThreads) {
         // the 16 warps in a fixed order
         double s = 0.0;
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kWideThreads, 2) gram_mma_wide_kernel(const __
         const int cb = e >> 7, ln = (e >> 2) & 31, k = e & 3;
         const int bi = k >> 1, bj = cb;                                   // 8 x 8 block, row and column inside it:
         const int row = ln >> 2, col = 2 * (ln & 3) + (k & 1);
-        if (bi > bj || bj >= tiles8) continue;                            // below the diagonal or absent: not wanted
+        if (bi > bj || bi >= tiles8) continue;                            // below the diagonal: not wanted
         int tp = 0;
         for (int q = 0; q < bi; ++q) tp += tiles8 - q;
         tp += bj - bi;

@@ -1,5 +1,5 @@
-// Gram matrix G = X X^T of one, or 9 to 24, binary32 gradients of short vectors on CUDA cores, reading every gradient ONCE
-// (longer vectors and more gradients: the digits of gaf_gram_digits.cuh, which take about 1 us longer to start and end;
+// Gram matrix G = X X^T of one, or 9 to 24, binary32 gradients of short vectors, and of one bfloat16 gradient, on CUDA cores, reading
+// every gradient ONCE (longer vectors and more gradients: the digits of gaf_gram_digits.cuh, which take 2 us longer to start and end;
 // the rule is beside use_panel_gram in gaf_api.cu).
 //
 // The K x K matrix is cut into 8 x 8 tiles of pairs (upper triangle: P = T(T+1)/2 tile pairs for
@@ -29,7 +29,7 @@ constexpr int kPanelMaxWarps = 12;          // warps per CTA (384 threads leave 
 constexpr int kPanelFlushEvery = 32;        // steps of two products per accumulator between binary64 flushes
 
 struct GramPanelArgs {
-    const float *g[GAF_MAX_K];
+    const void *g[GAF_MAX_K];
     int K;
     int64_t D;
     int tiles;              // T = ceil(K / 8)
@@ -48,9 +48,25 @@ __device__ __forceinline__ void panel_cp_async_commit() { asm volatile("cp.async
 template <int N>
 __device__ __forceinline__ void panel_cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+template <typename T> struct PanelLane;     // two consecutive elements of one row, as a lane reads them
+template <> struct PanelLane<float> {
+    static constexpr int kBytes = 8;
+    static __device__ __forceinline__ void load(const unsigned char *p, float (&v)[2]) {
+        const float2 x = *reinterpret_cast<const float2 *>(p);
+        v[0] = x.x; v[1] = x.y;
+    }
+};
+template <> struct PanelLane<__nv_bfloat16> {
+    static constexpr int kBytes = 4;
+    static __device__ __forceinline__ void load(const unsigned char *p, float (&v)[2]) {
+        const unsigned int w = *reinterpret_cast<const unsigned int *>(p);
+        v[0] = bf16_bits_to_float(w & 0xFFFFu); v[1] = __uint_as_float(w & 0xFFFF0000u);
+    }
+};
+
 // SHIFT: bytes of one gradient in one panel = 16 << SHIFT; WPP: warps that share a tile pair.  Both
 // are compile-time so that shared-memory addresses are immediates and a warp's steps unroll.
-template <int SHIFT, int WPP>
+template <typename T, int SHIFT, int WPP>
 __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(const __grid_constant__ GramPanelArgs a) {
     extern __shared__ uint4 panel_smem[];                       // [stage][8 T rows][row_bytes]
     __shared__ double wsum[kPanelMaxWarps][64];
@@ -61,7 +77,7 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
     const size_t stage_bytes = (size_t)rows_padded * RB;
     unsigned char *smem = reinterpret_cast<unsigned char *>(panel_smem);
 
-    for (int i = tid; i < a.K; i += nthreads) rowp[i] = reinterpret_cast<const unsigned char *>(a.g[i]);
+    for (int i = tid; i < a.K; i += nthreads) rowp[i] = static_cast<const unsigned char *>(a.g[i]);
     for (int p = lane; p < 64; p += 32) wsum[warp][p] = 0.0;
     // rows of absent gradients (K not a multiple of 8) stay zero in every stage
     {
@@ -115,13 +131,13 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
 
     // panels are dealt round-robin to the CTAs of a group: at any moment the grid reads one
     // compact window of every gradient
-    const int64_t chunk_elems = RB / 4;
+    const int64_t chunk_elems = RB / (int)sizeof(T);
     const int64_t n_chunks = (a.D + chunk_elems - 1) / chunk_elems;
     const int64_t G = gridDim.x;
     const int n_mine = blockIdx.x < n_chunks ? (int)((n_chunks - blockIdx.x + G - 1) / G) : 0;
     constexpr int pieces_per_row = RB / 16;
     const int pieces = a.K * pieces_per_row;
-    const int64_t total_bytes = a.D * 4;
+    const int64_t total_bytes = a.D * (int64_t)sizeof(T);
 
     // Every panel has the same shape: which 16-byte pieces this thread copies, from where (relative to
     // the panel's first byte in the row) and to where (relative to the stage) is worked out once.
@@ -162,12 +178,8 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
         panel_cp_async_commit();                                                    // (an empty group keeps the count in step)
     };
 
-    constexpr int LB = 8;                               // two consecutive elements of a row, as a lane reads them
+    constexpr int LB = PanelLane<T>::kBytes;
     constexpr int steps = RB / (32 * LB);
-    auto pair_at = [](const unsigned char *p, float (&v)[2]) {
-        const float2 x = *reinterpret_cast<const float2 *>(p);
-        v[0] = x.x; v[1] = x.y;
-    };
     static_assert(steps % WPP == 0, "a panel's steps divide evenly between the warps of a pair");
     // (one copy of the loop for diagonal tiles and one for the others: with the choice inside, its two sides keep the
     // accumulators in different registers and every step ends with 64 moves)
@@ -189,7 +201,7 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
                 const int s = s0 + sub;
                 float xi[8][2];
 #pragma unroll
-                for (int r = 0; r < 8; ++r) pair_at(bi + (size_t)r * RB + s * (32 * LB), xi[r]);
+                for (int r = 0; r < 8; ++r) PanelLane<T>::load(bi + (size_t)r * RB + s * (32 * LB), xi[r]);
                 if constexpr (DIAG) {
 #pragma unroll
                     for (int r = 0; r < 8; ++r)
@@ -199,7 +211,7 @@ __global__ void __launch_bounds__(kPanelMaxWarps * 32, 1) gram_panel_kernel(cons
                 } else {
                     float xj[8][2];
 #pragma unroll
-                    for (int r = 0; r < 8; ++r) pair_at(bj + (size_t)r * RB + s * (32 * LB), xj[r]);
+                    for (int r = 0; r < 8; ++r) PanelLane<T>::load(bj + (size_t)r * RB + s * (32 * LB), xj[r]);
 #pragma unroll
                     for (int r = 0; r < 8; ++r)
 #pragma unroll

@@ -794,6 +794,18 @@ def test_wide_mma_gram_kernel_shapes_and_long_runs(ws):
     check_pairwise(_mix(12, D, "bf16", seed=777).grads, ws)
 
 
+def test_square_of_one_bf16_gradient(ws):
+    """All pairs of a single bfloat16 gradient: |g|^2 from chains of 64 products in binary32, rounded to nearest.  Roundings of either
+    sign cancel over the chains: 2^-23 is three times what is left of them (4e-8, from ties of short significands); accumulators that
+    cut off, in longer chains of products that are all positive, leave 3.5e-7."""
+    gen = torch.Generator(device="cuda").manual_seed(8)
+    for x in (torch.randn(3_000_001, generator=gen, device="cuda"), torch.rand(3_000_001, generator=gen, device="cuda")):
+        x = x.bfloat16()
+        _, gram = gaf.gaf_pairwise_cosdist([x], ws)
+        want = (x.double() ** 2).sum()
+        assert float((gram[0, 0] - want).abs() / want) < 2.0 ** -23
+
+
 def test_mma_gram_kernel_long_runs(ws):
     """7 and 8 bfloat16 gradients take the warp-level tensor-core Gram kernel; from about 19 M elements on its
     CTAs walk the vectors in runs of several trips.  Both mappings, with ragged ends, against the oracle."""
