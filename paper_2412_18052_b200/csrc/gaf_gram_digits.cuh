@@ -28,8 +28,8 @@
 // Bound by HBM in short runs, by the power cap in long ones (tensor pipe 36 % busy, issue slots 55 %).  All pairs, D = 11.2 M, against the
 // kernel on the binary32 pipes (bound by these and by shared memory): 9 / 16 / 24 / 32 / 40 / 64 gradients 142 / 140 / 307 / 459 / 903 / 1954 us, now
 // 98 / 120 / 205 / 245 / 325 / 508; a second of calls on end 16 / 24 x 3 M / 32 gradients 153 / 88 / 459, now 148 / 64 / 287 (the SM
-// clock falls to 1.1 to 1.5 GHz).  What decided the shape: loads under a condition, or in a ring of single registers, wait for one another
-// (32 gradients: 900 us); eight gradients for the whole kernel per warp, 20 warps and more (300 -> 265); the MMAs issued by a converged warp with
+// clock falls to 1.1 to 1.5 GHz).  What decided the shape: loads under a branch, or in a ring of single registers, wait for one another
+// (32 gradients: 900 us; the warp with the absent gradients loads under predicates: 15 x 8.2 M 112 -> 107, binary32 pipes 109); eight gradients for the whole kernel per warp, 20 warps and more (300 -> 265); the MMAs issued by a converged warp with
 // an elected lane (their operands are scalars then; 16 gradients 147 -> 118 with two chunks a product).  Products of 64 rows, which waste less, cost the
 // same time and no less power.  The mean written meanwhile under the pattern of a sample: 16 x 11.2 M 199 us, 179 with a pass of its own.
 #pragma once
@@ -133,6 +133,15 @@ __device__ __forceinline__ void dg_mma(uint32_t tmem_d, uint64_t desc_a, uint64_
 __host__ __device__ constexpr uint32_t dg_idesc(int n) {
     return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24);
 }
+// 16 bytes if `wanted`, else r stays as it is: a load under a predicate.  (Under a branch the loads of a tile wait for one another.)
+__device__ __forceinline__ void dg_ld16_if(uint4 &r, bool wanted, const void *p, uint64_t policy) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "@p ld.global.nc.L1::no_allocate.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;\n\t}"
+        : "+r"(r.x), "+r"(r.y), "+r"(r.z), "+r"(r.w)
+        : "l"(p), "l"(policy), "r"((unsigned int)wanted));
+}
 // 32 lanes x 4 columns of 32-bit accumulators.
 __device__ __forceinline__ void dg_tmem_ld4(uint32_t taddr, int (&r)[4]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
@@ -221,15 +230,17 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
         const int first = (int)((int64_t)count * team / TEAMS);
         return v == 0 ? first : (v == first ? 0 : v);
     };
-    uint4 x[8];
+    uint4 x[8] = {};
     auto fetch = [&](auto full_tag, int n, int chunk) {
         const int64_t q = quad_of(n) + chunk * 32, left = n_quads - q;
         // lanes past the end of the vectors read the last four elements and count them as zeros
         const bool inside = lane < left;
         const int mine = inside ? lane * 16 : ((int)left - 1) * 16;
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (decltype(full_tag)::value || row0 + u < K) x[u] = ld16_policy(row(u) + q * 16 + mine, policy);
+        for (int u = 0; u < 8; ++u) {
+            if constexpr (decltype(full_tag)::value) x[u] = ld16_policy(row(u) + q * 16 + mine, policy);
+            else dg_ld16_if(x[u], row0 + u < K, row(u) + q * 16 + mine, policy);
+        }
         if (left < 32) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) x[u] = inside ? x[u] : make_uint4(0u, 0u, 0u, 0u);

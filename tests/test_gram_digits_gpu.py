@@ -66,6 +66,13 @@ def test_tiles_and_remainders(K):
         _check(_grads(K, D, "", K + D))
 
 
+@pytest.mark.parametrize("K", [15, 23, 31, 39, 47, 55, 63])
+def test_one_absent_gradient(K):
+    """The warp with the absent gradient loads the other seven under predicates."""
+    for D in ((1 << 20) + 129, 148 * 256 * 11 + 5) if K <= 16 else (327_680 + 127, 148 * 128 * 21 + 6):
+        _check(_grads(K, D, "", K + D))
+
+
 @pytest.mark.parametrize("kind", ["scales", "outlier", "segments", "sparse", "tiny", "huge"])
 @pytest.mark.parametrize("K, D", [(12, 1_100_001), (40, 300_001)])
 def test_ranges_of_values(K, D, kind):
