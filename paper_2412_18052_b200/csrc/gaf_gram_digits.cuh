@@ -10,12 +10,23 @@
 // gradient's root mean square, at random over the vector: less than the chains of 64 rounded products of a kernel on the
 // binary32 pipes left (24 x 3 M: 2e-10 of the norms' product against 4e-9).
 //
-// The power of two.  A CTA looks at the first tile of each of its teams and allows for elements 2^5 times as
-// large.  Anything beyond that (or an infinity or a NaN) is noticed in
-// the conversion; the CTA then takes the largest finite magnitude of its share and does its share again.
-// Infinities and NaNs count as zero there; their products with the other gradients, whose sums do not depend on an order
-// either, are added at the end.
-//
+// The power of two.  A CTA takes its share in periods of at most 1023 x 128 elements.  At the start of each it looks at the first tile of
+// each of its teams and allows for elements 2^5 times as large: half a unit is at most 2^-25 of the largest magnitude that the CTA sampled of
+// the gradient.  A tile with anything beyond that is noticed in the conversion and left out of the sums; at the end of the period the
+// tiles left out come again, under scales that hold the largest of their values (half a unit: 2^-30 of it), and
+// their sums are added.  Which tiles these are depends on the values alone, so that results repeat bit for bit.
+// Gradients with infinities or NaNs are left out of the digits, the products of their infinities found afterwards.
+// What values of many sizes cost (all pairs of 16 x 11.2 M, 24 x 3 M, 32 x 11.2 M, 64 x 3 M, us, short runs one after the other, so that the power
+// state moves them by a tenth; when a tile beyond its bound was noticed at the end only, the CTA did its whole share again):
+//                                                          here            whole share           binary32 pipes
+//     normal values                                  123  56 241 155     122   54  237  139     140  89 458 521
+//     one element of 10^6                            150  74 258 150     473  144  686  496     142  90 459 522
+//     lognormal, sigma 2                             128  67 251 171     478  151  748  535     142  89 459 522
+//     97 % of all rows of 512 elements zero          143  69 253 163     489  159  739  518     140  89 458 521
+//     200 tensors with lognormal scales, sigma 2     127  60 253 153     482  156  767  553     140  89 458 521
+//     6 % of the vector 1000 times as large          126  76 285 184     504   56  231  557     142  92 459 522
+//     one gradient of NaNs                           162  72 302 175    3426 1212 8184 2880     148  93 459 523
+//     infinities in a gradient                       152  85 321 231    1305  544 2583 1524     141  89 459 523
 // Work split.  One CTA per SM.  A tile is 128 consecutive elements of all K gradients (256 up to 16); tiles are dealt round-robin to the
 // CTAs, and inside a CTA to teams of KP / 8 warps.  Every warp of a team has eight gradients for the whole kernel (their
 // addresses and scales stay in registers); it reads 512 consecutive bytes of each, writes their digits into the team's tile
@@ -173,23 +184,33 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
     extern __shared__ unsigned char dg_smem[];
     __shared__ uint64_t full[NB], empty[NB], drained;
     __shared__ uint32_t tmem_base_s;
-    __shared__ int abort_s, over_s, nonfinite_s;
+    __shared__ int abort_s, issued_s;
     __shared__ int expo[KP];                            // value = fixed point x 2^-expo
-    __shared__ unsigned int rowmax[KP];
+    __shared__ unsigned int rowmax[KP];                 // largest finite magnitude of the period's sample,
+    __shared__ unsigned int rowtop[KP];                 // and of what was found beyond the bound
+    __shared__ unsigned int beyond_map[32];             // the period's tiles with a value beyond its bound,
+    __shared__ int beyond_buffer[NB];                   // and the buffers that hold one
+    __shared__ unsigned long long nan_rows[2], inf_rows[2];     // gradients with a NaN, an infinity: [0] known before the period, [1] found in it
     // (the warp's number from a shuffle: known to be the same in all lanes, so that a row's address is a scalar and the lane's part 32 bits)
     const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;
     unsigned char *tiles = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(dg_smem) + 1023) & ~uintptr_t(1023));
     const uint32_t tiles_u32 = tc_smem_u32(tiles);
     volatile int *const abort_flag = &abort_s;
 
-    for (int r = tid; r < KP; r += S::kThreads) rowmax[r] = 0u;
+    auto clear_period = [&]() {
+        if (tid < KP) { rowmax[tid] = 0u; rowtop[tid] = 0u; }
+        if (tid < 32) beyond_map[tid] = 0u;
+    };
+    clear_period();
     if (tid == 0) {
         for (int b = 0; b < NB; ++b) {
             tc_mbar_init(&full[b], TEAM + (b == 0 && a.test_extra_arrival ? 1 : 0));
             tc_mbar_init(&empty[b], 1);
+            beyond_buffer[b] = 0;
         }
         tc_mbar_init(&drained, 1);
-        abort_s = 0; over_s = 0; nonfinite_s = 0;
+        abort_s = 0;
+        nan_rows[0] = nan_rows[1] = inf_rows[0] = inf_rows[1] = 0ull;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == W) {
@@ -224,13 +245,20 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
     };
 
     // The team takes its tiles of a period [n0, n1) (n0 a multiple of the teams) in ascending order, but for one that changes places
-    // with its first: the first tiles of all teams, from which the scales are taken, are spread over the CTA's share.
+    // with its first: the first tiles of all teams, from which the scales are taken, are spread over the CTA's share, one in every
+    // TEAMS-th part of it at an uneven place (equal distances fall in step with rows of 2^n elements), the same in all CTAs: places
+    // of their own cost a page each (24 x 3 M: 1.5 us).
+    const unsigned int place = ((unsigned int)team * 2654435761u + 1234567u) >> 20;
     auto tiles_of = [&](int n0, int n1) { return n1 - n0 > team ? (n1 - n0 - team + TEAMS - 1) / TEAMS : 0; };
-    auto visit = [&](int v, int count) {
-        const int first = (int)((int64_t)count * team / TEAMS);
-        return v == 0 ? first : (v == first ? 0 : v);
-    };
+    auto first_of = [&](int count) { return (int)((unsigned int)count * ((unsigned int)team * 4096u + place) / (TEAMS * 4096u)); };
     uint4 x[8] = {};
+    // The warp's gradients that take part: those that are there and hold no NaN or infinity, as far as the CTA knows.  (All products of a
+    // gradient that does are NaN or infinite, whatever the digits say.)
+    unsigned int live = 0u;
+    auto update_live = [&](unsigned long long odd) {
+        const int here = min(max(K - row0, 0), 8);
+        live = warp < W ? ((1u << here) - 1u) & ~(unsigned int)(odd >> row0) : 0u;
+    };
     auto fetch = [&](auto full_tag, int n, int chunk) {
         const int64_t q = quad_of(n) + chunk * 32, left = n_quads - q;
         // lanes past the end of the vectors read the last four elements and count them as zeros
@@ -239,55 +267,91 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             if constexpr (decltype(full_tag)::value) x[u] = ld16_policy(row(u) + q * 16 + mine, policy);
-            else dg_ld16_if(x[u], row0 + u < K, row(u) + q * 16 + mine, policy);
+            else dg_ld16_if(x[u], (live >> u) & 1u, row(u) + q * 16 + mine, policy);
         }
         if (left < 32) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) x[u] = inside ? x[u] : make_uint4(0u, 0u, 0u, 0u);
         }
     };
-    if (warp < W && n_mine > team) {
-        const int n = visit(0, tiles_of(0, min(n_mine, S::kPeriodTiles))) * TEAMS + team;
-        if (row0 + 8 <= K) fetch(std::true_type(), n, 0);
-        else fetch(std::false_type(), n, 0);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const unsigned int top = __reduce_max_sync(0xFFFFFFFFu, finite_max(x[u]));
-            if (lane == 0 && row0 + u < K) atomicMax(&rowmax[row0 + u], top);
+    // What v holds of the warp's gradient u, 32 pieces of it: the largest finite magnitude, a NaN, an infinity.
+    auto look = [&](int u, const uint4 &v, unsigned int *top, int when) {
+        const unsigned int m[4] = {v.x & 0x7FFFFFFFu, v.y & 0x7FFFFFFFu, v.z & 0x7FFFFFFFu, v.w & 0x7FFFFFFFu};
+        const unsigned int finite = __reduce_max_sync(0xFFFFFFFFu, finite_max(v));
+        const unsigned int any = __reduce_max_sync(0xFFFFFFFFu, max(max(m[0], m[1]), max(m[2], m[3])));
+        if (any >= 0x7F800000u) {
+            const bool inf = __any_sync(0xFFFFFFFFu, m[0] == 0x7F800000u || m[1] == 0x7F800000u || m[2] == 0x7F800000u || m[3] == 0x7F800000u);
+            if (lane == 0 && any > 0x7F800000u) atomicOr(&nan_rows[when], 1ull << (row0 + u));
+            if (lane == 0 && inf) atomicOr(&inf_rows[when], 1ull << (row0 + u));
         }
-    }
-    __syncthreads();
-    if (tid < KP) expo[tid] = dg_exponent(rowmax[tid], kDgHeadroom);        // (read behind the next barrier)
+        if (lane == 0) atomicMax(&top[row0 + u], finite);
+    };
+    // The period's scales come from the first tiles of its teams, and for a gradient that has nothing but zeros there, from single pieces of
+    // 16 bytes, 32 times as many places.
+    auto sample = [&](int n0, int n1) {
+        update_live(nan_rows[0] | inf_rows[0]);
+        const int count = tiles_of(n0, n1);
+        if (warp < W && count > 0) {
+            const int n = n0 + team + first_of(count) * TEAMS;
+            if (live == 0xFFu) fetch(std::true_type(), n, 0);
+            else fetch(std::false_type(), n, 0);
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if ((live >> u) & 1u) look(u, x[u], rowmax, 0);
+        }
+        __syncthreads();
+        const unsigned long long odd = nan_rows[0] | inf_rows[0];
+        auto zeros = [&](int r) { return r < K && rowmax[r] == 0u && !((odd >> r) & 1ull); };
+        if (!__any_sync(0xFFFFFFFFu, zeros(lane) || zeros(lane + 32))) return;      // (the same for all warps)
+        unsigned int dark = 0u;
+        for (int u = 0; u < 8; ++u) dark |= warp < W && count > 0 && zeros(row0 + u) ? 1u << u : 0u;
+        __syncthreads();
+        if (dark) {
+            const int at = (int)((unsigned int)count * ((unsigned int)lane * 4096u + place) / (32u * 4096u));
+            const int64_t q = min(quad_of(n0 + team + at * TEAMS) + (int)((place + (unsigned int)lane * 11u) % (CH * 32u)), n_quads - 1);
+            for (int u = 0; u < 8; ++u)
+                if ((dark >> u) & 1u) look(u, ld16_policy(row(u) + q * 16, policy), rowmax, 0);
+        }
+        __syncthreads();
+    };
+    auto is_beyond = [&](int t) { return (beyond_map[t >> 5] >> (t & 31)) & 1u; };
 
     uint32_t done_tiles = 0;                            // tiles this warp's team has handed over so far
-    uint32_t phase = 0, n_drained = 0;                  // issuing warp: parity of the next tile in buffer `lane`; periods so far
-    // This warp's digits of the team's tiles of [n0, n1), into the team's buffers in turn.
-    auto convert_tiles = [&](auto exact_tag, auto full_tag, int n0, int n1, bool fetched) {
+    uint32_t phase = 0, n_drained = 0;                  // issuing warp: parity of the next tile in buffer `lane`; drains so far
+    // This warp's digits of the team's tiles of [n0, n1), into the team's buffers in turn: of all of them under the sample's scales (the
+    // first is in x already), or, EXACT, of those with a value beyond its bound under scales that hold every finite value in them.
+    auto convert_tiles = [&](auto exact_tag, auto full_tag, int n0, int n1) {
         constexpr bool EXACT = decltype(exact_tag)::value, FULL = decltype(full_tag)::value;
         float scale[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) scale[u] = __uint_as_float((unsigned int)(dg_exponent(rowmax[row0 + u], EXACT ? 0 : kDgHeadroom) + 127) << 23);
-        float most = 0.0f;
-        bool odd = false;
+        for (int u = 0; u < 8; ++u) {
+            const int sampled = dg_exponent(rowmax[row0 + u], kDgHeadroom);
+            const int k = EXACT ? min(sampled, dg_exponent(rowtop[row0 + u], 0)) : sampled;
+            scale[u] = __uint_as_float((unsigned int)(k + 127) << 23);
+        }
         const int count = tiles_of(n0, n1);
-        if (count > 0 && !fetched) fetch(full_tag, n0 + team + visit(0, count) * TEAMS, 0);
-        for (int v = 0, chunk = 0; v < count;) {
+        auto next_beyond = [&](int n) {
+            while (n < n1 && !is_beyond(n - n0)) n += TEAMS;
+            return n;
+        };
+        const int first = first_of(count);
+        int v = 0, n = n1;
+        if (EXACT) {
+            n = next_beyond(n0 + team);
+            if (n < n1) fetch(full_tag, n, 0);
+        } else if (count > 0) {
+            n = n0 + team + first * TEAMS;
+        }
+        for (int chunk = 0; n < n1;) {
             const int buffer = team * TB + (int)(done_tiles % TB);
             // the MMAs on what this buffer held before are complete
             if (chunk == 0 && done_tiles >= TB && !__all_sync(0xFFFFFFFFu, dg_mbar_wait(&empty[buffer], (done_tiles / TB - 1) & 1u, abort_flag, kDgPollLimit))) break;
             const uint32_t block = tiles_u32 + (uint32_t)(buffer * S::kTileBytes + chunk * S::kChunkBytes + row0 * 128);
+            float most = 0.0f;
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-                if (FULL || row0 + u < K) {
+                if (FULL || ((live >> u) & 1u)) {
                     float f[4] = {__uint_as_float(x[u].x), __uint_as_float(x[u].y), __uint_as_float(x[u].z), __uint_as_float(x[u].w)};
-                    if constexpr (EXACT) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const bool finite = fabsf(f[i]) <= 3.402823466e+38f;
-                            f[i] = finite ? f[i] : 0.0f;
-                            odd |= !finite;
-                        }
-                    }
 #pragma unroll
                     for (int i = 0; i < 4; ++i) f[i] *= scale[u];
                     if constexpr (!EXACT) most = dg_max_abs(dg_max_abs(most, f[0], f[1]), f[2], f[3]);
@@ -304,30 +368,42 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
                     dg_st<2 * KP * 128>(dst, __byte_perm(t0, t2, 0x7632) ^ 0x80808080u);
                     dg_st<3 * KP * 128>(dst, __byte_perm(t0, t2, 0x5410) ^ 0x80808080u);
                 }
+            if constexpr (!EXACT) {
+                if (__any_sync(0xFFFFFFFFu, !(most <= 1073741824.0f))) {
+                    // beyond the bound (or not finite): the tile is left out, and comes again under other scales
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        if ((live >> u) & 1u) look(u, x[u], rowtop, 1);
+                    if (lane == 0) {
+                        atomicOr(&beyond_map[(n - n0) >> 5], 1u << ((n - n0) & 31));
+                        *(volatile int *)&beyond_buffer[buffer] = 1;
+                    }
+                    __syncwarp();
+                }
+            }
             if (++chunk == CH) {
                 tc_fence_async_smem();
                 __syncwarp();
                 if (lane == 0) tc_mbar_arrive(&full[buffer]);
                 ++done_tiles;
                 chunk = 0;
-                ++v;
+                if (EXACT) n = next_beyond(n + TEAMS);
+                else n = ++v < count ? n0 + team + (v == first ? 0 : v) * TEAMS : n1;
             }
-            if (v < count) fetch(full_tag, n0 + team + visit(v, count) * TEAMS, chunk);
-        }
-        odd |= !(most <= 1073741824.0f);
-        if (__any_sync(0xFFFFFFFFu, odd) && lane == 0) {
-            if (EXACT) nonfinite_s = 1;
-            else over_s = 1;
+            if (n < n1) fetch(full_tag, n, chunk);
         }
     };
     // MMAs of `total` tiles in the order they come, by lane 0 of the issuing warp; back when all are complete (or a wait gave
-    // up).  Lane b looks at buffer b's barrier.  (In a fixed order the teams wait for one another: 32 x 2 M 69 us for 59.)
+    // up).  Tiles with a value beyond its bound are passed over.  Lane b looks at buffer b's barrier.  (In a fixed order the teams wait for one another: 32 x 2 M 69 us for 59.)
     auto issue_tiles = [&](int total) {
         uint32_t accumulate = 0;
         while (total > 0) {
             unsigned int ready = 0;
+            bool beyond = false;
             for (unsigned int idle = 0; idle <= a.wait_limit; ++idle) {
-                ready = __ballot_sync(0xFFFFFFFFu, dg_mbar_test(&full[lane < NB ? lane : 0], phase) && lane < NB);
+                const bool here = dg_mbar_test(&full[lane < NB ? lane : 0], phase) && lane < NB;
+                beyond = *(volatile int *)&beyond_buffer[lane < NB ? lane : 0] != 0 && here;
+                ready = __ballot_sync(0xFFFFFFFFu, here);
                 if (ready || __any_sync(0xFFFFFFFFu, *abort_flag)) break;
                 __nanosleep(32);                        // (without it the polls take issue slots from the conversion: 3 us on short calls)
             }
@@ -337,6 +413,12 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
             }
             phase ^= (ready >> lane) & 1u;
             total -= __popc(ready);
+            if (beyond) {
+                // (no MMA reads this buffer: it is free at once)
+                *(volatile int *)&beyond_buffer[lane] = 0;
+                tc_mbar_arrive(&empty[lane]);
+            }
+            ready &= ~__ballot_sync(0xFFFFFFFFu, beyond);
             __syncwarp();
             tc_fence_after_sync();
             for (; ready; ready &= ready - 1u) {
@@ -360,6 +442,7 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
         if (dg_elect()) tc_commit(&drained);            // (the lane that issued the MMAs)
         __syncwarp();
         if (lane == 0) {
+            issued_s = (int)accumulate;
             // (this last commit arrives when everything issued so far has completed: also before tensor memory is freed after a
             // wait that gave up)
             bool complete = false;
@@ -369,11 +452,12 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
         ++n_drained;
     };
 
-    // The sums of a period out of tensor memory, put together and added to what the periods before it left.
+    // The sums of what was issued out of tensor memory, put together and added to what came before.
     auto collect = [&](bool first) {
+        const bool any = issued_s != 0;
         constexpr int P = KP + 1;                       // (a pitch of 2 banks between rows)
         double *red = reinterpret_cast<double *>(tiles);
-        if (n_mine > 0 && warp < W) {
+        if (any && warp < W) {
             const int row = (warp & 3) * 32 + lane, s = row / KP % 4;
             const bool valid = row < S::kRowsValid;
             const double weight = dg_pow2(24 - 8 * s), weight2 = dg_pow2(8 - 8 * s);
@@ -416,7 +500,7 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
             const int i = ti * 8 + ((e >> 3) & 7), j = tj * 8 + (e & 7);
             if (i > j || j >= K) continue;
             double v = 0.0;
-            if (n_mine > 0) {
+            if (any) {
                 if constexpr (S::kTwo) {
                     const double *const low = red + (size_t)2 * KP * P;
 #pragma unroll
@@ -441,39 +525,99 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
         __syncthreads();
     };
 
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        for (int n0 = 0; n0 == 0 || n0 < n_mine; n0 += S::kPeriodTiles) {
-            const int n1 = min(n_mine, n0 + S::kPeriodTiles);
-            if (warp < W) {
-                if (attempt == 1) convert_tiles(std::true_type(), std::false_type(), n0, n1, false);
-                else if (row0 + 8 <= K) convert_tiles(std::false_type(), std::true_type(), n0, n1, n0 == 0);
-                else convert_tiles(std::false_type(), std::false_type(), n0, n1, n0 == 0);
-            } else {
-                issue_tiles(n1 - n0);
-            }
-            __syncwarp();
-            tc_fence_before_sync();
-            __syncthreads();
-            tc_fence_after_sync();
-            if (abort_s || (attempt == 0 && over_s)) break;     // (the same for every thread)
-            collect(n0 == 0);
-        }
-        if (abort_s || !over_s || attempt == 1) break;
-        // a sum of four beyond its bound: the largest finite magnitude of every gradient's share, and again
-        for (int r = tid; r < KP; r += S::kThreads) rowmax[r] = 0u;
+    // Gradients with NaNs and infinities: NaN for all products of the former; the products of infinities with the other gradients, infinite or
+    // NaN whatever the order, from the period's tiles beyond their bounds or, of a gradient that was left out from the start, from all.
+    // Once all products of a gradient are known to be NaN, or infinite of both signs, it is not looked at any more.
+    auto nonfinite_products = [&](int n0, int n1) {
+        unsigned long long *const pos_of = reinterpret_cast<unsigned long long *>(tiles), *const neg_of = pos_of + KP, *const nan_of = neg_of + KP;
+        for (int r = tid; r < 3 * KP; r += S::kThreads) pos_of[r] = 0ull;       // (bit j of word i; the tile buffers are free here)
         __syncthreads();
-        if (warp < W)
-            for (int n = team * CH; n < n_mine * CH; n += (n + 1) % CH == 0 ? (TEAMS - 1) * CH + 1 : 1) {
-                const int64_t q = min(quad_of(n / CH) + (n % CH) * 32 + lane, n_quads - 1);
+        const unsigned long long nans = nan_rows[0] | nan_rows[1], infs = inf_rows[0] | inf_rows[1], all = K == 64 ? ~0ull : (1ull << K) - 1ull;
+        for (int t = warp; warp < W && infs && t < (n1 - n0) * CH; t += W) {
+            const int64_t q = quad_of(n0 + t / CH) + (t % CH) * 32 + lane;
+            const bool inside = q < n_quads;
+            unsigned long long rows = (inf_rows[0] | (is_beyond(t / CH) ? inf_rows[1] : 0ull)) & ~nans;
+            for (; rows; rows &= rows - 1ull) {
+                const int r = __ffsll((long long)rows) - 1;
+                const unsigned long long known = *(volatile unsigned long long *)&nan_of[r] |
+                    (*(volatile unsigned long long *)&pos_of[r] & *(volatile unsigned long long *)&neg_of[r]) | (1ull << r) | nans;
+                if (!__any_sync(0xFFFFFFFFu, (~known & all) != 0ull)) continue;
+                const float4 f = inside ? reinterpret_cast<const float4 *>(a.g[r])[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+                const float xs[4] = {f.x, f.y, f.z, f.w};
+                if (!__any_sync(0xFFFFFFFFu, isinf(xs[0]) || isinf(xs[1]) || isinf(xs[2]) || isinf(xs[3]))) continue;
+                for (int j0 = 0; j0 < K; j0 += 4) {
+                    float4 g[4];                    // (loads in flight together)
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const unsigned int top = __reduce_max_sync(0xFFFFFFFFu, finite_max(ld16_policy(row(row0 + u < K ? u : -row0) + q * 16, policy)));
-                    if (lane == 0) atomicMax(&rowmax[row0 + u], top);
+                    for (int k = 0; k < 4; ++k)
+                        g[k] = inside && j0 + k < K ? reinterpret_cast<const float4 *>(a.g[j0 + k])[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float ys[4] = {g[k].x, g[k].y, g[k].z, g[k].w};
+                        bool pos = false, neg = false, nan = false;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float p = isinf(xs[i]) ? xs[i] * ys[i] : 0.0f;
+                            pos |= p > 0.0f; neg |= p < 0.0f; nan |= isnan(p);
+                        }
+                        pos = __any_sync(0xFFFFFFFFu, pos); neg = __any_sync(0xFFFFFFFFu, neg); nan = __any_sync(0xFFFFFFFFu, nan);
+                        const unsigned long long bit = lane == 0 && j0 + k < K ? 1ull << (j0 + k) : 0ull;
+                        if (pos && bit) atomicOr(&pos_of[r], bit);
+                        if (neg && bit) atomicOr(&neg_of[r], bit);
+                        if (nan && bit) atomicOr(&nan_of[r], bit);
+                    }
                 }
             }
+        }
         __syncthreads();
-        for (int r = tid; r < K; r += S::kThreads) expo[r] = dg_exponent(rowmax[r], 0);
+        for (int e = tid; e < a.pairs * 64; e += S::kThreads) {      // (the slots that this thread wrote)
+            int ti, tj;
+            tile_pair(e >> 6, a.tiles, ti, tj);
+            const int i = ti * 8 + ((e >> 3) & 7), j = tj * 8 + (e & 7);
+            if (i > j || j >= K) continue;
+            double *const dst = a.partials + ((size_t)(e >> 6) * gridDim.x + blockIdx.x) * 64 + (e & 63);
+            const double inf = __longlong_as_double(0x7FF0000000000000ll);
+            auto bit = [&](const unsigned long long *w) { return (((w[i] >> j) | (w[j] >> i)) & 1ull) != 0ull; };
+            const bool pos = i == j ? (infs >> i) & 1ull : bit(pos_of), neg = i != j && bit(neg_of);
+            if (((nans >> i) | (nans >> j)) & 1ull || (i != j && bit(nan_of))) *dst = __longlong_as_double(0x7FF8000000000000ll);
+            else *dst += (pos ? inf : 0.0) - (neg ? inf : 0.0);
+        }
         __syncthreads();
+    };
+    // (every thread takes the same turns: the conditions are read behind a barrier)
+    auto convert_and_issue = [&](auto exact_tag, int n0, int n1, int total) {
+        if (warp < W) {
+            if (!decltype(exact_tag)::value && live == 0xFFu) convert_tiles(std::false_type(), std::true_type(), n0, n1);
+            else convert_tiles(exact_tag, std::false_type(), n0, n1);
+        } else {
+            issue_tiles(total);
+        }
+        __syncwarp();
+        tc_fence_before_sync();
+        __syncthreads();
+        tc_fence_after_sync();
+    };
+    for (int n0 = 0; n0 == 0 || n0 < n_mine; n0 += S::kPeriodTiles) {
+        const int n1 = min(n_mine, n0 + S::kPeriodTiles);
+        if (n0 > 0) {
+            clear_period();
+            if (tid == 0) { nan_rows[0] |= nan_rows[1]; inf_rows[0] |= inf_rows[1]; }
+            __syncthreads();
+        }
+        sample(n0, n1);
+        update_live(nan_rows[0] | inf_rows[0]);
+        if (tid < KP) expo[tid] = dg_exponent(rowmax[tid], kDgHeadroom);        // (read behind the next barrier)
+        convert_and_issue(std::false_type(), n0, n1, n1 - n0);
+        if (abort_s) break;
+        const int beyond = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned int)__popc(beyond_map[lane]));
+        collect(n0 == 0);
+        if (beyond) {
+            update_live(nan_rows[0] | nan_rows[1] | inf_rows[0] | inf_rows[1]);
+            if (tid < KP) expo[tid] = min(expo[tid], dg_exponent(rowtop[tid], 0));
+            convert_and_issue(std::true_type(), n0, n1, beyond);
+            if (abort_s) break;
+            collect(false);
+        }
+        if (nan_rows[0] | nan_rows[1] | inf_rows[0] | inf_rows[1]) nonfinite_products(n0, n1);
     }
     // the streaming part of this CTA is over: the finishing kernel may be placed (it waits for this grid)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -484,26 +628,6 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
     if (abort_s) {
         if (tid == 0) atomicOr(&a.ctl->status, kStatusTimeoutBit);
         return;
-    }
-    if (nonfinite_s && warp < W) {
-        auto slot_of = [&](int i, int j) {
-            const int ti = i >> 3, tj = j >> 3, tp = ti * a.tiles - ti * (ti - 1) / 2 + (tj - ti);
-            return a.partials + ((size_t)tp * gridDim.x + blockIdx.x) * 64 + (i & 7) * 8 + (j & 7);
-        };
-        // the products of infinities and NaNs, element by element: infinite or NaN, whatever the order
-        for (int n = warp; n < n_mine * CH; n += W) {
-            const int64_t off = (quad_of(n / CH) + (n % CH) * 32 + lane) * 16;
-            if (off >= n_quads * 16) continue;
-            for (int r = 0; r < K; ++r)
-                for (int i = 0; i < 4; ++i) {
-                    const float v = *reinterpret_cast<const float *>(reinterpret_cast<const unsigned char *>(a.g[r]) + off + 4 * i);
-                    if (fabsf(v) <= 3.402823466e+38f) continue;
-                    for (int j = 0; j < K; ++j) {
-                        const float y = *reinterpret_cast<const float *>(reinterpret_cast<const unsigned char *>(a.g[j]) + off + 4 * i);
-                        atomicAdd(slot_of(min(r, j), max(r, j)), (double)v * (double)y);
-                    }
-                }
-        }
     }
 }
 
