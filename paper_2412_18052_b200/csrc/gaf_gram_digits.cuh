@@ -275,16 +275,33 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
         }
     };
     // What v holds of the warp's gradient u, 32 pieces of it: the largest finite magnitude, a NaN, an infinity.
-    auto look = [&](int u, const uint4 &v, unsigned int *top, int when) {
+    auto note = [&](int u, const uint4 &v, unsigned int *top, int when) {
         const unsigned int m[4] = {v.x & 0x7FFFFFFFu, v.y & 0x7FFFFFFFu, v.z & 0x7FFFFFFFu, v.w & 0x7FFFFFFFu};
         const unsigned int finite = __reduce_max_sync(0xFFFFFFFFu, finite_max(v));
-        const unsigned int any = __reduce_max_sync(0xFFFFFFFFu, max(max(m[0], m[1]), max(m[2], m[3])));
-        if (any >= 0x7F800000u) {
-            const bool inf = __any_sync(0xFFFFFFFFu, m[0] == 0x7F800000u || m[1] == 0x7F800000u || m[2] == 0x7F800000u || m[3] == 0x7F800000u);
-            if (lane == 0 && any > 0x7F800000u) atomicOr(&nan_rows[when], 1ull << (row0 + u));
-            if (lane == 0 && inf) atomicOr(&inf_rows[when], 1ull << (row0 + u));
+        const bool nan = __any_sync(0xFFFFFFFFu, max(max(m[0], m[1]), max(m[2], m[3])) > 0x7F800000u);
+        const bool inf = __any_sync(0xFFFFFFFFu, m[0] == 0x7F800000u || m[1] == 0x7F800000u || m[2] == 0x7F800000u || m[3] == 0x7F800000u);
+        if (lane == 0) {
+            if (nan) atomicOr(&nan_rows[when], 1ull << (row0 + u));
+            if (inf) atomicOr(&inf_rows[when], 1ull << (row0 + u));
+            atomicMax(&top[row0 + u], finite);
         }
-        if (lane == 0) atomicMax(&top[row0 + u], finite);
+    };
+    // The same of all that x holds, for the sample.
+    auto note_all = [&]() {
+        unsigned int most[8], mine = 0u;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            most[u] = __reduce_max_sync(0xFFFFFFFFu, max(max(x[u].x & 0x7FFFFFFFu, x[u].y & 0x7FFFFFFFu), max(x[u].z & 0x7FFFFFFFu, x[u].w & 0x7FFFFFFFu)));
+#pragma unroll
+        for (int u = 0; u < 8; ++u) mine = lane == u ? most[u] : mine;
+        const bool takes_part = lane < 8 && ((live >> lane) & 1u);
+        if (!__any_sync(0xFFFFFFFFu, takes_part && mine >= 0x7F800000u)) {
+            if (takes_part) atomicMax(&rowmax[row0 + lane], mine);
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if ((live >> u) & 1u) note(u, x[u], rowmax, 0);
+        }
     };
     // The period's scales come from the first tiles of its teams, and for a gradient that has nothing but zeros there, from single pieces of
     // 16 bytes, 32 times as many places.
@@ -295,9 +312,7 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
             const int n = n0 + team + first_of(count) * TEAMS;
             if (live == 0xFFu) fetch(std::true_type(), n, 0);
             else fetch(std::false_type(), n, 0);
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if ((live >> u) & 1u) look(u, x[u], rowmax, 0);
+            note_all();
         }
         __syncthreads();
         const unsigned long long odd = nan_rows[0] | inf_rows[0];
@@ -310,7 +325,7 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
             const int at = (int)((unsigned int)count * ((unsigned int)lane * 4096u + place) / (32u * 4096u));
             const int64_t q = min(quad_of(n0 + team + at * TEAMS) + (int)((place + (unsigned int)lane * 11u) % (CH * 32u)), n_quads - 1);
             for (int u = 0; u < 8; ++u)
-                if ((dark >> u) & 1u) look(u, ld16_policy(row(u) + q * 16, policy), rowmax, 0);
+                if ((dark >> u) & 1u) note(u, ld16_policy(row(u) + q * 16, policy), rowmax, 0);
         }
         __syncthreads();
     };
@@ -330,19 +345,16 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
             scale[u] = __uint_as_float((unsigned int)(k + 127) << 23);
         }
         const int count = tiles_of(n0, n1);
-        auto next_beyond = [&](int n) {
-            while (n < n1 && !is_beyond(n - n0)) n += TEAMS;
-            return n;
+        // v: how many tiles the team is through; EXACT: its tile, counted within the period
+        const int first = first_of(count), end = EXACT ? n1 - n0 : count;
+        auto tile_at = [&](int v) { return EXACT ? v : team + (v == 0 ? first : v == first ? 0 : v) * TEAMS; };
+        auto next_beyond = [&](int t) {
+            while (t < end && !is_beyond(t)) t += TEAMS;
+            return t;
         };
-        const int first = first_of(count);
-        int v = 0, n = n1;
-        if (EXACT) {
-            n = next_beyond(n0 + team);
-            if (n < n1) fetch(full_tag, n, 0);
-        } else if (count > 0) {
-            n = n0 + team + first * TEAMS;
-        }
-        for (int chunk = 0; n < n1;) {
+        int v = EXACT ? next_beyond(team) : 0;
+        if (EXACT && v < end) fetch(full_tag, n0 + v, 0);
+        for (int chunk = 0; v < end;) {
             const int buffer = team * TB + (int)(done_tiles % TB);
             // the MMAs on what this buffer held before are complete
             if (chunk == 0 && done_tiles >= TB && !__all_sync(0xFFFFFFFFu, dg_mbar_wait(&empty[buffer], (done_tiles / TB - 1) & 1u, abort_flag, kDgPollLimit))) break;
@@ -373,9 +385,10 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
                     // beyond the bound (or not finite): the tile is left out, and comes again under other scales
 #pragma unroll
                     for (int u = 0; u < 8; ++u)
-                        if ((live >> u) & 1u) look(u, x[u], rowtop, 1);
+                        if (FULL || ((live >> u) & 1u)) note(u, x[u], rowtop, 1);
                     if (lane == 0) {
-                        atomicOr(&beyond_map[(n - n0) >> 5], 1u << ((n - n0) & 31));
+                        const int t = tile_at(v);
+                        atomicOr(&beyond_map[t >> 5], 1u << (t & 31));
                         *(volatile int *)&beyond_buffer[buffer] = 1;
                     }
                     __syncwarp();
@@ -387,10 +400,9 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
                 if (lane == 0) tc_mbar_arrive(&full[buffer]);
                 ++done_tiles;
                 chunk = 0;
-                if (EXACT) n = next_beyond(n + TEAMS);
-                else n = ++v < count ? n0 + team + (v == first ? 0 : v) * TEAMS : n1;
+                v = EXACT ? next_beyond(v + TEAMS) : v + 1;
             }
-            if (n < n1) fetch(full_tag, n, chunk);
+            if (v < end) fetch(full_tag, n0 + tile_at(v), chunk);
         }
     };
     // MMAs of `total` tiles in the order they come, by lane 0 of the issuing warp; back when all are complete (or a wait gave
