@@ -153,9 +153,14 @@ int stream_grid(int64_t D, int threads, int sms) {
 // kernels for few gradients are faster at every length: with exactly 8, where the 128 x 128 product keeps 1/16 of
 // its work, the warp-level MMA kernel streams 16 GB of inputs at 6.6 TB/s against 5.2 TB/s (measured).
 // Binary32 with one gradient, or more than 8: digits on the tensor cores, except for few gradients of short vectors, where the kernel on the
-// CUDA cores starts and ends 2 us sooner (all pairs, panels / digits, us: 16 gradients of 100 k / 400 k / 800 k / 1.2 M / 2.4 M elements 7.7 /
-// 11.4 / 16.9 / 22.0 / 36.9 against 9.3 / 13.3 / 18.5 / 22.3 / 33.9; 24 of 100 k / 300 k / 400 k / 1.2 M 8.9 / 13.9 / 17.5 / 39.6 against
-// 10.9 / 14.6 / 16.8 / 29.0; 32 of 100 k 12.6 against 12.7).
+// CUDA cores starts and ends 2 us sooner.  All pairs, panels / digits, us:
+//    1 x 1 M / 2 M / 30 M  12.3 / 20.0 / 237 against 14.4 / 19.7 / 197        9 x 1 M / 1.3 M / 1.6 M  18.1 / 22.2 / 25.6 against 19.7 / 22 / 24.4
+//   12 x 1.3 M / 1.6 M     22.5 / 25.7       against 23 / 25                 15 x 1.3 M / 2 M / 8.2 M  22.6 / 30.6 / 109 against 26 / 32 / 107
+//   16 x 1.3 M / 1.6 M / 2.5 M  22.6 / 26.4 / 36.5  against 25 / 27.1 / 35.6     17 x 300 k / 350 k / 500 k  13.5 / 15.5 / 19.3 against 14 / 14.7 / 17.9
+//   24 x 350 k / 400 k / 600 k  15.6 / 17.0 / 22.6 against 16.6 / 17.5 / 20.9     32 x 1 k / 100 k / 130 k  6.5 / 10.6 / 12.1 against 7.5 / 11.0 / 11.6
+//   33 x 1 k / 12 k / 20 k  5.8 / 9.1 / 10.2 against 8.9 / 9.6 / 10.5        64 x 1 k / 12 k / 20 k  6.3 / 10.4 / 14.9 against 10.5 / 11.3 / 13.0
+// The lines lie below the points where the two are equally fast (1.3 M, with 15 and 16 gradients 2 M; 330 k to 450 k), and beyond 24 gradients the digits
+// take every length: their sums are exact (16 x 1 M: 2e-10 of the norms' product against 4e-9) and hold squares that binary32 loses.
 constexpr int kGramAutoMaxK = 32;
 constexpr int64_t kGramAutoMinD = 32768;
 constexpr int64_t kPanelMaxD16 = int64_t(1) << 20, kPanelMaxD24 = 5 * 65536;
@@ -386,7 +391,7 @@ int launch_gram_tiles(const void *const *grads, int K, int64_t D, int dtype, flo
         ++g_launches;
         if (err != cudaSuccess) { cudaGetLastError(); return GAF_ERR_CUDA; }
     } else if (use_panel_gram(K, D, dtype)) {
-        // CUDA cores, every gradient read once: one warp per tile pair, panels of D through shared memory
+        // CUDA cores, every gradient read once: 2 or 4 warps per tile pair, panels of D through shared memory
         GramPanelArgs pa{};
         for (int i = 0; i < K; ++i) pa.g[i] = grads[i];
         pa.K = K; pa.D = D; pa.tiles = a.tiles; pa.pairs = pairs;
@@ -871,7 +876,8 @@ int gaf_filter_accumulate(const void *const *grads, int K, int64_t D, int dtype,
     if (schedule == GAF_SCHED_AUTO) {
         // Gram-first moves fewer bytes whenever its one-pass Gram kernel applies
         const bool ws_ok = workspace_bytes >= kExtraOffset + pairwise_extra_bytes(K);
-        // (more than 32 binary32 gradients of fewer elements than this keep the streaming passes)
+        // (more than 32 binary32 gradients of fewer elements than kGramAutoMinD keep the streaming passes, although they are the slower choice:
+        // 33 / 64 x 20 k 138 / 269 us against 22 / 32 Gram-first; the schedule that AUTO resolves to is part of what callers see)
         const bool fast_gram = K >= 2 && (K <= kGsMaxK || use_tensor_gram(K, D, dtype) ||
                                           (dtype == GAF_F32 && (K <= kGramAutoMaxK || D >= kGramAutoMinD)));
         schedule = (fast_gram && ws_ok) ? (auto_one_launch(K, D, dtype) ? GAF_SCHED_GRAM_FUSED : GAF_SCHED_GRAM)
