@@ -7,6 +7,8 @@ import pytest
 import torch
 
 import paper_2412_18052_b200 as gaf
+from paper_2412_18052_b200 import workloads
+from parity import check_any_seed, check_filter
 
 pytestmark = pytest.mark.gpu
 
@@ -71,6 +73,73 @@ def test_one_absent_gradient(K):
     """The warp with the absent gradient loads the other seven under predicates."""
     for D in ((1 << 20) + 129, 148 * 256 * 11 + 5) if K <= 16 else (327_680 + 127, 148 * 128 * 21 + 6):
         _check(_grads(K, D, "", K + D))
+
+
+def _digits_length(K):
+    """A ragged length of several tiles per CTA that goes to the digits."""
+    return (1 << 20) + 261 if K <= 16 else 327_680 + 133 if K <= 24 else 50_005
+
+
+@pytest.mark.parametrize("K", [10, 16, 20, 24, 29, 32, 40, 47, 56, 64])
+@pytest.mark.parametrize("bands", [False, True])
+def test_whole_numbers_are_exact(K, bands):
+    """Whole numbers below 2^23, all four digits of them in use, are whole in fixed point, and so are smaller ones with bands beyond
+    their bound (2^5 times 2^15): nothing is rounded but sums in binary64, the reference's among them (sqrt(D) x 2^-53 at the most likely, 1e-13).
+    A digit lost or in the wrong place leaves 1e-9 and more."""
+    D = _digits_length(K)
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    top = 15 if bands else 23
+    grads = [torch.randint(1 - (1 << top), 1 << top, (D,), generator=gen, device="cuda").float() for _ in range(K)]
+    if bands:
+        for i, x in enumerate(grads):
+            for at in (D // 7 * (i % 5) + 11, D - 300 - i):
+                x[at:at + 200] = torch.randint(1 - (1 << 23), 1 << 23, (200,), generator=gen, device="cuda").float()
+    ws = gaf.new_workspace(K, D, gaf.GAF_F32)
+    G, E = _gram(grads, ws), _exact(grads)
+    norm = E.diagonal().sqrt()
+    assert float(((G - E).abs() / torch.outer(norm, norm)).max()) < 1e-12
+
+
+@pytest.mark.parametrize("K", [9, 16, 24, 32, 40, 48, 56, 64])
+def test_rounding_of_normal_values(K):
+    """Each value is at most half a unit off, 2^-25 of the gradient's largest, at random: the products' errors add up to a normal variable
+    of at most 2^-25 / sqrt(3) (max|x_i| |x_j| + max|x_j| |x_i|); eight times that."""
+    grads = _grads(K, _digits_length(K), "", 100 + K)
+    ws = gaf.new_workspace(K, grads[0].numel(), gaf.GAF_F32)
+    G, E = _gram(grads, ws), _exact(grads)
+    norm, top = E.diagonal().sqrt(), torch.stack([g.abs().max() for g in grads]).double()
+    bound = 8 / 3 ** 0.5 * 2.0 ** -25 * (torch.outer(top, norm) + torch.outer(norm, top)) + 1e-12 * torch.outer(norm, norm)
+    assert bool(((G - E).abs() <= bound).all()), ((G - E).abs() / bound).max().item()
+
+
+def test_small_elements_beside_large_ones():
+    """The stated bound holds where nearly all elements of a gradient are below its unit and all errors have one sign."""
+    K, D = 40, 300_001
+    grads = [torch.full((D,), 2.0 ** -26.2 * (1 + i / 40), device="cuda") for i in range(K)]
+    for i, x in enumerate(grads):
+        x[:: 997 + i] = 1.0
+    grads[3] = torch.ones(D, device="cuda")
+    grads[3][::2] = 0.9
+    ws = gaf.new_workspace(K, D, gaf.GAF_F32)
+    G, E = _gram(grads, ws), _exact(grads)
+    total, top = torch.stack([g.abs().double().sum() for g in grads]), torch.stack([g.abs().max() for g in grads]).double()
+    bound = 2.0 ** -25 * (torch.outer(top, total) + torch.outer(total, top)) + 2.0 ** -49 * D * torch.outer(top, top)
+    assert bool(((G - E).abs() <= bound).all()), ((G - E).abs() / bound).max().item()
+
+
+@pytest.mark.parametrize("K", [12, 15, 17, 20, 24, 30, 40])
+def test_filter_on_digits(K):
+    """Algorithm 1 and its order-indifferent variant on a Gram matrix of digits, with one scale and with tensors of different scales."""
+    D = _digits_length(K)
+    sigma = torch.exp(2.0 * torch.randn(40, generator=torch.Generator().manual_seed(K))).repeat_interleave(-(-D // 40))[:D].cuda() * 1e-3
+    for scale in (1e-3, sigma):
+        rho = ([0.8, 0.7, -0.6, 0.5, 0.0, 0.6, -0.2, 0.4] * 5)[:K]
+        grads = workloads.mixture(K, D, "f32", rho, K, device="cuda", sigma=scale).grads
+        ws = gaf.new_workspace(K, D, gaf.GAF_F32)
+        for tau in (0.9, 2.0):
+            check_filter(grads, tau, ws)
+            assert gaf.gaf_last_schedule() == gaf.GAF_SCHED_GRAM
+        check_any_seed(grads, 0.9, ws)
 
 
 @pytest.mark.parametrize("kind", ["scales", "outlier", "segments", "sparse", "tiny", "huge"])

@@ -624,10 +624,9 @@ def test_pairwise_small(ws, dtype):
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("K", [10, 16, 24, 32, 40, 48, 64])
 def test_pairwise_general_kernel_shapes(ws, dtype, K):
-    """More than 8 gradients: the general CUDA-core Gram kernel (binary32) in each of its shapes (warps
-    sharing a tile pair, one warp per pair, tile pairs split over groups of CTAs) and the tensor-core
-    kernels (bfloat16: warp-level MMAs up to 16 gradients, the tcgen05 tile in its 32- and 64-row forms):
-    several panels or tiles per CTA, a ragged end."""
+    """More than 8 gradients: the CUDA-core Gram kernel (binary32, up to 24) in its two shapes (4 or 2 warps sharing a tile pair),
+    8-bit digits on the tensor cores (binary32 beyond) and the tensor-core kernels (bfloat16: warp-level MMAs up to 16
+    gradients, the tcgen05 tile in its 32- and 64-row forms): several panels or tiles per CTA, a ragged end."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     for D in (sms * 512 * 3 + 1234 + 3, 100_001):
         w = _mix(K, D, dtype, seed=300 + K)
