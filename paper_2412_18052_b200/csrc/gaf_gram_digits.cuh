@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
 #pragma unroll
         for (int u = 0; u < 8; ++u) mine = lane == u ? most[u] : mine;
         const bool takes_part = lane < 8 && ((live >> lane) & 1u);
-        if (!__any_sync(0xFFFFFFFFu, takes_part && mine >= 0x7F800000u)) {
+        if (__builtin_expect(!__any_sync(0xFFFFFFFFu, takes_part && mine >= 0x7F800000u), 1)) {
             if (takes_part) atomicMax(&rowmax[row0 + lane], mine);
         } else {
 #pragma unroll
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
         __syncthreads();
         const unsigned long long odd = nan_rows[0] | inf_rows[0];
         auto zeros = [&](int r) { return r < K && rowmax[r] == 0u && !((odd >> r) & 1ull); };
-        if (!__any_sync(0xFFFFFFFFu, zeros(lane) || zeros(lane + 32))) return;      // (the same for all warps)
+        if (__builtin_expect(!__any_sync(0xFFFFFFFFu, zeros(lane) || zeros(lane + 32)), 1)) return;      // (the same for all warps)
         unsigned int dark = 0u;
         for (int u = 0; u < 8; ++u) dark |= warp < W && count > 0 && zeros(row0 + u) ? 1u << u : 0u;
         __syncthreads();
@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
                     dg_st<3 * KP * 128>(dst, __byte_perm(t0, t2, 0x5410) ^ 0x80808080u);
                 }
             if constexpr (!EXACT) {
-                if (__any_sync(0xFFFFFFFFu, !(most <= 1073741824.0f))) {
+                if (__builtin_expect(__any_sync(0xFFFFFFFFu, !(most <= 1073741824.0f)), 0)) {
                     // beyond the bound (or not finite): the tile is left out, and comes again under other scales
 #pragma unroll
                     for (int u = 0; u < 8; ++u)
@@ -622,14 +622,14 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
         if (abort_s) break;
         const int beyond = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned int)__popc(beyond_map[lane]));
         collect(n0 == 0);
-        if (beyond) {
+        if (__builtin_expect(beyond != 0, 0)) {
             update_live(nan_rows[0] | nan_rows[1] | inf_rows[0] | inf_rows[1]);
             if (tid < KP) expo[tid] = min(expo[tid], dg_exponent(rowtop[tid], 0));
             convert_and_issue(std::true_type(), n0, n1, beyond);
             if (abort_s) break;
             collect(false);
         }
-        if (nan_rows[0] | nan_rows[1] | inf_rows[0] | inf_rows[1]) nonfinite_products(n0, n1);
+        if (__builtin_expect((nan_rows[0] | nan_rows[1] | inf_rows[0] | inf_rows[1]) != 0ull, 0)) nonfinite_products(n0, n1);
     }
     // the streaming part of this CTA is over: the finishing kernel may be placed (it waits for this grid)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
