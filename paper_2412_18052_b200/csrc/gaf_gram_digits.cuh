@@ -16,17 +16,17 @@
 // tiles left out come again, under scales that hold the largest of their values (half a unit: 2^-30 of it), and
 // their sums are added.  Which tiles these are depends on the values alone, so that results repeat bit for bit.
 // Gradients with infinities or NaNs are left out of the digits, the products of their infinities found afterwards.
-// What values of many sizes cost (all pairs of 16 x 11.2 M, 24 x 3 M, 32 x 11.2 M, 64 x 3 M, us, short runs one after the other, so that the power
-// state moves them by a tenth; when a tile beyond its bound was noticed at the end only, the CTA did its whole share again):
+// What values of many sizes cost (all pairs of 16 x 11.2 M, 24 x 3 M, 32 x 11.2 M, 64 x 3 M, us, short runs; when a tile beyond its bound was
+// noticed at the end only, the CTA did its whole share again):
 //                                                          here            whole share           binary32 pipes
-//     normal values                                  123  56 241 155     122   54  237  139     140  89 458 521
-//     one element of 10^6                            150  74 258 150     473  144  686  496     142  90 459 522
-//     lognormal, sigma 2                             128  67 251 171     478  151  748  535     142  89 459 522
-//     97 % of all rows of 512 elements zero          143  69 253 163     489  159  739  518     140  89 458 521
-//     200 tensors with lognormal scales, sigma 2     127  60 253 153     482  156  767  553     140  89 458 521
-//     6 % of the vector 1000 times as large          126  76 285 184     504   56  231  557     142  92 459 522
-//     one gradient of NaNs                           162  72 302 175    3426 1212 8184 2880     148  93 459 523
-//     infinities in a gradient                       152  85 321 231    1305  544 2583 1524     141  89 459 523
+//     normal values                                  121  57 238 140     122   54  237  139     140  89 459 522
+//     one element of 10^6                            122  58 239 142     470  145  686  496     141  89 459 522
+//     lognormal, sigma 2                             121  60 238 145     480  151  743  524     141  89 459 522
+//     97 % of all rows of 512 elements zero          128  69 246 158     492  160  742  521     140  89 459 522
+//     200 tensors with lognormal scales, sigma 2     124  60 245 145     485  157  766  530     140  89 459 522
+//     6 % of the vector 1000 times as large          117  64 260 155     494   55  240  529     140  89 459 522
+//     one gradient of NaNs                           119  58 247 141    3417 1201 7912 2905     141  89 459 523
+//     infinities in a gradient                       135  79 274 196    1309  546 2588 1522     141  89 459 523
 // Work split.  One CTA per SM.  A tile is 128 consecutive elements of all K gradients (256 up to 16); tiles are dealt round-robin to the
 // CTAs, and inside a CTA to teams of KP / 8 warps.  Every warp of a team has eight gradients for the whole kernel (their
 // addresses and scales stay in registers); it reads 512 consecutive bytes of each, writes their digits into the team's tile
@@ -36,11 +36,13 @@
 // among themselves (what is missing of the 4 KP x 4 KP products then is the mirror image of something present).
 // Rows of absent gradients, and the rows of the 128 beyond 4 KP, hold whatever the memory holds: their sums are not read.
 //
-// Bound by HBM in short runs, by the power cap in long ones (tensor pipe 36 % busy, issue slots 55 %).  All pairs, D = 11.2 M, against the
-// kernel on the binary32 pipes (bound by these and by shared memory): 9 / 16 / 24 / 32 / 40 / 64 gradients 142 / 140 / 307 / 459 / 903 / 1954 us, now
-// 98 / 120 / 205 / 245 / 325 / 508; a second of calls on end 16 / 24 x 3 M / 32 gradients 153 / 88 / 459, now 148 / 64 / 287 (the SM
+// Bound by the conversion up to 9 gradients (0.61 of the copy rate), by HBM in short runs from there on (16 gradients 0.91, 24 and more 0.88 to 0.93; 24 x 3 M 0.77,
+// with 8 us of launch, first tiles and last sums), by the power cap in long ones (24 x 3 M: tensor pipe 33 % busy, issue slots 52 %).  All pairs, D = 11.2 M, against
+// the kernel on the binary32 pipes (bound by these and by shared memory): 9 / 15 / 16 / 24 / 32 / 40 / 64 gradients 143 / 141 / 140 / 306 / 459 / 901 / 1905 us,
+// now 102 / 118 / 121 / 183 / 238 / 320 / 501; a second of calls on end 142 / 143 / 145 / 306 / 459 / 901 / 1947, now 112 / 135 / 138 / 211 / 277 / 369 / 581 (the SM
 // clock falls to 1.1 to 1.5 GHz).  What decided the shape: loads under a branch, or in a ring of single registers, wait for one another
-// (32 gradients: 900 us; the warp with the absent gradients loads under predicates: 15 x 8.2 M 112 -> 107, binary32 pipes 109); eight gradients for the whole kernel per warp, 20 warps and more (300 -> 265); the MMAs issued by a converged warp with
+// (32 gradients: 900 us; a warp with absent gradients loads under predicates and
+// converts zeros for them, without a branch: 15 / 31 x 8.2 M 108 / 220 us with branches, 100 / 198 so, binary32 pipes 105 / 338); eight gradients for the whole kernel per warp, 20 warps and more (300 -> 265); the MMAs issued by a converged warp with
 // an elected lane (their operands are scalars then; 16 gradients 147 -> 118 with two chunks a product).  Products of 64 rows, which waste less, cost the
 // same time and no less power.  The mean written meanwhile under the pattern of a sample: 16 x 11.2 M 199 us, 179 with a pass of its own.
 #pragma once
@@ -57,6 +59,10 @@ constexpr int kDgChunk = 128;                   // elements of a digit row in on
 constexpr int kDgHeadroom = 5;                  // bits between the largest sampled magnitude and the bound
 constexpr unsigned int kDgPollLimit = 1u << 23; // looks at all barriers without a tile: a second
 constexpr int kDgMaxChain = 1023;               // chunks: 1023 x 128 products of at most 2^14 fit a 32-bit sum
+
+// How a warp goes through a tile: all of its eight gradients; some of them, loads under predicates and zeros for the others; or none beyond the fourth.
+enum { kDgAll, kDgSome, kDgFour };
+template <int FORM> using DigitsForm = std::integral_constant<int, FORM>;
 
 template <int KP> struct DigitsShape {
     // Chunks of 128 elements of a tile.  Up to 16 gradients two of them lie one above the other in the 128 rows of a product, each
@@ -257,21 +263,26 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
     unsigned int live = 0u;
     auto update_live = [&](unsigned long long odd) {
         const int here = min(max(K - row0, 0), 8);
-        live = warp < W ? ((1u << here) - 1u) & ~(unsigned int)(odd >> row0) : 0u;
+        const unsigned int mask = warp < W ? ((1u << here) - 1u) & ~(unsigned int)(odd >> row0) : 0u;
+        live = __shfl_sync(0xFFFFFFFFu, mask, 0);           // (known to be the same in all lanes, as `warp` is)
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (!((live >> u) & 1u)) x[u] = make_uint4(0u, 0u, 0u, 0u);         // (and stays so: loads are under predicates)
     };
-    auto fetch = [&](auto full_tag, int n, int chunk) {
+    auto fetch = [&](auto form, int n, int chunk) {
+        constexpr int ROWS = decltype(form)::value == kDgFour ? 4 : 8;
         const int64_t q = quad_of(n) + chunk * 32, left = n_quads - q;
         // lanes past the end of the vectors read the last four elements and count them as zeros
         const bool inside = lane < left;
         const int mine = inside ? lane * 16 : ((int)left - 1) * 16;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if constexpr (decltype(full_tag)::value) x[u] = ld16_policy(row(u) + q * 16 + mine, policy);
+        for (int u = 0; u < ROWS; ++u) {
+            if constexpr (decltype(form)::value == kDgAll) x[u] = ld16_policy(row(u) + q * 16 + mine, policy);
             else dg_ld16_if(x[u], (live >> u) & 1u, row(u) + q * 16 + mine, policy);
         }
         if (left < 32) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) x[u] = inside ? x[u] : make_uint4(0u, 0u, 0u, 0u);
+            for (int u = 0; u < ROWS; ++u) x[u] = inside ? x[u] : make_uint4(0u, 0u, 0u, 0u);
         }
     };
     // What v holds of the warp's gradient u, 32 pieces of it: the largest finite magnitude, a NaN, an infinity.
@@ -310,8 +321,8 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
         const int count = tiles_of(n0, n1);
         if (warp < W && count > 0) {
             const int n = n0 + team + first_of(count) * TEAMS;
-            if (live == 0xFFu) fetch(std::true_type(), n, 0);
-            else fetch(std::false_type(), n, 0);
+            if (live == 0xFFu) fetch(DigitsForm<kDgAll>(), n, 0);
+            else fetch(DigitsForm<kDgSome>(), n, 0);
             note_all();
         }
         __syncthreads();
@@ -335,11 +346,12 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
     uint32_t phase = 0, n_drained = 0;                  // issuing warp: parity of the next tile in buffer `lane`; drains so far
     // This warp's digits of the team's tiles of [n0, n1), into the team's buffers in turn: of all of them under the sample's scales (the
     // first is in x already), or, EXACT, of those with a value beyond its bound under scales that hold every finite value in them.
-    auto convert_tiles = [&](auto exact_tag, auto full_tag, int n0, int n1) {
-        constexpr bool EXACT = decltype(exact_tag)::value, FULL = decltype(full_tag)::value;
-        float scale[8];
+    auto convert_tiles = [&](auto exact_tag, auto form, int n0, int n1) {
+        constexpr bool EXACT = decltype(exact_tag)::value;
+        constexpr int ROWS = decltype(form)::value == kDgFour ? 4 : 8;
+        float scale[ROWS];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        for (int u = 0; u < ROWS; ++u) {
             const int sampled = dg_exponent(rowmax[row0 + u], kDgHeadroom);
             const int k = EXACT ? min(sampled, dg_exponent(rowtop[row0 + u], 0)) : sampled;
             scale[u] = __uint_as_float((unsigned int)(k + 127) << 23);
@@ -353,7 +365,7 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
             return t;
         };
         int v = EXACT ? next_beyond(team) : 0;
-        if (EXACT && v < end) fetch(full_tag, n0 + v, 0);
+        if (EXACT && v < end) fetch(form, n0 + v, 0);
         for (int chunk = 0; v < end;) {
             const int buffer = team * TB + (int)(done_tiles % TB);
             // the MMAs on what this buffer held before are complete
@@ -361,31 +373,30 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
             const uint32_t block = tiles_u32 + (uint32_t)(buffer * S::kTileBytes + chunk * S::kChunkBytes + row0 * 128);
             float most = 0.0f;
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (FULL || ((live >> u) & 1u)) {
-                    float f[4] = {__uint_as_float(x[u].x), __uint_as_float(x[u].y), __uint_as_float(x[u].z), __uint_as_float(x[u].w)};
+            for (int u = 0; u < ROWS; ++u) {
+                float f[4] = {__uint_as_float(x[u].x), __uint_as_float(x[u].y), __uint_as_float(x[u].z), __uint_as_float(x[u].w)};
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) f[i] *= scale[u];
-                    if constexpr (!EXACT) most = dg_max_abs(dg_max_abs(most, f[0], f[1]), f[2], f[3]);
-                    // signed digits: carries by an addition, then the lower three bytes without their bias
-                    unsigned int d[4];
+                for (int i = 0; i < 4; ++i) f[i] *= scale[u];
+                if constexpr (!EXACT) most = dg_max_abs(dg_max_abs(most, f[0], f[1]), f[2], f[3]);
+                // signed digits: carries by an addition, then the lower three bytes without their bias
+                unsigned int d[4];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) d[i] = (unsigned int)__float2int_rn(f[i]) + 0x00808080u;
-                    // 4 x 4 bytes turned: word s = digit s of the four elements
-                    const unsigned int t0 = __byte_perm(d[0], d[1], 0x5140), t1 = __byte_perm(d[0], d[1], 0x7362);
-                    const unsigned int t2 = __byte_perm(d[2], d[3], 0x5140), t3 = __byte_perm(d[2], d[3], 0x7362);
-                    const uint32_t dst = block + (uint32_t)(u * 128) + (uint32_t)((lane * 4) ^ (u << 4));
-                    dg_st<0>(dst, __byte_perm(t1, t3, 0x7632));
-                    dg_st<KP * 128>(dst, __byte_perm(t1, t3, 0x5410) ^ 0x80808080u);
-                    dg_st<2 * KP * 128>(dst, __byte_perm(t0, t2, 0x7632) ^ 0x80808080u);
-                    dg_st<3 * KP * 128>(dst, __byte_perm(t0, t2, 0x5410) ^ 0x80808080u);
-                }
+                for (int i = 0; i < 4; ++i) d[i] = (unsigned int)__float2int_rn(f[i]) + 0x00808080u;
+                // 4 x 4 bytes turned: word s = digit s of the four elements
+                const unsigned int t0 = __byte_perm(d[0], d[1], 0x5140), t1 = __byte_perm(d[0], d[1], 0x7362);
+                const unsigned int t2 = __byte_perm(d[2], d[3], 0x5140), t3 = __byte_perm(d[2], d[3], 0x7362);
+                const uint32_t dst = block + (uint32_t)(u * 128) + (uint32_t)((lane * 4) ^ (u << 4));
+                dg_st<0>(dst, __byte_perm(t1, t3, 0x7632));
+                dg_st<KP * 128>(dst, __byte_perm(t1, t3, 0x5410) ^ 0x80808080u);
+                dg_st<2 * KP * 128>(dst, __byte_perm(t0, t2, 0x7632) ^ 0x80808080u);
+                dg_st<3 * KP * 128>(dst, __byte_perm(t0, t2, 0x5410) ^ 0x80808080u);
+            }
             if constexpr (!EXACT) {
                 if (__builtin_expect(__any_sync(0xFFFFFFFFu, !(most <= 1073741824.0f)), 0)) {
                     // beyond the bound (or not finite): the tile is left out, and comes again under other scales
 #pragma unroll
-                    for (int u = 0; u < 8; ++u)
-                        if (FULL || ((live >> u) & 1u)) note(u, x[u], rowtop, 1);
+                    for (int u = 0; u < ROWS; ++u)
+                        if ((live >> u) & 1u) note(u, x[u], rowtop, 1);
                     if (lane == 0) {
                         const int t = tile_at(v);
                         atomicOr(&beyond_map[t >> 5], 1u << (t & 31));
@@ -402,7 +413,7 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
                 chunk = 0;
                 v = EXACT ? next_beyond(v + TEAMS) : v + 1;
             }
-            if (v < end) fetch(full_tag, n0 + tile_at(v), chunk);
+            if (v < end) fetch(form, n0 + tile_at(v), chunk);
         }
     };
     // MMAs of `total` tiles in the order they come, by lane 0 of the issuing warp; back when all are complete (or a wait gave
@@ -598,8 +609,10 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
     // (every thread takes the same turns: the conditions are read behind a barrier)
     auto convert_and_issue = [&](auto exact_tag, int n0, int n1, int total) {
         if (warp < W) {
-            if (!decltype(exact_tag)::value && live == 0xFFu) convert_tiles(std::false_type(), std::true_type(), n0, n1);
-            else convert_tiles(exact_tag, std::false_type(), n0, n1);
+            if (decltype(exact_tag)::value) convert_tiles(exact_tag, DigitsForm<kDgSome>(), n0, n1);
+            else if (live == 0xFFu) convert_tiles(std::false_type(), DigitsForm<kDgAll>(), n0, n1);
+            else if (live < 16u) convert_tiles(std::false_type(), DigitsForm<kDgFour>(), n0, n1);
+            else convert_tiles(std::false_type(), DigitsForm<kDgSome>(), n0, n1);
         } else {
             issue_tiles(total);
         }
