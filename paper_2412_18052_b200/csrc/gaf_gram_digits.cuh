@@ -183,6 +183,28 @@ __device__ __forceinline__ int dg_exponent(unsigned int max_bits, int headroom) 
     return max_bits == 0u ? 126 : min(30 - e - headroom, 126);
 }
 
+// What the 32 lanes' pieces v of gradient r hold: the largest finite magnitude, a NaN, an infinity.  (Called where little else goes on; inlined at
+// every call it is half of the kernel's code.)
+__device__ __noinline__ void dg_note(uint4 v, int r, unsigned int *top, unsigned long long *nan_rows, unsigned long long *inf_rows) {
+    const unsigned int m[4] = {v.x & 0x7FFFFFFFu, v.y & 0x7FFFFFFFu, v.z & 0x7FFFFFFFu, v.w & 0x7FFFFFFFu};
+    unsigned int finite = 0u;
+    bool nan = false, inf = false;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        finite = m[i] < 0x7F800000u ? max(finite, m[i]) : finite;
+        nan |= m[i] > 0x7F800000u;
+        inf |= m[i] == 0x7F800000u;
+    }
+    finite = __reduce_max_sync(0xFFFFFFFFu, finite);
+    nan = __any_sync(0xFFFFFFFFu, nan);
+    inf = __any_sync(0xFFFFFFFFu, inf);
+    if ((threadIdx.x & 31) == 0) {
+        if (nan) atomicOr(nan_rows, 1ull << r);
+        if (inf) atomicOr(inf_rows, 1ull << r);
+        atomicMax(&top[r], finite);
+    }
+}
+
 template <int KP>
 __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kernel(const __grid_constant__ GramDigitsArgs a) {
     using S = DigitsShape<KP>;
@@ -242,14 +264,6 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
     // this warp's eight gradients (absent ones: never read)
     const int team = warp / TEAM, row0 = (warp - team * TEAM) * 8;
     auto row = [&](int u) { return reinterpret_cast<const unsigned char *>(a.g[row0 + u]); };
-    auto finite_max = [&](const uint4 &x) {
-        unsigned int m = 0u;
-        const unsigned int v[4] = {x.x & 0x7FFFFFFFu, x.y & 0x7FFFFFFFu, x.z & 0x7FFFFFFFu, x.w & 0x7FFFFFFFu};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) m = v[i] < 0x7F800000u ? max(m, v[i]) : m;
-        return m;
-    };
-
     // The team takes its tiles of a period [n0, n1) (n0 a multiple of the teams) in ascending order, but for one that changes places
     // with its first: the first tiles of all teams, from which the scales are taken, are spread over the CTA's share, one in every
     // TEAMS-th part of it at an uneven place (equal distances fall in step with rows of 2^n elements), the same in all CTAs: places
@@ -285,18 +299,6 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
             for (int u = 0; u < ROWS; ++u) x[u] = inside ? x[u] : make_uint4(0u, 0u, 0u, 0u);
         }
     };
-    // What v holds of the warp's gradient u, 32 pieces of it: the largest finite magnitude, a NaN, an infinity.
-    auto note = [&](int u, const uint4 &v, unsigned int *top, int when) {
-        const unsigned int m[4] = {v.x & 0x7FFFFFFFu, v.y & 0x7FFFFFFFu, v.z & 0x7FFFFFFFu, v.w & 0x7FFFFFFFu};
-        const unsigned int finite = __reduce_max_sync(0xFFFFFFFFu, finite_max(v));
-        const bool nan = __any_sync(0xFFFFFFFFu, max(max(m[0], m[1]), max(m[2], m[3])) > 0x7F800000u);
-        const bool inf = __any_sync(0xFFFFFFFFu, m[0] == 0x7F800000u || m[1] == 0x7F800000u || m[2] == 0x7F800000u || m[3] == 0x7F800000u);
-        if (lane == 0) {
-            if (nan) atomicOr(&nan_rows[when], 1ull << (row0 + u));
-            if (inf) atomicOr(&inf_rows[when], 1ull << (row0 + u));
-            atomicMax(&top[row0 + u], finite);
-        }
-    };
     // The same of all that x holds, for the sample.
     auto note_all = [&]() {
         unsigned int most[8], mine = 0u;
@@ -311,7 +313,7 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
         } else {
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-                if ((live >> u) & 1u) note(u, x[u], rowmax, 0);
+                if ((live >> u) & 1u) dg_note(x[u], row0 + u, rowmax, &nan_rows[0], &inf_rows[0]);
         }
     };
     // The period's scales come from the first tiles of its teams, and for a gradient that has nothing but zeros there, from single pieces of
@@ -336,7 +338,7 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
             const int at = (int)((unsigned int)count * ((unsigned int)lane * 4096u + place) / (32u * 4096u));
             const int64_t q = min(quad_of(n0 + team + at * TEAMS) + (int)((place + (unsigned int)lane * 11u) % (CH * 32u)), n_quads - 1);
             for (int u = 0; u < 8; ++u)
-                if ((dark >> u) & 1u) note(u, ld16_policy(row(u) + q * 16, policy), rowmax, 0);
+                if ((dark >> u) & 1u) dg_note(ld16_policy(row(u) + q * 16, policy), row0 + u, rowmax, &nan_rows[0], &inf_rows[0]);
         }
         __syncthreads();
     };
@@ -396,7 +398,7 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
                     // beyond the bound (or not finite): the tile is left out, and comes again under other scales
 #pragma unroll
                     for (int u = 0; u < ROWS; ++u)
-                        if ((live >> u) & 1u) note(u, x[u], rowtop, 1);
+                        if ((live >> u) & 1u) dg_note(x[u], row0 + u, rowtop, &nan_rows[1], &inf_rows[1]);
                     if (lane == 0) {
                         const int t = tile_at(v);
                         atomicOr(&beyond_map[t >> 5], 1u << (t & 31));
