@@ -35,8 +35,12 @@
  *     take from 7 gradients on: binary32 accumulators over at most 512 products);
  *     the Gram sums of up to 4 binary32 gradients are taken in binary64
  *     throughout, where every product is exact, and those of more than 8 (up to
- *     16 from 2^20 elements on, up to 24 from 327680 on) as exact integers of
- *     values brought to 31-bit fixed point under a power of two of each gradient.  Sums are carried in binary64
+ *     16 from 2^20 elements on, up to 24 from 327680 on; one from 2^20 on) as exact integers of
+ *     values brought to fixed point: each off, absolutely, by at most 2^-25 of the
+ *     largest magnitude in a sample of its gradient (one sample for each SM's
+ *     share), in the tiles that hold values beyond 2^5 of that by 2^-25 of it or
+ *     2^-30 of the largest of them, and by 2^-127 in any case; elements much
+ *     smaller count as zero.  Sums are carried in binary64
  *     from the thread level up and reduced in a fixed order, so results are
  *     bitwise reproducible on the same GPU model.  The scalar arithmetic of
  *     Eq. 4 and the comparison with tau are binary64.

@@ -6,9 +6,12 @@
 // matrix, row s KP + i = digit s of gradient i (KP = K rounded up to 8, 16 at least), so that its product with itself
 // (tcgen05.mma.kind::i8, 8-bit x 8-bit -> 32-bit integers) holds every product of digits of every pair.  Integer sums
 // are exact and do not depend on their order, up to 2^17 products a sum; they are put together in 64-bit integers and
-// binary64 at the end.  What is rounded at all is the value to fixed point: half a unit of 2^-k, about 2^-23 of the
-// gradient's root mean square, at random over the vector: less than the chains of 64 rounded products of a kernel on the
-// binary32 pipes left (24 x 3 M: 2e-10 of the norms' product against 4e-9).
+// binary64 at the end.  What is rounded at all is the value to fixed point, by half a unit of 2^-k at most: a fixed part of the largest
+// magnitudes, so that elements far below them lose bits, the smallest all.  For normal values half a unit is about 2^-23 of their
+// root mean square.  Largest error of all pairs, of the norms' product, against the chains of 64 rounded products of a kernel on the binary32
+// pipes (24 x 3 M): normal values 1e-10 / 3e-9, Student's t of 3 degrees 3e-10 / 7e-9, lognormal of sigma 2 2e-9 / 8e-8, 200 tensors of
+// lognormal scales 7e-12 / 5e-9.  (A gradient with one element of 1 and all others 2^-26, against one of ones: 4e-6 of the norms' product, where
+// chains leave 3e-9.)
 //
 // The power of two.  A CTA takes its share in periods of at most 1023 x 128 elements.  At the start of each it looks at the first tile of
 // each of its teams and allows for elements 2^5 times as large: half a unit is at most 2^-25 of the largest magnitude that the CTA sampled of
@@ -36,15 +39,19 @@
 // among themselves (what is missing of the 4 KP x 4 KP products then is the mirror image of something present).
 // Rows of absent gradients, and the rows of the 128 beyond 4 KP, hold whatever the memory holds: their sums are not read.
 //
-// Bound by the conversion up to 9 gradients (0.61 of the copy rate), by HBM in short runs from there on (16 gradients 0.91, 24 and more 0.88 to 0.93; 24 x 3 M 0.77,
-// with 8 us of launch, first tiles and last sums), by the power cap in long ones (24 x 3 M: tensor pipe 33 % busy, issue slots 52 %).  All pairs, D = 11.2 M, against
-// the kernel on the binary32 pipes (bound by these and by shared memory): 9 / 15 / 16 / 24 / 32 / 40 / 64 gradients 143 / 141 / 140 / 306 / 459 / 901 / 1905 us,
-// now 102 / 118 / 121 / 183 / 238 / 320 / 501; a second of calls on end 142 / 143 / 145 / 306 / 459 / 901 / 1947, now 112 / 135 / 138 / 211 / 277 / 369 / 581 (the SM
-// clock falls to 1.1 to 1.5 GHz).  What decided the shape: loads under a branch, or in a ring of single registers, wait for one another
-// (32 gradients: 900 us; a warp with absent gradients loads under predicates and
-// converts zeros for them, without a branch: 15 / 31 x 8.2 M 108 / 220 us with branches, 100 / 198 so, binary32 pipes 105 / 338); eight gradients for the whole kernel per warp, 20 warps and more (300 -> 265); the MMAs issued by a converged warp with
-// an elected lane (their operands are scalars then; 16 gradients 147 -> 118 with two chunks a product).  Products of 64 rows, which waste less, cost the
-// same time and no less power.  The mean written meanwhile under the pattern of a sample: 16 x 11.2 M 199 us, 179 with a pass of its own.
+// Bound by HBM in short runs (of the copy rate: 16 gradients 0.91, 24 to 40 0.86 to 0.92, 64 0.88; up to 12, whose rows are padded to 16, 0.61 to 0.76; 24 x 3 M 0.77,
+// with 8 us of launch, first tiles and last sums), by the power cap in long ones (24 x 3 M: tensor pipe 33 % busy, issue slots 52 %).  All
+// pairs, D = 11.2 M, against the kernel on the binary32 pipes (bound by these and by shared memory), us:
+//     gradients                    9    15    16    24    32    40    64
+//     short runs                 102   118   121   183   238   320   501    (binary32 pipes 143  141  140  306  459  901  1905)
+//     a second of calls on end   112   135   138   211   277   369   581    (142  143  145  306  459  901  1947; the SM clock falls to 1.1 to 1.5 GHz)
+// What decided the shape: loads under a branch, or in a ring of single registers, wait for one another (32 gradients: 900 us; a warp with
+// absent gradients loads under predicates and converts zeros for them, without a branch: 15 / 31 x 8.2 M 108 / 220 us with branches,
+// 100 / 198 so, binary32 pipes 105 / 338); eight gradients for the whole kernel per warp, 20 warps and more (300 -> 265); the MMAs issued by a
+// converged warp with an elected lane (their operands are scalars then; 16 gradients 147 -> 118 with two chunks a product); shared memory of
+// less than 196 KB in all, beyond which the first-level cache that loads in flight need shrinks (64 x 4.1 M 230 -> 245).  Products of 64 rows,
+// which waste less, cost the same time and no less power.  The mean written meanwhile under the pattern of a sample: 16 x 11.2 M 199 us, 179 with a
+// pass of its own.
 #pragma once
 
 #include "gaf_device.cuh"

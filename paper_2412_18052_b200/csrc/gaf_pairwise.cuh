@@ -4,7 +4,7 @@
 // What the Gram kernels for more than 8 gradients share (gaf_gram_digits.cuh and gaf_gram_tc.cuh on tensor cores,
 // gaf_gram_mma.cuh, gaf_gram_panel.cuh on CUDA cores): the K x K matrix cut into 8 x 8 tiles of pairs, per-CTA
 // binary64 partial sums in a [tile pair][slice][64] layout, and the finishing kernel that totals
-// the slices in a fixed order and whose last CTA derives the distances, or walks Algorithm 1 on the matrix.
+// the slices in a fixed order and derives the distances, or whose last CTA walks Algorithm 1 on the matrix.
 #pragma once
 
 #include "gaf_device.cuh"
