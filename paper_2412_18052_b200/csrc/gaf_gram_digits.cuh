@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(DigitsShape<KP>::kThreads, 1) gram_digits_kern
             for (int u = 0; u < ROWS; ++u) x[u] = inside ? x[u] : make_uint4(0u, 0u, 0u, 0u);
         }
     };
-    // The same of all that x holds, for the sample.
+    // dg_note of all that x holds, for the sample: one operation a gradient where everything is finite.
     auto note_all = [&]() {
         unsigned int most[8], mine = 0u;
 #pragma unroll
